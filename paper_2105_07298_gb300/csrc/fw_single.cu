@@ -11,8 +11,9 @@
 //                           round's TB values of k.
 // Relaxation rule: Algorithm 1 with a strict "<" (see apsp_fw.h).
 //
-// Rounds overlap: phase 4 of round r first updates row and column r+1, then
-// the rest of the matrix while K1/K2 of round r+1 run on a second stream.
+// Rounds overlap: what round r+1 waits for (phase 4 of round r on row and
+// column r+1, then K1 and K2 of round r+1) runs on a second stream of higher
+// priority beside the rest of round r's phase 4.
 //
 // Differences from the Pascal design of §3.2 (one output per thread, TB <= 32):
 //  * K3 runs two CTAs per 128 x 128 block, three per SM, an 8 x 4 register
@@ -27,8 +28,8 @@
 //    (lane-parallel for dense 8-row groups, warp-cooperative otherwise).
 //    Either way P is exactly that of the sequential loop (ascending k, strict
 //    "<" keeps the first k reaching the final minimum).
-//  * K1 keeps only minima in its step loop and recovers P afterwards from a
-//    per-step history; K2 keeps each row/column line in registers.
+//  * K1 is one cluster of eight CTAs, K2 keeps each row/column line in
+//    registers; both keep only minima per step and settle P afterwards.
 //  * Nothing reads P: K1/K2/K3 write P only where D strictly improved.
 #include <stdint.h>
 
@@ -41,179 +42,492 @@
 namespace apsp {
 
 // --------------------------------------------------------------------------
-// K0: P := -1 over an n x n region with leading dimension ld.
+// K0: P := -1 over an n x n region with leading dimension ld, but for its
+// first skip x skip block.
 // --------------------------------------------------------------------------
-__global__ void fw_path_init(int32_t *__restrict__ P, int64_t n, int64_t ld) {
+__global__ void fw_path_init(int32_t *__restrict__ P, int64_t n, int64_t ld, int64_t skip) {
   const int64_t total = n * n;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
        e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = e / n, j = e - i * n;
-    P[i * ld + j] = -1;
+    if (i >= skip || j >= skip) P[i * ld + j] = -1;
   }
 }
 
-__global__ void __launch_bounds__(k2::THREADS, 2) fw_phase2_lines_f32(float *__restrict__ D, int64_t ld,
-                                                                  int32_t *__restrict__ P, int n, int r,
-                                                                  int R, Panels pan) {
-  using namespace k2;
+// Alignment of the caller's matrices: every row of D (of P) starts on a
+// 16-byte boundary.
+constexpr int kVecD = 1, kVecP = 2;
+
+// The closed diagonal block of a round in K2's operand layouts (K1 writes them).
+struct DiagOps {
+  unsigned long long *A, *B;
+};
+
+// __byte_perm selector that replaces byte c of its first operand with byte 0 of its second.
+__device__ __forceinline__ constexpr unsigned byte_sel(int c) {
+  return 0x3210 ^ ((0x3210 & (0xF << (4 * c))) ^ (4 << (4 * c)));
+}
+
+// --------------------------------------------------------------------------
+// K1 (FP32): phase 1, Algorithm 1 on the diagonal block (r,r), by one cluster
+// of eight CTAs of four warps.  A warp owns the four rows 4 kq .. 4 kq + 3,
+// lane l their columns 4l..4l+3 in registers; the four steps k = 4 kq + s are
+// taken together.  The warp owning rows kq brings each to its value at its own
+// step and publishes them k-paired in its CTA's history; the CTAs form a ring
+// and pass each published quad on (16-byte st.async, counted by the receiver's
+// barrier of that quad), so no SM sends more than its share.  Every warp then
+// relaxes its rows through the four steps: the pivots of a row come by
+// shuffle, are brought to their steps against the quad's own 4 x 4 entries,
+// and two packed adds and two three-input mins per element do the rest.
+//   hist[kp][j] = (row 2 kp at step 2 kp, row 2 kp + 1 at step 2 kp + 1)
+//   hcol[i][kp] = (column 2 kp of row i at its step, column 2 kp + 1 likewise)
+// Step k never changes row or column k (D[k][k] = 0), so these are the values
+// the sequential loop uses.  Only minima are kept in the loop; with a path
+// matrix the element is compared once per 16 steps (strictly lower: the last
+// improvement lies there), and afterwards the first k of those 16 whose
+// candidate from the histories equals the final value is the path entry - the
+// k of the sequential loop's last strict improvement.
+//
+// What bounds it: the serial chain of 32 quads (shuffles, a few dependent
+// adds and mins, publish, barrier), not arithmetic.  One CTA that keeps the
+// block in the registers of 256 threads is bound by its one SM's pipes
+// (2.1e6 relaxations: 12 us at the measured pair rate) and a barrier per step.
+// Measured per launch between events, n = 1024: 21 us, 25 us with a path
+// matrix (such a one-CTA kernel: 39 and 64 us); 0.3 us a quad and about 8 us
+// of launch, load and store.  Publishing to all seven peers at once, by
+// st.async or by bulk copies, measured 29 and 34 us: the sends hold up the
+// owner SM's own shared-memory accesses.  Two rows a warp: 23 us.
+//
+// Also writes the final block as K2's operands: diagA[kp][i] = (D[i][2kp],
+// D[i][2kp+1]), diagB[kp][j] = (D[2kp][j], D[2kp+1][j]), +inf past n.
+// --------------------------------------------------------------------------
+namespace k1 {
+constexpr int T = mp32::T, CTAS = 8, WARPS = 4, ROWS = T / CTAS, PAIRS = T / 2, QUADS = T / 4;
+struct Smem {
+  unsigned long long hist[PAIRS][T];
+  unsigned long long hcol[ROWS][PAIRS];
+  uint64_t bar[QUADS];
+};
+}  // namespace k1
+
+template <bool PATH>
+__global__ void __cluster_dims__(k1::CTAS, 1, 1) __launch_bounds__(32 * k1::WARPS, 1)
+    fw_phase1_diag_f32(float *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r, int vec,
+                       int first, DiagOps ops) {
+  using namespace k1;
+  using mp32::pack2;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
+  const int base = r * T, m = min(T, n - base), nquad = (m + 3) / 4;
+  const int cta = (int)cluster_cta_rank(), tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int own = cta * WARPS + w;  // this warp's row quad
+  const int i0 = 4 * own, j0 = 4 * lane;
+  const float INF = inf<float>();
+  // A quad another CTA owns completes its barrier here by its 2 KiB; the
+  // quads owned here use the CTA barrier instead.
+  if (tid < QUADS) {
+    mbar_init(&sm.bar[tid], 1);
+    fence_mbar_init();
+    if (tid / WARPS != cta) mbar_expect_tx(&sm.bar[tid], 4 * T * 4);
+  }
+  grid_dep_wait();
+  float d[4][4];
+#pragma unroll
+  for (int rr = 0; rr < 4; ++rr) {
+    const float *row = D + (int64_t)(base + i0 + rr) * ld + base;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) d[rr][c] = INF;
+    if (i0 + rr < m) {
+      if ((vec & kVecD) && j0 + 3 < m) {
+        const float4 t = *reinterpret_cast<const float4 *>(row + j0);
+        d[rr][0] = t.x, d[rr][1] = t.y, d[rr][2] = t.z, d[rr][3] = t.w;
+      } else {
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          if (j0 + c < m) d[rr][c] = row[j0 + c];
+      }
+    }
+  }
+  cluster_sync();  // every barrier of the cluster is set up before anyone publishes
+  float prev[4][4];   // the elements at the start of the current 16 steps (without P: the input)
+  unsigned chunk[4];  // PATH: byte c: last group of 16 steps that lowered element c, 0xFF none
+#pragma unroll
+  for (int rr = 0; rr < 4; ++rr) {
+    chunk[rr] = 0xFFFFFFFFu;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) prev[rr][c] = d[rr][c];
+  }
+  bool ok = true;
+  const unsigned next = (unsigned)(cta + 1) % CTAS;
+  const uint32_t next_base = cluster_map(smem_addr(smem_raw), next) - smem_addr(smem_raw);
+#pragma unroll 1
+  for (int kq = 0; kq < nquad; ++kq) {
+    const int g = kq / WARPS;  // the owning CTA
+    // The rows' values at the quad's columns, before its steps.
+    float x[4][4];
+#pragma unroll
+    for (int rr = 0; rr < 4; ++rr)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) x[rr][c] = __shfl_sync(kFullMask, d[rr][c], kq);
+    // e: row 4 kq + s at its step, at the quad's column t > s.
+    float e01, e02, e03, e12, e13, e23;
+    unsigned long long ha[4], hb[4];  // this lane's columns: rows (0, 1) and (2, 3) of the quad
+    auto pivots = [&](float (&p)[4]) {  // a row's pivots brought to their steps
+      p[1] = fminf(p[1], __fadd_rn(p[0], e01));
+      p[2] = mp32::min3f(p[2], __fadd_rn(p[0], e02), __fadd_rn(p[1], e12));
+      p[3] = fminf(mp32::min3f(p[3], __fadd_rn(p[0], e03), __fadd_rn(p[1], e13)), __fadd_rn(p[2], e23));
+    };
+    const bool mine = kq == own;
+    if (mine) {  // warp-uniform
+      e01 = x[0][1], e02 = x[0][2], e03 = x[0][3];
+      e12 = fminf(x[1][2], __fadd_rn(x[1][0], e02));
+      e13 = fminf(x[1][3], __fadd_rn(x[1][0], e03));
+      const float y21 = fminf(x[2][1], __fadd_rn(x[2][0], e01));
+      e23 = mp32::min3f(x[2][3], __fadd_rn(x[2][0], e03), __fadd_rn(y21, e13));
+#pragma unroll
+      for (int rr = 0; rr < 4; ++rr) pivots(x[rr]);
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const float r0 = d[0][c], r1 = fminf(d[1][c], __fadd_rn(x[1][0], r0));
+        const float r2 = mp32::min3f(d[2][c], __fadd_rn(x[2][0], r0), __fadd_rn(x[2][1], r1));
+        const float r3 = fminf(mp32::min3f(d[3][c], __fadd_rn(x[3][0], r0), __fadd_rn(x[3][1], r1)),
+                               __fadd_rn(x[3][2], r2));
+        ha[c] = pack2(r0, r1);
+        hb[c] = pack2(r2, r3);
+      }
+#pragma unroll
+      for (int c = 0; c < 4; c += 2) {
+        *reinterpret_cast<ulonglong2 *>(&sm.hist[2 * kq][j0 + c]) = make_ulonglong2(ha[c], ha[c + 1]);
+        *reinterpret_cast<ulonglong2 *>(&sm.hist[2 * kq + 1][j0 + c]) = make_ulonglong2(hb[c], hb[c + 1]);
+      }
+    }
+    if (cta == g) __syncthreads();
+    else if (ok) ok = mbar_spin(&sm.bar[kq], 0);
+    if (!mine) {
+#pragma unroll
+      for (int c = 0; c < 4; c += 2) {
+        const ulonglong2 ta = *reinterpret_cast<const ulonglong2 *>(&sm.hist[2 * kq][j0 + c]);
+        const ulonglong2 tb = *reinterpret_cast<const ulonglong2 *>(&sm.hist[2 * kq + 1][j0 + c]);
+        ha[c] = ta.x, ha[c + 1] = ta.y, hb[c] = tb.x, hb[c + 1] = tb.y;
+      }
+      const ulonglong2 q0 = *reinterpret_cast<const ulonglong2 *>(&sm.hist[2 * kq][4 * kq]);
+      const ulonglong2 q1 = *reinterpret_cast<const ulonglong2 *>(&sm.hist[2 * kq][4 * kq + 2]);
+      e01 = __uint_as_float((unsigned)q0.y);
+      e02 = __uint_as_float((unsigned)q1.x);
+      e03 = __uint_as_float((unsigned)q1.y);
+      e12 = __uint_as_float((unsigned)(q1.x >> 32));
+      e13 = __uint_as_float((unsigned)(q1.y >> 32));
+      e23 = __uint_as_float((unsigned)sm.hist[2 * kq + 1][4 * kq + 3]);
+#pragma unroll
+      for (int rr = 0; rr < 4; ++rr) pivots(x[rr]);
+    }
+    if (w == kq % WARPS && next != (unsigned)g) {  // pass the quad on to the next CTA of the ring
+      const uint32_t to = next_base + smem_addr(&sm.hist[2 * kq][j0]), bar = next_base + smem_addr(&sm.bar[kq]);
+      st_async16(to, ha[0], ha[1], bar);
+      st_async16(to + 16, ha[2], ha[3], bar);
+      st_async16(to + T * 8, hb[0], hb[1], bar);
+      st_async16(to + T * 8 + 16, hb[2], hb[3], bar);
+    }
+#pragma unroll
+    for (int rr = 0; rr < 4; ++rr) {
+      const unsigned long long xa = pack2(x[rr][0], x[rr][1]), xb = pack2(x[rr][2], x[rr][3]);
+      if (PATH && lane == 0)
+        *reinterpret_cast<ulonglong2 *>(&sm.hcol[4 * w + rr][2 * kq]) = make_ulonglong2(xa, xb);
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        mp32::relax2(d[rr][c], xa, ha[c]);
+        mp32::relax2(d[rr][c], xb, hb[c]);
+      }
+    }
+    if (PATH && ((kq & 3) == 3 || kq + 1 == nquad)) {
+#pragma unroll
+      for (int rr = 0; rr < 4; ++rr)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          if (d[rr][c] < prev[rr][c]) chunk[rr] = __byte_perm(chunk[rr], (unsigned)(kq >> 2), byte_sel(c));
+          prev[rr][c] = d[rr][c];
+        }
+    }
+  }
+  grid_dep_launch();
+  __syncwarp();
+  if (!ok) report_wait_timeout();  // D and P stay as they are
+  if (ok) {
+    if (ops.A) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int c = 0; c < 4; c += 2)
+          *reinterpret_cast<ulonglong2 *>(&ops.B[(int64_t)(2 * own + h) * T + j0 + c]) =
+              make_ulonglong2(pack2(d[2 * h][c], d[2 * h + 1][c]), pack2(d[2 * h][c + 1], d[2 * h + 1][c + 1]));
+#pragma unroll
+      for (int c = 0; c < 4; c += 2)
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          *reinterpret_cast<ulonglong2 *>(&ops.A[(int64_t)(2 * lane + c / 2) * T + i0 + 2 * h]) =
+              make_ulonglong2(pack2(d[2 * h][c], d[2 * h][c + 1]), pack2(d[2 * h + 1][c], d[2 * h + 1][c + 1]));
+    }
+#pragma unroll
+    for (int rr = 0; rr < 4; ++rr) {
+      const int i = i0 + rr;
+      if (i >= m) continue;
+      const int64_t row = (int64_t)(base + i) * ld + base;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        if (j0 + c >= m) continue;
+        const unsigned g = (chunk[rr] >> (8 * c)) & 0xFFu;
+        if (PATH ? g != 0xFFu : d[rr][c] < prev[rr][c]) D[row + j0 + c] = d[rr][c];
+        if (!PATH) continue;
+        int k = -1;
+        if (g != 0xFFu) {
+#pragma unroll
+          for (int q = 7; q >= 0; --q) {
+            const float2 t = mp32::sum2(sm.hcol[4 * w + rr][8 * g + q], sm.hist[8 * g + q][j0 + c]);
+            k = t.y == d[rr][c] ? 16 * (int)g + 2 * q + 1 : k;
+            k = t.x == d[rr][c] ? 16 * (int)g + 2 * q : k;
+          }
+        }
+        // the first round's block is not initialised: every entry is written
+        if (first || k >= 0) P[row + j0 + c] = k >= 0 ? base + k : -1;
+      }
+    }
+  }
+  cluster_sync();  // no CTA leaves while another may still write its history
+}
+
+// --------------------------------------------------------------------------
+// K2 (FP32): phases 2 and 3.  Blocks b < R-1 of the grid cover row block
+// (r, J), the others column block (I, r); PARTS CTAs share a block.  Within a
+// row block every column evolves on its own, within a column block every row:
+//   row block, column j:  own[i][j] = min(own[i][j], diag[i][k] + own[k][j])
+//   column block, row i:  own[i][j] = min(own[i][j], own[i][k] + diag[k][j])
+// for k ascending over the round's vertices (the diagonal block is final
+// after K1).  A warp keeps LINES such lines in registers, lane l holding
+// positions 2l, 2l+1, 2l+64, 2l+65 of each.  Steps 2 kp and 2 kp + 1 are taken
+// together: the two pivot values come by shuffle, the second is brought to its
+// step with one add and min, and each position takes both candidates with one
+// packed add against the k-paired diagonal block in shared memory (one bulk
+// copy of K1's operands) and one three-input min.  No barrier in the loop.
+// Paths as in K1: one comparison per 16 steps in the loop, the k inside the
+// last improving 16 settled afterwards from the pivot history in shared
+// memory.  The finished blocks are also written, padded with +inf to T x T,
+// in the layouts phase 4 reads this round:
+//   row block (r,J):    Bpan[J][j/64][kp][j%64] = (own[2kp][j], own[2kp+1][j]),
+//                       Bt[J][j][k] = own[k][j]
+//   column block (I,r): Apan[I][kp][i] = (own[i][2kp], own[i][2kp+1]),
+//                       Acp[I][i][k] = own[i][k]
+// Bound: issue and the shuffle-add-min chain of a step pair (latency) where a
+// launch has few CTAs, the FP32 pipes where it fills the chip.  Measured per
+// launch, n = 1024: 10.5 us, 13.7 us with a path matrix (a compare and two
+// selects per relaxation, one step at a time, the block read element by
+// element: 29.5 us); with four lines a warp instead of two 13.5 and 20 us
+// there, since 56 CTAs leave SMs idle.
+// --------------------------------------------------------------------------
+namespace k2s {
+constexpr int T = mp32::T, THREADS = 256, PAIRS = T / 2;
+__host__ __device__ constexpr int parts(int lines) { return T / (THREADS / 32 * lines); }  // CTAs per block
+template <int LINES>
+struct Smem {
+  unsigned long long M[PAIRS][T];  // row block: diagA, column block: diagB
+  unsigned long long hist[PAIRS][THREADS / 32 * LINES];
+  uint64_t bar;
+};
+}  // namespace k2s
+
+template <bool PATH, int LINES>
+__global__ void __launch_bounds__(k2s::THREADS, 2)
+    fw_phase2_lines_f32(float *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r, int R, int vec_in,
+                        DiagOps ops, Panels pan) {
+  using namespace k2s;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  static_assert(LINES == 2 || LINES == 4, "the lines of a position are one 8- or 16-byte access");
+  constexpr int PARTS = parts(LINES), CTA_LINES = T / PARTS;
+  Smem<LINES> &sm = *reinterpret_cast<Smem<LINES> *>(smem_raw);
   const int b = blockIdx.x / PARTS, part = blockIdx.x % PARTS;
   const bool is_row = b < R - 1;
   int other = is_row ? b : b - (R - 1);
   other += (other >= r);
-  lines_load_diag(D, ld, n, r, is_row);
+  const int base_r = r * T, m_r = min(T, n - base_r);
+  const int base_o = other * T, m_o = min(T, n - base_o);
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const float INF = inf<float>();
+  if (tid == 0) {
+    mbar_init(&sm.bar, 1);
+    fence_mbar_init();
+    mbar_expect_tx(&sm.bar, sizeof(sm.M));
+  }
+  grid_dep_wait();
+  if (tid == 0) {
+    fence_proxy_async_global();
+    bulk_g2s(&sm.M[0][0], is_row ? ops.A : ops.B, sizeof(sm.M), &sm.bar);
+  }
+  const int wl = w * LINES, line0 = part * CTA_LINES + wl;
+  // Element (line, pos) of the own block sits at D[g0 + line * sl + pos * sp];
+  // slot q of a lane is position 2 lane + (q & 1) + 64 (q >> 1).
+  const int64_t g0 = is_row ? (int64_t)base_r * ld + base_o : (int64_t)base_o * ld + base_r;
+  const int64_t sl = is_row ? 1 : ld, sp = is_row ? ld : 1;
+  float v[LINES][4];
+#pragma unroll
+  for (int c = 0; c < LINES; ++c)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[c][q] = INF;
+  // row blocks: the LINES lines of a position are one access
+  const bool whole = line0 + LINES <= m_o, vec = (vec_in & kVecD) && whole;
+  const bool vec_out = vec && (!PATH || (vec_in & kVecP));
+  if (is_row && vec) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int pos = 2 * lane + (q & 1) + 64 * (q >> 1);
+      if (pos < m_r) {
+        const float *src = &D[g0 + line0 + pos * sp];
+        if constexpr (LINES == 4) {
+          const float4 t = *reinterpret_cast<const float4 *>(src);
+          v[0][q] = t.x, v[1][q] = t.y, v[2][q] = t.z, v[3][q] = t.w;
+        } else {
+          const float2 t = *reinterpret_cast<const float2 *>(src);
+          v[0][q] = t.x, v[1][q] = t.y;
+        }
+      }
+    }
+  } else {
+#pragma unroll
+    for (int c = 0; c < LINES; ++c)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int line = line0 + c, pos = 2 * lane + (q & 1) + 64 * (q >> 1);
+        if (line < m_o && pos < m_r) v[c][q] = D[g0 + line * sl + pos * sp];
+      }
+  }
+  float prev[LINES][4];   // the lines at the start of the current 16 steps
+  unsigned chunk[LINES];  // byte q: last group of 16 steps that lowered slot q, 0xFF none
+#pragma unroll
+  for (int c = 0; c < LINES; ++c) {
+    chunk[c] = 0xFFFFFFFFu;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) prev[c][q] = v[c][q];
+  }
   __syncthreads();
-  lines_part_f32(D, ld, P, n, r, other, is_row, part, pan);
+  const bool ok = mbar_wait(&sm.bar, 0);
+  if (__syncthreads_or(!ok)) {  // the diagonal block never arrived: leave D, P and the panels as they are
+    if (tid == 0) report_wait_timeout();
+    return;
+  }
+  // Positions 2 kp, 2 kp + 1: slots 2 h, 2 h + 1 of lane kp mod 32, h = kp / 32.
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+#pragma unroll 1
+    for (int g = 0; g < 4; ++g) {
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int src = 8 * g + u, kp = 32 * h + src;
+        const ulonglong2 ma = *reinterpret_cast<const ulonglong2 *>(&sm.M[kp][2 * lane]);
+        const ulonglong2 mb = *reinterpret_cast<const ulonglong2 *>(&sm.M[kp][64 + 2 * lane]);
+        // step 2 kp's diagonal entry for position 2 kp + 1
+        const float e = __uint_as_float((unsigned)sm.M[kp][2 * kp + 1]);
+        unsigned long long xx[LINES];
+#pragma unroll
+        for (int c = 0; c < LINES; ++c) {
+          const float x0 = __shfl_sync(kFullMask, v[c][2 * h], src);
+          const float x1 = fminf(__shfl_sync(kFullMask, v[c][2 * h + 1], src), __fadd_rn(x0, e));
+          xx[c] = mp32::pack2(x0, x1);
+          mp32::relax2(v[c][0], xx[c], ma.x);
+          mp32::relax2(v[c][1], xx[c], ma.y);
+          mp32::relax2(v[c][2], xx[c], mb.x);
+          mp32::relax2(v[c][3], xx[c], mb.y);
+        }
+        if (PATH && lane == 0) {
+#pragma unroll
+          for (int c = 0; c < LINES; c += 2)
+            *reinterpret_cast<ulonglong2 *>(&sm.hist[kp][wl + c]) = make_ulonglong2(xx[c], xx[c + 1]);
+        }
+      }
+#pragma unroll
+      for (int c = 0; c < LINES; ++c)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (PATH) {
+            if (v[c][q] < prev[c][q]) chunk[c] = __byte_perm(chunk[c], (unsigned)(4 * h + g), byte_sel(q));
+            prev[c][q] = v[c][q];
+          }
+    }
+  }
+  grid_dep_launch();
+  __syncwarp();  // lane 0's history writes
+  if (!PATH) {  // which positions improved (prev still holds the input)
+#pragma unroll
+    for (int c = 0; c < LINES; ++c)
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (v[c][q] < prev[c][q]) chunk[c] = __byte_perm(chunk[c], 0u, byte_sel(q));
+  }
+  // The phase-4 panels (padded): position pair hq of a line is k-pair lane + 32 hq.
+  const int64_t blk = other;
+#pragma unroll
+  for (int hq = 0; hq < 2; ++hq) {
+    const int kp = lane + 32 * hq;
+    unsigned long long *dst = is_row ? &pan.Bpan[((blk * 2 + (line0 >> 6)) * (T / 2) + kp) * (T / 2) + (line0 & 63)]
+                                     : &pan.Apan[(blk * (T / 2) + kp) * T + line0];
+    float *rows = is_row ? pan.Bt : pan.Acp;
+#pragma unroll
+    for (int c = 0; c < LINES; c += 2)
+      *reinterpret_cast<ulonglong2 *>(dst + c) = make_ulonglong2(mp32::pack2(v[c][2 * hq], v[c][2 * hq + 1]),
+                                                                 mp32::pack2(v[c + 1][2 * hq], v[c + 1][2 * hq + 1]));
+#pragma unroll
+    for (int c = 0; c < LINES; ++c)
+      *reinterpret_cast<float2 *>(&rows[(blk * T + line0 + c) * T + 2 * kp]) = make_float2(v[c][2 * hq], v[c][2 * hq + 1]);
+  }
+  // D and P where the line improved (such positions lie inside the matrix).
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int pos = 2 * lane + (q & 1) + 64 * (q >> 1);
+    unsigned gq[LINES];
+    bool all = true;  // every line improved at this position
+#pragma unroll
+    for (int c = 0; c < LINES; ++c) {
+      gq[c] = (chunk[c] >> (8 * q)) & 0xFFu;
+      all = all && gq[c] != 0xFFu;
+    }
+    int k[LINES];
+    if (PATH) {
+#pragma unroll
+      for (int c = 0; c < LINES; ++c) {
+        k[c] = 0;
+        if (gq[c] == 0xFFu) continue;
+#pragma unroll
+        for (int u = 7; u >= 0; --u) {
+          const int kp = 8 * (int)gq[c] + u;
+          const float2 t = mp32::sum2(sm.hist[kp][wl + c], sm.M[kp][pos]);
+          k[c] = t.y == v[c][q] ? 2 * kp + 1 : k[c];
+          k[c] = t.x == v[c][q] ? 2 * kp : k[c];
+        }
+      }
+    }
+    const int64_t gp = g0 + line0 * sl + pos * sp;
+    if (is_row && vec_out && all) {
+      if constexpr (LINES == 4) {
+        *reinterpret_cast<float4 *>(&D[gp]) = make_float4(v[0][q], v[1][q], v[2][q], v[3][q]);
+        if (PATH)
+          *reinterpret_cast<int4 *>(&P[gp]) = make_int4(base_r + k[0], base_r + k[1], base_r + k[2], base_r + k[3]);
+      } else {
+        *reinterpret_cast<float2 *>(&D[gp]) = make_float2(v[0][q], v[1][q]);
+        if (PATH) *reinterpret_cast<int2 *>(&P[gp]) = make_int2(base_r + k[0], base_r + k[1]);
+      }
+    } else {
+#pragma unroll
+      for (int c = 0; c < LINES; ++c)
+        if (gq[c] != 0xFFu) {
+          D[gp + c * sl] = v[c][q];
+          if (PATH) P[gp + c * sl] = base_r + k[c];
+        }
+    }
+  }
 }
 
 // --------------------------------------------------------------------------
-// K1 (FP32): phase 1 with the register-resident closure of minplus_f32.cuh.
-// K3 (FP32): phase 4, one 128 x 128 block product per CTA (minplus_f32.cuh).
-// Grid: (R-1)^2 CTAs in row-major (I', J') order over the blocks I, J != r,
+// K3 (FP32): phase 4, two CTAs per 128 x 128 block product.
+// Grid: (R-1)^2 blocks in row-major (I', J') order over the blocks I, J != r,
 // so consecutive CTAs share the column-panel block A and sweep the row panel.
 // --------------------------------------------------------------------------
-// K1 (FP32): Algorithm 1 on the diagonal block, minima only in the step
-// loop, path entries recovered afterwards.  Each thread keeps its 8 x 8
-// elements in registers; at step k the owners of row k and column k publish
-// them into a per-step history in shared memory (k-paired layout:
-// hr[k/2][j] = (row 2kp at its step, row 2kp+1 at its step), hc likewise for
-// columns), one barrier per step.  Step k never changes row or column k
-// (D[k][k] = 0), so the published values are the ones every thread uses.
-// Within the round an element's last strict improvement is the first step
-// whose candidate hc[k][i] + hr[k][j] equals the element's final value, so
-// after the loop each improved element finds that k by scanning its
-// candidate sums from the history (folded 8 k at a time, lowest matching
-// chunk kept, then the first k inside it) - the P of the sequential loop.
-namespace k1 {
-constexpr int T = mp32::T, TM = 8;
-struct Hist {
-  unsigned long long hc[T / 2][T];  // (D[i][2kp], D[i][2kp+1]) as published at steps 2kp, 2kp+1
-  unsigned long long hr[T / 2][T];  // (D[2kp][j], D[2kp+1][j]) likewise
-};
-}  // namespace k1
-
-__global__ void __launch_bounds__(mp32::THREADS)
-    fw_phase1_diag_f32(float *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r) {
-  using namespace k1;
-  using mp32::col_at;
-  using mp32::row_at;
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  Hist &h = *reinterpret_cast<Hist *>(smem_raw);
-  float *hc = reinterpret_cast<float *>(&h.hc[0][0]), *hr = reinterpret_cast<float *>(&h.hr[0][0]);
-  const int base = r * T, m = min(T, n - base);
-  const int ty = mp32::thread_ty(), tx = mp32::thread_tx();
-  const float INF = inf<float>();
-  float d[TM][TM];
-#pragma unroll
-  for (int rr = 0; rr < TM; ++rr)
-#pragma unroll
-    for (int cc = 0; cc < TM; ++cc) {
-      const int i = row_at(rr, ty), j = col_at(cc, tx);
-      d[rr][cc] = (i < m && j < m) ? D[(int64_t)(base + i) * ld + base + j] : INF;
-    }
-  // k = 32 kb + 2 kk + q: row_at / col_at index 2 kb + q of owner kk; k-pair 16 kb + kk.
-#pragma unroll
-  for (int kb = 0; kb < TM / 2; ++kb) {
-#pragma unroll 1
-    for (int kk = 0; kk < 16; ++kk) {
-      const int kp = 16 * kb + kk;
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        if (ty == kk) {
-#pragma unroll
-          for (int cc = 0; cc < TM; ++cc) hr[(kp * T + col_at(cc, tx)) * 2 + q] = d[2 * kb + q][cc];
-        }
-        if (tx == kk) {
-#pragma unroll
-          for (int rr = 0; rr < TM; ++rr) hc[(kp * T + row_at(rr, ty)) * 2 + q] = d[rr][2 * kb + q];
-        }
-        __syncthreads();
-        float a[TM], b[TM];
-#pragma unroll
-        for (int rr = 0; rr < TM; ++rr) a[rr] = hc[(kp * T + row_at(rr, ty)) * 2 + q];
-#pragma unroll
-        for (int cc = 0; cc < TM; ++cc) b[cc] = hr[(kp * T + col_at(cc, tx)) * 2 + q];
-#pragma unroll
-        for (int rr = 0; rr < TM; ++rr) {
-          const unsigned long long aa = mp32::pack2(a[rr], a[rr]);
-#pragma unroll
-          for (int c2 = 0; c2 < TM / 2; ++c2) {
-            const float2 cand = mp32::sum2(aa, mp32::pack2(b[2 * c2], b[2 * c2 + 1]));
-            d[rr][2 * c2] = fminf(d[rr][2 * c2], cand.x);
-            d[rr][2 * c2 + 1] = fminf(d[rr][2 * c2 + 1], cand.y);
-          }
-        }
-      }
-    }
-  }
-  // D where improved (the old value is still in global memory).
-  unsigned long long imp = 0ull;  // bit 8 rr + cc
-#pragma unroll
-  for (int rr = 0; rr < TM; ++rr)
-#pragma unroll
-    for (int cc = 0; cc < TM; ++cc) {
-      const int i = row_at(rr, ty), j = col_at(cc, tx);
-      if (i < m && j < m) {
-        const int64_t g = (int64_t)(base + i) * ld + base + j;
-        if (d[rr][cc] < D[g]) {
-          D[g] = d[rr][cc];
-          imp |= 1ull << (TM * rr + cc);
-        }
-      }
-    }
-  if (!P || __syncthreads_count(imp != 0ull) == 0) return;  // the history is complete past this barrier
-  if (imp == 0ull) return;
-  // P: lowest 8-k chunk (4 k-pairs) whose minimum candidate equals the final
-  // value, then the first k inside it.  Chunks are walked from high to low
-  // and the byte of an element is overwritten on every match.
-  unsigned ch[TM][TM / 4];
-#pragma unroll
-  for (int rr = 0; rr < TM; ++rr)
-#pragma unroll
-    for (int c4 = 0; c4 < TM / 4; ++c4) ch[rr][c4] = 0u;
-#pragma unroll 1
-  for (int c = T / 8 - 1; c >= 0; --c) {
-    unsigned long long bq[4][TM];
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-#pragma unroll
-      for (int cc = 0; cc < TM; ++cc) bq[q][cc] = h.hr[4 * c + q][col_at(cc, tx)];
-#pragma unroll
-    for (int rr = 0; rr < TM; ++rr) {
-      unsigned long long aq[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) aq[q] = h.hc[4 * c + q][row_at(rr, ty)];
-#pragma unroll
-      for (int cc = 0; cc < TM; ++cc) {
-        const float2 s0 = mp32::sum2(aq[0], bq[0][cc]), s1 = mp32::sum2(aq[1], bq[1][cc]);
-        const float2 s2 = mp32::sum2(aq[2], bq[2][cc]), s3 = mp32::sum2(aq[3], bq[3][cc]);
-        float mm = mp32::min3f(s0.x, s0.y, s1.x);
-        mm = mp32::min3f(mm, s1.y, s2.x);
-        mm = mp32::min3f(mm, s2.y, s3.x);
-        mm = fminf(mm, s3.y);
-        if (mm == d[rr][cc])
-          ch[rr][cc / 4] = __byte_perm(ch[rr][cc / 4], (unsigned)c,
-                                       0x3210 ^ ((0x3210 & (0xF << (4 * (cc & 3)))) ^ (4 << (4 * (cc & 3)))));
-      }
-    }
-  }
-#pragma unroll
-  for (int rr = 0; rr < TM; ++rr)
-#pragma unroll
-    for (int cc = 0; cc < TM; ++cc) {
-      if (!((imp >> (TM * rr + cc)) & 1ull)) continue;
-      const int c = (ch[rr][cc / 4] >> (8 * (cc & 3))) & 0xFF;  // an improved element's chunk
-      const int i = row_at(rr, ty), j = col_at(cc, tx);
-      int kf = 8 * c + 7;
-#pragma unroll
-      for (int q = 3; q >= 0; --q) {
-        const float2 sv = mp32::sum2(h.hc[4 * c + q][i], h.hr[4 * c + q][j]);
-        kf = sv.y == d[rr][cc] ? 8 * c + 2 * q + 1 : kf;
-        kf = sv.x == d[rr][cc] ? 8 * c + 2 * q : kf;
-      }
-      P[(int64_t)(base + i) * ld + base + j] = base + kf;
-    }
-}
-
 template <bool EAGER>
 __global__ void __launch_bounds__(mp32::THREADS, EAGER ? APSP_K3_EAGER_MIN_BLOCKS : APSP_K3_MIN_BLOCKS)
     fw_phase3_minplus_f32(float *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r,
@@ -617,18 +931,38 @@ std::vector<cudaEvent_t> g_prof_pool;
 constexpr int kMaxN = 1 << 18;
 
 constexpr int kT32 = mp32::T, kT64 = 128;
-static int g_smem_k1f[64], g_smem_p2f[64], g_smem_k3[64], g_smem_k3e[64];
+constexpr int kSms = 152;
+static int g_smem_k1[2][64], g_smem_k2[2][2][64], g_smem_k3[64], g_smem_k3e[64];
 
 int run_fw_f64_interval(double *D, int n, int64_t ld, int32_t *P, cudaStream_t s);
 int take_device_error_f64();
 int take_device_error_checks();
 int take_device_error_int32();
 
-static void path_init(int32_t *P, int64_t n, int64_t ld, cudaStream_t s) {
+// Launches `kernel` so that it may start before the previous kernel of the
+// stream has ended (it waits for it with grid_dep_wait before it reads or
+// writes anything that kernel does): the launch latency, about 3 us, is hidden.
+template <typename... A>
+static void launch_after(void (*kernel)(A...), int grid, int threads, size_t smem, cudaStream_t s, bool overlap,
+                         A... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = overlap ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+static void path_init(int32_t *P, int64_t n, int64_t ld, int64_t skip, cudaStream_t s) {
   const int64_t total = n * n;
   const int blocks = (int)((total + 255) / 256 < 152 * 32 ? (total + 255) / 256 : 152 * 32);
   PhaseScope ps(0, s);
-  fw_path_init<<<blocks, 256, 0, s>>>(P, n, ld);
+  fw_path_init<<<blocks, 256, 0, s>>>(P, n, ld, skip);
 }
 
 static int check_args(const void *D, int64_t n, int64_t ld) {
@@ -644,21 +978,29 @@ static int run_fw_f32(float *D, int64_t n64, int64_t ld, int32_t *P, void *strea
   const int n = (int)n64;
   constexpr int T = kT32;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  if ((st = ensure_smem(fw_phase1_diag_f32, (int)sizeof(k1::Hist), g_smem_k1f))) return st;
-  if ((st = ensure_smem(fw_phase2_lines_f32, k2::SMEM, g_smem_p2f))) return st;
+  const int R = (n + T - 1) / T;
+  if ((st = ensure_smem(fw_phase1_diag_f32<false>, (int)sizeof(k1::Smem), g_smem_k1[0]))) return st;
+  if ((st = ensure_smem(fw_phase1_diag_f32<true>, (int)sizeof(k1::Smem), g_smem_k1[1]))) return st;
+  // K2 with two lines a warp while four would not fill the chip.
+  const int lines = 2 * (R - 1) * k2s::parts(4) < kSms ? 2 : 4;
+  const auto lines_kernel = lines == 2 ? (P ? fw_phase2_lines_f32<true, 2> : fw_phase2_lines_f32<false, 2>)
+                                       : (P ? fw_phase2_lines_f32<true, 4> : fw_phase2_lines_f32<false, 4>);
+  const int lines_smem = (int)(lines == 2 ? sizeof(k2s::Smem<2>) : sizeof(k2s::Smem<4>));
+  if ((st = ensure_smem(lines_kernel, lines_smem, g_smem_k2[lines / 4][P != nullptr]))) return st;
   if ((st = ensure_smem(fw_phase3_minplus_f32<false>, (int)sizeof(k3::Smem), g_smem_k3))) return st;
   if ((st = ensure_smem(fw_phase3_minplus_f32<true>, (int)sizeof(k3::Smem), g_smem_k3e))) return st;
   cudaGetLastError();  // clear any stale error so the checks below are ours
-  const int R = (n + T - 1) / T;
   // Phase-4 operand panels, written by K2 each round: two sets (round parity)
   // of 4 arrays of R*T*T 4-byte words, so that K2 of round r+1 can run while
-  // phase 4 of round r still reads round r's panels.  Stream-ordered scratch,
-  // freed after the last round.
+  // phase 4 of round r still reads round r's panels; then K1's two copies of
+  // the closed diagonal block.  Stream-ordered scratch, freed after the last
+  // round.
   Panels pan[2]{};
+  DiagOps ops{};
   char *scratch = nullptr;
   if (R > 1) {
     const size_t words = (size_t)R * T * T;
-    if (cudaMallocAsync((void **)&scratch, 8 * words * 4, s) != cudaSuccess) {
+    if (cudaMallocAsync((void **)&scratch, (8 * words + 2 * (size_t)T * T) * 4, s) != cudaSuccess) {
       cudaGetLastError();
       return APSP_ENOMEM;
     }
@@ -669,35 +1011,13 @@ static int run_fw_f32(float *D, int64_t n64, int64_t ld, int32_t *P, void *strea
       pan[q].Acp = reinterpret_cast<float *>(base + 2 * words * 4);
       pan[q].Bt = reinterpret_cast<float *>(base + 3 * words * 4);
     }
+    ops.A = reinterpret_cast<unsigned long long *>(scratch + 8 * words * 4);
+    ops.B = ops.A + T * T / 2;
   }
-  if (P) path_init(P, n64, ld, s);
-  const int vec_ok = (ld % 4 == 0) && ((reinterpret_cast<uintptr_t>(D) & 15) == 0);
-  auto diag_and_panels = [&](int r, cudaStream_t st) {
-    {
-      PhaseScope ps(1, st);
-      fw_phase1_diag_f32<<<1, mp32::THREADS, sizeof(k1::Hist), st>>>(D, ld, P, n, r);
-    }
-    if (R > 1) {
-      PhaseScope ps(2, st);
-      fw_phase2_lines_f32<<<2 * (R - 1) * k2::PARTS, k2::THREADS, k2::SMEM, st>>>(D, ld, P, n, r, R, pan[r & 1]);
-    }
-  };
-  auto phase4 = [&](int r, int set, int blocks) {
-    if (blocks <= 0) return;
-    PhaseScope ps(3, s);
-    if (P && r < kEagerRounds)
-      fw_phase3_minplus_f32<true><<<2 * blocks, mp32::THREADS, sizeof(k3::Smem), s>>>(D, ld, P, n, r, R, vec_ok,
-                                                                                   pan[r & 1], set);
-    else
-      fw_phase3_minplus_f32<false><<<2 * blocks, mp32::THREADS, sizeof(k3::Smem), s>>>(D, ld, P, n, r, R, vec_ok,
-                                                                                    pan[r & 1], set);
-  };
-  // Look-ahead: phase 4 of round r first updates row and column r+1 (the
-  // blocks K1/K2 of round r+1 read), then the rest of the matrix while K1/K2
-  // of round r+1 run on a second, higher-priority stream; the two touch
-  // disjoint blocks and write/read different panel sets.
-  cudaStream_t s2 = nullptr;
-  cudaEvent_t ev_next = nullptr, ev_panels = nullptr;
+  const bool aligned = ld % 4 == 0;
+  const int vec = (aligned && (reinterpret_cast<uintptr_t>(D) & 15) == 0 ? kVecD : 0) |
+                  (aligned && (reinterpret_cast<uintptr_t>(P) & 15) == 0 ? kVecP : 0);
+  const int vec_ok = vec & kVecD;
   // While the caller's stream is being captured into a CUDA graph every
   // phase stays on that stream (no stream is created or destroyed mid-capture).
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -706,39 +1026,83 @@ static int run_fw_f32(float *D, int64_t n64, int64_t ld, int32_t *P, void *strea
     cudaGetLastError();
     return APSP_ECUDA;
   }
+  const bool overlap = cap == cudaStreamCaptureStatusNone;
+  auto diag = [&](int r, cudaStream_t st) {
+    PhaseScope ps(1, st);
+    launch_after(P ? fw_phase1_diag_f32<true> : fw_phase1_diag_f32<false>, k1::CTAS, 32 * k1::WARPS, sizeof(k1::Smem),
+                 st, overlap, D, ld, P, n, r, vec, (int)(P && r == 0), ops);
+  };
+  auto panels = [&](int r, cudaStream_t st) {
+    if (R == 1) return;
+    PhaseScope ps(2, st);
+    launch_after(lines_kernel, 2 * (R - 1) * k2s::parts(lines), k2s::THREADS, lines_smem, st, overlap, D, ld, P, n, r, R,
+                 vec, ops, pan[r & 1]);
+  };
+  auto phase4 = [&](int r, int set, int blocks, cudaStream_t st) {
+    if (blocks <= 0) return;
+    PhaseScope ps(3, st);
+    if (P && r < kEagerRounds)
+      fw_phase3_minplus_f32<true><<<2 * blocks, mp32::THREADS, sizeof(k3::Smem), st>>>(D, ld, P, n, r, R, vec_ok,
+                                                                                    pan[r & 1], set);
+    else
+      fw_phase3_minplus_f32<false><<<2 * blocks, mp32::THREADS, sizeof(k3::Smem), st>>>(D, ld, P, n, r, R, vec_ok,
+                                                                                     pan[r & 1], set);
+  };
+  // Look-ahead: everything the next round waits for runs on a second stream of
+  // higher priority: phase 4 of round r on row and column r+1, then K1 and K2
+  // of round r+1.  The rest of round r's phase 4 runs on the caller's stream
+  // beside it, filling the SMs the chain leaves free; the two touch disjoint
+  // blocks and write/read different panel sets.
+  cudaStream_t s2 = nullptr;
+  cudaEvent_t ev_rest = nullptr, ev_panels = nullptr;
   if (R > 2 && cap == cudaStreamCaptureStatusNone) {
     int lo = 0, hi = 0;
     cudaDeviceGetStreamPriorityRange(&lo, &hi);
     if (cudaStreamCreateWithPriority(&s2, cudaStreamNonBlocking, hi) != cudaSuccess ||
-        cudaEventCreateWithFlags(&ev_next, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&ev_rest, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&ev_panels, cudaEventDisableTiming) != cudaSuccess) {
       if (s2) cudaStreamDestroy(s2);
-      if (ev_next) cudaEventDestroy(ev_next);
+      if (ev_rest) cudaEventDestroy(ev_rest);
       if (scratch) cudaFreeAsync(scratch, s);
       cudaGetLastError();
       return APSP_ECUDA;
     }
   }
-  diag_and_panels(0, s);
-  for (int r = 0; r < R; ++r) {
-    if (R == 1) break;
-    if (r + 1 < R && s2) {
-      phase4(r, k3::kSetNext, 2 * R - 3);
-      cudaEventRecord(ev_next, s);
-      cudaStreamWaitEvent(s2, ev_next, 0);
-      diag_and_panels(r + 1, s2);
-      cudaEventRecord(ev_panels, s2);
-      phase4(r, k3::kSetRest, (R - 2) * (R - 2));
-      cudaStreamWaitEvent(s, ev_panels, 0);
-    } else {
-      phase4(r, k3::kSetAll, (R - 1) * (R - 1));
-      if (r + 1 < R) diag_and_panels(r + 1, s);
-    }
-  }
+  // K1 of round 0 writes all of P's first block; the rest of P is set to -1
+  // beside it.
   if (s2) {
+    cudaEventRecord(ev_panels, s);
+    if (P) path_init(P, n64, ld, T, s);
+    cudaStreamWaitEvent(s2, ev_panels, 0);
+    diag(0, s2);
+    if (P) {
+      cudaEventRecord(ev_rest, s);
+      cudaStreamWaitEvent(s2, ev_rest, 0);
+    }
+    panels(0, s2);
+    cudaEventRecord(ev_panels, s2);
+    for (int r = 0; r + 1 < R; ++r) {
+      phase4(r, k3::kSetNext, 2 * R - 3, s2);
+      diag(r + 1, s2);
+      cudaStreamWaitEvent(s, ev_panels, 0);  // round r's panels
+      panels(r + 1, s2);
+      cudaEventRecord(ev_panels, s2);
+      phase4(r, k3::kSetRest, (R - 2) * (R - 2), s);
+      cudaEventRecord(ev_rest, s);
+      cudaStreamWaitEvent(s2, ev_rest, 0);
+    }
+    cudaStreamWaitEvent(s, ev_panels, 0);
+    phase4(R - 1, k3::kSetAll, (R - 1) * (R - 1), s);
     cudaStreamDestroy(s2);
-    cudaEventDestroy(ev_next);
+    cudaEventDestroy(ev_rest);
     cudaEventDestroy(ev_panels);
+  } else {
+    if (P && R > 1) path_init(P, n64, ld, T, s);
+    for (int r = 0; r < R; ++r) {
+      diag(r, s);
+      panels(r, s);
+      phase4(r, k3::kSetAll, (R - 1) * (R - 1), s);
+    }
   }
   cudaError_t e = cudaGetLastError();
   if (scratch) {
@@ -753,7 +1117,7 @@ static int run_fw_f64(double *D, int64_t n64, int64_t ld, int32_t *P, void *stre
   if (st || n64 == 0) return st;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   cudaGetLastError();
-  if (P) path_init(P, n64, ld, s);
+  if (P) path_init(P, n64, ld, 0, s);
   return run_fw_f64_interval(D, (int)n64, ld, P, s);
 }
 
