@@ -197,7 +197,7 @@ def kernel_source_hash() -> str:
     txt = open(os.path.join(d, "phases_f32.cuh")).read()
     h.update(txt[txt.index("namespace k3 {"):txt.index("}  // namespace k3")].encode())
     txt = open(os.path.join(d, "fw_single.cu")).read()
-    h.update(txt[txt.index("template <bool EAGER>\n__global__"):txt.index("// Phase timing state")].encode())
+    h.update(txt[txt.index("// K3 (FP32): phase 4"):txt.index("// Phase timing state")].encode())
     return h.hexdigest()[:16]
 
 

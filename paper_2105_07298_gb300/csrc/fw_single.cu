@@ -16,18 +16,18 @@
 // priority beside the rest of round r's phase 4.
 //
 // Differences from the Pascal design of §3.2 (one output per thread, TB <= 32):
-//  * K3 runs two CTAs per 128 x 128 block, three per SM, an 8 x 4 register
-//    tile per thread (FP32, TB = 128), and pairs consecutive k: one packed
-//    add.rn.f32x2 forms the two candidates of an output and one three-input
-//    min.f32 folds both into the accumulator (FADD2 and FMNMX3 run on
-//    different pipes).  Operands arrive by bulk copy into a two-stage ring.
-//  * Path state: in rounds 0-15 (nearly every output improves) an eager
-//    instance of K3 keeps, per output, the k-pair of the last strict decrease
-//    as a byte; later rounds keep none in the inner loop, and after the loop
-//    the improved outputs recover the first k that attains the new minimum
-//    (lane-parallel for dense 8-row groups, warp-cooperative otherwise).
-//    Either way P is exactly that of the sequential loop (ascending k, strict
-//    "<" keeps the first k reaching the final minimum).
+//  * K3 pairs consecutive k: one packed add.rn.f32x2 forms the two candidates
+//    of an output and one three-input min.f32 folds both into the accumulator
+//    (FADD2 and FMNMX3 run on different pipes).  Large launches run two CTAs
+//    per 128 x 128 block, three per SM, an 8 x 4 register tile per thread,
+//    operands by bulk copy into a two-stage ring; small ones, and the first
+//    rounds with a path matrix, run 32- or 64-row pieces of a block.
+//  * Path state: the pieces note once per 16 k which outputs fell; the ring
+//    kernel keeps none in the loop, and afterwards the improved outputs
+//    recover the first k that attains the new minimum (lane-parallel for dense
+//    8-row groups, warp-cooperative otherwise).  Either way P is exactly that
+//    of the sequential loop (ascending k, strict "<" keeps the first k
+//    reaching the final minimum).
 //  * K1 is one cluster of eight CTAs, K2 keeps each row/column line in
 //    registers; both keep only minima per step and settle P afterwards.
 //  * Nothing reads P: K1/K2/K3 write P only where D strictly improved.
@@ -528,8 +528,7 @@ __global__ void __launch_bounds__(k2s::THREADS, 2)
 // Grid: (R-1)^2 blocks in row-major (I', J') order over the blocks I, J != r,
 // so consecutive CTAs share the column-panel block A and sweep the row panel.
 // --------------------------------------------------------------------------
-template <bool EAGER>
-__global__ void __launch_bounds__(mp32::THREADS, EAGER ? APSP_K3_EAGER_MIN_BLOCKS : APSP_K3_MIN_BLOCKS)
+__global__ void __launch_bounds__(mp32::THREADS, APSP_K3_MIN_BLOCKS)
     fw_phase3_minplus_f32(float *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r,
                           int R, int vec_ok, Panels pan, int set) {
   using namespace k3;
@@ -537,31 +536,9 @@ __global__ void __launch_bounds__(mp32::THREADS, EAGER ? APSP_K3_EAGER_MIN_BLOCK
   using mp32::row_at;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
-  const int Rm = R - 1, tile = blockIdx.x >> 1, hJ = blockIdx.x & 1;
+  const int tile = blockIdx.x >> 1, hJ = blockIdx.x & 1;
   int I, J;
-  if (set == kSetAll) {  // every block off row and column r
-    I = tile / Rm;
-    J = tile % Rm;
-    I += (I >= r);
-    J += (J >= r);
-  } else if (set == kSetNext) {  // row r+1, then column r+1: the next round's K1/K2 input
-    if (tile < Rm) {
-      I = r + 1;
-      J = tile + (tile >= r);
-    } else {
-      I = tile - Rm;
-      I += (I >= r);
-      I += (I >= r + 1);
-      J = r + 1;
-    }
-  } else {  // the rest: rows and columns other than r and r+1
-    I = tile / (R - 2);
-    J = tile % (R - 2);
-    I += (I >= r);
-    I += (I >= r + 1);
-    J += (J >= r);
-    J += (J >= r + 1);
-  }
+  block_of(set, tile, r, R, I, J);
   const int baseI = I * T, baseJ = J * T + hJ * H, baseK = r * T;
   const int mI = min(T, n - baseI), mJ = min(H, n - baseJ), mK = min(T, n - baseK);
   if (mJ <= 0) return;  // empty half of the last (narrow) block; uniform exit
@@ -584,10 +561,8 @@ __global__ void __launch_bounds__(mp32::THREADS, EAGER ? APSP_K3_EAGER_MIN_BLOCK
   __syncthreads();
 
   float acc[8][4];
-  unsigned kid[8];  // EAGER: byte c of kid[a] = the round's k-pair of the last strict decrease, 0xFF none
 #pragma unroll
   for (int a = 0; a < 8; ++a) {
-    kid[a] = 0xFFFFFFFFu;
 #pragma unroll
     for (int c = 0; c < 4; ++c) acc[a][c] = INF;
   }
@@ -618,7 +593,6 @@ __global__ void __launch_bounds__(mp32::THREADS, EAGER ? APSP_K3_EAGER_MIN_BLOCK
         b[cc + 1] = t.y;
       }
     };
-    const unsigned kbase = (unsigned)(s * KP);
     auto compute = [&](int kp, const unsigned long long (&b)[4]) {
       ulonglong2 an = *reinterpret_cast<const ulonglong2 *>(&Asl[kp * T + row_at(0, ty)]);
 #pragma unroll
@@ -627,58 +601,13 @@ __global__ void __launch_bounds__(mp32::THREADS, EAGER ? APSP_K3_EAGER_MIN_BLOCK
         if (rp < 3) an = *reinterpret_cast<const ulonglong2 *>(&Asl[kp * T + row_at(2 * rp + 2, ty)]);
 #pragma unroll
         for (int cc = 0; cc < 4; ++cc) {
-          if constexpr (EAGER) {
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              const float m = mp32::min3f_pair(acc[2 * rp + h][cc], h ? ac.y : ac.x, b[cc]);
-              if (m < acc[2 * rp + h][cc])
-                kid[2 * rp + h] = __byte_perm(kid[2 * rp + h], kbase + kp,
-                                              0x3210 ^ ((0x3210 & (0xF << (4 * cc))) ^ (4 << (4 * cc))));
-              acc[2 * rp + h][cc] = m;
-            }
-          } else {
-            mp32::relax2(acc[2 * rp][cc], ac.x, b[cc]);
-            mp32::relax2(acc[2 * rp + 1][cc], ac.y, b[cc]);
-          }
+          mp32::relax2(acc[2 * rp][cc], ac.x, b[cc]);
+          mp32::relax2(acc[2 * rp + 1][cc], ac.y, b[cc]);
         }
       }
     };
     unsigned long long b0[4], b1[4];
     load_b(0, b0);
-    if constexpr (EAGER) {
-      // Both k-pairs of a step per output, one compare and one byte permute
-      // per four candidates: the byte keeps the step's first k-pair.
-      auto compute2 = [&](int kp, const unsigned long long (&p0)[4], const unsigned long long (&p1)[4]) {
-        ulonglong2 n0 = *reinterpret_cast<const ulonglong2 *>(&Asl[kp * T + row_at(0, ty)]);
-        ulonglong2 n1 = *reinterpret_cast<const ulonglong2 *>(&Asl[(kp + 1) * T + row_at(0, ty)]);
-#pragma unroll
-        for (int rp = 0; rp < 4; ++rp) {
-          const ulonglong2 c0 = n0, c1 = n1;
-          if (rp < 3) {
-            n0 = *reinterpret_cast<const ulonglong2 *>(&Asl[kp * T + row_at(2 * rp + 2, ty)]);
-            n1 = *reinterpret_cast<const ulonglong2 *>(&Asl[(kp + 1) * T + row_at(2 * rp + 2, ty)]);
-          }
-#pragma unroll
-          for (int cc = 0; cc < 4; ++cc)
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              float &acc_o = acc[2 * rp + h][cc];
-              const float m1 = mp32::min3f_pair(acc_o, h ? c0.y : c0.x, p0[cc]);
-              const float m2 = mp32::min3f_pair(m1, h ? c1.y : c1.x, p1[cc]);
-              if (m2 < acc_o)
-                kid[2 * rp + h] = __byte_perm(kid[2 * rp + h], kbase + kp,
-                                              0x3210 ^ ((0x3210 & (0xF << (4 * cc))) ^ (4 << (4 * cc))));
-              acc_o = m2;
-            }
-        }
-      };
-#pragma unroll 4
-      for (int kp = 0; kp < KP; kp += 2) {
-        load_b(kp + 1, b1);
-        compute2(kp, b0, b1);
-        if (kp + 2 < KP) load_b(kp + 2, b0);
-      }
-    } else {
 // Unrolled by four (measured best of 1, 2, 4 and 8).
 #pragma unroll 4
     for (int kp = 0; kp < KP; kp += 2) {
@@ -686,7 +615,6 @@ __global__ void __launch_bounds__(mp32::THREADS, EAGER ? APSP_K3_EAGER_MIN_BLOCK
       compute(kp, b0);
       if (kp + 2 < KP) load_b(kp + 2, b0);
       compute(kp + 1, b1);
-    }
     }
     __syncthreads();  // stage st fully read
     if (tid == 0 && s + STAGES < nslab) {
@@ -703,18 +631,13 @@ __global__ void __launch_bounds__(mp32::THREADS, EAGER ? APSP_K3_EAGER_MIN_BLOCK
   // owning 16 whole rows (lane l: columns 2l, 2l+1), which keeps the code small
   // (instruction-cache friendly) and every global access coalesced.
   float *Cs = reinterpret_cast<float *>(smem_raw);  // [T][H]
-  unsigned char *Ks = smem_raw + sizeof(Smem::As);  // EAGER: [T][H] k-pair bytes, in the B ring
   __syncthreads();
 #pragma unroll
   for (int rr = 0; rr < 8; ++rr)
 #pragma unroll
-    for (int cc = 0; cc < 4; cc += 2) {
+    for (int cc = 0; cc < 4; cc += 2)
       *reinterpret_cast<float2 *>(&Cs[row_at(rr, ty) * H + col_at(cc, tx)]) =
           make_float2(acc[rr][cc], acc[rr][cc + 1]);
-      if constexpr (EAGER)
-        *reinterpret_cast<unsigned short *>(&Ks[row_at(rr, ty) * H + col_at(cc, tx)]) =
-            (unsigned short)(kid[rr] >> (8 * cc));
-    }
   __syncthreads();
   const float *acp = pan.Acp + (int64_t)I * T * T;
   const float *bt = pan.Bt + ((int64_t)J * T + hJ * H) * T;
@@ -755,32 +678,6 @@ __global__ void __launch_bounds__(mp32::THREADS, EAGER ? APSP_K3_EAGER_MIN_BLOCK
     }
   }
   if (!P) return;
-  if constexpr (EAGER) {
-    // The k inside each improved output's last decreasing step (two k-pairs):
-    // the first whose candidate equals the new value (the sequential loop
-    // keeps the first k reaching a minimum).
-#pragma unroll 1
-    for (int t = 0; t < 16; ++t)
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        if (!((flags >> (2 * t + q)) & 1u)) continue;
-        const int i = i0 + t, j = j0 + q;
-        const int kp = Ks[i * H + j];  // an improved output has one
-        const float g = Cs[i * H + j];
-        const float2 c = mp32::sum2(srcA[(int64_t)kp * T + i], srcB[(int64_t)kp * H + j]);
-        int k;
-        if (c.x == g) {
-          k = 2 * kp;
-        } else if (c.y == g) {
-          k = 2 * kp + 1;
-        } else {  // the second k-pair of the step
-          const float2 c2 = mp32::sum2(srcA[(int64_t)(kp + 1) * T + i], srcB[(int64_t)(kp + 1) * H + j]);
-          k = c2.x == g ? 2 * kp + 2 : 2 * kp + 3;
-        }
-        P[(int64_t)(baseI + i) * ld + baseJ + j] = baseK + k;
-      }
-    return;
-  }
   // Pass 2a: each 8-row group of the warp with many improved outputs (the
   // early rounds, where most outputs improve) is resolved lane-parallel: lane
   // l scans the 128 candidates of its own two columns in the paired panel
@@ -916,6 +813,165 @@ __global__ void __launch_bounds__(mp32::THREADS, EAGER ? APSP_K3_EAGER_MIN_BLOCK
   }
 }
 
+// --------------------------------------------------------------------------
+// K3 in small pieces: one CTA computes a TR x 64 piece of an output block (TR =
+// 32 where a launch has few blocks, so that it still uses every SM and a CTA's
+// serial time is short; 64 otherwise).  The operands of all 128 k come in one
+// go; the old values load while they are under way and start the accumulators,
+// so an output improves exactly when its accumulator falls.  Thread tile 4 x 2
+// or 4 x 4.  With a path matrix the outputs are compared once per 16 k (one
+// compare, one byte permute and one move per 16 relaxations) and the k of an
+// improved one is found afterwards among those 16, from the operands still in
+// shared memory.
+// Bound: the FP32 pipes once a launch fills the chip (52 relax/clk/SM at
+// n = 8192 with 32 rows, 56 with 64, 57 for the ring kernel above), latency
+// below.  Measured per launch of 13 blocks (n = 1024, row and column r+1):
+// 12 us, 17 us with a path matrix; the 128 x 64 tile 19 and 36 us.  Tracking
+// here costs about 20 % in every round; the ring kernel's recovery after the
+// loop costs more while most outputs improve and less when few do.
+// --------------------------------------------------------------------------
+namespace k3s {
+constexpr int T = mp32::T, THREADS = 256, TC = 64, PAIRS = T / 2;
+__host__ __device__ constexpr int per_block(int tr) { return (T / tr) * (T / TC); }
+template <int TR>
+struct Smem {
+  unsigned long long A[PAIRS][TR];  // A[kp][i] = (A[i][2kp], A[i][2kp+1])
+  unsigned long long B[PAIRS][TC];  // B[kp][j] = (B[2kp][j], B[2kp+1][j])
+  uint64_t bar;
+};
+}  // namespace k3s
+
+template <bool PATH, int TR>
+__global__ void __launch_bounds__(k3s::THREADS, TR == 32 ? 4 : 3)
+    fw_phase3_small_f32(float *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r, int R, int vec_ok,
+                        Panels pan, int set) {
+  using namespace k3s;
+  static_assert(TR == 32 || TR == 64, "eight warps of 16 x 16 or 16 x 32 outputs");
+  constexpr int CW = TR / 16, PER = per_block(TR);  // columns per thread
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  Smem<TR> &sm = *reinterpret_cast<Smem<TR> *>(smem_raw);
+  const int tile = blockIdx.x / PER, sub = blockIdx.x % PER;
+  int I, J;
+  k3::block_of(set, tile, r, R, I, J);
+  const int si = sub >> 1, hJ = sub & 1;
+  const int baseI = I * T + si * TR, baseJ = J * T + hJ * TC, baseK = r * T;
+  const int mI = min(TR, n - baseI), mJ = min(TC, n - baseJ), mK = min(T, n - baseK);
+  if (mI <= 0 || mJ <= 0) return;  // past the matrix (uniform exit)
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int nkp = (mK + 1) / 2;
+  if (tid == 0) {
+    mbar_init(&sm.bar, 1);
+    fence_mbar_init();
+    mbar_expect_tx(&sm.bar, (uint32_t)(nkp * (TR + TC) * 8));
+  }
+  grid_dep_wait();
+  if (tid == 0) {
+    fence_proxy_async_global();
+    bulk_g2s(&sm.B[0][0], pan.Bpan + ((int64_t)J * 2 + hJ) * PAIRS * TC, (uint32_t)(nkp * TC * 8), &sm.bar);
+  }
+  __syncthreads();
+  if (w == 0) {
+    const unsigned long long *srcA = pan.Apan + (int64_t)I * PAIRS * T + si * TR;
+    fence_proxy_async_global();
+    for (int kp = lane; kp < nkp; kp += 32) bulk_g2s(&sm.A[kp][0], srcA + (int64_t)kp * T, TR * 8, &sm.bar);
+  }
+  // A warp owns 16 x 8 CW outputs; lane (ty, tx) = (l / 8, l % 8) rows
+  // 2 ty + (a & 1) + 8 (a >> 1) and columns 2 tx + (c & 1) + 16 (c >> 1) of them.
+  constexpr int WC = TC / (8 * CW);  // warps side by side
+  const int r0 = (w / WC) * 16 + 2 * (lane >> 3), c0 = (w % WC) * 8 * CW + 2 * (lane & 7);
+  float acc[4][CW], prev[4][CW];
+  unsigned chunk[CW];  // byte a of chunk[c]: last group of 16 k that lowered output (a, c), 0xFF none
+#pragma unroll
+  for (int c = 0; c < CW; ++c) chunk[c] = 0xFFFFFFFFu;
+#pragma unroll
+  for (int a = 0; a < 4; ++a) {
+    const int i = r0 + (a & 1) + 8 * (a >> 1);
+#pragma unroll
+    for (int c = 0; c < CW; c += 2) {
+      const int j = c0 + 8 * c;
+      const float *src = D + (int64_t)(baseI + i) * ld + baseJ + j;
+      float2 t = make_float2(inf<float>(), inf<float>());
+      if (i < mI) {
+        if (vec_ok && j + 1 < mJ) {
+          t = *reinterpret_cast<const float2 *>(src);
+        } else {
+          if (j < mJ) t.x = src[0];
+          if (j + 1 < mJ) t.y = src[1];
+        }
+      }
+      prev[a][c] = acc[a][c] = t.x;
+      prev[a][c + 1] = acc[a][c + 1] = t.y;
+    }
+  }
+  __syncwarp();
+  const bool ok = mbar_wait(&sm.bar, 0);
+  if (__syncthreads_or(!ok)) {  // the operands never arrived: the block stays as it is
+    if (tid == 0) report_wait_timeout();
+    return;
+  }
+  auto step = [&](int kp) {
+    const ulonglong2 a01 = *reinterpret_cast<const ulonglong2 *>(&sm.A[kp][r0]);
+    const ulonglong2 a23 = *reinterpret_cast<const ulonglong2 *>(&sm.A[kp][r0 + 8]);
+#pragma unroll
+    for (int c = 0; c < CW; c += 2) {
+      const ulonglong2 b = *reinterpret_cast<const ulonglong2 *>(&sm.B[kp][c0 + 8 * c]);
+      mp32::relax2(acc[0][c], a01.x, b.x);
+      mp32::relax2(acc[0][c + 1], a01.x, b.y);
+      mp32::relax2(acc[1][c], a01.y, b.x);
+      mp32::relax2(acc[1][c + 1], a01.y, b.y);
+      mp32::relax2(acc[2][c], a23.x, b.x);
+      mp32::relax2(acc[2][c + 1], a23.x, b.y);
+      mp32::relax2(acc[3][c], a23.y, b.x);
+      mp32::relax2(acc[3][c + 1], a23.y, b.y);
+    }
+  };
+  auto note = [&](int g) {
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int c = 0; c < CW; ++c) {
+        if (acc[a][c] < prev[a][c]) chunk[c] = __byte_perm(chunk[c], (unsigned)g, byte_sel(a));
+        prev[a][c] = acc[a][c];
+      }
+  };
+  int g = 0;
+#pragma unroll 1
+  for (; g < nkp / 8; ++g) {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) step(8 * g + u);
+    if (PATH) note(g);
+  }
+  if (8 * g < nkp) {  // the last round's remainder
+#pragma unroll 1
+    for (int kp = 8 * g; kp < nkp; ++kp) step(kp);
+    if (PATH) note(g);
+  }
+  grid_dep_launch();
+#pragma unroll
+  for (int a = 0; a < 4; ++a) {
+    const int i = r0 + (a & 1) + 8 * (a >> 1);
+#pragma unroll
+    for (int c = 0; c < CW; ++c) {
+      const unsigned gc = (chunk[c] >> (8 * a)) & 0xFFu;
+      if (PATH ? gc == 0xFFu : !(acc[a][c] < prev[a][c])) continue;  // (improved outputs lie inside the matrix)
+      const int j = c0 + 16 * (c >> 1) + (c & 1);
+      const int64_t e = (int64_t)(baseI + i) * ld + baseJ + j;
+      D[e] = acc[a][c];
+      if (PATH) {
+        int k = 0;
+#pragma unroll
+        for (int u = 7; u >= 0; --u) {
+          const int kp = min(8 * (int)gc + u, nkp - 1);
+          const float2 t = mp32::sum2(sm.A[kp][i], sm.B[kp][j]);
+          k = t.y == acc[a][c] ? 2 * kp + 1 : k;
+          k = t.x == acc[a][c] ? 2 * kp : k;
+        }
+        P[e] = baseK + k;
+      }
+    }
+  }
+}
+
 // Phase timing state (see profile.h).
 std::mutex g_prof_mu;
 bool g_prof_on = false;
@@ -932,7 +988,18 @@ constexpr int kMaxN = 1 << 18;
 
 constexpr int kT32 = mp32::T, kT64 = 128;
 constexpr int kSms = 152;
-static int g_smem_k1[2][64], g_smem_k2[2][2][64], g_smem_k3[64], g_smem_k3e[64];
+// Phase-4 kernels by blocks per side R (measured, whole solves, ms):
+//  * 32-row pieces for every launch while the whole of phase 4 is about a wave
+//    of CTAs or less (n = 2049: 0.93 against 0.97 with 64 rows, 1.12 with the
+//    ring kernel; with P 1.29 / 1.38 / 1.74), and for row and column r+1 alone,
+//    which the next round waits for, a little longer;
+//  * 64-row pieces in the first rounds with a path matrix, where most outputs
+//    improve (n = 16384: 16 / 32 / 48 rounds 301.1 / 299.1 / 301.5; n = 4096:
+//    6.97 / 6.65 / 6.64), and without one up to n = 5120 (n = 4096: 4.55
+//    against 4.69);
+//  * the ring kernel otherwise (n = 8192 without P: 32.7 against 33.3).
+constexpr int kR32 = 21, kRNext32 = 40, kR64 = 40, kDenseRounds = 32;
+static int g_smem_k1[2][64], g_smem_k2[2][2][64], g_smem_k3s[2][2][64], g_smem_k3[64];
 
 int run_fw_f64_interval(double *D, int n, int64_t ld, int32_t *P, cudaStream_t s);
 int take_device_error_f64();
@@ -987,8 +1054,12 @@ static int run_fw_f32(float *D, int64_t n64, int64_t ld, int32_t *P, void *strea
                                        : (P ? fw_phase2_lines_f32<true, 4> : fw_phase2_lines_f32<false, 4>);
   const int lines_smem = (int)(lines == 2 ? sizeof(k2s::Smem<2>) : sizeof(k2s::Smem<4>));
   if ((st = ensure_smem(lines_kernel, lines_smem, g_smem_k2[lines / 4][P != nullptr]))) return st;
-  if ((st = ensure_smem(fw_phase3_minplus_f32<false>, (int)sizeof(k3::Smem), g_smem_k3))) return st;
-  if ((st = ensure_smem(fw_phase3_minplus_f32<true>, (int)sizeof(k3::Smem), g_smem_k3e))) return st;
+  // Phase 4 in pieces of 32 or 64 rows.
+  const auto kernel32 = P ? fw_phase3_small_f32<true, 32> : fw_phase3_small_f32<false, 32>;
+  const auto kernel64 = P ? fw_phase3_small_f32<true, 64> : fw_phase3_small_f32<false, 64>;
+  if ((st = ensure_smem(kernel32, (int)sizeof(k3s::Smem<32>), g_smem_k3s[0][P != nullptr]))) return st;
+  if ((st = ensure_smem(kernel64, (int)sizeof(k3s::Smem<64>), g_smem_k3s[1][P != nullptr]))) return st;
+  if ((st = ensure_smem(fw_phase3_minplus_f32, (int)sizeof(k3::Smem), g_smem_k3))) return st;
   cudaGetLastError();  // clear any stale error so the checks below are ours
   // Phase-4 operand panels, written by K2 each round: two sets (round parity)
   // of 4 arrays of R*T*T 4-byte words, so that K2 of round r+1 can run while
@@ -1041,12 +1112,15 @@ static int run_fw_f32(float *D, int64_t n64, int64_t ld, int32_t *P, void *strea
   auto phase4 = [&](int r, int set, int blocks, cudaStream_t st) {
     if (blocks <= 0) return;
     PhaseScope ps(3, st);
-    if (P && r < kEagerRounds)
-      fw_phase3_minplus_f32<true><<<2 * blocks, mp32::THREADS, sizeof(k3::Smem), st>>>(D, ld, P, n, r, R, vec_ok,
-                                                                                    pan[r & 1], set);
+    if (R <= kR32 || (set == k3::kSetNext && R <= kRNext32))
+      launch_after(kernel32, k3s::per_block(32) * blocks, k3s::THREADS, sizeof(k3s::Smem<32>), st, overlap, D, ld, P, n,
+                   r, R, vec_ok, pan[r & 1], set);
+    else if (P ? r < kDenseRounds : R <= kR64)
+      launch_after(kernel64, k3s::per_block(64) * blocks, k3s::THREADS, sizeof(k3s::Smem<64>), st, overlap, D, ld, P, n,
+                   r, R, vec_ok, pan[r & 1], set);
     else
-      fw_phase3_minplus_f32<false><<<2 * blocks, mp32::THREADS, sizeof(k3::Smem), st>>>(D, ld, P, n, r, R, vec_ok,
-                                                                                     pan[r & 1], set);
+      fw_phase3_minplus_f32<<<2 * blocks, mp32::THREADS, sizeof(k3::Smem), st>>>(D, ld, P, n, r, R, vec_ok, pan[r & 1],
+                                                                              set);
   };
   // Look-ahead: everything the next round waits for runs on a second stream of
   // higher priority: phase 4 of round r on row and column r+1, then K1 and K2

@@ -170,22 +170,30 @@ struct Smem {
   unsigned long long Bs[STAGES][KP][H];  // Bs[kp][j] = (B[2kp][j], B[2kp+1][j]), this half
   uint64_t bar[STAGES];
 };
+// The output block (I, J) of a launch's tile-th block in round r (R blocks a side).
+__device__ __forceinline__ void block_of(int set, int tile, int r, int R, int &I, int &J) {
+  if (set == kSetNext) {  // row r+1, then column r+1
+    const bool row = tile < R - 1;
+    const int o = row ? tile : tile - (R - 1);
+    I = row ? r + 1 : o + (o >= r);
+    I += !row && I >= r + 1;
+    J = row ? o + (o >= r) : r + 1;
+    return;
+  }
+  const int side = set == kSetAll ? R - 1 : R - 2;
+  I = tile / side;
+  J = tile % side;
+  I += (I >= r);
+  J += (J >= r);
+  if (set == kSetRest) {
+    I += (I >= r + 1);
+    J += (J >= r + 1);
+  }
+}
 }  // namespace k3
 
 #ifndef APSP_K3_MIN_BLOCKS
 #define APSP_K3_MIN_BLOCKS 3
-#endif
-#ifndef APSP_K3_EAGER_ROUNDS
-#define APSP_K3_EAGER_ROUNDS 16
-#endif
-// Rounds that track P in the main loop (EAGER): in the first rounds nearly
-// every output improves, and one compare and one byte permute per k-pair
-// (per two k-pairs in the single-graph kernel) cost less than recomputing
-// every candidate afterwards.
-constexpr int kEagerRounds = APSP_K3_EAGER_ROUNDS;
-
-#ifndef APSP_K3_EAGER_MIN_BLOCKS
-#define APSP_K3_EAGER_MIN_BLOCKS 2
 #endif
 template <bool NC, typename V>
 __device__ __forceinline__ V ld_panel(const V *p) {

@@ -1,0 +1,51 @@
+"""The FP32 single-graph kernels at the sizes where their dispatch changes or a
+tile is ragged, bit for bit against the oracle's blocked FW at the library's
+block size on real weights (one rounded sum per candidate, ascending k)."""
+import numpy as np
+import pytest
+import torch
+
+import graphgen
+import oracle
+import paper_2105_07298_gb300 as apsp
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+def _expect(n, p, seed):
+    W = graphgen.dense_graph(n, p, seed, weights="real", lo=0.5, hi=2.0, dtype=np.float32)
+    return W, *oracle.bfw(W, apsp.block_size(torch.float32))
+
+
+# One quad of the diagonal block; a block less one; two blocks, the last one
+# vertex wide; the last size with two lines a warp in the panels and the first
+# with four; the first past the 32-row pieces; the first on the ring kernel.
+@pytest.mark.parametrize("n", [1, 3, 5, 127, 129, 258, 2305, 2433, 2689, 5121])
+def test_real_weights_bitwise_at_dispatch_limits(n):
+    W, Db, Pb = _expect(n, 0.3 if n < 300 else 0.05, 900 + n)
+    D, P = torch.from_numpy(W).to(DEV), torch.full((n, n), 77, dtype=torch.int32, device=DEV)
+    apsp.apsp_fw(D, P)
+    np.testing.assert_array_equal(D.cpu().numpy(), Db)
+    np.testing.assert_array_equal(P.cpu().numpy(), Pb)
+    D = torch.from_numpy(W).to(DEV)
+    apsp.apsp_fw(D)
+    np.testing.assert_array_equal(D.cpu().numpy(), Db)
+    assert apsp.device_status() == apsp.APSP_OK
+
+
+@pytest.mark.parametrize("ld,d_off,p_off", [(263, 0, 0), (264, 1, 0), (264, 0, 1), (264, 3, 2)])
+def test_unaligned_rows_and_buffers(ld, d_off, p_off):
+    """Odd leading dimensions and buffers that start off a 16-byte boundary, D
+    and P apart; the columns past n stay as they are."""
+    n = 261
+    W, Db, Pb = _expect(n, 0.3, 5)
+    dbuf = torch.full((n * ld + 4,), -3.0, device=DEV)
+    pbuf = torch.full((n * ld + 4,), -9, dtype=torch.int32, device=DEV)
+    D = dbuf[d_off:d_off + n * ld].view(n, ld)
+    P = pbuf[p_off:p_off + n * ld].view(n, ld)
+    D[:, :n].copy_(torch.from_numpy(W))
+    apsp.apsp_fw(D[:, :n], P[:, :n])
+    np.testing.assert_array_equal(D[:, :n].cpu().numpy(), Db)
+    np.testing.assert_array_equal(P[:, :n].cpu().numpy(), Pb)
+    assert bool((D[:, n:] == -3.0).all()) and bool((P[:, n:] == -9).all())
