@@ -1,36 +1,28 @@
 // FP64 blocked Floyd-Warshall for sm_103a, exact, on the FP32 pipes.
 //
-// GB300 executes FP64 adds and mins at about 2 per clock per SM, 1/64 of its
-// FP32 rate, so a native FP64 min-plus product runs ~60x slower than FP32.
-// This path keeps every result bit-exact with IEEE FP64 (round to nearest)
-// while doing almost all of the work in FP32:
+// GB300 executes FP64 adds at about 2 per clock per SM, 1/64 of its FP32 rate,
+// so a native FP64 min-plus product runs ~60x slower than FP32.  This path
+// keeps every result bit-exact with IEEE FP64 (round to nearest) while doing
+// almost all of the work in FP32:
 //
-//  * each FP64 operand x is held as the float interval [rd(x), ru(x)]
-//    (largest float <= x, smallest float >= x);
-//  * a candidate a + b then lies in [lo, up] with lo = rd(rd(a) + rd(b)) and
-//    up = ru(ru(a) + ru(b)) (add.rm / add.rp), and so does its FP64 rounding
-//    fl(a + b), since rounding is monotone;
-//  * the min-plus product runs on the lower bounds alone (one packed
-//    add.rm.f32x2 and one three-input min per two candidates, as the FP32
-//    kernel) and keeps X = min lo per output.  If X >= ru(old) nothing can
-//    beat the old value.  Otherwise the exact FP64 minimum is X when some
-//    candidate with lo = X has an exact sum X (its upper bound is X, or one
-//    FP64 add says so; integer-valued weights always land here), and the
-//    first such k is the path entry; if none has, the candidates with
-//    lo <= min(ru(old), their up) are evaluated with a real FP64 add.
+//  * each FP64 operand x has a lower bound rd(x), the largest float <= x;
+//  * a candidate a + b is at least lo = rd(rd(a) + rd(b)) (add.rm), and so is
+//    its FP64 rounding fl(a + b), since rounding is monotone;
+//  * a group of candidates is taken by its lower bounds alone (one packed
+//    add.rm.f32x2 and one three-input min per two).  If their minimum X is not
+//    below ru(old), the smallest float >= the old value, nothing improves.
+//    Otherwise the first candidate with lo = X gets one FP64 add, s.  If s = X,
+//    or no other candidate has lo <= ru(s), s is the exact minimum and its k
+//    the first that reaches it; if some has (rare: sums within one float step
+//    of each other), every candidate with lo <= ru(s) is added in FP64.
 //
 // Schedule per round r (TB = 128), the blocked FW of §2.2, every phase in the
 // paper's k order:
-//  K1  fw64_diag         phase 1: Algorithm 1 on block (r,r), k sequential,
-//                        with the interval filter per relaxation.
-//  K2  fw64_lines        phases 2 and 3: the row blocks (r,J) and column
-//                        blocks (I,r), k sequential per line with the same
-//                        filter; packs the finished blocks as phase-4 operands.
-//  K3  fw64_product      phase 4: (I,J) <- min(C, D(I,r) (x) D(r,J)); rounds
-//                        0-15 run an eager instance that also keeps, per
-//                        output, the k-pair where min lo last decreased.
-// As in the FP32 path, phase 4 of round r updates row and column r+1 first,
-// then the rest while K1/K2 of round r+1 run on a second stream.
+//  K1  fw64_diag     phase 1: Algorithm 1 on block (r,r), k sequential.
+//  K2  fw64_lines    phases 2 and 3: the row blocks (r,J) and column blocks
+//                    (I,r), k sequential per line; writes the phase-4 operands.
+//  K3  fw64_pieces   phase 4: (I,J) <- min(C, D(I,r) (x) D(r,J)).
+// Rounds overlap as in the FP32 path (rounds.cuh).
 // Every candidate sum is one IEEE FP64 addition rounded to nearest, taken in
 // the order of the sequential blocked FW, so D and P are bit-exact with it on
 // any weights (and with every correct FW on integer-valued weights).
@@ -40,38 +32,30 @@
 #include "bulk.cuh"
 #include "common.cuh"
 #include "profile.h"
+#include "rounds.cuh"
 
 namespace apsp {
 namespace f64 {
 
-constexpr int T = 128;
-constexpr int THREADS = 256;  // product: 8 warps, 4 x 8 outputs per thread, 128 x 64 per CTA
-constexpr int H = T / 2;      // output columns per CTA (one half of a block)
-constexpr int KS = 32, KP = 16, STAGES = 2;
-constexpr uint32_t SLAB_BYTES = KP * H * 8;  // one half of one paired array, one slab
-#ifndef APSP_F64_DENSE_MIN
-#define APSP_F64_DENSE_MIN 40
-#endif
-// Quick improvements (of 512) above which an 8-row group takes recovery pass 2a.
-constexpr int kDenseMin64 = APSP_F64_DENSE_MIN;
+constexpr int T = 128, PAIRS = T / 2, QUADS = T / 4;
 
-// One operand block packed for the product kernel.  For an A operand
-// (A[i][k]): lo[i/64][kp][i%64] = (rd A[i][2kp], rd A[i][2kp+1]), hi likewise
-// with ru, rlo[i][k] = rd A[i][k], rhi[i][k] = ru A[i][k], r64[i][k] = A[i][k].
-// For a B operand (B[k][j]): lo[j/64][kp][j%64] = (rd B[2kp][j],
-// rd B[2kp+1][j]), ..., rlo[j][k] = rd B[k][j], rhi[j][k], r64[j][k] = B[k][j]
-// (transposed).  The paired arrays are split in two 64-wide halves so that a
-// 16-k-pair slab of one half is one contiguous 8 KiB piece.  Entries outside
-// the matrix hold +inf.
-// 128-byte aligned so that every pack of an array starts on a 16-byte
-// boundary (bulk copies and 16-byte loads read from it).
-struct __align__(128) Pack {
-  unsigned long long lo[2][T / 2][T / 2];
-  unsigned long long hi[2][T / 2][T / 2];
-  float rlo[T][T];
-  float rhi[T][T];
-  double r64[T][T];
-  int exact;  // 1: every value is a float (rlo == rhi), so upper bounds follow from rlo
+// Operands of phase 4, written by K2 each round (entries outside the matrix
+// are +inf):
+//   column block (I,r): A[I][kp][i] = (rd D[i][2kp], rd D[i][2kp+1]),
+//                       A64[I][i][k] = D[i][k]
+//   row block (r,J):    B[J][j/64][kp][j%64] = (rd D[2kp][j], rd D[2kp+1][j]),
+//                       B64[J][j][k] = D[k][j]
+struct Panels64 {
+  unsigned long long *A, *B;
+  double *A64, *B64;
+};
+// The closed diagonal block in K2's layouts, written by K1: lower bounds
+// k-paired, Alo[kp][i] = (rd D[i][2kp], rd D[i][2kp+1]), Blo[kp][j] =
+// (rd D[2kp][j], rd D[2kp+1][j]), and values A64[k][i] = D[i][k], B64[k][j] =
+// D[k][j].
+struct DiagOps64 {
+  unsigned long long *Alo, *Blo;
+  double *A64, *B64;
 };
 
 // ---------------------------------------------------------------- bounds
@@ -79,37 +63,17 @@ struct __align__(128) Pack {
 // bit pattern (integer pipes only).  Tight in the normal float range; below
 // it the bound is loosened to 0 / +-FLT_MIN, which keeps it valid.
 __device__ __forceinline__ float f64_up(double x) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  if ((b << 1) == 0) return 0.0f;
-  const unsigned hi = (unsigned)(b >> 32), lo = (unsigned)b;
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
   const unsigned sign = hi & 0x80000000u;
-  const int e = (int)((hi >> 20) & 0x7ff);
-  if (e == 0x7ff) return sign ? -__int_as_float(0x7f800000) : __int_as_float(0x7f800000);
-  const int fe = e - 1023 + 127;
-  if (fe >= 255) return sign ? -FLT_MAX : __int_as_float(0x7f800000);
-  if (fe <= 0) return sign ? -0.0f : FLT_MIN;
-  const unsigned m23 = ((hi & 0xfffffu) << 3) | (lo >> 29);
-  unsigned f = sign | ((unsigned)fe << 23) | m23;  // toward zero
-  if ((lo & 0x1fffffffu) && !sign) f += 1u;
-  return __uint_as_float(f);
+  const int e = (int)((hi >> 20) & 0x7ff), fe = e - 1023 + 127;
+  unsigned f = ((unsigned)fe << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);  // magnitude toward zero
+  f += (lo & 0x1fffffffu) && !sign ? 1u : 0u;
+  if (fe >= 255) f = e == 0x7ff || !sign ? 0x7f800000u : 0x7f7fffffu;            // infinity, or beyond the floats
+  if (fe <= 0) f = sign || ((hi << 1) | lo) == 0u ? 0u : 0x00800000u;           // below the normal floats
+  return __uint_as_float(f | sign);
 }
 
 __device__ __forceinline__ float f64_down(double x) { return -f64_up(-x); }
-
-// Exact x < d for a float x and a double d (no NaN).  Equal to x < ru(d),
-// since a float below d is below the smallest float >= d.  Both non-negative
-// with x normal: the doubles' bit patterns order as unsigned integers, so x's
-// double pattern is built (exponent rebiased, mantissa shifted) and compared.
-__device__ __forceinline__ bool f32_lt_f64(float x, double d) {
-  const unsigned ux = __float_as_uint(x);
-  const unsigned long long ud = (unsigned long long)__double_as_longlong(d);
-  const unsigned e = ux >> 23;  // sign bit clear: the biased exponent
-  if (!(ud >> 63) && e - 1u < 254u) {
-    const unsigned long long bx = ((unsigned long long)(e + 896u) << 52) | ((unsigned long long)(ux & 0x7fffffu) << 29);
-    return bx < ud;
-  }
-  return x < f64_up(d);
-}
 
 // Exact float -> double bits (integer pipes; subnormal floats via cvt).
 __device__ __forceinline__ unsigned long long f32_to_f64_bits(float f) {
@@ -124,28 +88,25 @@ __device__ __forceinline__ unsigned long long f32_to_f64_bits(float f) {
   return sign | ((unsigned long long)(e - 127 + 1023) << 52) | ((unsigned long long)(u & 0x7fffffu) << 29);
 }
 
-// Signed integer key with the order of the doubles (-0 sorts just below +0;
-// neither arises from sums of the non-negative-cycle inputs except -0 + -0).
-__device__ __forceinline__ long long dkey(unsigned long long b) {
-  return (long long)(b ^ ((unsigned long long)((long long)b >> 63) >> 1));
-}
-__device__ __forceinline__ unsigned long long dkey_bits(long long k) {
-  return (unsigned long long)k ^ ((unsigned long long)(k >> 63) >> 1);
+__device__ __forceinline__ double f32_as_f64(float x) { return __longlong_as_double((long long)f32_to_f64_bits(x)); }
+
+// a < b for doubles (no NaN) on the integer pipes: as signed integers, with
+// the order of two negative values reversed, and -0 equal to +0.
+__device__ __forceinline__ bool dless(double a, double b) {
+  const long long x = __double_as_longlong(a), y = __double_as_longlong(b);
+  const long long kx = x ^ (long long)((unsigned long long)(x >> 63) >> 1);
+  const long long ky = y ^ (long long)((unsigned long long)(y >> 63) >> 1);
+  return kx < ky && ((x | y) << 1) != 0;
 }
 
 __device__ __forceinline__ unsigned long long packf2(float lo, float hi) {
   return ((unsigned long long)__float_as_uint(hi) << 32) | __float_as_uint(lo);
 }
 
-// Lower- and upper-bound sums of two candidates (add.rm / add.rp, as the main loop).
+// Lower-bound sums of two candidates (add.rm, as the main loop).
 __device__ __forceinline__ float2 sum2_rm(unsigned long long a, unsigned long long b) {
   unsigned long long t;
   asm("add.rm.f32x2 %0, %1, %2;" : "=l"(t) : "l"(a), "l"(b));
-  return make_float2(__uint_as_float((unsigned)t), __uint_as_float((unsigned)(t >> 32)));
-}
-__device__ __forceinline__ float2 sum2_rp(unsigned long long a, unsigned long long b) {
-  unsigned long long t;
-  asm("add.rp.f32x2 %0, %1, %2;" : "=l"(t) : "l"(a), "l"(b));
   return make_float2(__uint_as_float((unsigned)t), __uint_as_float((unsigned)(t >> 32)));
 }
 __device__ __forceinline__ float min3f(float a, float b, float c) {
@@ -163,129 +124,408 @@ __device__ __forceinline__ void relax2_rm(float &acc, unsigned long long a, unsi
       : "l"(a), "l"(b));
 }
 
-// ---------------------------------------------------------------- K1
-// Phase 1 on block (r,r): Algorithm 1 (strict "<", k ascending), k
-// sequential as the paper's phase 1.  The block's values live in shared
-// memory as doubles (d) with their lower float bounds (dlo = rd d); each
-// thread keeps the upper bounds (dhi = ru d) of its 4 x 8 elements in
-// registers.  At step k a candidate d[i][k] + d[k][j] is skipped without an
-// FP64 add when its lower bound rd(dlo[i][k] + dlo[k][j]) is not below dhi[i][j]
-// (then fl(d[i][k] + d[k][j]) >= d[i][j]); otherwise one FP64 add decides.
-// Step k never changes row or column k (D[k][k] = 0), so every thread reads
-// them straight from shared memory while the step writes other elements; one
-// barrier per step.  Element (i, j) of thread (ty, tx) = (tid / 16, tid % 16):
-// i = ty + 32 rr (rr 0..3), j = 2 tx + q + 32 cb (cb 0..3, q 0..1).
-// Also marks every operand pack of the round's set exact (the phase-2/3
-// kernel clears the flag of a pack holding a value that is not a float).
-constexpr int K1_THREADS = 512;
-struct K1Smem {
-  double d[T * T];
-  float dlo[T * T];
-  unsigned char pk[T * T];  // block-local k of the last improvement, 0xFF none
-};
-
-__global__ void __launch_bounds__(K1_THREADS, 1)
-    fw64_diag(double *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r, int R, Pack *packA,
-              Pack *packB) {
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  K1Smem &sm = *reinterpret_cast<K1Smem *>(smem_raw);
-  const int base = r * T, m = min(T, n - base), tid = threadIdx.x;
-  const int ty = tid >> 4, tx = tid & 15;
-  const double INF = inf<double>();
-  for (int e = tid; e < T * T; e += K1_THREADS) {
-    const int i = e / T, j = e % T;
-    const double v = (i < m && j < m) ? D[(int64_t)(base + i) * ld + base + j] : INF;
-    sm.d[e] = v;
-    sm.dlo[e] = f64_down(v);
-    sm.pk[e] = 0xFF;
-  }
-  if (packA)
-    for (int b = tid; b < R; b += K1_THREADS) {
-      packA[b].exact = 1;
-      packB[b].exact = 1;
-    }
-  __syncthreads();
-  // element t = 8 rr + c of this thread: i = ty + 32 rr, j = 2 tx + (c & 1) + 32 (c >> 1)
-  float dhi[32];
-#pragma unroll
-  for (int t = 0; t < 32; ++t)
-    dhi[t] = f64_up(sm.d[(ty + 32 * (t >> 3)) * T + 2 * tx + (t & 1) + 32 * ((t & 7) >> 1)]);
-#pragma unroll 1
-  for (int k = 0; k < m; ++k) {
-    float alo[4];
-    unsigned long long blo[4];
-#pragma unroll
-    for (int rr = 0; rr < 4; ++rr) alo[rr] = sm.dlo[(ty + 32 * rr) * T + k];
-#pragma unroll
-    for (int cb = 0; cb < 4; ++cb) blo[cb] = *reinterpret_cast<const unsigned long long *>(&sm.dlo[k * T + 2 * tx + 32 * cb]);
-    unsigned cand_mask = 0u;  // bit t: the candidate's lower bound is below element t's upper bound
-#pragma unroll
-    for (int rr = 0; rr < 4; ++rr) {
-      const unsigned long long aa = packf2(alo[rr], alo[rr]);
-#pragma unroll
-      for (int cb = 0; cb < 4; ++cb) {
-        const float2 lo = sum2_rm(aa, blo[cb]);
-        cand_mask |= (lo.x < dhi[8 * rr + 2 * cb] ? 1u : 0u) << (8 * rr + 2 * cb);
-        cand_mask |= (lo.y < dhi[8 * rr + 2 * cb + 1] ? 1u : 0u) << (8 * rr + 2 * cb + 1);
-      }
-    }
-    // The exact test, once per flagged element (rolled: the code stays small).
-#pragma unroll 1
-    while (cand_mask) {
-      const int t = __ffs(cand_mask) - 1;
-      cand_mask &= cand_mask - 1;
-      const int i = ty + 32 * (t >> 3), j = 2 * tx + (t & 1) + 32 * ((t & 7) >> 1);
-      const double cand = __dadd_rn(sm.d[i * T + k], sm.d[k * T + j]);
-      if (cand < sm.d[i * T + j]) {
-        sm.d[i * T + j] = cand;
-        sm.dlo[i * T + j] = f64_down(cand);
-        sm.pk[i * T + j] = (unsigned char)k;
-        const float up = f64_up(cand);
-#pragma unroll
-        for (int u = 0; u < 32; ++u) dhi[u] = u == t ? up : dhi[u];
-      }
-    }
-    __syncthreads();
-  }
-  for (int e = tid; e < T * T; e += K1_THREADS) {
-    const int i = e / T, j = e % T;
-    const unsigned kl = sm.pk[e];
-    if (kl != 0xFFu && i < m && j < m) {
-      const int64_t g = (int64_t)(base + i) * ld + base + j;
-      D[g] = sm.d[e];
-      if (P) P[g] = base + (int)kl;
-    }
-  }
+// __byte_perm selector that replaces byte c of its first operand with byte 0 of its second.
+__device__ __forceinline__ constexpr unsigned byte_sel64(int c) {
+  return 0x3210 ^ ((0x3210 & (0xF << (4 * c))) ^ (4 << (4 * c)));
 }
 
-// ---------------------------------------------------------------- K2
-// Phases 2 and 3, k sequential in the paper's order (as the FP32 path):
+// ---------------------------------------------------------------- K1, K2
+// Both phases take four steps k = 4 kq + s at a time on lines held four
+// elements a lane: a line's pivots p[s] (its values at positions 4 kq + s, each
+// at its own step) against the quad's rows r[s].
+//
+// The pivots of up to four lines at once: lane 4 c + t (c, t < 4) holds line
+// c's value v at position 4 kq + t.  e[s]: row s of the quad at position
+// 4 kq + t, at its own step; elo[s]: its lower bound.  Brings v to its step; vlo
+// is its lower bound.  The FP64 additions run only if some lane's candidates
+// may improve.  All lanes call.
+template <typename E>
+__device__ __forceinline__ void quad_pivots(double &v, float &vlo, const float (&elo)[3], int lane, E e) {
+  const int t = lane & 3;
+  vlo = f64_down(v);
+  const float vhi = f64_up(v);
+  bool may = false;
+#pragma unroll
+  for (int s = 0; s < 3; ++s) {
+    const float pivot = __shfl_sync(kFullMask, vlo, (lane & ~3) | s);
+    may |= t > s && __fadd_rd(pivot, elo[s]) < vhi;
+  }
+  if (!__any_sync(kFullMask, may && lane < 16)) return;
+#pragma unroll
+  for (int s = 0; s < 3; ++s) {
+    const double cand = __dadd_rn(__shfl_sync(kFullMask, v, (lane & ~3) | s), e(s));
+    if (t > s && dless(cand, v)) v = cand;
+  }
+  vlo = f64_down(v);
+}
+// The same for the quad's own four rows (line c = row c), whose entries are
+// each other's e (returned too).
+__device__ __forceinline__ void quad_pivots_own(double &v, float &vlo, double (&e)[3], int lane) {
+  const int t = lane & 3;
+  vlo = f64_down(v);
+  const float vhi = f64_up(v);
+  bool may = false;
+#pragma unroll
+  for (int s = 0; s < 3; ++s) {
+    e[s] = __shfl_sync(kFullMask, v, 4 * s + t);
+    // row s itself takes D[k][k] + its own value: no change unless D[k][k] < 0
+    const float pivot = __shfl_sync(kFullMask, vlo, (lane & ~3) | s);
+    const float row = __shfl_sync(kFullMask, vlo, 4 * s + t);
+    may |= t > s && __fadd_rd(pivot, row) < vhi && !(lane >> 2 == s && pivot >= 0.0f);
+  }
+  if (!__any_sync(kFullMask, may && lane < 16)) return;
+#pragma unroll
+  for (int s = 0; s < 3; ++s) {
+    e[s] = __shfl_sync(kFullMask, v, 4 * s + t);
+    const double cand = __dadd_rn(__shfl_sync(kFullMask, v, (lane & ~3) | s), e[s]);
+    if (t > s && dless(cand, v)) v = cand;
+  }
+  vlo = f64_down(v);
+}
+
+// A warp's four lines, in shared memory.
+struct WarpLines {
+  double d[4][T];
+  float hi[4][T];          // ru(d)
+  double ps[4][4];         // the quad's pivots [line][s]
+  float plo[4][4];         // their lower bounds
+  unsigned short list[4 * T];
+  unsigned char pk[4][T];  // k of the last improvement, 0xFF none
+};
+
+// The warp's lines through the quad's four steps.  rlo01, rlo23: the rows'
+// lower bounds (rows 0, 1 and 2, 3, paired, by position), r64(s, pos): their
+// values.  Lane l tests its positions 4l..4l+3 of each line by lower bounds; the
+// elements that may improve are then listed and taken by all lanes together,
+// one each, so that the FP64 additions (16 clocks a warp per SM however many
+// lanes need them) and the work around them are shared.
+//
+// The element at position k itself takes D[k][k] + its own value at step k,
+// and (own: the lines are the quad's rows) so does every element of row k;
+// neither can lower it unless D[k][k] < 0.  Those candidates are left out,
+// since their lower bounds alone would list every value that is not a float.
+template <typename Rv>
+__device__ __forceinline__ void relax_lines(WarpLines &L, int kq, bool own, int lane, const unsigned long long *rlo01,
+                                            const unsigned long long *rlo23, Rv r64) {
+  auto bounds = [](float (&l)[4], unsigned long long pa, unsigned long long pb, unsigned long long ra,
+                   unsigned long long rb) {
+    const float2 l01 = sum2_rm(pa, ra), l23 = sum2_rm(pb, rb);
+    l[0] = l01.x, l[1] = l01.y, l[2] = l23.x, l[3] = l23.y;
+  };
+  auto leave_out = [](float (&l)[4], int c, unsigned long long ra, unsigned long long rb) {
+    const unsigned long long rc = c < 2 ? ra : rb;
+    if (__uint_as_float((unsigned)((c & 1) ? rc >> 32 : rc)) >= 0.0f) {
+#pragma unroll
+      for (int s = 0; s < 4; ++s) l[s] = s == c ? inf<float>() : l[s];
+    }
+  };
+  unsigned may = 0u;  // bit 4 c + q
+  {
+    unsigned long long ra[4], rb[4];
+#pragma unroll
+    for (int q = 0; q < 4; q += 2) {
+      const ulonglong2 ta = *reinterpret_cast<const ulonglong2 *>(&rlo01[4 * lane + q]);
+      const ulonglong2 tb = *reinterpret_cast<const ulonglong2 *>(&rlo23[4 * lane + q]);
+      ra[q] = ta.x, ra[q + 1] = ta.y, rb[q] = tb.x, rb[q + 1] = tb.y;
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      float4 p4 = *reinterpret_cast<const float4 *>(&L.plo[c][0]);
+      float &pc = c == 0 ? p4.x : c == 1 ? p4.y : c == 2 ? p4.z : p4.w;
+      if (own && pc >= 0.0f) pc = inf<float>();
+      const unsigned long long pa = packf2(p4.x, p4.y), pb = packf2(p4.z, p4.w);
+      const float4 h = *reinterpret_cast<const float4 *>(&L.hi[c][4 * lane]);
+      const float hi[4] = {h.x, h.y, h.z, h.w};
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        float l[4];
+        bounds(l, pa, pb, ra[q], rb[q]);
+        if (lane == kq) leave_out(l, q, ra[q], rb[q]);
+        may |= (fminf(min3f(l[0], l[1], l[2]), l[3]) < hi[q] ? 1u : 0u) << (4 * c + q);
+      }
+    }
+  }
+  if (!__any_sync(kFullMask, may != 0u)) return;
+  int end = __popc(may);  // inclusive prefix sum of the counts
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(kFullMask, end, o);
+    end += lane >= o ? t : 0;
+  }
+  const int total = __shfl_sync(kFullMask, end, 31);
+  for (int at = end - __popc(may); may; may &= may - 1) {
+    const int b = __ffs(may) - 1;
+    L.list[at++] = (unsigned short)((b >> 2) * T + 4 * lane + (b & 3));
+  }
+  __syncwarp();
+#pragma unroll 1
+  for (int t = lane; t < total; t += 32) {
+    const int c = L.list[t] / T, pos = L.list[t] % T;
+    const ulonglong2 pp = *reinterpret_cast<const ulonglong2 *>(&L.plo[c][0]);
+    const unsigned long long ra = rlo01[pos], rb = rlo23[pos];
+    float l[4];
+    bounds(l, pp.x, pp.y, ra, rb);
+    if (pos >> 2 == kq) leave_out(l, pos & 3, ra, rb);
+    if (own && L.plo[c][c] >= 0.0f) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) l[u] = u == c ? inf<float>() : l[u];
+    }
+    const float X = fminf(min3f(l[0], l[1], l[2]), l[3]);
+    int s = l[0] == X ? 0 : l[1] == X ? 1 : l[2] == X ? 2 : 3;
+    double best = __dadd_rn(L.ps[c][s], r64(s, pos));
+    float up = f64_up(best);
+    const int near = (l[0] <= up) + (l[1] <= up) + (l[2] <= up) + (l[3] <= up);
+    if (near > 1 && best != f32_as_f64(X)) {  // others within one float step: add them too
+      best = inf<double>();
+#pragma unroll 1
+      for (int u = 0; u < 4; ++u) {
+        const float lu = u == 0 ? l[0] : u == 1 ? l[1] : u == 2 ? l[2] : l[3];
+        if (lu > up) continue;
+        const double cand = __dadd_rn(L.ps[c][u], r64(u, pos));
+        if (dless(cand, best)) {
+          best = cand;
+          s = u;
+        }
+      }
+      up = f64_up(best);
+    }
+    if (dless(best, L.d[c][pos])) {
+      L.d[c][pos] = best;
+      L.hi[c][pos] = up;
+      L.pk[c][pos] = (unsigned char)(4 * kq + s);
+    }
+  }
+  __syncwarp();
+}
+
+// K1: phase 1 on block (r,r) by one cluster of eight CTAs of four warps, as
+// the FP32 path's: a warp owns four adjacent rows, lane l their columns
+// 4l..4l+3, and takes the four steps of a quad together.  The quad's own rows
+// are brought to their steps by all four warps of the owning CTA (a column a
+// lane) and passed around the ring of CTAs by st.async.  The buffers hold
+// eight quads (so that the kernel leaves room beside phase-4 CTAs): a CTA's
+// four quads reuse the space of the quads eight before, which every CTA has
+// left behind by then (a split cluster barrier per four quads).
+// Bound: the chain of 32 quads (up to six dependent FP64 adds each), and while
+// many elements still improve the FP64 adds of their candidates.  Measured per
+// launch at n = 1000, real weights: 65-105 us, of which 1.9 us a quad (one CTA
+// that took each flagged element in a serial loop per step: 245-600 us);
+// taking a lane's own flagged elements in place instead of listing them for
+// the warp 125-218 us.
+namespace k1 {
+constexpr int CTAS = 8, WARPS = 4, RING = 2 * WARPS;
+struct Smem {
+  double r64[RING][4][T];              // row s of the quad at its step
+  unsigned long long rlo[RING][2][T];  // their lower bounds, rows (0, 1) and (2, 3)
+  WarpLines wl[WARPS];
+  double es[3][4];                     // the own quad's rows at its columns, at their steps
+  uint64_t bar[QUADS];
+};
+constexpr uint32_t QUAD_BYTES = 4 * T * 8 + 2 * T * 8;
+}  // namespace k1
+
+__global__ void __cluster_dims__(k1::CTAS, 1, 1) __launch_bounds__(32 * k1::WARPS, 1)
+    fw64_diag(double *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r, int vec, int first,
+              DiagOps64 ops) {
+  using namespace k1;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
+  const int base = r * T, m = min(T, n - base), nquad = (m + 3) / 4;
+  const int cta = (int)cluster_cta_rank(), tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int own = cta * WARPS + w;  // this warp's row quad
+  const int i0 = 4 * own, j0 = 4 * lane;
+  if (tid < QUADS) {
+    mbar_init(&sm.bar[tid], 1);
+    fence_mbar_init();
+    if (tid / WARPS != cta) mbar_expect_tx(&sm.bar[tid], QUAD_BYTES);
+  }
+  grid_dep_wait();
+  WarpLines &L = sm.wl[w];
+#pragma unroll
+  for (int rr = 0; rr < 4; ++rr) {
+    const double *row = D + (int64_t)(base + i0 + rr) * ld + base;
+    *reinterpret_cast<unsigned *>(&L.pk[rr][j0]) = 0xFFFFFFFFu;
+#pragma unroll
+    for (int c = 0; c < 4; c += 2) {
+      double2 t = make_double2(inf<double>(), inf<double>());
+      if (i0 + rr < m) {
+        if (vec && j0 + c + 1 < m) {
+          t = *reinterpret_cast<const double2 *>(row + j0 + c);
+        } else {
+          if (j0 + c < m) t.x = row[j0 + c];
+          if (j0 + c + 1 < m) t.y = row[j0 + c + 1];
+        }
+      }
+      *reinterpret_cast<double2 *>(&L.d[rr][j0 + c]) = t;
+      *reinterpret_cast<float2 *>(&L.hi[rr][j0 + c]) = make_float2(f64_up(t.x), f64_up(t.y));
+    }
+  }
+  __syncwarp();
+  cluster_sync();  // every barrier of the cluster is set up before anyone publishes
+  bool ok = true;
+  const unsigned next = (unsigned)(cta + 1) % CTAS;
+  const uint32_t next_base = cluster_map(smem_addr(smem_raw), next) - smem_addr(smem_raw);
+#pragma unroll 1
+  for (int kq = 0; kq < nquad; ++kq) {
+    const int g = kq / WARPS, ow = kq % WARPS, slot = kq % RING;
+    const bool mine = kq == own;
+    double v = L.d[(lane >> 2) & 3][4 * kq + (lane & 3)];
+    float vlo;
+    if (cta == g) {
+      if (mine) {
+        double e[3];
+        quad_pivots_own(v, vlo, e, lane);
+        if (lane < 4) {
+#pragma unroll
+          for (int u = 0; u < 3; ++u) sm.es[u][lane] = e[u];
+        }
+        if (lane < 16) {
+          (&L.ps[0][0])[lane] = v;
+          (&L.plo[0][0])[lane] = vlo;
+        }
+      }
+      __syncthreads();
+      {  // column tid: the quad's rows at their steps
+        double q[4];
+        float qlo[4];
+        bool may = false;
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+          q[s] = sm.wl[ow].d[s][tid];
+          qlo[s] = f64_down(q[s]);
+#pragma unroll
+          for (int u = 0; u < 3; ++u)
+            if (u < s) may |= __fadd_rd(sm.wl[ow].plo[s][u], qlo[u]) < sm.wl[ow].hi[s][tid];
+        }
+        if (may) {  // (a column whose rows cannot improve keeps its values)
+#pragma unroll
+          for (int s = 1; s < 4; ++s) {
+#pragma unroll
+            for (int u = 0; u < 3; ++u)
+              if (u < s) {
+                const double cand = __dadd_rn(sm.wl[ow].ps[s][u], q[u]);
+                if (dless(cand, q[s])) q[s] = cand;
+              }
+            qlo[s] = f64_down(q[s]);
+          }
+        }
+#pragma unroll
+        for (int s = 0; s < 4; ++s) sm.r64[slot][s][tid] = q[s];
+        sm.rlo[slot][0][tid] = packf2(qlo[0], qlo[1]);
+        sm.rlo[slot][1][tid] = packf2(qlo[2], qlo[3]);
+      }
+      if (!mine) {
+        float elo[3];
+#pragma unroll
+        for (int s = 0; s < 3; ++s) elo[s] = f64_down(sm.es[s][lane & 3]);
+        quad_pivots(v, vlo, elo, lane, [&](int s) { return sm.es[s][lane & 3]; });
+      }
+      __syncthreads();
+    } else {
+      if (ok) ok = mbar_spin(&sm.bar[kq], 0);
+    }
+    if (next != (unsigned)g) {  // pass the quad on to the next CTA of the ring
+      const uint32_t bar = next_base + smem_addr(&sm.bar[kq]);
+      const ulonglong2 *src = reinterpret_cast<const ulonglong2 *>(&sm.r64[slot][0][0]);
+      const ulonglong2 *srl = reinterpret_cast<const ulonglong2 *>(&sm.rlo[slot][0][0]);
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const ulonglong2 t = src[tid + 128 * u];
+        st_async16(next_base + smem_addr(src + tid + 128 * u), t.x, t.y, bar);
+      }
+      const ulonglong2 t = srl[tid];
+      st_async16(next_base + smem_addr(srl + tid), t.x, t.y, bar);
+    }
+    if (!mine) {
+      if (cta != g) {
+        const int t = 4 * kq + (lane & 3);
+        const unsigned long long e01 = sm.rlo[slot][0][t], e23 = sm.rlo[slot][1][t];
+        const float elo[3] = {__uint_as_float((unsigned)e01), __uint_as_float((unsigned)(e01 >> 32)),
+                              __uint_as_float((unsigned)e23)};
+        quad_pivots(v, vlo, elo, lane, [&](int s) { return sm.r64[slot][s][t]; });
+      }
+      if (lane < 16) {
+        (&L.ps[0][0])[lane] = v;
+        (&L.plo[0][0])[lane] = vlo;
+      }
+    }
+    __syncwarp();
+    relax_lines(L, kq, mine, lane, sm.rlo[slot][0], sm.rlo[slot][1], [&](int s, int pos) { return sm.r64[slot][s][pos]; });
+    if (ow == WARPS - 1 || kq + 1 == nquad) {  // done with CTA g's quads
+      if (g > 0) cluster_wait();               // and so is everyone with CTA g-1's, whose space comes next
+      cluster_arrive();
+    }
+  }
+  grid_dep_launch();
+  cluster_wait();  // no CTA leaves while another may still write its buffers
+  if (!ok) {       // D and P stay as they are
+    report_wait_timeout();
+    return;
+  }
+  double d[4][4];
+#pragma unroll
+  for (int rr = 0; rr < 4; ++rr)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) d[rr][c] = L.d[rr][j0 + c];
+  if (ops.Alo) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        ops.Blo[(2 * own + h) * T + j0 + c] = packf2(f64_down(d[2 * h][c]), f64_down(d[2 * h + 1][c]));
+        ops.Alo[(2 * lane + h) * T + i0 + c] = packf2(f64_down(d[c][2 * h]), f64_down(d[c][2 * h + 1]));
+      }
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int c = 0; c < 4; c += 2) {
+        *reinterpret_cast<double2 *>(&ops.B64[(i0 + a) * T + j0 + c]) = make_double2(d[a][c], d[a][c + 1]);
+        *reinterpret_cast<double2 *>(&ops.A64[(j0 + a) * T + i0 + c]) = make_double2(d[c][a], d[c + 1][a]);
+      }
+  }
+#pragma unroll
+  for (int rr = 0; rr < 4; ++rr)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const int i = i0 + rr, j = j0 + c;
+      if (i >= m || j >= m) continue;
+      const unsigned k = L.pk[rr][j];
+      const int64_t e = (int64_t)(base + i) * ld + base + j;
+      if (k != 0xFFu) D[e] = d[rr][c];
+      // the first round's block is not initialised: every entry is written
+      if (P && (first || k != 0xFFu)) P[e] = k != 0xFFu ? base + (int)k : -1;
+    }
+}
+
+// K2: phases 2 and 3, k sequential in the paper's order (as the FP32 path):
 // within a row block (r,J) every column j evolves on its own,
 //   own[i][j] <- min(own[i][j], diag[i][k] + own[k][j])   (k ascending),
 // within a column block (I,r) every row i does,
 //   own[i][j] <- min(own[i][j], own[i][k] + diag[k][j]),
-// with the diagonal block final after K1.  A warp keeps four such lines in
-// registers as doubles with their float bounds (lane l: positions 2l, 2l+1,
-// 2l+64, 2l+65).  At step k the lower bound of the pivot own[k] is broadcast
-// by a shuffle and paired with the diagonal's lower bounds from shared memory
-// (one add.rm.f32x2 per two candidates); only when some lane's candidate
-// lower bound is below its upper bound does the warp fetch the pivot's double
-// and run the exact FP64 adds.  Then the finished lines are written (D and P
-// where improved) and packed as phase-4 operands: a row block as the B
-// operand packB[J] (B[k][j] = own[k][j]), a column block as the A operand
-// packA[I] (A[i][k] = own[i][k]); in (line, position) terms both are
-// lo[line / 64][pos / 2][line % 64] = (rd at pos, rd at pos + 1), hi likewise
-// with ru, and rlo/rhi/r64[line][pos].  Entries outside the matrix are +inf.
+// with the diagonal block final after K1.  A warp keeps four such lines, lane
+// l their positions 4l..4l+3, and takes the four steps of a quad together
+// against the diagonal block's lower bounds in shared memory (one bulk copy);
+// the values are read from global memory only where a candidate may improve.
+// Then D and P are written where improved, and the blocks packed as phase-4
+// operands.  Four warps a CTA, so that few blocks still use many SMs.
+// Bound: the chain of 32 quads, as K1.  Measured per launch at n = 1000, real
+// weights: 31-66 us (one step at a time, each flagged element in a serial
+// loop: 94-156 us).
 namespace k2 {
-constexpr int K2_THREADS = 256, LINES = 2, PARTS = T / (K2_THREADS / 32 * LINES), MS = T + 2;
-constexpr int SMEM = T * MS * 4;
+constexpr int WARPS = 4, LINES = 4 /* of a WarpLines */, CTA_LINES = WARPS * LINES, PARTS = T / CTA_LINES;
+struct Smem {
+  unsigned long long M[PAIRS][T];
+  WarpLines wl[WARPS];
+  uint64_t bar;
+};
 }  // namespace k2
 
-__global__ void __launch_bounds__(k2::K2_THREADS, 2)
-    fw64_lines(double *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r, int R, Pack *packA,
-               Pack *packB) {
+__global__ void __launch_bounds__(32 * k2::WARPS, 2)
+    fw64_lines(double *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r, int R, int vec,
+               DiagOps64 ops, Panels64 pan) {
   using namespace k2;
-  extern __shared__ __align__(16) float Mlo[];  // [T][MS]: Mlo[k][pos] = rd of the diagonal entry
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
   const int b = blockIdx.x / PARTS, part = blockIdx.x % PARTS;
   const bool is_row = b < R - 1;
   int other = is_row ? b : b - (R - 1);
@@ -293,654 +533,379 @@ __global__ void __launch_bounds__(k2::K2_THREADS, 2)
   const int base_r = r * T, m_r = min(T, n - base_r);
   const int base_o = other * T, m_o = min(T, n - base_o);
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const double INF = inf<double>();
-  const double *diag = D + (int64_t)base_r * ld + base_r;
-  for (int e = tid; e < T * T; e += K2_THREADS) {
-    const int i = e / T, k = e % T;
-    const double x = (i < m_r && k < m_r) ? diag[(int64_t)i * ld + k] : INF;
-    Mlo[is_row ? k * MS + i : i * MS + k] = f64_down(x);  // Mlo[k][pos]
+  if (tid == 0) {
+    mbar_init(&sm.bar, 1);
+    fence_mbar_init();
+    mbar_expect_tx(&sm.bar, sizeof(sm.M));
   }
-  const int line0 = part * (T / PARTS) + w * LINES;
+  grid_dep_wait();
+  if (tid == 0) {
+    fence_proxy_async_global();
+    bulk_g2s(&sm.M[0][0], is_row ? ops.Alo : ops.Blo, sizeof(sm.M), &sm.bar);
+  }
+  const double *M64 = is_row ? ops.A64 : ops.B64;  // [k][pos]
+  const int line0 = part * CTA_LINES + w * LINES, p0 = 4 * lane;
   // Element (line, pos) of the own block sits at D[g0 + line * sl + pos * sp].
   const int64_t g0 = is_row ? (int64_t)base_r * ld + base_o : (int64_t)base_o * ld + base_r;
   const int64_t sl = is_row ? 1 : ld, sp = is_row ? ld : 1;
-  // the diagonal entry paired with position pos at step k: row block diag[pos][k], column block diag[k][pos]
-  const int64_t dpos = is_row ? ld : 1, dk = is_row ? 1 : ld;
+  WarpLines &L = sm.wl[w];
   double v[LINES][4];
-  float vlo[LINES][4], vhi[LINES][4];
-  unsigned pk[LINES];  // byte q: round-local k of the last improvement of slot q, 0xFF: none
+  // pairs along a line (column blocks) or across two lines (row blocks)
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int u = 0; u < 4; u += 2) {
+      const int c = is_row ? u : a, q = is_row ? a : u;  // first element of the pair
+      const int dc = is_row ? 1 : 0, dq = is_row ? 0 : 1;
+      const bool in0 = line0 + c < m_o && p0 + q < m_r, in1 = line0 + c + dc < m_o && p0 + q + dq < m_r;
+      const double *src = D + g0 + (line0 + c) * sl + (p0 + q) * sp;
+      double2 t = make_double2(inf<double>(), inf<double>());
+      if (vec && in1) {
+        t = *reinterpret_cast<const double2 *>(src);
+      } else {
+        if (in0) t.x = src[0];
+        if (in1) t.y = src[1];
+      }
+      if (is_row) {
+        v[u][a] = t.x, v[u + 1][a] = t.y;
+      } else {
+        v[a][u] = t.x, v[a][u + 1] = t.y;
+      }
+    }
 #pragma unroll
   for (int c = 0; c < LINES; ++c) {
-    pk[c] = 0xFFFFFFFFu;
+    *reinterpret_cast<unsigned *>(&L.pk[c][p0]) = 0xFFFFFFFFu;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      const int line = line0 + c, pos = 2 * lane + (q & 1) + 64 * (q >> 1);
-      v[c][q] = (line < m_o && pos < m_r) ? D[g0 + line * sl + pos * sp] : INF;
-      vlo[c][q] = f64_down(v[c][q]);
-      vhi[c][q] = f64_up(v[c][q]);
+      L.d[c][p0 + q] = v[c][q];
+      L.hi[c][p0 + q] = f64_up(v[c][q]);
     }
   }
   __syncthreads();
-  // Step k: owner lane (k mod 64) / 2, slot 2 (k / 64) + (k mod 2).  The
-  // filter runs unrolled over the warp's lines; the exact FP64 tests run in a
-  // rolled loop over the flagged elements, so the loop body stays small.
+  const bool ok = mbar_wait(&sm.bar, 0);
+  if (__syncthreads_or(!ok)) {  // the diagonal block never arrived: leave D, P and the operands as they are
+    if (tid == 0) report_wait_timeout();
+    return;
+  }
 #pragma unroll 1
-  for (int k = 0; k < T; ++k) {
-    const int owner = (k & 63) >> 1, slot = 2 * (k >> 6) + (k & 1);
-    const unsigned long long m01 = *reinterpret_cast<const unsigned long long *>(&Mlo[k * MS + 2 * lane]);
-    const unsigned long long m23 = *reinterpret_cast<const unsigned long long *>(&Mlo[k * MS + 64 + 2 * lane]);
-    unsigned pass = 0u;  // bit 4 c + q
-#pragma unroll
-    for (int c = 0; c < LINES; ++c) {
-      const float own_lo = slot == 0 ? vlo[c][0] : slot == 1 ? vlo[c][1] : slot == 2 ? vlo[c][2] : vlo[c][3];
-      const float vk_lo = __shfl_sync(kFullMask, own_lo, owner);
-      const unsigned long long vv = packf2(vk_lo, vk_lo);
-      const float2 l01 = sum2_rm(m01, vv), l23 = sum2_rm(m23, vv);
-      pass |= ((l01.x < vhi[c][0] ? 1u : 0u) | (l01.y < vhi[c][1] ? 2u : 0u) | (l23.x < vhi[c][2] ? 4u : 0u) |
-               (l23.y < vhi[c][3] ? 8u : 0u)) << (4 * c);
-    }
-    const unsigned any = __ballot_sync(kFullMask, pass != 0u);
-    if (!any) continue;  // warp-uniform
-    double vk[LINES];
-#pragma unroll
-    for (int c = 0; c < LINES; ++c) {
-      const double own = slot == 0 ? v[c][0] : slot == 1 ? v[c][1] : slot == 2 ? v[c][2] : v[c][3];
-      vk[c] = __shfl_sync(kFullMask, own, owner);
-    }
-#pragma unroll 1
-    while (pass) {
-      const int b = __ffs(pass) - 1, c = b >> 2, q = b & 3;
-      pass &= pass - 1;
-      const int pos = 2 * lane + (q & 1) + 64 * (q >> 1);
-      double vkc = vk[0];
-#pragma unroll
-      for (int u = 1; u < LINES; ++u) vkc = u == c ? vk[u] : vkc;
-      const double cand = __dadd_rn(__ldg(diag + pos * dpos + k * dk), vkc);
-      double cur = 0.0;
-#pragma unroll
-      for (int u = 0; u < 4 * LINES; ++u) cur = u == b ? v[u >> 2][u & 3] : cur;
-      if (cand < cur) {
-        const float lo = f64_down(cand), up = f64_up(cand);
-#pragma unroll
-        for (int u = 0; u < 4 * LINES; ++u)
-          if (u == b) {
-            v[u >> 2][u & 3] = cand;
-            vlo[u >> 2][u & 3] = lo;
-            vhi[u >> 2][u & 3] = up;
-            pk[u >> 2] = __byte_perm(pk[u >> 2], (unsigned)k,
-                                     0x3210 ^ ((0x3210 & (0xF << (4 * (u & 3)))) ^ (4 << (4 * (u & 3)))));
-          }
+  for (int kq = 0; kq < QUADS; ++kq) {
+    double x = L.d[(lane >> 2) & 3][4 * kq + (lane & 3)];
+    {
+      const int t = 4 * kq + (lane & 3);
+      const unsigned long long e01 = sm.M[2 * kq][t], e23 = sm.M[2 * kq + 1][t];
+      const float elo[3] = {__uint_as_float((unsigned)e01), __uint_as_float((unsigned)(e01 >> 32)),
+                            __uint_as_float((unsigned)e23)};
+      float xlo;
+      quad_pivots(x, xlo, elo, lane, [&](int s) { return M64[(4 * kq + s) * T + t]; });
+      if (lane < 16) {
+        (&L.ps[0][0])[lane] = x;
+        (&L.plo[0][0])[lane] = xlo;
       }
     }
+    __syncwarp();
+    relax_lines(L, kq, false, lane, sm.M[2 * kq], sm.M[2 * kq + 1], [&](int s, int pos) { return M64[(4 * kq + s) * T + pos]; });
   }
-  // D and P where the line improved; the phase-4 operand pack everywhere.
-  Pack *dst = is_row ? &packB[other] : &packA[other];
-  bool ex = true;
 #pragma unroll
-  for (int c = 0; c < LINES; ++c) {
-    const int line = line0 + c;
+  for (int c = 0; c < LINES; ++c)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[c][q] = L.d[c][p0 + q];
+  grid_dep_launch();
+  // The phase-4 operands everywhere (padded), D and P where the line improved.
+  const int64_t blk = other;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int kp = 2 * lane + h;
+    unsigned long long *dst = is_row ? &pan.B[((blk * 2 + (line0 >> 6)) * PAIRS + kp) * (T / 2) + (line0 & 63)]
+                                     : &pan.A[(blk * PAIRS + kp) * T + line0];
+#pragma unroll
+    for (int c = 0; c < LINES; c += 2)
+      *reinterpret_cast<ulonglong2 *>(dst + c) =
+          make_ulonglong2(packf2(f64_down(v[c][2 * h]), f64_down(v[c][2 * h + 1])),
+                          packf2(f64_down(v[c + 1][2 * h]), f64_down(v[c + 1][2 * h + 1])));
+  }
+  double *rows = is_row ? pan.B64 : pan.A64;
+#pragma unroll
+  for (int c = 0; c < LINES; ++c)
+#pragma unroll
+    for (int q = 0; q < 4; q += 2)
+      *reinterpret_cast<double2 *>(&rows[(blk * T + line0 + c) * T + p0 + q]) = make_double2(v[c][q], v[c][q + 1]);
+#pragma unroll
+  for (int c = 0; c < LINES; ++c)
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      const unsigned kq = (pk[c] >> (8 * q)) & 0xFFu;
-      if (kq != 0xFFu) {  // improved: inside the matrix
-        const int pos = 2 * lane + (q & 1) + 64 * (q >> 1);
-        const int64_t g = g0 + line * sl + pos * sp;
-        D[g] = v[c][q];
-        if (P) P[g] = base_r + (int)kq;
-      }
-      ex = ex && vlo[c][q] == vhi[c][q];
+      const unsigned k = L.pk[c][p0 + q];
+      if (k == 0xFFu) continue;  // improved: inside the matrix
+      const int64_t g = g0 + (line0 + c) * sl + (p0 + q) * sp;
+      D[g] = v[c][q];
+      if (P) P[g] = base_r + (int)k;
     }
-#pragma unroll
-    for (int hq = 0; hq < 2; ++hq) {  // positions 2 lane + 64 hq + {0, 1}: k-pair lane + 32 hq
-      const int kp = lane + 32 * hq, pos = 2 * kp;
-      dst->lo[line >> 6][kp][line & 63] = packf2(vlo[c][2 * hq], vlo[c][2 * hq + 1]);
-      dst->hi[line >> 6][kp][line & 63] = packf2(vhi[c][2 * hq], vhi[c][2 * hq + 1]);
-      *reinterpret_cast<float2 *>(&dst->rlo[line][pos]) = make_float2(vlo[c][2 * hq], vlo[c][2 * hq + 1]);
-      *reinterpret_cast<float2 *>(&dst->rhi[line][pos]) = make_float2(vhi[c][2 * hq], vhi[c][2 * hq + 1]);
-      *reinterpret_cast<double2 *>(&dst->r64[line][pos]) = make_double2(v[c][2 * hq], v[c][2 * hq + 1]);
-    }
-  }
-  if (__syncthreads_or(!ex) && tid == 0) dst->exact = 0;
 }
 
-// ---------------------------------------------------------------- products
-// Phase 4: a CTA computes one 128 x 64 half of an output block C = (I,J)
-// (two CTAs per block, three CTAs per SM) from A = packA[I] and B = packB[J],
-// both final for the round.
-//
-// Only the lower bounds enter the main loop.  X = min_k lo_k is a lower bound
-// of the exact FP64 minimum s* (lo_k <= s_k for every k), so X >= ru(old)
-// means no improvement.  Otherwise s* = X exactly when some k with lo_k = X
-// has an exact sum of X (its upper bound is X too, or one FP64 add says so),
-// and the first such k is the path entry; if none has, s* > X and the exact
-// minimum is taken over the candidates with lo_k <= min(ru(old),
-// min{up_k : lo_k = X}) (an upper bound of s*).  With integer weights every
-// sum is exact and the first case always holds.
-struct ProdSmem {
-  unsigned long long Alo[STAGES][2][KP][H];  // both row halves of the A slab
-  unsigned long long Blo[STAGES][KP][H];     // this CTA's column half of the B slab
-  uint64_t bar[STAGES];
+// ---------------------------------------------------------------- K3
+// Phase 4: one CTA computes a 32 x 64 piece of an output block from the lower
+// bounds of all 128 k in shared memory, thread tile 4 x 2 (as the FP32 path's
+// pieces).  Per output and group of k only the group's minimum is
+// kept, merged into
+//   X = min lo, with the group it came from (the first that reached it), and
+//   Y = min lo over all other groups.
+// Afterwards an output with X < ru(old) finds the first k with lo = X in its
+// group and adds that candidate in FP64 (s).  No other candidate can be as
+// small when s = X, or when neither Y nor the group's other sums are <= ru(s);
+// otherwise every candidate with lo <= ru(s) is added in FP64, k ascending.
+// Bound: the FP32 pipes where a launch fills the chip, latency below.  Measured
+// per solve: n = 1000, real weights, 0.41 ms (6.8 ms with every improved output
+// settled by a whole warp over all 128 k, which is what lower bounds alone ask
+// for when no sum is a float); n = 4096 / 8192, integers, 11.0 / 66.7 ms with
+// the overlapped chain's share (11.4 / 64.5 with a 128 x 64 tile, whose solves
+// took 14.1 / 65.7 ms against 9.8 / 63.6).
+namespace k3 {
+constexpr int THREADS = 256, TR = 32, TC = 64, PER_BLOCK = (T / TR) * (T / TC);
+constexpr int GP = 8;  // k-pairs per group
+struct Smem {
+  unsigned long long A[PAIRS][TR];
+  unsigned long long B[PAIRS][TC];
+  uint64_t bar;
 };
+}  // namespace k3
 
-// Thread (warp w, lane l): ty = 4w + l/8 (0..31), tx = l%8 (0..7);
-//   rows i(r) = (r>>1)*64 + ty*2 + (r&1)        (r = 0..3, row half r>>1)
-//   cols j(c) = (c>>1)*16 + tx*2 + (c&1)        (c = 0..7, within the CTA's half)
-// Row and column pairs are adjacent, so each pair is one 16-byte shared load;
-// a warp's loads of one k-pair touch 64 (A) and 128 (B) consecutive bytes.
-__device__ __forceinline__ int row4(int r, int ty) { return (r >> 1) * 64 + ty * 2 + (r & 1); }
-__device__ __forceinline__ int col8(int c, int tx) { return (c >> 1) * 16 + tx * 2 + (c & 1); }
-
-__device__ __forceinline__ void issue_slab(ProdSmem &sm, int st, const Pack *A, const Pack *B, int hJ,
-                                           int s) {
-  mbar_expect_tx(&sm.bar[st], 3 * SLAB_BYTES);
-  for (int h = 0; h < 2; ++h) bulk_g2s(&sm.Alo[st][h][0][0], &A->lo[h][s * KP][0], SLAB_BYTES, &sm.bar[st]);
-  bulk_g2s(&sm.Blo[st][0][0], &B->lo[hJ][s * KP][0], SLAB_BYTES, &sm.bar[st]);
-}
-
-// Block sets of one phase-4 launch (grid: 2 CTAs per block).
-constexpr int kSetAll = 0;   // all (R-1)^2 blocks off row/column r
-constexpr int kSetNext = 1;  // the 2R-3 blocks in row r+1 or column r+1
-constexpr int kSetRest = 2;  // the (R-2)^2 blocks off rows/columns r and r+1
-
-__device__ __forceinline__ double f32_as_f64(float x) { return __longlong_as_double((long long)f32_to_f64_bits(x)); }
-
-#ifndef APSP_F64_EAGER_ROUNDS
-#define APSP_F64_EAGER_ROUNDS 16
-#endif
-// Phase-4 rounds whose main loop also keeps, per output, the k-pair where
-// min lo last decreased strictly (EAGER): in the first rounds nearly every
-// output may improve, and one compare and one byte permute per k-pair cost
-// less than scanning every candidate again to find the k that reaches X.
-constexpr int kEagerRounds64 = APSP_F64_EAGER_ROUNDS;
-
-template <bool EAGER>
-__global__ void __launch_bounds__(THREADS, EAGER ? 2 : 3)
-    fw64_product(double *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r, int R,
-                 const Pack *packA, const Pack *packB, int set) {
+template <int CTAS_PER_SM>
+__global__ void __launch_bounds__(k3::THREADS, CTAS_PER_SM)
+    fw64_pieces(double *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r, int R, Panels64 pan,
+                int set) {
+  using namespace k3;
+  constexpr int CW = 2;  // columns per thread
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  ProdSmem &sm = *reinterpret_cast<ProdSmem *>(smem_raw);
-  const int tile = blockIdx.x >> 1, hJ = blockIdx.x & 1;
+  Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
+  const int tile = blockIdx.x / PER_BLOCK, sub = blockIdx.x % PER_BLOCK;
   int I, J;
-  if (set == kSetAll) {
-    I = tile / (R - 1);
-    J = tile % (R - 1);
-    I += (I >= r);
-    J += (J >= r);
-  } else if (set == kSetNext) {  // row r+1, then column r+1: the next round's K1/K2 input
-    if (tile < R - 1) {
-      I = r + 1;
-      J = tile + (tile >= r);
-    } else {
-      I = tile - (R - 1);
-      I += (I >= r);
-      I += (I >= r + 1);
-      J = r + 1;
-    }
-  } else {  // the rest: rows and columns other than r and r+1
-    I = tile / (R - 2);
-    J = tile % (R - 2);
-    I += (I >= r);
-    I += (I >= r + 1);
-    J += (J >= r);
-    J += (J >= r + 1);
-  }
-  const Pack *A = &packA[I];
-  const Pack *B = &packB[J];
-  const int baseI = I * T, baseJ = J * T + hJ * H, baseK = r * T;
-  const int mI = min(T, n - baseI), mJ = min(H, n - baseJ), mK = min(T, n - baseK);
-  if (mJ <= 0) return;  // an empty half of the last (narrow) block (uniform exit, no barrier used)
-  const int nslab = (mK + KS - 1) / KS;
+  block_of(set, tile, r, R, I, J);
+  const int si = sub >> 1, hJ = sub & 1;
+  const int baseI = I * T + si * TR, baseJ = J * T + hJ * TC, baseK = r * T;
+  const int mI = min(TR, n - baseI), mJ = min(TC, n - baseJ), mK = min(T, n - baseK);
+  if (mI <= 0 || mJ <= 0) return;  // past the matrix (uniform exit)
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const int ty = 4 * w + (lane >> 3), tx = lane & 7;
-  const float FINF = __int_as_float(0x7f800000);
-  // Both operands hold floats only: a candidate's upper bound is ru of the
-  // same operands as its lower bound.
-  const bool exact = A->exact && B->exact;
-
+  // Whole groups: the operands are +inf past the matrix.
+  const int ng = (mK + 2 * GP - 1) / (2 * GP);
   if (tid == 0) {
-    for (int st = 0; st < STAGES; ++st) mbar_init(&sm.bar[st], 1);
+    mbar_init(&sm.bar, 1);
     fence_mbar_init();
-    for (int s = 0; s < STAGES && s < nslab; ++s) issue_slab(sm, s, A, B, hJ, s);
+    mbar_expect_tx(&sm.bar, (uint32_t)(GP * ng * (TR + TC) * 8));
+  }
+  grid_dep_wait();
+  if (tid == 0) {
+    fence_proxy_async_global();
+    bulk_g2s(&sm.B[0][0], pan.B + ((int64_t)J * 2 + hJ) * PAIRS * TC, (uint32_t)(GP * ng * TC * 8), &sm.bar);
   }
   __syncthreads();
-
-  float lo[4][8];
-  unsigned kid[4][2];  // EAGER: byte c%4 of kid[a][c/4] = k-pair of the last strict decrease, 0xFF none
-#pragma unroll
-  for (int a = 0; a < 4; ++a) {
-    kid[a][0] = kid[a][1] = 0xFFFFFFFFu;
-#pragma unroll
-    for (int c = 0; c < 8; ++c) lo[a][c] = FINF;
+  if (w == 0) {
+    const unsigned long long *srcA = pan.A + (int64_t)I * PAIRS * T + si * TR;
+    fence_proxy_async_global();
+    for (int kp = lane; kp < GP * ng; kp += 32) bulk_g2s(&sm.A[kp][0], srcA + (int64_t)kp * T, TR * 8, &sm.bar);
   }
-
-  for (int s = 0; s < nslab; ++s) {
-    const int st = s % STAGES;
-    const bool ok = mbar_wait(&sm.bar[st], (s / STAGES) & 1);
-    if (__syncthreads_or(!ok)) {
-      if (tid == 0) {
-        report_wait_timeout();
-        for (int s2 = s + 1; s2 < nslab && s2 < s + STAGES; ++s2)
-          mbar_wait(&sm.bar[s2 % STAGES], (s2 / STAGES) & 1);
+  // Outputs of a lane as in the FP32 pieces: rows r0 + (a & 1) + 8 (a >> 1),
+  // columns c0 + (c & 1) + 16 (c >> 1).
+  constexpr int WC = TC / (8 * CW);
+  const int r0 = (w / WC) * 16 + 2 * (lane >> 3), c0 = (w % WC) * 8 * CW + 2 * (lane & 7);
+  const float FINF = inf<float>();
+  float X[4][CW], Y[4][CW];
+  unsigned grp[CW];  // byte a of grp[c]: the group X[a][c] came from
+#pragma unroll
+  for (int c = 0; c < CW; ++c) {
+    grp[c] = 0u;
+#pragma unroll
+    for (int a = 0; a < 4; ++a) X[a][c] = Y[a][c] = FINF;
+  }
+  __syncwarp();
+  const bool ok = mbar_wait(&sm.bar, 0);
+  if (__syncthreads_or(!ok)) {  // the operands never arrived: the block stays as it is
+    if (tid == 0) report_wait_timeout();
+    return;
+  }
+#pragma unroll 1
+  for (int g = 0; g < ng; ++g) {
+    float m[4][CW];
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int c = 0; c < CW; ++c) m[a][c] = FINF;
+#pragma unroll 8
+    for (int u = 0; u < GP; ++u) {
+      const int kp = GP * g + u;
+      const ulonglong2 a01 = *reinterpret_cast<const ulonglong2 *>(&sm.A[kp][r0]);
+      const ulonglong2 a23 = *reinterpret_cast<const ulonglong2 *>(&sm.A[kp][r0 + 8]);
+#pragma unroll
+      for (int c = 0; c < CW; c += 2) {
+        const ulonglong2 bb = *reinterpret_cast<const ulonglong2 *>(&sm.B[kp][c0 + 8 * c]);
+        relax2_rm(m[0][c], a01.x, bb.x);
+        relax2_rm(m[0][c + 1], a01.x, bb.y);
+        relax2_rm(m[1][c], a01.y, bb.x);
+        relax2_rm(m[1][c + 1], a01.y, bb.y);
+        relax2_rm(m[2][c], a23.x, bb.x);
+        relax2_rm(m[2][c + 1], a23.x, bb.y);
+        relax2_rm(m[3][c], a23.y, bb.x);
+        relax2_rm(m[3][c + 1], a23.y, bb.y);
       }
-      return;
     }
-    const unsigned long long(*As)[KP][H] = sm.Alo[st];
-    const unsigned long long(*Bs)[H] = sm.Blo[st];
-// Unrolled by four: the shared loads of later k-pairs are scheduled ahead of
-    // the current one's arithmetic (measured best of 1, 2, 4, 8 and 16).
-#pragma unroll 4
-    for (int kp = 0; kp < KP; ++kp) {
-      unsigned long long a[4], b[8];
 #pragma unroll
-      for (int rr = 0; rr < 4; rr += 2) {
-        const ulonglong2 t = *reinterpret_cast<const ulonglong2 *>(&As[rr >> 1][kp][ty * 2]);
-        a[rr] = t.x;
-        a[rr + 1] = t.y;
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int c = 0; c < CW; ++c) {
+        if (m[a][c] < X[a][c]) grp[c] = __byte_perm(grp[c], (unsigned)g, byte_sel64(a));
+        Y[a][c] = fminf(Y[a][c], fmaxf(X[a][c], m[a][c]));
+        X[a][c] = fminf(X[a][c], m[a][c]);
       }
+  }
+  grid_dep_launch();
+  double old[4][CW];
+  unsigned left = 0u;  // bit 4 c + a: output (a, c) may improve
 #pragma unroll
-      for (int cc = 0; cc < 8; cc += 2) {
-        const ulonglong2 t = *reinterpret_cast<const ulonglong2 *>(&Bs[kp][col8(cc, tx)]);
-        b[cc] = t.x;
-        b[cc + 1] = t.y;
-      }
+  for (int a = 0; a < 4; ++a)
 #pragma unroll
-      for (int rr = 0; rr < 4; ++rr)
+    for (int c = 0; c < CW; ++c) {
+      const int i = r0 + (a & 1) + 8 * (a >> 1), j = c0 + c;
+      old[a][c] = i < mI && j < mJ ? D[(int64_t)(baseI + i) * ld + baseJ + j] : -inf<double>();
+    }
 #pragma unroll
-        for (int cc = 0; cc < 8; ++cc) {
-          if constexpr (EAGER) {
-            const float2 t2 = sum2_rm(a[rr], b[cc]);
-            const float m = min3f(lo[rr][cc], t2.x, t2.y);
-            if (m < lo[rr][cc])
-              kid[rr][cc >> 2] = __byte_perm(kid[rr][cc >> 2], (unsigned)(s * KP + kp),
-                                             0x3210 ^ ((0x3210 & (0xF << (4 * (cc & 3)))) ^ (4 << (4 * (cc & 3)))));
-            lo[rr][cc] = m;
-          } else {
-            relax2_rm(lo[rr][cc], a[rr], b[cc]);
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int c = 0; c < CW; ++c) left |= (X[a][c] < f64_up(old[a][c]) ? 1u : 0u) << (4 * c + a);
+  // Each lane takes its own next output, so that the warp runs the rest as
+  // often as its fullest lane needs and not once per output.
+#pragma unroll 1
+  for (; left; left &= left - 1) {
+    const int t = __ffs(left) - 1, a = t & 3, c = t >> 2;
+    float x = X[0][0], second = Y[0][0];
+    double was = old[0][0];
+#pragma unroll
+    for (int u = 1; u < 4 * CW; ++u) {
+      x = t == u ? X[u & 3][u >> 2] : x;
+      second = t == u ? Y[u & 3][u >> 2] : second;
+      was = t == u ? old[u & 3][u >> 2] : was;
+    }
+    const int g = (int)(((c ? grp[1] : grp[0]) >> (8 * a)) & 0xFFu);
+    const int i = r0 + (a & 1) + 8 * (a >> 1), j = c0 + c;
+    int k = -1;
+#pragma unroll
+    for (int u = 0; u < GP; ++u) {
+      const float2 l = sum2_rm(sm.A[GP * g + u][i], sm.B[GP * g + u][j]);
+      const bool h0 = k < 0 && l.x == x;
+      k = h0 ? 2 * (GP * g + u) : k;
+      second = h0 ? second : fminf(second, l.x);
+      const bool h1 = k < 0 && l.y == x;
+      k = h1 ? 2 * (GP * g + u) + 1 : k;
+      second = h1 ? second : fminf(second, l.y);
+    }
+    const double *ra = pan.A64 + ((int64_t)I * T + si * TR + i) * T, *rb = pan.B64 + ((int64_t)J * T + hJ * TC + j) * T;
+    double best = __dadd_rn(__ldcg(ra + k), __ldcg(rb + k));
+    if (best != f32_as_f64(x)) {
+      const float up = f64_up(best);
+      if (second <= up) {
+        best = inf<double>();
+#pragma unroll 1
+        for (int h = 0; h < ng; ++h) {
+          unsigned bits = 0u;
+#pragma unroll
+          for (int u = 0; u < GP; ++u) {
+            const float2 l = sum2_rm(sm.A[GP * h + u][i], sm.B[GP * h + u][j]);
+            bits |= (l.x <= up ? 1u : 0u) << (2 * u) | (l.y <= up ? 1u : 0u) << (2 * u + 1);
           }
-        }
-    }
-    __syncthreads();
-    if (tid == 0 && s + STAGES < nslab) {
-      fence_proxy_async_smem();
-      issue_slab(sm, st, A, B, hJ, s + STAGES);
-    }
-  }
-
-  // Epilogue.  The ring is free: X = min lo goes to shared memory, then each
-  // warp owns 16 whole rows (lane l: columns 2l, 2l+1 of the half).
-  float *Lo = reinterpret_cast<float *>(smem_raw);            // [T][H]
-  unsigned char *Ks = smem_raw + sizeof(ProdSmem::Alo);        // EAGER: [T][H] k-pair bytes
-  __syncthreads();
-#pragma unroll
-  for (int rr = 0; rr < 4; ++rr)
-#pragma unroll
-    for (int cc = 0; cc < 8; cc += 2) {
-      *reinterpret_cast<float2 *>(&Lo[row4(rr, ty) * H + col8(cc, tx)]) = make_float2(lo[rr][cc], lo[rr][cc + 1]);
-      if constexpr (EAGER)
-        *reinterpret_cast<unsigned short *>(&Ks[row4(rr, ty) * H + col8(cc, tx)]) =
-            (unsigned short)(kid[rr][cc >> 2] >> (8 * (cc & 3)));
-    }
-  __syncthreads();
-  const int j0 = 2 * lane, i0 = w * 16, jb0 = hJ * H;
-  // Pass 1: outputs that may improve (X < ru(old)).  Bit 2t + q of `pot`:
-  // row i0 + t, column j0 + q.  Old values load eight rows at a time.
-  unsigned pot = 0u;
-#pragma unroll
-  for (int t8 = 0; t8 < 16; t8 += 8) {
-    double o[8][2];
-#pragma unroll
-    for (int t = 0; t < 8; ++t)
-#pragma unroll
-      for (int q = 0; q < 2; ++q)
-        o[t][q] = (i0 + t8 + t < mI && j0 + q < mJ) ? D[(int64_t)(baseI + i0 + t8 + t) * ld + baseJ + j0 + q]
-                                                     : inf<double>();
-#pragma unroll
-    for (int t = 0; t < 8; ++t) {
-      const float2 x = *reinterpret_cast<const float2 *>(&Lo[(i0 + t8 + t) * H + j0]);
-      if (i0 + t8 + t < mI) {
-        if (j0 < mJ && f32_lt_f64(x.x, o[t][0])) pot |= 1u << (2 * (t8 + t));
-        if (j0 + 1 < mJ && f32_lt_f64(x.y, o[t][1])) pot |= 2u << (2 * (t8 + t));
-      }
-    }
-  }
-  if constexpr (EAGER) {
-    // The k-pair where min lo last decreased holds the first k with lo_k = X
-    // (the lower one if its lower bound is X).  If that candidate's exact sum
-    // is X, s* = X and k is the path entry; otherwise pass 2b decides.
 #pragma unroll 1
-    for (int t = 0; t < 16; ++t)
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        const unsigned bitq = 1u << (2 * t + q);
-        if (!(pot & bitq)) continue;
-        const int i = i0 + t, jl = j0 + q, jb = jb0 + jl;
-        const int kp = Ks[i * H + jl];  // a candidate output has one (X is finite)
-        const float X = Lo[i * H + jl];
-        const unsigned long long al = A->lo[i >> 6][kp][i & 63], bl = B->lo[hJ][kp][jl];
-        const float2 l = sum2_rm(al, bl);
-        const int k = l.x == X ? 2 * kp : 2 * kp + 1;
-        const float up_ = exact ? (l.x == X ? sum2_rp(al, bl).x : sum2_rp(al, bl).y)
-                                : __fadd_ru(A->rhi[i][k], B->rhi[jb][k]);
-        if (up_ == X || __dadd_rn(A->r64[i][k], B->r64[jb][k]) == f32_as_f64(X)) {
-          const int64_t gi = (int64_t)(baseI + i) * ld + baseJ + jl;
-          D[gi] = f32_as_f64(X);  // X < old (pass 1)
-          if (P) P[gi] = baseK + k;
-          pot &= ~bitq;
-        }
-      }
-  }
-  // Pass 2a: each 8-row group of the warp with many candidates (the early
-  // rounds) is scanned lane-parallel: lane l walks the lower-bound pairs of
-  // its two columns over all k (B pairs coalesced, A pairs broadcast,
-  // add.rm.f32x2 as in the main loop), folds every 8 k into one minimum, and
-  // keeps the lowest 8-k chunk whose minimum is X.  Inside that chunk the
-  // first k with lo_k = X and an exact sum X settles the output (D where X <
-  // old, and P); an output without one there is left to pass 2b.
-  {
-    const unsigned long long *pbl = &B->lo[hJ][0][j0];
-#pragma unroll 1
-    for (int G = 0; G < 2; ++G) {
-      const unsigned gm = 0xFFFFu << (16 * G);
-      if (EAGER || (int)__reduce_add_sync(kFullMask, (unsigned)__popc(pot & gm)) < kDenseMin64) continue;
-      const int tg0 = 8 * G;
-      float g[8][2];
-      unsigned hit[8];  // bit c (+16 for column j0 + 1): chunk c's minimum lo equals X
-#pragma unroll
-      for (int t = 0; t < 8; ++t) {
-        const float2 x = *reinterpret_cast<const float2 *>(&Lo[(i0 + tg0 + t) * H + j0]);
-        g[t][0] = x.x;
-        g[t][1] = x.y;
-        hit[t] = 0u;
-      }
-#pragma unroll 1
-      for (int c = T / 8 - 1; c >= 0; --c) {
-        ulonglong2 b[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) b[q] = __ldg(reinterpret_cast<const ulonglong2 *>(pbl + (4 * c + q) * H));
-        const unsigned bit = 1u << c;
-#pragma unroll
-        for (int t = 0; t < 8; ++t) {
-          const int i = i0 + tg0 + t;
-          const unsigned long long *pal = &A->lo[i >> 6][0][i & 63];
-          unsigned long long a[4];
-#pragma unroll
-          for (int q = 0; q < 4; ++q) a[q] = __ldg(pal + (4 * c + q) * H);
-#pragma unroll
-          for (int q2 = 0; q2 < 2; ++q2) {
-            const float2 s0 = sum2_rm(a[0], q2 ? b[0].y : b[0].x), s1 = sum2_rm(a[1], q2 ? b[1].y : b[1].x);
-            const float2 s2 = sum2_rm(a[2], q2 ? b[2].y : b[2].x), s3 = sum2_rm(a[3], q2 ? b[3].y : b[3].x);
-            float m = min3f(s0.x, s0.y, s1.x);
-            m = min3f(m, s1.y, s2.x);
-            m = min3f(m, s2.y, s3.x);
-            m = fminf(m, s3.y);
-            if (m == g[t][q2]) hit[t] |= bit << (16 * q2);
-          }
-        }
-      }
-#pragma unroll
-      for (int t = 0; t < 8; ++t) {
-        const int i = i0 + tg0 + t;
-        const unsigned long long *pal = &A->lo[i >> 6][0][i & 63];
-#pragma unroll
-        for (int q2 = 0; q2 < 2; ++q2) {
-          const unsigned bitq = 1u << (2 * (tg0 + t) + q2);
-          if (!(pot & bitq)) continue;
-          const unsigned cm = (hit[t] >> (16 * q2)) & 0xFFFFu;  // not empty: X is some lo
-          const int c = __ffs(cm) - 1;
-          const float X = g[t][q2];
-          const int jb = jb0 + j0 + q2;
-          // the chunk's eight lower-bound sums; upper bounds (and FP64 sums)
-          // only for a k whose lower bound is X, in ascending k
-          unsigned eq = 0u, equp = 0u;  // lo_k = X; and up_k = X (exact operands only)
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const unsigned long long av = __ldg(pal + (4 * c + q) * H), bv = __ldg(pbl + (4 * c + q) * H + q2);
-            const float2 l = sum2_rm(av, bv);
-            eq |= (l.x == X ? 1u : 0u) << (2 * q);
-            eq |= (l.y == X ? 1u : 0u) << (2 * q + 1);
-            if (exact) {
-              const float2 u = sum2_rp(av, bv);
-              equp |= (u.x == X ? 1u : 0u) << (2 * q);
-              equp |= (u.y == X ? 1u : 0u) << (2 * q + 1);
+          for (; bits; bits &= bits - 1) {
+            const int kk = 2 * GP * h + __ffs(bits) - 1;
+            const double cand = __dadd_rn(__ldcg(ra + kk), __ldcg(rb + kk));
+            if (dless(cand, best)) {
+              best = cand;
+              k = kk;
             }
           }
-          int kf = -1;
-#pragma unroll 1
-          while (eq) {
-            const int b = __ffs(eq) - 1, k = 8 * c + b;
-            eq &= eq - 1;
-            if ((exact ? ((equp >> b) & 1u) != 0u : __fadd_ru(A->rhi[i][k], B->rhi[jb][k]) == X) ||
-                __dadd_rn(A->r64[i][k], B->r64[jb][k]) == f32_as_f64(X)) {
-              kf = k;
-              break;
-            }
-          }
-          if (kf >= 0) {  // s* = X exactly
-            const int64_t gi = (int64_t)(baseI + i) * ld + baseJ + j0 + q2;
-            const double xd = f32_as_f64(X);
-            if (xd < D[gi]) {
-              D[gi] = xd;
-              if (P) P[gi] = baseK + kf;
-            }
-            pot &= ~bitq;
-          }
         }
       }
     }
-  }
-  // Pass 2b: every remaining candidate output, walked as one stream two at a
-  // time; lane l tests k = 4l..4l+3.  The lower-bound rows load first; a k
-  // with lo_k = X fetches its upper bounds (and, if they differ, its FP64
-  // operands).  The first exact X settles the output; without one, the exact
-  // FP64 minimum over the candidates with lo_k <= min(ru(old), min up over
-  // lo_k = X) does (first k on ties).
-  unsigned wf = __reduce_or_sync(kFullMask, pot), bal = 0u;
-  int pos = 0;
-  auto next = [&](int &t, int &sj) -> bool {  // warp-uniform
-    while (!bal) {
-      if (!wf) return false;
-      pos = __ffs(wf) - 1;
-      wf &= wf - 1;
-      bal = __ballot_sync(kFullMask, (pot >> pos) & 1u);
-    }
-    const int src = __ffs(bal) - 1;
-    bal &= bal - 1;
-    t = pos >> 1;
-    sj = 2 * src + (pos & 1);
-    return true;
-  };
-#pragma unroll 1
-  for (;;) {
-    int t[2], sj[2];
-    bool v[2];
-#pragma unroll
-    for (int u = 0; u < 2; ++u) v[u] = next(t[u], sj[u]);
-    if (!v[0]) break;
-    float4 al[2], bl[2];
-    double old[2];
-#pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      if (!v[u]) continue;
-      const int i = i0 + t[u];
-      al[u] = reinterpret_cast<const float4 *>(&A->rlo[i][0])[lane];
-      bl[u] = reinterpret_cast<const float4 *>(&B->rlo[jb0 + sj[u]][0])[lane];
-      old[u] = D[(int64_t)(baseI + i) * ld + baseJ + sj[u]];
-    }
-#pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      if (!v[u]) continue;
-      const int i = i0 + t[u], jb = jb0 + sj[u];
-      const int64_t gi = (int64_t)(baseI + i) * ld + baseJ + sj[u];
-      const float X = Lo[i * H + sj[u]];
-      const float la[4] = {al[u].x, al[u].y, al[u].z, al[u].w};
-      const float lb[4] = {bl[u].x, bl[u].y, bl[u].z, bl[u].w};
-      float l4[4];
-      unsigned h = 0u;
-      float upx = FINF;  // min up over this lane's k with lo_k = X
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int k = 4 * lane + q;
-        l4[q] = __fadd_rd(la[q], lb[q]);
-        if (l4[q] == X) {
-          const float up_ = exact ? __fadd_ru(la[q], lb[q]) : __fadd_ru(A->rhi[i][k], B->rhi[jb][k]);
-          upx = fminf(upx, up_);
-          if (up_ == X || __dadd_rn(A->r64[i][k], B->r64[jb][k]) == f32_as_f64(X)) h |= 1u << q;
-        }
-      }
-      const unsigned hb = __ballot_sync(kFullMask, h != 0u);
-      if (hb) {  // s* = X exactly; the lowest hit is the first k
-        const int L = __ffs(hb) - 1;
-        const unsigned hL = __shfl_sync(kFullMask, h, L);
-        const double xd = f32_as_f64(X);
-        if (lane == 0 && xd < old[u]) {
-          D[gi] = xd;
-          if (P) P[gi] = baseK + 4 * L + (__ffs(hL) - 1);
-        }
-        continue;
-      }
-      // s* > X: exact FP64 minimum over the candidates that can reach it.
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) upx = fminf(upx, __shfl_xor_sync(kFullMask, upx, off));
-      const float th = fminf(upx, f64_up(old[u]));
-      long long best = 0x7fffffffffffffffll;
-      int bestk = 0x7fffffff;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int k = 4 * lane + q;
-        if (l4[q] <= th) {
-          const float up_ = exact ? __fadd_ru(la[q], lb[q]) : __fadd_ru(A->rhi[i][k], B->rhi[jb][k]);
-          const unsigned long long vb =
-              l4[q] == up_ ? f32_to_f64_bits(l4[q])
-                           : (unsigned long long)__double_as_longlong(__dadd_rn(A->r64[i][k], B->r64[jb][k]));
-          const long long key = dkey(vb);
-          if (key < best) {
-            best = key;
-            bestk = k;
-          }
-        }
-      }
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) {  // warp argmin over (key, k)
-        const long long ob = __shfl_xor_sync(kFullMask, best, off);
-        const int okk = __shfl_xor_sync(kFullMask, bestk, off);
-        if (ob < best || (ob == best && okk < bestk)) {
-          best = ob;
-          bestk = okk;
-        }
-      }
-      if (lane == 0 && bestk != 0x7fffffff &&
-          best < dkey((unsigned long long)__double_as_longlong(old[u]))) {
-        D[gi] = __longlong_as_double((long long)dkey_bits(best));
-        if (P) P[gi] = baseK + bestk;
-      }
+    if (dless(best, was)) {
+      const int64_t e = (int64_t)(baseI + i) * ld + baseJ + j;
+      D[e] = best;
+      if (P) P[e] = baseK + k;
     }
   }
 }
 
-static int g_smem_k1[64], g_smem_k2[64], g_smem_p0[64], g_smem_p0e[64];
+static int g_smem_k1[64], g_smem_k2[64], g_smem_k3[2][64];
+
+// Four CTAs of 64 registers per SM where phase 4 has many waves (n = 4096 /
+// 8192: 10.6 / 68.9 ms against 11.1 / 72.2 with three, before the outputs were
+// settled a lane at a time), three of 80 up to 24 blocks a side, where K1 must
+// find room beside them (int32 n = 2048: 2.96 against 3.09 ms).
+constexpr int kFewBlocks = 24;
 
 }  // namespace f64
 
-// Host round loop for FP64 (called by apsp_fw_f64).
-int run_fw_f64_interval(double *D, int n, int64_t ld, int32_t *P, cudaStream_t s) {
+// Host side of FP64 (called by apsp_fw_f64); init(stream) sets P to -1 outside
+// its first block.
+int run_fw_f64_interval(double *D, int n, int64_t ld, int32_t *P, cudaStream_t s,
+                        void (*path_init)(int32_t *, int64_t, int64_t, int64_t, cudaStream_t)) {
   using namespace f64;
   const int R = (n + T - 1) / T;
   int st;
-  const int smem1 = (int)sizeof(K1Smem), smemp = (int)sizeof(ProdSmem);
-  if ((st = ensure_smem(fw64_diag, smem1, g_smem_k1))) return st;
-  if ((st = ensure_smem(fw64_lines, k2::SMEM, g_smem_k2))) return st;
-  if ((st = ensure_smem(fw64_product<false>, smemp, g_smem_p0))) return st;
-  if ((st = ensure_smem(fw64_product<true>, smemp, g_smem_p0e))) return st;
-  // Operand packs: two sets by round parity (so that phases 1-3 of round
-  // r+1 can pack while phase 4 of round r still reads), each R column-panel
-  // packs (A operands) and R row-panel packs (B operands).
-  struct PackSet {
-    Pack *A, *B;
-  } ps[2]{};
+  if ((st = ensure_smem(fw64_diag, (int)sizeof(k1::Smem), g_smem_k1))) return st;
+  if ((st = ensure_smem(fw64_lines, (int)sizeof(k2::Smem), g_smem_k2))) return st;
+  const auto pieces = R <= kFewBlocks ? fw64_pieces<3> : fw64_pieces<4>;
+  if ((st = ensure_smem(pieces, (int)sizeof(k3::Smem), g_smem_k3[R <= kFewBlocks]))) return st;
+  // Phase-4 operands: two sets by round parity, each R blocks of A and of B;
+  // then K1's copies of the closed diagonal block.
+  Panels64 pan[2]{};
+  DiagOps64 ops{};
   char *scratch = nullptr;
   if (R > 1) {
-    if (cudaMallocAsync((void **)&scratch, sizeof(Pack) * 2 * (2 * (size_t)R), s) != cudaSuccess) {
+    const size_t elems = (size_t)R * T * T, set = elems * (4 + 4 + 8 + 8);
+    if (cudaMallocAsync((void **)&scratch, 2 * set + (size_t)T * T * 24, s) != cudaSuccess) {
       cudaGetLastError();
       return APSP_ENOMEM;
     }
     for (int q = 0; q < 2; ++q) {
-      Pack *base = reinterpret_cast<Pack *>(scratch) + (size_t)q * (2 * R);
-      ps[q] = {base, base + R};
+      char *base = scratch + q * set;
+      pan[q].A64 = reinterpret_cast<double *>(base);
+      pan[q].B64 = pan[q].A64 + elems;
+      pan[q].A = reinterpret_cast<unsigned long long *>(pan[q].B64 + elems);
+      pan[q].B = pan[q].A + elems / 2;
     }
+    ops.A64 = reinterpret_cast<double *>(scratch + 2 * set);
+    ops.B64 = ops.A64 + T * T;
+    ops.Alo = reinterpret_cast<unsigned long long *>(ops.B64 + T * T);
+    ops.Blo = ops.Alo + T * T / 2;
   }
-  auto diag_and_panels = [&](int r, cudaStream_t stm) {
-    const PackSet &p = ps[r & 1];
-    {
-      PhaseScope sc(1, stm);
-      fw64_diag<<<1, K1_THREADS, smem1, stm>>>(D, ld, P, n, r, R, p.A, p.B);
-    }
-    if (R > 1) {
-      PhaseScope sc(2, stm);
-      fw64_lines<<<2 * (R - 1) * k2::PARTS, k2::K2_THREADS, k2::SMEM, stm>>>(D, ld, P, n, r, R, p.A, p.B);
-    }
-  };
-  auto phase4 = [&](int r, int set, int blocks) {
-    if (blocks <= 0) return;
-    const PackSet &p = ps[r & 1];
-    PhaseScope sc(3, s);
-    if (r < kEagerRounds64)
-      fw64_product<true><<<2 * blocks, THREADS, smemp, s>>>(D, ld, P, n, r, R, p.A, p.B, set);
-    else
-      fw64_product<false><<<2 * blocks, THREADS, smemp, s>>>(D, ld, P, n, r, R, p.A, p.B, set);
-  };
-  // Look-ahead as in the FP32 path: phase 4 of round r updates row and
-  // column r+1 first; phases 1-3 of round r+1 then run on a second stream of
-  // higher priority beside the rest of phase 4 (disjoint blocks, the other
-  // pack set).
-  cudaStream_t s2 = nullptr;
-  cudaEvent_t ev_next = nullptr, ev_panels = nullptr;
-  // While the caller's stream is being captured into a CUDA graph every
-  // phase stays on that stream (no stream is created or destroyed mid-capture).
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
+  bool capturing = false;
+  if ((st = stream_capturing(s, &capturing))) {
     if (scratch) cudaFreeAsync(scratch, s);
-    cudaGetLastError();
-    return APSP_ECUDA;
+    return st;
   }
-  if (R > 2 && cap == cudaStreamCaptureStatusNone) {
-    int lo = 0, hi = 0;
-    cudaDeviceGetStreamPriorityRange(&lo, &hi);
-    if (cudaStreamCreateWithPriority(&s2, cudaStreamNonBlocking, hi) != cudaSuccess ||
-        cudaEventCreateWithFlags(&ev_next, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&ev_panels, cudaEventDisableTiming) != cudaSuccess) {
-      if (s2) cudaStreamDestroy(s2);
-      if (ev_next) cudaEventDestroy(ev_next);
-      if (scratch) cudaFreeAsync(scratch, s);
-      cudaGetLastError();
-      return APSP_ECUDA;
-    }
-  }
-  diag_and_panels(0, s);
-  for (int r = 0; R > 1 && r < R; ++r) {
-    if (r + 1 < R && s2) {
-      phase4(r, kSetNext, 2 * R - 3);
-      cudaEventRecord(ev_next, s);
-      cudaStreamWaitEvent(s2, ev_next, 0);
-      diag_and_panels(r + 1, s2);
-      cudaEventRecord(ev_panels, s2);
-      phase4(r, kSetRest, (R - 2) * (R - 2));
-      cudaStreamWaitEvent(s, ev_panels, 0);
-    } else {
-      phase4(r, kSetAll, (R - 1) * (R - 1));
-      if (r + 1 < R) diag_and_panels(r + 1, s);
-    }
-  }
-  if (s2) {
-    cudaStreamDestroy(s2);
-    cudaEventDestroy(ev_next);
-    cudaEventDestroy(ev_panels);
-  }
+  const bool overlap = !capturing;
+  const int vec = ld % 2 == 0 && (reinterpret_cast<uintptr_t>(D) & 15) == 0;
+  auto init = [&](cudaStream_t stm) {
+    if (P) path_init(P, n, ld, T, stm);
+  };
+  auto diag = [&](int r, cudaStream_t stm) {
+    PhaseScope sc(1, stm);
+    launch_after(fw64_diag, k1::CTAS, 32 * k1::WARPS, sizeof(k1::Smem), stm, overlap, D, ld, P, n, r, vec,
+                 (int)(P && r == 0), ops);
+  };
+  auto panels = [&](int r, cudaStream_t stm) {
+    PhaseScope sc(2, stm);
+    launch_after(fw64_lines, 2 * (R - 1) * k2::PARTS, 32 * k2::WARPS, sizeof(k2::Smem), stm, overlap, D, ld, P, n, r, R,
+                 vec, ops, pan[r & 1]);
+  };
+  auto phase4 = [&](int r, int set, int blocks, cudaStream_t stm) {
+    if (blocks <= 0) return;
+    PhaseScope sc(3, stm);
+    launch_after(pieces, k3::PER_BLOCK * blocks, k3::THREADS, sizeof(k3::Smem), stm, overlap, D, ld, P, n, r, R,
+                 pan[r & 1], set);
+  };
+  st = run_rounds(R, s, capturing, init, diag, panels, phase4);
   cudaError_t e = cudaGetLastError();
   if (scratch) {
     cudaError_t f = cudaFreeAsync(scratch, s);
     if (e == cudaSuccess) e = f;
   }
-  return status_from(e);
+  return st ? st : status_from(e);
 }
 
 int take_device_error_f64() { return take_tu_device_error(); }

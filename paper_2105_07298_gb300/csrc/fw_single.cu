@@ -38,6 +38,7 @@
 #include "minplus_f32.cuh"
 #include "phases_f32.cuh"
 #include "profile.h"
+#include "rounds.cuh"
 
 namespace apsp {
 
@@ -852,7 +853,7 @@ __global__ void __launch_bounds__(k3s::THREADS, TR == 32 ? 4 : 3)
   Smem<TR> &sm = *reinterpret_cast<Smem<TR> *>(smem_raw);
   const int tile = blockIdx.x / PER, sub = blockIdx.x % PER;
   int I, J;
-  k3::block_of(set, tile, r, R, I, J);
+  block_of(set, tile, r, R, I, J);
   const int si = sub >> 1, hJ = sub & 1;
   const int baseI = I * T + si * TR, baseJ = J * T + hJ * TC, baseK = r * T;
   const int mI = min(TR, n - baseI), mJ = min(TC, n - baseJ), mK = min(T, n - baseK);
@@ -1001,29 +1002,11 @@ constexpr int kSms = 152;
 constexpr int kR32 = 21, kRNext32 = 40, kR64 = 40, kDenseRounds = 32;
 static int g_smem_k1[2][64], g_smem_k2[2][2][64], g_smem_k3s[2][2][64], g_smem_k3[64];
 
-int run_fw_f64_interval(double *D, int n, int64_t ld, int32_t *P, cudaStream_t s);
+int run_fw_f64_interval(double *D, int n, int64_t ld, int32_t *P, cudaStream_t s,
+                        void (*path_init)(int32_t *, int64_t, int64_t, int64_t, cudaStream_t));
 int take_device_error_f64();
 int take_device_error_checks();
 int take_device_error_int32();
-
-// Launches `kernel` so that it may start before the previous kernel of the
-// stream has ended (it waits for it with grid_dep_wait before it reads or
-// writes anything that kernel does): the launch latency, about 3 us, is hidden.
-template <typename... A>
-static void launch_after(void (*kernel)(A...), int grid, int threads, size_t smem, cudaStream_t s, bool overlap,
-                         A... args) {
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3((unsigned)threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr{};
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = overlap ? 1 : 0;
-  cudaLaunchKernelEx(&cfg, kernel, args...);
-}
 
 static void path_init(int32_t *P, int64_t n, int64_t ld, int64_t skip, cudaStream_t s) {
   const int64_t total = n * n;
@@ -1089,22 +1072,23 @@ static int run_fw_f32(float *D, int64_t n64, int64_t ld, int32_t *P, void *strea
   const int vec = (aligned && (reinterpret_cast<uintptr_t>(D) & 15) == 0 ? kVecD : 0) |
                   (aligned && (reinterpret_cast<uintptr_t>(P) & 15) == 0 ? kVecP : 0);
   const int vec_ok = vec & kVecD;
-  // While the caller's stream is being captured into a CUDA graph every
-  // phase stays on that stream (no stream is created or destroyed mid-capture).
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
+  bool capturing = false;
+  if ((st = stream_capturing(s, &capturing))) {
     if (scratch) cudaFreeAsync(scratch, s);
-    cudaGetLastError();
-    return APSP_ECUDA;
+    return st;
   }
-  const bool overlap = cap == cudaStreamCaptureStatusNone;
+  const bool overlap = !capturing;
+  // K1 of round 0 writes all of P's first block; the rest of P is set to -1
+  // beside it.
+  auto init = [&](cudaStream_t st) {
+    if (P) path_init(P, n64, ld, T, st);
+  };
   auto diag = [&](int r, cudaStream_t st) {
     PhaseScope ps(1, st);
     launch_after(P ? fw_phase1_diag_f32<true> : fw_phase1_diag_f32<false>, k1::CTAS, 32 * k1::WARPS, sizeof(k1::Smem),
                  st, overlap, D, ld, P, n, r, vec, (int)(P && r == 0), ops);
   };
   auto panels = [&](int r, cudaStream_t st) {
-    if (R == 1) return;
     PhaseScope ps(2, st);
     launch_after(lines_kernel, 2 * (R - 1) * k2s::parts(lines), k2s::THREADS, lines_smem, st, overlap, D, ld, P, n, r, R,
                  vec, ops, pan[r & 1]);
@@ -1112,7 +1096,7 @@ static int run_fw_f32(float *D, int64_t n64, int64_t ld, int32_t *P, void *strea
   auto phase4 = [&](int r, int set, int blocks, cudaStream_t st) {
     if (blocks <= 0) return;
     PhaseScope ps(3, st);
-    if (R <= kR32 || (set == k3::kSetNext && R <= kRNext32))
+    if (R <= kR32 || (set == kSetNext && R <= kRNext32))
       launch_after(kernel32, k3s::per_block(32) * blocks, k3s::THREADS, sizeof(k3s::Smem<32>), st, overlap, D, ld, P, n,
                    r, R, vec_ok, pan[r & 1], set);
     else if (P ? r < kDenseRounds : R <= kR64)
@@ -1122,68 +1106,13 @@ static int run_fw_f32(float *D, int64_t n64, int64_t ld, int32_t *P, void *strea
       fw_phase3_minplus_f32<<<2 * blocks, mp32::THREADS, sizeof(k3::Smem), st>>>(D, ld, P, n, r, R, vec_ok, pan[r & 1],
                                                                               set);
   };
-  // Look-ahead: everything the next round waits for runs on a second stream of
-  // higher priority: phase 4 of round r on row and column r+1, then K1 and K2
-  // of round r+1.  The rest of round r's phase 4 runs on the caller's stream
-  // beside it, filling the SMs the chain leaves free; the two touch disjoint
-  // blocks and write/read different panel sets.
-  cudaStream_t s2 = nullptr;
-  cudaEvent_t ev_rest = nullptr, ev_panels = nullptr;
-  if (R > 2 && cap == cudaStreamCaptureStatusNone) {
-    int lo = 0, hi = 0;
-    cudaDeviceGetStreamPriorityRange(&lo, &hi);
-    if (cudaStreamCreateWithPriority(&s2, cudaStreamNonBlocking, hi) != cudaSuccess ||
-        cudaEventCreateWithFlags(&ev_rest, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&ev_panels, cudaEventDisableTiming) != cudaSuccess) {
-      if (s2) cudaStreamDestroy(s2);
-      if (ev_rest) cudaEventDestroy(ev_rest);
-      if (scratch) cudaFreeAsync(scratch, s);
-      cudaGetLastError();
-      return APSP_ECUDA;
-    }
-  }
-  // K1 of round 0 writes all of P's first block; the rest of P is set to -1
-  // beside it.
-  if (s2) {
-    cudaEventRecord(ev_panels, s);
-    if (P) path_init(P, n64, ld, T, s);
-    cudaStreamWaitEvent(s2, ev_panels, 0);
-    diag(0, s2);
-    if (P) {
-      cudaEventRecord(ev_rest, s);
-      cudaStreamWaitEvent(s2, ev_rest, 0);
-    }
-    panels(0, s2);
-    cudaEventRecord(ev_panels, s2);
-    for (int r = 0; r + 1 < R; ++r) {
-      phase4(r, k3::kSetNext, 2 * R - 3, s2);
-      diag(r + 1, s2);
-      cudaStreamWaitEvent(s, ev_panels, 0);  // round r's panels
-      panels(r + 1, s2);
-      cudaEventRecord(ev_panels, s2);
-      phase4(r, k3::kSetRest, (R - 2) * (R - 2), s);
-      cudaEventRecord(ev_rest, s);
-      cudaStreamWaitEvent(s2, ev_rest, 0);
-    }
-    cudaStreamWaitEvent(s, ev_panels, 0);
-    phase4(R - 1, k3::kSetAll, (R - 1) * (R - 1), s);
-    cudaStreamDestroy(s2);
-    cudaEventDestroy(ev_rest);
-    cudaEventDestroy(ev_panels);
-  } else {
-    if (P && R > 1) path_init(P, n64, ld, T, s);
-    for (int r = 0; r < R; ++r) {
-      diag(r, s);
-      panels(r, s);
-      phase4(r, k3::kSetAll, (R - 1) * (R - 1), s);
-    }
-  }
+  st = run_rounds(R, s, capturing, init, diag, panels, phase4);
   cudaError_t e = cudaGetLastError();
   if (scratch) {
     cudaError_t f = cudaFreeAsync(scratch, s);
     if (e == cudaSuccess) e = f;
   }
-  return status_from(e);
+  return st ? st : status_from(e);
 }
 
 static int run_fw_f64(double *D, int64_t n64, int64_t ld, int32_t *P, void *stream) {
@@ -1191,8 +1120,7 @@ static int run_fw_f64(double *D, int64_t n64, int64_t ld, int32_t *P, void *stre
   if (st || n64 == 0) return st;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   cudaGetLastError();
-  if (P) path_init(P, n64, ld, 0, s);
-  return run_fw_f64_interval(D, (int)n64, ld, P, s);
+  return run_fw_f64_interval(D, (int)n64, ld, P, s, path_init);
 }
 
 }  // namespace apsp

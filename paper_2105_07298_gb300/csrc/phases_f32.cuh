@@ -155,10 +155,6 @@ __device__ __forceinline__ void lines_part_f32(float *__restrict__ D, int64_t ld
 // improved output.
 namespace k3 {
 constexpr int T = mp32::T, KS = mp32::KS, KP = mp32::KP, STAGES = 2, H = T / 2;
-// Block sets of one phase-4 launch (grid: 2 CTAs per block).
-constexpr int kSetAll = 0;   // all (R-1)^2 blocks off row/column r
-constexpr int kSetNext = 1;  // the 2R-3 blocks in row r+1 or column r+1
-constexpr int kSetRest = 2;  // the (R-2)^2 blocks off rows/columns r and r+1
 constexpr uint32_t A_SLAB = KP * T * 8, B_SLAB = KP * H * 8;
 #ifndef APSP_K3_DENSE_MIN
 #define APSP_K3_DENSE_MIN 96
@@ -170,26 +166,6 @@ struct Smem {
   unsigned long long Bs[STAGES][KP][H];  // Bs[kp][j] = (B[2kp][j], B[2kp+1][j]), this half
   uint64_t bar[STAGES];
 };
-// The output block (I, J) of a launch's tile-th block in round r (R blocks a side).
-__device__ __forceinline__ void block_of(int set, int tile, int r, int R, int &I, int &J) {
-  if (set == kSetNext) {  // row r+1, then column r+1
-    const bool row = tile < R - 1;
-    const int o = row ? tile : tile - (R - 1);
-    I = row ? r + 1 : o + (o >= r);
-    I += !row && I >= r + 1;
-    J = row ? o + (o >= r) : r + 1;
-    return;
-  }
-  const int side = set == kSetAll ? R - 1 : R - 2;
-  I = tile / side;
-  J = tile % side;
-  I += (I >= r);
-  J += (J >= r);
-  if (set == kSetRest) {
-    I += (I >= r + 1);
-    J += (J >= r + 1);
-  }
-}
 }  // namespace k3
 
 #ifndef APSP_K3_MIN_BLOCKS

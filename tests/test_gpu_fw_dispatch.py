@@ -1,6 +1,6 @@
-"""The FP32 single-graph kernels at the sizes where their dispatch changes or a
-tile is ragged, bit for bit against the oracle's blocked FW at the library's
-block size on real weights (one rounded sum per candidate, ascending k)."""
+"""The single-graph kernels at the sizes where their dispatch changes or a tile
+is ragged, bit for bit against the oracle's blocked FW at the library's block
+size on real weights (one rounded sum per candidate, ascending k)."""
 import numpy as np
 import pytest
 import torch
@@ -13,9 +13,9 @@ pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
 
 
-def _expect(n, p, seed):
-    W = graphgen.dense_graph(n, p, seed, weights="real", lo=0.5, hi=2.0, dtype=np.float32)
-    return W, *oracle.bfw(W, apsp.block_size(torch.float32))
+def _expect(n, p, seed, dtype=np.float32):
+    W = graphgen.dense_graph(n, p, seed, weights="real", lo=0.5, hi=2.0, dtype=dtype)
+    return W, *oracle.bfw(W, 128)
 
 
 # One quad of the diagonal block; a block less one; two blocks, the last one
@@ -34,13 +34,44 @@ def test_real_weights_bitwise_at_dispatch_limits(n):
     assert apsp.device_status() == apsp.APSP_OK
 
 
+# The same edges in FP64; the first size with four phase-4 CTAs per SM.
+@pytest.mark.parametrize("n", [1, 3, 5, 127, 129, 258, 3073])
+def test_real_weights_f64_bitwise_at_dispatch_limits(n):
+    W, Db, Pb = _expect(n, 0.3 if n < 300 else 0.05, 700 + n, np.float64)
+    assert apsp.block_size(torch.float64) == 128
+    D, P = torch.from_numpy(W).to(DEV), torch.full((n, n), 77, dtype=torch.int32, device=DEV)
+    apsp.apsp_fw(D, P)
+    np.testing.assert_array_equal(D.cpu().numpy(), Db)
+    np.testing.assert_array_equal(P.cpu().numpy(), Pb)
+    D = torch.from_numpy(W).to(DEV)
+    apsp.apsp_fw(D)
+    np.testing.assert_array_equal(D.cpu().numpy(), Db)
+    assert apsp.device_status() == apsp.APSP_OK
+
+
+def test_f64_sums_within_a_float_step():
+    """Weights 1 + j 2^-40 + i 2^-52: every sum shares one float, so candidates can
+    only be told apart in FP64, and many tie exactly (the first k wins)."""
+    n = 200
+    rng = np.random.default_rng(4)
+    W = 1.0 + rng.integers(0, 3, (n, n)) * 2.0 ** -40 + rng.integers(0, 3, (n, n)) * 2.0 ** -52
+    W[rng.random((n, n)) >= 0.1] = np.inf
+    np.fill_diagonal(W, 0)
+    Db, Pb = oracle.bfw(W, 128)
+    D, P = torch.from_numpy(W).to(DEV), torch.empty((n, n), dtype=torch.int32, device=DEV)
+    apsp.apsp_fw(D, P)
+    np.testing.assert_array_equal(D.cpu().numpy(), Db)
+    np.testing.assert_array_equal(P.cpu().numpy(), Pb)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
 @pytest.mark.parametrize("ld,d_off,p_off", [(263, 0, 0), (264, 1, 0), (264, 0, 1), (264, 3, 2)])
-def test_unaligned_rows_and_buffers(ld, d_off, p_off):
+def test_unaligned_rows_and_buffers(ld, d_off, p_off, dtype):
     """Odd leading dimensions and buffers that start off a 16-byte boundary, D
     and P apart; the columns past n stay as they are."""
     n = 261
-    W, Db, Pb = _expect(n, 0.3, 5)
-    dbuf = torch.full((n * ld + 4,), -3.0, device=DEV)
+    W, Db, Pb = _expect(n, 0.3, 5, np.float32 if dtype == torch.float32 else np.float64)
+    dbuf = torch.full((n * ld + 4,), -3.0, dtype=dtype, device=DEV)
     pbuf = torch.full((n * ld + 4,), -9, dtype=torch.int32, device=DEV)
     D = dbuf[d_off:d_off + n * ld].view(n, ld)
     P = pbuf[p_off:p_off + n * ld].view(n, ld)
