@@ -948,28 +948,46 @@ __global__ void __launch_bounds__(k3s::THREADS, TR == 32 ? 4 : 3)
     if (PATH) note(g);
   }
   grid_dep_launch();
+  if (!PATH) {
 #pragma unroll
-  for (int a = 0; a < 4; ++a) {
-    const int i = r0 + (a & 1) + 8 * (a >> 1);
+    for (int a = 0; a < 4; ++a)
 #pragma unroll
-    for (int c = 0; c < CW; ++c) {
-      const unsigned gc = (chunk[c] >> (8 * a)) & 0xFFu;
-      if (PATH ? gc == 0xFFu : !(acc[a][c] < prev[a][c])) continue;  // (improved outputs lie inside the matrix)
-      const int j = c0 + 16 * (c >> 1) + (c & 1);
-      const int64_t e = (int64_t)(baseI + i) * ld + baseJ + j;
-      D[e] = acc[a][c];
-      if (PATH) {
-        int k = 0;
-#pragma unroll
-        for (int u = 7; u >= 0; --u) {
-          const int kp = min(8 * (int)gc + u, nkp - 1);
-          const float2 t = mp32::sum2(sm.A[kp][i], sm.B[kp][j]);
-          k = t.y == acc[a][c] ? 2 * kp + 1 : k;
-          k = t.x == acc[a][c] ? 2 * kp : k;
-        }
-        P[e] = baseK + k;
+      for (int c = 0; c < CW; ++c) {
+        const int i = r0 + (a & 1) + 8 * (a >> 1), j = c0 + 16 * (c >> 1) + (c & 1);
+        // (improved outputs lie inside the matrix)
+        if (acc[a][c] < prev[a][c]) D[(int64_t)(baseI + i) * ld + baseJ + j] = acc[a][c];
       }
+    return;
+  }
+  // Each lane takes its own next improved output, so that the warp runs the
+  // rest as often as its fullest lane needs and not once per output.
+  unsigned left = 0u;  // bit 4 c + a: output (a, c) improved
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int c = 0; c < CW; ++c) left |= (((chunk[c] >> (8 * a)) & 0xFFu) != 0xFFu ? 1u : 0u) << (4 * c + a);
+#pragma unroll 1
+  for (; left; left &= left - 1) {
+    const int t = __ffs(left) - 1, a = t & 3, c = t >> 2;
+    float x = acc[0][0];
+#pragma unroll
+    for (int u = 1; u < 4 * CW; ++u) x = t == u ? acc[u & 3][u >> 2] : x;
+    unsigned ch = chunk[0];
+#pragma unroll
+    for (int u = 1; u < CW; ++u) ch = c == u ? chunk[u] : ch;
+    const int i = r0 + (a & 1) + 8 * (a >> 1), j = c0 + 16 * (c >> 1) + (c & 1);
+    const int gc = (int)((ch >> (8 * a)) & 0xFFu);
+    int k = 0;
+#pragma unroll
+    for (int u = 7; u >= 0; --u) {
+      const int kp = min(8 * gc + u, nkp - 1);
+      const float2 s = mp32::sum2(sm.A[kp][i], sm.B[kp][j]);
+      k = s.y == x ? 2 * kp + 1 : k;
+      k = s.x == x ? 2 * kp : k;
     }
+    const int64_t e = (int64_t)(baseI + i) * ld + baseJ + j;
+    D[e] = x;
+    P[e] = baseK + k;
   }
 }
 
