@@ -21,9 +21,10 @@
 //     path matrix: variant 0 recovers each improved output's first argmin k
 //     from the operands after the product (lazy), variant 1 keeps the index
 //     of the last improving k-pair in the inner loop (eager);
-//     variant 1, and every variant run without a path matrix, pipelines the
-//     products of a phase group: the operands of the next product are copied
-//     into a second shared-memory stage while the current one computes.
+//     variant 1, and every variant run without a path matrix, closes the
+//     diagonal block four steps per barrier and pipelines the products of a
+//     phase group: the operands the next product does not share with this one
+//     are copied while this one computes.
 //   variant 2, 128 x 128 blocks, 8 x 4 register tile per thread: the
 //     single-graph kernels' code run by one CTA: the register-resident closure
 //     for phase 1, the k-sequential line kernel for phases 2+3 (the paper's
@@ -87,45 +88,36 @@ struct ProdSmem {
   unsigned long long Bs[KP][ST];  // Bs[kp][j] = (B[2kp][j], B[2kp+1][j])
   float Cs[T][CS];                // new candidates
 };
-// Operand stage of the pipelined products: the same k-pair layout.
-struct Stage {
-  unsigned long long As[KP][ST];
-  unsigned long long Bs[KP][ST];
-};
-// Output tile of thread (warp w, lane l) in the pipelined products:
-// ty = 2 w + l / 16, tx = l % 16 (rows and columns from mp32::row_at/col_at).
-// A quarter-warp shares its A pairs with the next one and its B pairs with
-// the one two further (measured 2 % faster than the phase-4 mapping here).
-__device__ __forceinline__ int prod_ty() { return (threadIdx.x >> 5) * 2 + ((threadIdx.x & 31) >> 4); }
-__device__ __forceinline__ int prod_tx() { return threadIdx.x & 15; }
 }  // namespace b64
+
+// Copies of operand blocks in shared memory: the k-paired layout of the A and
+// the B operand, two buffers each.
+struct Bufs64 {
+  unsigned long long A[2][b64::KP][b64::ST];  // A[kp][i] = (A[i][2kp], A[i][2kp+1])
+  unsigned long long B[2][b64::KP][b64::ST];  // B[kp][j] = (B[2kp][j], B[2kp+1][j])
+};
+// The closure's histories.
+struct Quad64 {
+  unsigned long long hr[b64::KP][b64::T];    // (row 2kp, row 2kp+1), each at its own step
+  unsigned long long hcol[b64::T][b64::KP];  // (column 2kp, column 2kp+1) likewise
+  float x[2][b64::T][4];                     // columns of the current quad before its steps
+};
 
 union BatchedSmem {
   b64::ProdSmem prod;
-  b64::Stage stage[2];
+  Bufs64 bufs;
+  Quad64 quad;
   mp32::DiagSmemT<64> diag;
   mp32::DiagSmemT<128> diag128;
   float lines_M[k2::T * k2::MS];
   k3::Smem prod128;
 };
 
-// Eager path tracking per k-pair: the three-input min writes the new
-// accumulator, and the pair index is kept when it lowered the accumulator
-// strictly.  Which k of the last such pair reached the final value is settled
-// once per output after the loop (the lower k if its candidate equals the
-// final value: the strict "<" of the sequential loop keeps the first k
-// reaching a minimum).
-__device__ __forceinline__ void relax2_argpair(float &acc, int &kp_last, unsigned long long a,
-                                               unsigned long long b, int kp) {
-  float m;
-  asm("{\n\t.reg .b64 t;\n\t.reg .f32 lo, hi;\n\t"
-      "add.rn.f32x2 t, %1, %2;\n\t"
-      "mov.b64 {lo, hi}, t;\n\t"
-      "min.f32 %0, %3, lo, hi;\n\t}"
-      : "=f"(m)
-      : "l"(a), "l"(b), "f"(acc));
-  kp_last = m < acc ? kp : kp_last;
-  acc = m;
+__device__ __forceinline__ void cp_async8(void *dst, const void *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(
+                   static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
+               "l"(src)
+               : "memory");
 }
 
 // C(baseI, baseJ) <- min(C, A(baseI, baseK) (x) B(baseK, baseJ)), TB = 64,
@@ -292,178 +284,314 @@ __device__ __forceinline__ void solve_graph_lazy_f32(float *__restrict__ D, int3
 }
 
 // --------------------------------------------------------------------------
-// Pipelined 64-block products (variant 1, and every variant without a path
-// matrix).  The products of one group (phases 2+3 of a round, or its phase 4)
-// neither read nor write a block another product of the group writes, so the
-// operands of product p+1 are copied into the second stage while product p
-// computes.  The accumulator starts at C itself, so an output's pair index is
-// set only when a candidate beats C strictly, which is the sequential loop's
-// rule, and only such outputs are resolved and written (from registers).
+// Variant 1, and every variant without a path matrix: 64-block closure by
+// quads of steps, then pipelined 64-block products.
 // --------------------------------------------------------------------------
 
-// Both operand blocks of one product into a stage (4-byte asynchronous
-// copies into the k-pair layout, +inf outside the valid extents), committed
-// as one group.
-__device__ __forceinline__ void stage_operands(b64::Stage &s, const float *__restrict__ D, int ld, int baseI,
-                                               int baseJ, int baseK, int mI, int mJ, int mK) {
+// Phase 1 on the diagonal block at `base` (m valid vertices, 256 threads): each
+// thread keeps 4 x 4 adjacent elements, and the four steps of a quad share one
+// barrier.  The threads of the quad's rows (one half-warp) take the quad's own
+// 4 x 4 entries by shuffle, bring their rows to each row's step and publish
+// them; the threads of its columns publish those as they are; after the
+// barrier every thread brings its rows' four column values to their steps
+// against the published 4 x 4 entries and relaxes its elements (two packed
+// adds and two three-input mins each).  Step k never changes row or column k.
+// TRACK: elements are compared once per quad, and the k of the last improvement
+// found among its four steps afterwards (the first whose candidate from the
+// histories equals the final value).
+template <bool TRACK>
+__device__ __forceinline__ void closure64(float *__restrict__ D, int ld, int32_t *__restrict__ P, int base, int m,
+                                          Quad64 &sm) {
+  using mp32::pack2;
+  const int tid = threadIdx.x, w = tid >> 5, ty = tid >> 4, tx = tid & 15;
+  const int i0 = 4 * ty, j0 = 4 * tx;
+  const float INF = inf<float>();
+  float d[4][4];
+  int aux[4][4];  // TRACK: last quad that lowered the element, -1 none; else its input's bits
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      d[a][c] = (i0 + a < m && j0 + c < m) ? D[(base + i0 + a) * ld + base + j0 + c] : INF;
+      aux[a][c] = TRACK ? -1 : __float_as_int(d[a][c]);
+    }
+  const int nq = (m + 3) / 4;
+  const bool idle = 8 * w >= m;  // warp-uniform: no valid row
+#pragma unroll 1
+  for (int q = 0; q < nq; ++q) {
+    float e01, e02, e03, e12, e13, e23;
+    auto pivots = [&](float (&p)[4]) {  // a row's values at the quad's columns brought to their steps
+      p[1] = fminf(p[1], __fadd_rn(p[0], e01));
+      p[2] = mp32::min3f(p[2], __fadd_rn(p[0], e02), __fadd_rn(p[1], e12));
+      p[3] = fminf(mp32::min3f(p[3], __fadd_rn(p[0], e03), __fadd_rn(p[1], e13)), __fadd_rn(p[2], e23));
+    };
+    if (tx == q) {
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+        *reinterpret_cast<float4 *>(&sm.x[q & 1][i0 + a][0]) = make_float4(d[a][0], d[a][1], d[a][2], d[a][3]);
+    }
+    if (w == q >> 1) {
+      float x[4][4];
+      const int src = (q & 1) * 16 + q;
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) x[a][c] = __shfl_sync(kFullMask, d[a][c], src);
+      if (ty == q) {
+        e01 = x[0][1], e02 = x[0][2], e03 = x[0][3];
+        e12 = fminf(x[1][2], __fadd_rn(x[1][0], e02));
+        e13 = fminf(x[1][3], __fadd_rn(x[1][0], e03));
+        const float y21 = fminf(x[2][1], __fadd_rn(x[2][0], e01));
+        e23 = mp32::min3f(x[2][3], __fadd_rn(x[2][0], e03), __fadd_rn(y21, e13));
+#pragma unroll
+        for (int a = 1; a < 4; ++a) pivots(x[a]);
+        unsigned long long ha[4], hb[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const float r0 = d[0][c], r1 = fminf(d[1][c], __fadd_rn(x[1][0], r0));
+          const float r2 = mp32::min3f(d[2][c], __fadd_rn(x[2][0], r0), __fadd_rn(x[2][1], r1));
+          const float r3 = fminf(mp32::min3f(d[3][c], __fadd_rn(x[3][0], r0), __fadd_rn(x[3][1], r1)),
+                                 __fadd_rn(x[3][2], r2));
+          ha[c] = pack2(r0, r1);
+          hb[c] = pack2(r2, r3);
+        }
+#pragma unroll
+        for (int c = 0; c < 4; c += 2) {
+          *reinterpret_cast<ulonglong2 *>(&sm.hr[2 * q][j0 + c]) = make_ulonglong2(ha[c], ha[c + 1]);
+          *reinterpret_cast<ulonglong2 *>(&sm.hr[2 * q + 1][j0 + c]) = make_ulonglong2(hb[c], hb[c + 1]);
+        }
+      }
+    }
+    __syncthreads();
+    if (idle) continue;
+    const ulonglong2 q0 = *reinterpret_cast<const ulonglong2 *>(&sm.hr[2 * q][4 * q]);
+    const ulonglong2 q1 = *reinterpret_cast<const ulonglong2 *>(&sm.hr[2 * q][4 * q + 2]);
+    e01 = __uint_as_float((unsigned)q0.y);
+    e02 = __uint_as_float((unsigned)q1.x);
+    e03 = __uint_as_float((unsigned)q1.y);
+    e12 = __uint_as_float((unsigned)(q1.x >> 32));
+    e13 = __uint_as_float((unsigned)(q1.y >> 32));
+    e23 = __uint_as_float((unsigned)sm.hr[2 * q + 1][4 * q + 3]);
+    unsigned long long ha[4], hb[4];
+#pragma unroll
+    for (int c = 0; c < 4; c += 2) {
+      const ulonglong2 ta = *reinterpret_cast<const ulonglong2 *>(&sm.hr[2 * q][j0 + c]);
+      const ulonglong2 tb = *reinterpret_cast<const ulonglong2 *>(&sm.hr[2 * q + 1][j0 + c]);
+      ha[c] = ta.x, ha[c + 1] = ta.y, hb[c] = tb.x, hb[c + 1] = tb.y;
+    }
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      const float4 t = *reinterpret_cast<const float4 *>(&sm.x[q & 1][i0 + a][0]);
+      float p[4] = {t.x, t.y, t.z, t.w};
+      pivots(p);
+      const unsigned long long pa = pack2(p[0], p[1]), pb = pack2(p[2], p[3]);
+      if (TRACK && tx == 0) *reinterpret_cast<ulonglong2 *>(&sm.hcol[i0 + a][2 * q]) = make_ulonglong2(pa, pb);
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const float v = mp32::min3f_pair(mp32::min3f_pair(d[a][c], pa, ha[c]), pb, hb[c]);
+        if (TRACK) aux[a][c] = v < d[a][c] ? q : aux[a][c];
+        d[a][c] = v;
+      }
+    }
+  }
+  if (idle) return;
+  __syncwarp();  // hcol is written and read by the same half-warps
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const int i = i0 + a, j = j0 + c, e = (base + i) * ld + base + j;
+      const float g = d[a][c];
+      if constexpr (TRACK) {
+        const int q = aux[a][c];
+        if (q < 0) continue;  // (improved elements are valid)
+        const float2 t0 = mp32::sum2(sm.hcol[i][2 * q], sm.hr[2 * q][j]);
+        const float2 t1 = mp32::sum2(sm.hcol[i][2 * q + 1], sm.hr[2 * q + 1][j]);
+        D[e] = g;
+        P[e] = base + 4 * q + (t0.x == g ? 0 : t0.y == g ? 1 : t1.x == g ? 2 : 3);
+      } else {
+        if (g < __int_as_float(aux[a][c])) D[e] = g;
+      }
+    }
+}
+
+// The A operand D(baseI.., baseK..) into a buffer (+inf outside the valid
+// extents), asynchronously: 8-byte copies of a k-pair where every pair starts
+// on an 8-byte boundary (even ld and an aligned D), else 4-byte ones.
+__device__ __forceinline__ void stage_a(unsigned long long (&dst)[b64::KP][b64::ST], const float *__restrict__ D,
+                                        int ld, int baseI, int baseK, int mI, int mK) {
   using namespace b64;
   const int tid = threadIdx.x;
   const float INF = inf<float>();
-  float *as = reinterpret_cast<float *>(&s.As[0][0]);
-  float *bs = reinterpret_cast<float *>(&s.Bs[0][0]);
+  if ((ld & 1) == 0 && (reinterpret_cast<uintptr_t>(D) & 7) == 0) {
 #pragma unroll
-  for (int q = 0; q < T * T / 256; ++q) {
-    const int idx = tid + q * 256, i = idx / T, k = idx % T;
-    float *dst = as + ((k >> 1) * ST + i) * 2 + (k & 1);
-    if (i < mI && k < mK) mp32::cp_async4(dst, D + (int64_t)(baseI + i) * ld + baseK + k);
-    else *dst = INF;
+    for (int q = 0; q < T * KP / 256; ++q) {
+      const int idx = tid + q * 256, i = idx / KP, kp = idx % KP;
+      unsigned long long *to = &dst[kp][i];
+      const float *from = D + (baseI + i) * ld + baseK + 2 * kp;
+      if (i < mI && 2 * kp + 1 < mK) {
+        cp_async8(to, from);
+      } else {
+        float *f = reinterpret_cast<float *>(to);
+        f[1] = INF;
+        if (i < mI && 2 * kp < mK) mp32::cp_async4(f, from);
+        else f[0] = INF;
+      }
+    }
+  } else {
+#pragma unroll
+    for (int q = 0; q < T * T / 256; ++q) {
+      const int idx = tid + q * 256, i = idx / T, k = idx % T;
+      float *to = reinterpret_cast<float *>(&dst[k >> 1][i]) + (k & 1);
+      if (i < mI && k < mK) mp32::cp_async4(to, D + (baseI + i) * ld + baseK + k);
+      else *to = INF;
+    }
   }
+}
+// The B operand D(baseK.., baseJ..).
+__device__ __forceinline__ void stage_b(unsigned long long (&dst)[b64::KP][b64::ST], const float *__restrict__ D,
+                                        int ld, int baseK, int baseJ, int mK, int mJ) {
+  using namespace b64;
+  const int tid = threadIdx.x;
+  const float INF = inf<float>();
 #pragma unroll
   for (int q = 0; q < T * T / 256; ++q) {
     const int idx = tid + q * 256, k = idx / T, j = idx % T;
-    float *dst = bs + ((k >> 1) * ST + j) * 2 + (k & 1);
-    if (j < mJ && k < mK) mp32::cp_async4(dst, D + (int64_t)(baseK + k) * ld + baseJ + j);
-    else *dst = INF;
+    float *to = reinterpret_cast<float *>(&dst[k >> 1][j]) + (k & 1);
+    if (j < mJ && k < mK) mp32::cp_async4(to, D + (baseK + k) * ld + baseJ + j);
+    else *to = INF;
   }
-  mp32::cp_async_commit();
 }
 
-// C(baseI, baseJ) <- min(C, A (x) B) from a filled stage, TB = 64, all 256
-// threads; TRACK writes P (the first k whose candidate beats C strictly).
+// C(baseI, baseJ) <- min(C, A (x) B) from filled buffers, all 256 threads.  A
+// warp owns eight rows (one without a valid row does nothing), a thread 4 x 4
+// outputs.  The accumulators start at C, so an output improves exactly
+// when its accumulator falls.  TRACK: compared once per four k (one compare and
+// one select per output); the first of the last improving four whose candidate
+// equals the new value is the path entry (the sequential loop's, strict "<").
+// Fewer comparisons lose here: with 8 or 16 candidates to look through for
+// every improved output (20-90 % of them in a round) the 4096-graph batch took
+// 23.3 and 26.2 ms against 21.0.
+// Bound: instruction issue and the ALU pipe (a min, a compare and a select per
+// two pairs).  Measured on that batch (n ~ U[16, 512]): 21.0 ms with P, 13.8
+// without (22.7 and 15.9 with every product copying both operands 4 bytes at a
+// time and computing all 64 rows of a ragged block); lanes two rows of pairs by
+// sixteen columns: four by eight took 21.6 ms.
 template <bool TRACK>
-__device__ __forceinline__ void product64_staged(float *__restrict__ D, int ld, int32_t *__restrict__ P, int baseI,
-                                                 int baseJ, int baseK, int mI, int mJ, int mK,
-                                                 const b64::Stage &s) {
-  using namespace b64;
-  using mp32::col_at;
-  using mp32::row_at;
-  const int ty = prod_ty(), tx = prod_tx();
+__device__ __forceinline__ void product64(float *__restrict__ D, int ld, int32_t *__restrict__ P, int baseI, int baseJ,
+                                          int baseK, int mI, int mJ, int mK,
+                                          const unsigned long long (&A)[b64::KP][b64::ST],
+                                          const unsigned long long (&B)[b64::KP][b64::ST]) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (8 * w >= mI) return;  // warp-uniform
+  const int r0 = 8 * w + 2 * (lane >> 4), c0 = 2 * (lane & 15);
   const float INF = inf<float>();
-  float acc[TM][TM];
-  // TRACK: the first pair of the last chunk that lowered the accumulator
-  // (-1: none); otherwise C itself, to find the improved outputs.
-  int aux[TM][TM];
+  float acc[4][4];
+  int aux[4][4];  // TRACK: last k-pair step (two pairs) that lowered the output, -1 none; else C's bits
+  const int e0 = (baseI + r0) * ld + baseJ + c0;  // output (a, c): row (a & 1) + 4 (a >> 1), column (c & 1) + 32 (c >> 1) further
 #pragma unroll
-  for (int rr = 0; rr < TM; ++rr)
+  for (int c = 0; c < 4; ++c)
 #pragma unroll
-    for (int cc = 0; cc < TM; ++cc) {
-      const int i = row_at(rr, ty), j = col_at(cc, tx);
-      acc[rr][cc] = (i < mI && j < mJ) ? D[(int64_t)(baseI + i) * ld + baseJ + j] : INF;
-      aux[rr][cc] = TRACK ? -1 : __float_as_int(acc[rr][cc]);
+    for (int a = 0; a < 4; ++a) {
+      const int di = (a & 1) + 4 * (a >> 1), dj = (c & 1) + 32 * (c >> 1);
+      acc[a][c] = (r0 + di < mI && c0 + dj < mJ) ? D[e0 + di * ld + dj] : INF;
+      aux[a][c] = TRACK ? -1 : __float_as_int(acc[a][c]);
     }
-  const int kpn = (mK + 1) / 2;
-  auto load_pair = [&](int kp, unsigned long long (&a)[TM], unsigned long long (&b)[TM]) {
+  auto load = [&](int kp, unsigned long long (&a)[4], unsigned long long (&b)[4]) {
 #pragma unroll
-    for (int rr = 0; rr < TM; rr += 2) {
-      const ulonglong2 t = *reinterpret_cast<const ulonglong2 *>(&s.As[kp][row_at(rr, ty)]);
-      a[rr] = t.x;
-      a[rr + 1] = t.y;
-    }
-#pragma unroll
-    for (int cc = 0; cc < TM; cc += 2) {
-      const ulonglong2 t = *reinterpret_cast<const ulonglong2 *>(&s.Bs[kp][col_at(cc, tx)]);
-      b[cc] = t.x;
-      b[cc + 1] = t.y;
+    for (int u = 0; u < 4; u += 2) {
+      const ulonglong2 t = *reinterpret_cast<const ulonglong2 *>(&A[kp][r0 + 2 * u]);
+      const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(&B[kp][c0 + 16 * u]);
+      a[u] = t.x, a[u + 1] = t.y, b[u] = v.x, b[u + 1] = v.y;
     }
   };
-  int kp0 = 0;
-  if constexpr (TRACK) {
-    // Two k-pairs (four k) per step, one compare and one select per output.
+  const int kpn = ((mK + 3) / 4) * 2;  // whole steps of two k-pairs: the operands are +inf past mK
 #pragma unroll 1
-    for (; kp0 + 1 < kpn; kp0 += 2) {
-      unsigned long long a0[TM], b0[TM], a1[TM], b1[TM];
-      load_pair(kp0, a0, b0);
-      load_pair(kp0 + 1, a1, b1);
+  for (int kp = 0; kp < kpn; kp += 2) {
+    unsigned long long a0[4], b0[4], a1[4], b1[4];
+    load(kp, a0, b0);
+    load(kp + 1, a1, b1);
 #pragma unroll
-      for (int rr = 0; rr < TM; ++rr)
+    for (int a = 0; a < 4; ++a)
 #pragma unroll
-        for (int cc = 0; cc < TM; ++cc) {
-          const float m1 = mp32::min3f_pair(acc[rr][cc], a0[rr], b0[cc]);
-          const float m2 = mp32::min3f_pair(m1, a1[rr], b1[cc]);
-          aux[rr][cc] = m2 < acc[rr][cc] ? kp0 : aux[rr][cc];
-          acc[rr][cc] = m2;
-        }
-    }
-  }
-#pragma unroll 1
-  for (int kp = kp0; kp < kpn; ++kp) {  // TRACK: an odd last pair only
-    unsigned long long a[TM], b[TM];
-    load_pair(kp, a, b);
-#pragma unroll
-    for (int rr = 0; rr < TM; ++rr)
-#pragma unroll
-      for (int cc = 0; cc < TM; ++cc) {
-        if (TRACK) relax2_argpair(acc[rr][cc], aux[rr][cc], a[rr], b[cc], kp);
-        else mp32::relax2(acc[rr][cc], a[rr], b[cc]);
+      for (int c = 0; c < 4; ++c) {
+        const float m = mp32::min3f_pair(mp32::min3f_pair(acc[a][c], a0[a], b0[c]), a1[a], b1[c]);
+        if (TRACK) aux[a][c] = m < acc[a][c] ? kp : aux[a][c];
+        acc[a][c] = m;
       }
   }
 #pragma unroll
-  for (int rr = 0; rr < TM; ++rr)
+  for (int a = 0; a < 4; ++a)
 #pragma unroll
-    for (int cc = 0; cc < TM; ++cc) {
-      const int i = row_at(rr, ty), j = col_at(cc, tx);
-      const float g = acc[rr][cc];
-      const int64_t e = (int64_t)(baseI + i) * ld + baseJ + j;
+    for (int c = 0; c < 4; ++c) {
+      const int di = (a & 1) + 4 * (a >> 1), dj = (c & 1) + 32 * (c >> 1), e = e0 + di * ld + dj;
+      const float g = acc[a][c];
       if constexpr (TRACK) {
-        const int kp = aux[rr][cc];
-        if (kp >= 0) {  // improved: the first k of the chunk whose candidate is the final value
-          // both pairs of the chunk, without branches (a lone last pair
-          // has its value in c0; c1 is then unused)
-          const int kq = min(kp + 1, KP - 1);
-          const float2 c0 = mp32::sum2(s.As[kp][i], s.Bs[kp][j]);
-          const float2 c1 = mp32::sum2(s.As[kq][i], s.Bs[kq][j]);
-          const int k = c0.x == g ? 2 * kp : c0.y == g ? 2 * kp + 1 : c1.x == g ? 2 * kp + 2 : 2 * kp + 3;
-          D[e] = g;
-          P[e] = baseK + k;
-        }
+        const int kp = aux[a][c];
+        if (kp < 0) continue;  // (improved outputs are valid)
+        const unsigned long long *pa = &A[kp][r0 + di], *pb = &B[kp][c0 + dj];
+        const float2 t0 = mp32::sum2(pa[0], pb[0]), t1 = mp32::sum2(pa[b64::ST], pb[b64::ST]);
+        D[e] = g;
+        P[e] = baseK + 2 * kp + (t0.x == g ? 0 : t0.y == g ? 1 : t1.x == g ? 2 : 3);
       } else {
-        if (g < __int_as_float(aux[rr][cc])) D[e] = g;
+        if (g < __int_as_float(aux[a][c])) D[e] = g;
       }
     }
 }
 
-// The products of round r (base = 64 r, m valid vertices) in group 0 (phases
-// 2+3: the row blocks (r, J), then the column blocks (I, r), each a product
-// with the closed diagonal block) or group 1 (phase 4), two stages deep.
+// The products of round r (m valid vertices) in group 0 (phases 2+3: the row
+// blocks (r, J), then the column blocks (I, r), each with the closed diagonal
+// block) or group 1 (phase 4, column by column).  No product of a group reads
+// a block another one writes, so the operands of the next product are copied
+// while the current one computes; an operand two products share is copied once.
 template <bool TRACK>
 __device__ __forceinline__ void run_group64(float *__restrict__ D, int ld, int32_t *__restrict__ P, int n, int r,
-                                            int group, b64::Stage (&st)[2]) {
+                                            int group, Bufs64 &sm) {
   constexpr int T = b64::T;
   const int R = (n + T - 1) / T, base = r * T, m = min(T, n - base);
   const int np = group == 0 ? 2 * (R - 1) : (R - 1) * (R - 1);
-  auto coords = [&](int p, int &bI, int &bJ, int &mI, int &mJ) {
-    int I, J;
+  auto coords = [&](int p, int &I, int &J) {
     if (group == 0) {
-      const int o = p % (R - 1), O = o < r ? o : o + 1;
+      const int o = p % (R - 1), O = o + (o >= r);
       I = p < R - 1 ? r : O;
       J = p < R - 1 ? O : r;
     } else {
-      const int a = p / (R - 1), b = p % (R - 1);
-      I = a < r ? a : a + 1;
-      J = b < r ? b : b + 1;
+      I = p % (R - 1);
+      J = p / (R - 1);
+      I += I >= r;
+      J += J >= r;
     }
-    bI = I * T;
-    bJ = J * T;
-    mI = min(T, n - bI);
-    mJ = min(T, n - bJ);
   };
-  int bI, bJ, mI, mJ;
-  coords(0, bI, bJ, mI, mJ);
-  stage_operands(st[0], D, ld, bI, bJ, base, mI, mJ, m);
+  int I, J, ba = 0, bb = 0;  // the product and the buffers that hold its operands
+  coords(0, I, J);
+  stage_a(sm.A[0], D, ld, I * T, base, min(T, n - I * T), m);
+  stage_b(sm.B[0], D, ld, base, J * T, m, min(T, n - J * T));
+  mp32::cp_async_commit();
 #pragma unroll 1
   for (int p = 0; p < np; ++p) {
-    int cI, cJ, cmI, cmJ;
-    coords(p, cI, cJ, cmI, cmJ);
+    int nI = I, nJ = J, na = ba, nb = bb;
     if (p + 1 < np) {
-      __syncthreads();  // product p-1 is done with the stage refilled here
-      coords(p + 1, bI, bJ, mI, mJ);
-      stage_operands(st[(p + 1) & 1], D, ld, bI, bJ, base, mI, mJ, m);
+      coords(p + 1, nI, nJ);
+      __syncthreads();  // product p-1 is done with the buffers refilled here
+      if (nI != I) {
+        na = ba ^ 1;
+        stage_a(sm.A[na], D, ld, nI * T, base, min(T, n - nI * T), m);
+      }
+      if (nJ != J) {
+        nb = bb ^ 1;
+        stage_b(sm.B[nb], D, ld, base, nJ * T, m, min(T, n - nJ * T));
+      }
+      mp32::cp_async_commit();
       mp32::cp_async_wait<1>();
     } else {
       mp32::cp_async_wait<0>();
     }
-    __syncthreads();  // every thread's copies into stage p & 1 are visible
-    product64_staged<TRACK>(D, ld, P, cI, cJ, base, cmI, cmJ, m, st[p & 1]);
+    __syncthreads();  // every thread's copies for product p are visible
+    product64<TRACK>(D, ld, P, I * T, J * T, base, min(T, n - I * T), min(T, n - J * T), m, sm.A[ba], sm.B[bb]);
+    I = nI;
+    J = nJ;
+    ba = na;
+    bb = nb;
   }
 }
 
@@ -475,13 +603,13 @@ __device__ __forceinline__ void solve_graph_pipe_f32(float *__restrict__ D, int3
   const int R = (n + T - 1) / T;
   for (int r = 0; r < R; ++r) {
     const int base = r * T, m = min(T, n - base);
-    __syncthreads();  // the previous round's products are done with the stages
-    mp32::diag_closure<4>(D, ld, P, base, m, sm.diag);
+    __syncthreads();  // the previous round's products are done with the buffers
+    closure64<TRACK>(D, ld, P, base, m, sm.quad);
     __syncthreads();
     if (R == 1) break;
-    run_group64<TRACK>(D, ld, P, n, r, 0, sm.stage);
+    run_group64<TRACK>(D, ld, P, n, r, 0, sm.bufs);
     __syncthreads();  // the panels are final (and visible) before phase 4 copies them
-    run_group64<TRACK>(D, ld, P, n, r, 1, sm.stage);
+    run_group64<TRACK>(D, ld, P, n, r, 1, sm.bufs);
   }
   __syncthreads();
 }

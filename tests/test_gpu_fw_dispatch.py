@@ -8,6 +8,7 @@ import torch
 import graphgen
 import oracle
 import paper_2105_07298_gb300 as apsp
+from paper_2105_07298_gb300 import batched
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
@@ -80,3 +81,24 @@ def test_unaligned_rows_and_buffers(ld, d_off, p_off, dtype):
     np.testing.assert_array_equal(D[:, :n].cpu().numpy(), Db)
     np.testing.assert_array_equal(P[:, :n].cpu().numpy(), Pb)
     assert bool((D[:, n:] == -3.0).all()) and bool((P[:, n:] == -9).all())
+
+
+@pytest.mark.parametrize("with_path", [True, False])
+@pytest.mark.parametrize("d_off", [0, 1])
+def test_batched_blocks_at_quad_and_tile_edges(d_off, with_path):
+    """Batched sizes around the quads of the closure, the eight rows of a warp
+    and the 64-blocks, even and odd, from a buffer on and off an 8-byte boundary."""
+    sizes = [1, 2, 3, 4, 5, 8, 9, 31, 33, 63, 64, 65, 66, 72, 73, 127, 128, 129, 130, 194]
+    off = batched.packed_offsets(sizes)
+    mats = [graphgen.dense_graph(n, 0.3, 40 + n) for n in sizes]
+    total = batched.packed_numel(sizes)
+    buf = torch.zeros(total + 1, device=DEV)[d_off:d_off + total]
+    for m, n, o in zip(mats, sizes, off):
+        buf[int(o):int(o) + n * n] = torch.from_numpy(m.reshape(-1)).to(DEV)
+    P = torch.full((total,), -7, dtype=torch.int32, device=DEV) if with_path else None
+    apsp.apsp_fw_batched(buf, sizes, off, P)
+    for m, n, o in zip(mats, sizes, off):
+        D = buf[int(o):int(o) + n * n].view(n, n).cpu().numpy()
+        np.testing.assert_array_equal(D, oracle.fw(m)[0])
+        if with_path:
+            assert oracle.check_paths(m, D, P[int(o):int(o) + n * n].view(n, n).cpu().numpy()) == 0
