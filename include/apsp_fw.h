@@ -90,7 +90,9 @@ int apsp_fw_block_size(int elem_bytes);
  *            captured into a CUDA graph: then every phase runs on `stream`.
  *            Scratch (operand panels: about 32 n TB bytes for FP32, 48 n TB
  *            bytes for FP64; 128 MiB / 192 MiB at n = 32768) is stream-ordered
- *            (cudaMallocAsync / cudaFreeAsync on `stream`).
+ *            (allocated on `stream` from a memory pool of the library's own,
+ *            which keeps at most 256 MiB per device between calls, and freed
+ *            with cudaFreeAsync; cudaMallocAsync while `stream` is captured).
  * Returns APSP_OK, APSP_EINVAL (null d_dist with n > 0, ld < n, n > 262144),
  * APSP_ENOMEM (scratch) or APSP_ECUDA.
  * ---------------------------------------------------------------------- */

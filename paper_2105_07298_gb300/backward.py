@@ -10,8 +10,6 @@ from __future__ import annotations
 
 import ctypes
 
-import numpy as np
-
 
 def _raise_status(status):
     from . import ApspError, APSP_OK
@@ -83,7 +81,7 @@ def _solve_stack(D, P):
     multiple of 4), otherwise through a copy in the aligned packed layout.
     Larger graphs are solved one by one by the single-graph path."""
     from . import apsp_fw_f32
-    from .batched import BatchedPlan, packed_offsets, packed_numel, MAX_N
+    from .batched import apsp_fw_batched_f32, packed_offsets, packed_numel, MAX_N
     B, n, _ = D.shape
     if n > MAX_N:
         for b in range(B):
@@ -91,9 +89,7 @@ def _solve_stack(D, P):
         return
     sizes = [n] * B
     if (n * n) % 4 == 0:
-        plan = BatchedPlan(sizes, [b * n * n for b in range(B)])
-        plan.run(D.view(-1), P.view(-1))
-        plan.close()
+        apsp_fw_batched_f32(D.view(-1), sizes, [b * n * n for b in range(B)], P.view(-1))
         return
     import torch
     off = packed_offsets(sizes)
@@ -102,9 +98,7 @@ def _solve_stack(D, P):
     Dp = torch.empty(total, dtype=D.dtype, device=D.device)
     Pp = torch.empty(total, dtype=torch.int32, device=D.device)
     Dp[idx] = D.view(B, -1)
-    plan = BatchedPlan(sizes, off)
-    plan.run(Dp, Pp)
-    plan.close()
+    apsp_fw_batched_f32(Dp, sizes, off, Pp)
     D.view(B, -1).copy_(Dp[idx])
     P.view(B, -1).copy_(Pp[idx])
 
@@ -148,7 +142,7 @@ class ShortestPathDistances:
     def get_packed(cls):
         if cls._packed is None:
             import torch
-            from .batched import BatchedPlan
+            from .batched import _host_arrays, apsp_fw_batched_f32
 
             class _Packed(torch.autograd.Function):
                 @staticmethod
@@ -157,11 +151,10 @@ class ShortestPathDistances:
                         raise TypeError("W must be a 1-D CUDA float32 packed buffer")
                     D = Wp.detach().contiguous().clone()
                     P = torch.full(D.shape, -1, dtype=torch.int32, device=D.device)
-                    plan = BatchedPlan(sizes, offsets)
-                    plan.run(D, P)
-                    plan.close()
-                    n_dev = torch.from_numpy(np.ascontiguousarray(plan.sizes)).to(D.device)
-                    off_dev = torch.from_numpy(np.ascontiguousarray(plan.offsets)).to(D.device)
+                    n, off = _host_arrays(sizes, offsets)
+                    apsp_fw_batched_f32(D, n, off, P)
+                    n_dev = torch.from_numpy(n).to(D.device)
+                    off_dev = torch.from_numpy(off).to(D.device)
                     ctx.save_for_backward(D, P, n_dev, off_dev)
                     return D
 

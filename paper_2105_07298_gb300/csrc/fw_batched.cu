@@ -39,13 +39,16 @@
 // 0 and 1 round phases 2/3 through the closed block instead.
 #include <stdint.h>
 #include <stdlib.h>
+#include <string.h>
 
 #include <algorithm>
+#include <exception>
 #include <numeric>
 #include <vector>
 
 #include "bulk.cuh"
 #include "common.cuh"
+#include "scratch.h"
 #include "minplus_f32.cuh"
 #include "phases_f32.cuh"
 
@@ -861,7 +864,7 @@ APSP_EXPORT int apsp_fw_batched_run_f32(const apsp_batched_plan *p, float *d_dis
 }
 
 APSP_EXPORT int apsp_fw_batched_f32(float *d_dist, int32_t *d_path, const int32_t *h_n,
-                                    const int64_t *h_off, int32_t num, void *stream) {
+                                    const int64_t *h_off, int32_t num, void *stream) try {
   int st = validate(h_n, h_off, num);
   if (st) return st;
   if (num == 0) return APSP_OK;
@@ -871,35 +874,39 @@ APSP_EXPORT int apsp_fw_batched_f32(float *d_dist, int32_t *d_path, const int32_
   std::vector<int32_t> order = lpt_order(h_n, num, &rmax);
   int grid = grid_for(num, rmax > 0);
   if (grid <= 0) return APSP_ECUDA;
-  // one scratch block: counter | order | n | offsets | panels of the
-  // 128-block variants (stream-ordered allocation)
-  const size_t list_bytes = (16 + (size_t)num * 8 + (size_t)num * 8 + (size_t)num * 8 + 255) & ~(size_t)255;
-  const size_t bytes = list_bytes + (rmax > 0 ? (size_t)grid * apsp::panel_bytes_per_cta(rmax) : 0);
+  // One scratch block: counter | order | n | offsets | panels of the 128-block
+  // variants.  The work list, its counter already zero, goes up in one copy.
+  const size_t list_bytes = 16 + (((size_t)num * 8 + 15) & ~(size_t)15) + (size_t)num * 8;
+  const size_t list_span = (list_bytes + 255) & ~(size_t)255;
+  std::vector<char> list(list_bytes, 0);
+  int32_t *l_order = reinterpret_cast<int32_t *>(list.data() + 16);
+  std::copy(order.begin(), order.end(), l_order);
+  std::copy(h_n, h_n + num, l_order + num);
+  memcpy(list.data() + list_bytes - (size_t)num * 8, h_off, (size_t)num * 8);
+  const size_t bytes = list_span + (rmax > 0 ? (size_t)grid * apsp::panel_bytes_per_cta(rmax) : 0);
   char *scratch = nullptr;
   cudaGetLastError();
-  if (cudaMallocAsync((void **)&scratch, bytes, s) != cudaSuccess) {
+  if (apsp::scratch_alloc((void **)&scratch, bytes, s) != cudaSuccess) {
     cudaGetLastError();
     return APSP_ENOMEM;
   }
-  unsigned char *panels = rmax > 0 ? reinterpret_cast<unsigned char *>(scratch + list_bytes) : nullptr;
+  unsigned char *panels = rmax > 0 ? reinterpret_cast<unsigned char *>(scratch + list_span) : nullptr;
   int *d_counter = reinterpret_cast<int *>(scratch);
   int32_t *d_order = reinterpret_cast<int32_t *>(scratch + 16);
   int32_t *d_n = d_order + num;
-  int64_t *d_off = reinterpret_cast<int64_t *>(scratch + 16 + (((size_t)num * 8 + 15) & ~(size_t)15));
-  // offsets region starts 16-byte aligned after order and n (2 * 4 * num bytes)
-  cudaError_t e = cudaMemsetAsync(d_counter, 0, sizeof(int), s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(d_order, order.data(), (size_t)num * 4, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(d_n, h_n, (size_t)num * 4, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(d_off, h_off, (size_t)num * 8, cudaMemcpyHostToDevice, s);
+  int64_t *d_off = reinterpret_cast<int64_t *>(scratch + list_bytes - (size_t)num * 8);
+  cudaError_t e = cudaMemcpyAsync(scratch, list.data(), list_bytes, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) {
     kernel_for(rmax > 0)<<<grid, apsp::mp32::THREADS, sizeof(apsp::BatchedSmem), s>>>(
         d_dist, d_path, d_order, d_n, d_off, num, d_counter, panels, rmax);
     e = cudaGetLastError();
   }
   // Copies from pageable host memory have consumed their sources when they
-  // return, so `order` may go out of scope; the scratch is freed in stream order.
+  // return, so `list` may go out of scope; the scratch is freed in stream order.
   cudaFreeAsync(scratch, s);
   return apsp::status_from(e);
+} catch (const std::exception &) {  // host memory for the work list (nothing enqueued yet)
+  return APSP_ENOMEM;
 }
 
 APSP_EXPORT int apsp_batched_num_classes(void) { return apsp::kNumClasses; }

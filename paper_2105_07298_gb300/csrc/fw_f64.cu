@@ -31,6 +31,7 @@
 
 #include "bulk.cuh"
 #include "common.cuh"
+#include "scratch.h"
 #include "profile.h"
 #include "rounds.cuh"
 
@@ -857,7 +858,7 @@ int run_fw_f64_interval(double *D, int n, int64_t ld, int32_t *P, cudaStream_t s
   char *scratch = nullptr;
   if (R > 1) {
     const size_t elems = (size_t)R * T * T, set = elems * (4 + 4 + 8 + 8);
-    if (cudaMallocAsync((void **)&scratch, 2 * set + (size_t)T * T * 24, s) != cudaSuccess) {
+    if (scratch_alloc((void **)&scratch, 2 * set + (size_t)T * T * 24, s) != cudaSuccess) {
       cudaGetLastError();
       return APSP_ENOMEM;
     }

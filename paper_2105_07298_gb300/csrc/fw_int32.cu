@@ -18,6 +18,7 @@
 
 #include "bulk.cuh"
 #include "common.cuh"
+#include "scratch.h"
 
 namespace apsp {
 
@@ -64,7 +65,7 @@ APSP_EXPORT int apsp_fw_i32(int32_t *d_dist, int64_t n, int64_t ld, int32_t *d_p
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   cudaGetLastError();
   double *tmp = nullptr;
-  if (cudaMallocAsync((void **)&tmp, (size_t)n * n * sizeof(double), s) != cudaSuccess) {
+  if (apsp::scratch_alloc((void **)&tmp, (size_t)n * n * sizeof(double), s) != cudaSuccess) {
     cudaGetLastError();
     return APSP_ENOMEM;
   }

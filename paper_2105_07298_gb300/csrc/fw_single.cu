@@ -34,6 +34,7 @@
 #include <stdint.h>
 
 #include "common.cuh"
+#include "scratch.h"
 #include "bulk.cuh"
 #include "minplus_f32.cuh"
 #include "phases_f32.cuh"
@@ -1072,7 +1073,7 @@ static int run_fw_f32(float *D, int64_t n64, int64_t ld, int32_t *P, void *strea
   char *scratch = nullptr;
   if (R > 1) {
     const size_t words = (size_t)R * T * T;
-    if (cudaMallocAsync((void **)&scratch, (8 * words + 2 * (size_t)T * T) * 4, s) != cudaSuccess) {
+    if (scratch_alloc((void **)&scratch, (8 * words + 2 * (size_t)T * T) * 4, s) != cudaSuccess) {
       cudaGetLastError();
       return APSP_ENOMEM;
     }
