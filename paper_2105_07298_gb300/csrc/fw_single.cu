@@ -28,10 +28,15 @@
 //    8-row groups, warp-cooperative otherwise).  Either way P is exactly that
 //    of the sequential loop (ascending k, strict "<" keeps the first k
 //    reaching the final minimum).
+//  * From round 8 on (n > 2688) a bf16 product on the tensor cores finds the
+//    outputs that may improve, and only those are relaxed.
 //  * K1 is one cluster of eight CTAs, K2 keeps each row/column line in
 //    registers; both keep only minima per step and settle P afterwards.
 //  * Nothing reads P: K1/K2/K3 write P only where D strictly improved.
+#include <stddef.h>
 #include <stdint.h>
+
+#include <algorithm>
 
 #include "common.cuh"
 #include "scratch.h"
@@ -64,6 +69,44 @@ constexpr int kVecD = 1, kVecP = 2;
 struct DiagOps {
   unsigned long long *A, *B;
 };
+
+// What the screened phase 4 needs of a round besides the panels (all NULL in a
+// round that is not screened), see fw_phase3_screen_f32.
+//   EA[I][i][k], EB[J][j][k]: bf16 weights of the column and the row panel, 8-k
+//     chunks of a line moved to chunk (k / 8) ^ (line % 8);
+//   base_a[I][i], base_b[J][j]: the least entry of the line (0 if none is finite);
+//   whole_a[I][p], whole_b[J][p]: part p of the block holds only integers below
+//     2^22 in magnitude (and +inf);
+//   range: of the closed diagonal block, ordered keys of its largest finite
+//     entry and of minus its smallest;
+//   dense_next, dense_rest: lists the screen makes for the dense kernel.
+struct Screen {
+  uint32_t *EA, *EB;
+  float *base_a, *base_b;
+  int *whole_a, *whole_b;
+  unsigned *range;
+  int *dense_next, *dense_rest;  // [0]: tiles listed, [1..]: the tiles to relax densely, by block set
+};
+constexpr int kScreenParts = 4;  // parts of a block K2 reports on
+
+// Unsigned keys with the order of the floats (no NaN), and back.
+__device__ __forceinline__ unsigned fkey(float x) {
+  const unsigned u = __float_as_uint(x);
+  return (u >> 31) ? ~u : u | 0x80000000u;
+}
+__device__ __forceinline__ float fkey_value(unsigned k) { return __uint_as_float((k >> 31) ? k & 0x7fffffffu : ~k); }
+
+// 1 / s of a round, s = (largest - smallest finite entry of the diagonal block) / 48.
+__device__ __forceinline__ float screen_scale(const unsigned *range) {
+  const unsigned hi = range[0], lo = range[1];
+  const float span = hi && lo ? fkey_value(hi) + fkey_value(lo) : 0.0f;
+  return span > 0.0f ? fminf(fmaxf(48.0f / span, 1e-30f), 1e30f) : 1e-30f;
+}
+__device__ __forceinline__ float ex2(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
 
 // __byte_perm selector that replaces byte c of its first operand with byte 0 of its second.
 __device__ __forceinline__ constexpr unsigned byte_sel(int c) {
@@ -115,7 +158,7 @@ struct Smem {
 template <bool PATH>
 __global__ void __cluster_dims__(k1::CTAS, 1, 1) __launch_bounds__(32 * k1::WARPS, 1)
     fw_phase1_diag_f32(float *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r, int vec,
-                       int first, DiagOps ops) {
+                       int first, DiagOps ops, unsigned *range) {
   using namespace k1;
   using mp32::pack2;
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -255,6 +298,23 @@ __global__ void __cluster_dims__(k1::CTAS, 1, 1) __launch_bounds__(32 * k1::WARP
   __syncwarp();
   if (!ok) report_wait_timeout();  // D and P stay as they are
   if (ok) {
+    if (range) {
+      unsigned hi = 0u, lo = 0u;
+#pragma unroll
+      for (int rr = 0; rr < 4; ++rr)
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          if (d[rr][c] < INF) {
+            hi = max(hi, fkey(d[rr][c]));
+            lo = max(lo, fkey(-d[rr][c]));
+          }
+      hi = __reduce_max_sync(kFullMask, hi);
+      lo = __reduce_max_sync(kFullMask, lo);
+      if (lane == 0) {
+        atomicMax(&range[0], hi);
+        atomicMax(&range[1], lo);
+      }
+    }
     if (ops.A) {
 #pragma unroll
       for (int h = 0; h < 2; ++h)
@@ -339,7 +399,7 @@ struct Smem {
 template <bool PATH, int LINES>
 __global__ void __launch_bounds__(k2s::THREADS, 2)
     fw_phase2_lines_f32(float *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r, int R, int vec_in,
-                        DiagOps ops, Panels pan) {
+                        DiagOps ops, Panels pan, Screen scr) {
   using namespace k2s;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   static_assert(LINES == 2 || LINES == 4, "the lines of a position are one 8- or 16-byte access");
@@ -477,6 +537,35 @@ __global__ void __launch_bounds__(k2s::THREADS, 2)
 #pragma unroll
     for (int c = 0; c < LINES; ++c)
       *reinterpret_cast<float2 *>(&rows[(blk * T + line0 + c) * T + 2 * kp]) = make_float2(v[c][2 * hq], v[c][2 * hq + 1]);
+  }
+  if (scr.EA) {
+    const float inv = screen_scale(scr.range);
+    uint32_t *E = (is_row ? scr.EB : scr.EA) + blk * (T * T / 2);
+    bool whole = true;
+#pragma unroll
+    for (int c = 0; c < LINES; ++c) {
+      const int line = line0 + c;
+      float least = fminf(mp32::min3f(v[c][0], v[c][1], v[c][2]), v[c][3]);
+      least = fkey_value(__reduce_min_sync(kFullMask, fkey(least)));
+      least = least < INF ? least : 0.0f;
+      float e[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float x = v[c][q];
+        // at least 2^-(x - least) / s: 1/128 above what covers ex2's error and the rounding to bf16
+        e[q] = x < INF ? ex2(-fminf(__fmul_rn(__fsub_rn(x, least), inv), 60.0f)) * 1.0078125f : 0.0f;
+        whole = whole && (!(x < INF) || (x == rintf(x) && fabsf(x) < 4194304.0f));
+      }
+#pragma unroll
+      for (int hq = 0; hq < 2; ++hq) {  // k = 2 lane + 64 hq, + 1: chunk lane / 4 + 8 hq
+        uint32_t two;
+        asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(two) : "f"(e[2 * hq + 1]), "f"(e[2 * hq]));
+        E[line * (T / 2) + (((lane >> 2) + 8 * hq) ^ (line & 7)) * 4 + (lane & 3)] = two;
+      }
+      if (lane == 0) (is_row ? scr.base_b : scr.base_a)[blk * T + line] = least;
+    }
+    whole = __syncthreads_and(whole);
+    if (tid == 0) (is_row ? scr.whole_b : scr.whole_a)[blk * kScreenParts + part * kScreenParts / PARTS] = whole;
   }
   // D and P where the line improved (such positions lie inside the matrix).
 #pragma unroll
@@ -843,18 +932,16 @@ struct Smem {
 };
 }  // namespace k3s
 
+// Piece `sub` of output block (I, J): all 256 threads, the launch's dynamic
+// shared memory from offset 0, its barrier in phase 0.
 template <bool PATH, int TR>
-__global__ void __launch_bounds__(k3s::THREADS, TR == 32 ? 4 : 3)
-    fw_phase3_small_f32(float *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r, int R, int vec_ok,
-                        Panels pan, int set) {
+__device__ __forceinline__ void piece_f32(float *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r,
+                                          int I, int J, int sub, int vec_ok, const Panels &pan) {
   using namespace k3s;
   static_assert(TR == 32 || TR == 64, "eight warps of 16 x 16 or 16 x 32 outputs");
-  constexpr int CW = TR / 16, PER = per_block(TR);  // columns per thread
+  constexpr int CW = TR / 16;  // columns per thread
   extern __shared__ __align__(128) unsigned char smem_raw[];
   Smem<TR> &sm = *reinterpret_cast<Smem<TR> *>(smem_raw);
-  const int tile = blockIdx.x / PER, sub = blockIdx.x % PER;
-  int I, J;
-  block_of(set, tile, r, R, I, J);
   const int si = sub >> 1, hJ = sub & 1;
   const int baseI = I * T + si * TR, baseJ = J * T + hJ * TC, baseK = r * T;
   const int mI = min(TR, n - baseI), mJ = min(TC, n - baseJ), mK = min(T, n - baseK);
@@ -911,6 +998,7 @@ __global__ void __launch_bounds__(k3s::THREADS, TR == 32 ? 4 : 3)
     if (tid == 0) report_wait_timeout();
     return;
   }
+  if (tid == 0) mbar_inval(&sm.bar);  // its one phase is over: the next piece may set it up again
   auto step = [&](int kp) {
     const ulonglong2 a01 = *reinterpret_cast<const ulonglong2 *>(&sm.A[kp][r0]);
     const ulonglong2 a23 = *reinterpret_cast<const ulonglong2 *>(&sm.A[kp][r0 + 8]);
@@ -992,6 +1080,285 @@ __global__ void __launch_bounds__(k3s::THREADS, TR == 32 ? 4 : 3)
   }
 }
 
+template <bool PATH, int TR>
+__global__ void __launch_bounds__(k3s::THREADS, TR == 32 ? 4 : 3)
+    fw_phase3_small_f32(float *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r, int R, int vec_ok,
+                        Panels pan, int set) {
+  constexpr int PER = k3s::per_block(TR);
+  int I, J;
+  block_of(set, blockIdx.x / PER, r, R, I, J);
+  piece_f32<PATH, TR>(D, ld, P, n, r, I, J, blockIdx.x % PER, vec_ok, pan);
+}
+
+// --------------------------------------------------------------------------
+// K3 screened: phase 4 in rounds where few outputs improve.  A bf16 product on
+// the tensor cores finds the outputs that may improve, and only those are
+// relaxed in FP32.
+//
+// With s > 0 and any bases a_i, b_j, a candidate below the old value, D[i][k] +
+// D[k][j] < old, gives 2^-(D[i][k] - a_i)/s * 2^-(D[k][j] - b_j)/s >
+// 2^-(old - a_i - b_j)/s =: T.  K2 writes weights at least as large as the two
+// factors (the bases are the lines' least entries, so weights are at most about
+// 1; entries further than 60 s above get the weight of 60 s, +inf gets 0), so
+// the sum X of a row's products over the round's k exceeds T whenever any
+// candidate improves.  Outputs with X <= 0.96 T', T' lowered by what rounding
+// in its argument can amount to, are left as they are; the FP32 accumulation of
+// at most 128 non-negative normal products loses less than the factor covers.
+// The other outputs may or may not improve: the test sees a candidate within
+// about s log2(how many) of the old value.  Where both blocks hold only
+// integers, a candidate below the old value is at most ceil(old) - 1, and with
+// s <= 1/8 (128 ties at the old value weigh half of one a step below) the test
+// is exact.
+//
+// Flagged outputs are listed and settled four to a warp, eight lanes each: the
+// lanes add the row of A and the row of B^T, and the minimum and its first k are
+// taken over them - the values and the tie rule of the sequential loop.
+// A tile with more than kScreenDense flagged outputs is listed for
+// fw_phase3_listed_f32, which relaxes it densely.
+//
+// Bound: the latency of a tile's loads (weights, old values, then the flagged
+// outputs' rows), overlapped over four CTAs per SM; a tile of 128 x 64 with two
+// CTAs measured 8 % slower, settling one output a warp 25 %.  Measured per round
+// at n = 16384 (U[1, 100], p = 0.5): 0.64 ms from round 60 on, of which the
+// screen 0.58 (the dense kernel 2.0 ms); the product itself 0.22 ms on mma.sync
+// with 128 x 128 tiles, so its rate is not what counts.  Solves with P: n = 4096
+// 6.2 -> 4.4 ms, 8192 40.9 -> 24.3, 16384 289 -> 120; real weights and sparse
+// graphs gain likewise (n = 8192: U[0.5, 2) 22.2 ms, 16 edges a vertex 52.9
+// against 81).
+// --------------------------------------------------------------------------
+namespace k3x {
+constexpr int T = mp32::T, THREADS = 256;
+constexpr int H = T / 2, PER_BLOCK = 4;  // a CTA's tile: H x H, a quarter of a block
+constexpr int kScreenDense = 800;  // of H H outputs (625, 800, 1000: within 1 %)
+struct Smem {
+  uint32_t EA[H][T / 2], EB[H][T / 2];
+  float base_a[H], base_b[H];  // adjacent; base_b is read in pairs
+  uint64_t bar;
+  int count, next;
+  unsigned short list[kScreenDense];  // flagged outputs, i H + j
+};
+static_assert(offsetof(Smem, base_b) % 8 == 0 && offsetof(Smem, EB) % 128 == 0, "pairs and bulk copies");
+__device__ __forceinline__ void ldmatrix4(uint32_t (&f)[4], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(f[0]), "=r"(f[1]), "=r"(f[2]), "=r"(f[3])
+               : "r"(addr));
+}
+__device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+               "{%0, %1, %2, %3};"
+               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+               : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+}  // namespace k3x
+
+template <bool PATH>
+__global__ void __launch_bounds__(k3x::THREADS, 4)
+    fw_phase3_screen_f32(float *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r, int R, int vec_ok,
+                         Panels pan, Screen scr, int set) {
+  using namespace k3x;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
+  int I, J;
+  block_of(set, blockIdx.x / PER_BLOCK, r, R, I, J);
+  const int hI = (blockIdx.x >> 1) & 1, hJ = blockIdx.x & 1;
+  const int baseI = I * T + hI * H, baseJ = J * T + hJ * H, baseK = r * T;
+  const int mI = min(H, n - baseI), mJ = min(H, n - baseJ);
+  if (mI <= 0 || mJ <= 0) return;  // past the matrix (uniform exit)
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const float INF = inf<float>();
+  if (tid == 0) {
+    mbar_init(&sm.bar, 1);
+    fence_mbar_init();
+    mbar_expect_tx(&sm.bar, 2 * H * T * 2);
+    sm.count = sm.next = 0;
+  }
+  grid_dep_wait();
+  if (tid == 0) {
+    fence_proxy_async_global();
+    bulk_g2s(&sm.EA[0][0], scr.EA + (int64_t)I * (T * T / 2) + hI * (H * T / 2), H * T * 2, &sm.bar);
+    bulk_g2s(&sm.EB[0][0], scr.EB + (int64_t)J * (T * T / 2) + hJ * (H * T / 2), H * T * 2, &sm.bar);
+  }
+  // Warp (w / 4, w % 4): rows wi .. wi + 31, columns wj .. wj + 15.  Output (a, h,
+  // b, q) of lane l: row wi + 16 a + 8 h + l / 4, column wj + 8 b + 2 (l % 4) + q.
+  // The old values are under way while the weights arrive and are multiplied.
+  const int wi = 32 * (w >> 2), wj = 16 * (w & 3);
+  float2 o[2][2][2];
+#pragma unroll
+  for (int a = 0; a < 2; ++a)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int i = wi + 16 * a + 8 * h + (lane >> 2);
+      const float *row = D + (int64_t)(baseI + i) * ld + baseJ;
+#pragma unroll
+      for (int b = 0; b < 2; ++b) {
+        const int j = wj + 8 * b + 2 * (lane & 3);
+        o[a][h][b] = make_float2(-INF, -INF);  // outside the matrix: never flagged
+        if (i < mI) {
+          if (vec_ok && j + 1 < mJ) {
+            o[a][h][b] = *reinterpret_cast<const float2 *>(row + j);
+          } else {
+            if (j < mJ) o[a][h][b].x = row[j];
+            if (j + 1 < mJ) o[a][h][b].y = row[j + 1];
+          }
+        }
+      }
+    }
+  const float inv = screen_scale(scr.range);
+  if (tid < 2 * H) {  // the bases in units of s, less their share of the argument's error
+    const float v = tid < H ? scr.base_a[I * T + hI * H + tid] : scr.base_b[J * T + hJ * H + tid - H];
+    (&sm.base_a[0])[tid] = fmaf(v, inv, -fabsf(v) * (4.76837158203125e-7f * inv) - 0.03f);
+  }
+  bool whole = true;
+#pragma unroll
+  for (int p = 0; p < kScreenParts; ++p)
+    whole = whole && scr.whole_a[I * kScreenParts + p] && scr.whole_b[J * kScreenParts + p];
+  __syncthreads();
+  const bool ok = mbar_wait(&sm.bar, 0);
+  if (__syncthreads_or(!ok)) {  // the weights never arrived: the block stays as it is
+    if (tid == 0) report_wait_timeout();
+    return;
+  }
+  float x[2][2][4];
+#pragma unroll
+  for (int a = 0; a < 2; ++a)
+#pragma unroll
+    for (int b = 0; b < 2; ++b)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) x[a][b][c] = 0.0f;
+  const uint32_t sa = smem_addr(&sm.EA[0][0]), sb = smem_addr(&sm.EB[0][0]);
+  const int ar = wi + (lane & 15), ac = lane >> 4;                       // A: row, chunk
+  const int br = wj + (lane & 7) + 8 * (lane >> 4), bc = (lane >> 3) & 1;  // B: line, chunk
+#pragma unroll
+  for (int ks = 0; ks < T / 16; ++ks) {
+    uint32_t fb[4];
+    ldmatrix4(fb, sb + (uint32_t)(br * (T * 2) + (((2 * ks + bc) ^ (br & 7)) << 4)));
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+      uint32_t fa[4];
+      ldmatrix4(fa, sa + (uint32_t)((ar + 16 * a) * (T * 2) + (((2 * ks + ac) ^ (ar & 7)) << 4)));
+      mma_bf16(x[a][0], fa, fb[0], fb[1]);
+      mma_bf16(x[a][1], fa, fb[2], fb[3]);
+    }
+  }
+  // log2(0.96 T') = (a_i + b_j - t) / s, less what its roundings and ex2's can
+  // amount to: kErr of each of its three terms, and 0.06.
+  constexpr float kErr = 4.76837158203125e-7f;  // 2^-21
+  unsigned mine[2][2];  // [a][h]: bit 2 b + q
+  int found = 0;
+  auto test = [&](auto limit) {  // limit(old): the largest value a candidate below old can have
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        mine[a][h] = 0u;
+        const float ai = sm.base_a[wi + 16 * a + 8 * h + (lane >> 2)];
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+          const float2 bj = *reinterpret_cast<const float2 *>(&sm.base_b[wj + 8 * b + 2 * (lane & 3)]);
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            const float t = limit(q ? o[a][h][b].y : o[a][h][b].x);
+            const float arg = fmaf(-fabsf(t), kErr * inv, fmaf(-t, inv, ai + (q ? bj.y : bj.x)));
+            if (x[a][b][2 * h + q] > ex2(arg)) mine[a][h] |= 1u << (2 * b + q);
+          }
+        }
+        found += __popc(mine[a][h]);
+      }
+  };
+  if (whole)
+    test([](float old) {  // the largest integer below old, by rounding to nearest (old itself beyond 2^22)
+      const float near = __fadd_rn(__fadd_rn(old, 12582912.0f), -12582912.0f);
+      return fabsf(old) < 4194304.0f ? (near < old ? near : near - 1.0f) : old;
+    });
+  else test([](float old) { return old; });
+  found = __reduce_add_sync(kFullMask, found);
+  if (lane == 0 && found) atomicAdd(&sm.count, found);
+  __syncthreads();
+  const int count = sm.count;
+  if (count == 0) return;
+  if (count > kScreenDense) {  // left to the dense kernel
+    if (tid == 0) {
+      int *list = set == kSetNext ? scr.dense_next : scr.dense_rest;
+      list[1 + atomicAdd(&list[0], 1)] = blockIdx.x;
+    }
+    return;
+  }
+  // The flagged outputs as a list, in any order.
+  int at = __popc(mine[0][0]) + __popc(mine[0][1]) + __popc(mine[1][0]) + __popc(mine[1][1]);
+  if (at) at = atomicAdd(&sm.next, at);
+#pragma unroll
+  for (int a = 0; a < 2; ++a)
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      for (unsigned bits = mine[a][h]; bits; bits &= bits - 1) {
+        const int t = __ffs(bits) - 1;
+        sm.list[at++] = (unsigned short)((wi + 16 * a + 8 * h + (lane >> 2)) * H + wj + 8 * (t >> 1) + 2 * (lane & 3) + (t & 1));
+      }
+  __syncthreads();
+  // Eight lanes an output, four outputs a warp: lane s of an output adds
+  // entries 4 (s + 8 u) + c (u, c < 4) of the row of A and the row of B^T.
+  const float4 *acp = reinterpret_cast<const float4 *>(pan.Acp + ((int64_t)I * T + hI * H) * T);
+  const float4 *bt = reinterpret_cast<const float4 *>(pan.Bt + ((int64_t)J * T + hJ * H) * T);
+  const int s8 = lane & 7;
+#pragma unroll 1
+  for (int g = 4 * w; g < count; g += THREADS / 32 * 4) {
+    const int it = g + (lane >> 3), e = sm.list[min(it, count - 1)], i = e / H, j = e % H;
+    float *out = D + (int64_t)(baseI + i) * ld + baseJ + j;
+    float4 av[4], bv[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      av[u] = acp[i * (T / 4) + s8 + 8 * u];
+      bv[u] = bt[j * (T / 4) + s8 + 8 * u];
+    }
+    const float old = *out;
+    float c[16], m = INF;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      c[4 * u] = __fadd_rn(av[u].x, bv[u].x);
+      c[4 * u + 1] = __fadd_rn(av[u].y, bv[u].y);
+      c[4 * u + 2] = __fadd_rn(av[u].z, bv[u].z);
+      c[4 * u + 3] = __fadd_rn(av[u].w, bv[u].w);
+      m = mp32::min3f(mp32::min3f(m, c[4 * u], c[4 * u + 1]), c[4 * u + 2], c[4 * u + 3]);
+    }
+#pragma unroll
+    for (int d = 1; d < 8; d <<= 1) m = fminf(m, __shfl_xor_sync(kFullMask, m, d));
+    const bool better = it < count && m < old;
+    if (!__any_sync(kFullMask, better)) continue;
+    int k = T;  // this lane's first k that reaches m
+    if (PATH) {
+#pragma unroll
+      for (int u = 3; u >= 0; --u)
+#pragma unroll
+        for (int q = 3; q >= 0; --q) k = c[4 * u + q] == m ? 4 * (s8 + 8 * u) + q : k;
+#pragma unroll
+      for (int d = 1; d < 8; d <<= 1) k = min(k, __shfl_xor_sync(kFullMask, k, d));
+    }
+    if (better && s8 == 0) {
+      *out = m;
+      if (PATH) P[out - D] = baseK + k;
+    }
+  }
+}
+
+// The tiles the screen listed, relaxed densely: CTAs take 64-row pieces in turn.
+template <bool PATH>
+__global__ void __launch_bounds__(k3s::THREADS, 3)
+    fw_phase3_listed_f32(float *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r, int R, int vec_ok,
+                         Panels pan, Screen scr, int set) {
+  grid_dep_wait();
+  const int *list = set == kSetNext ? scr.dense_next : scr.dense_rest;
+  const int tiles = list[0];
+#pragma unroll 1
+  for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
+    const int tile = list[1 + t];
+    int I, J;
+    block_of(set, tile / k3x::PER_BLOCK, r, R, I, J);
+    fence_proxy_async_smem();
+    __syncthreads();  // everyone is done with the previous piece's shared memory
+    piece_f32<PATH, 64>(D, ld, P, n, r, I, J, tile % k3x::PER_BLOCK, vec_ok, pan);
+  }
+}
+
 // Phase timing state (see profile.h).
 std::mutex g_prof_mu;
 bool g_prof_on = false;
@@ -1019,7 +1386,13 @@ constexpr int kSms = 152;
 //    against 4.69);
 //  * the ring kernel otherwise (n = 8192 without P: 32.7 against 33.3).
 constexpr int kR32 = 21, kRNext32 = 40, kR64 = 40, kDenseRounds = 32;
-static int g_smem_k1[2][64], g_smem_k2[2][2][64], g_smem_k3s[2][2][64], g_smem_k3[64];
+// Phase 4 is screened from round 8 on (5 and 12 rounds: within 2 % at n = 4096
+// and 16384; about one output in r + 1 improves in round r of a random graph)
+// above 21 blocks a side, where the chain of the next round no longer sets the
+// pace.
+constexpr int kScreenMinR = 22, kScreenFrom = 8;
+static_assert(2 * (kScreenMinR - 1) * k2s::parts(4) >= kSms, "a screened round's K2 runs kScreenParts parts");
+static int g_smem_k1[2][64], g_smem_k2[2][2][64], g_smem_k3s[2][2][64], g_smem_k3[64], g_smem_k3x[2][64], g_smem_k3l[2][64];
 
 int run_fw_f64_interval(double *D, int n, int64_t ld, int32_t *P, cudaStream_t s,
                         void (*path_init)(int32_t *, int64_t, int64_t, int64_t, cudaStream_t));
@@ -1062,6 +1435,11 @@ static int run_fw_f32(float *D, int64_t n64, int64_t ld, int32_t *P, void *strea
   if ((st = ensure_smem(kernel32, (int)sizeof(k3s::Smem<32>), g_smem_k3s[0][P != nullptr]))) return st;
   if ((st = ensure_smem(kernel64, (int)sizeof(k3s::Smem<64>), g_smem_k3s[1][P != nullptr]))) return st;
   if ((st = ensure_smem(fw_phase3_minplus_f32, (int)sizeof(k3::Smem), g_smem_k3))) return st;
+  if ((st = ensure_smem(P ? fw_phase3_screen_f32<true> : fw_phase3_screen_f32<false>, (int)sizeof(k3x::Smem),
+                        g_smem_k3x[P != nullptr])) ||
+      (st = ensure_smem(P ? fw_phase3_listed_f32<true> : fw_phase3_listed_f32<false>, (int)sizeof(k3s::Smem<64>),
+                        g_smem_k3l[P != nullptr])))
+    return st;
   cudaGetLastError();  // clear any stale error so the checks below are ours
   // Phase-4 operand panels, written by K2 each round: two sets (round parity)
   // of 4 arrays of R*T*T 4-byte words, so that K2 of round r+1 can run while
@@ -1071,9 +1449,19 @@ static int run_fw_f32(float *D, int64_t n64, int64_t ld, int32_t *P, void *strea
   Panels pan[2]{};
   DiagOps ops{};
   char *scratch = nullptr;
+  Screen scr[2]{};
+  unsigned *ranges = nullptr;
+  int *dense_next = nullptr, *dense_rest = nullptr;
+  const bool screened = R >= kScreenMinR;
   if (R > 1) {
-    const size_t words = (size_t)R * T * T;
-    if (scratch_alloc((void **)&scratch, (8 * words + 2 * (size_t)T * T) * 4, s) != cudaSuccess) {
+    const size_t words = (size_t)R * T * T, diag = 2 * (size_t)T * T;
+    // per set: EA, EB (half a word per entry), bases, whole flags; per round: the range
+    const size_t scr_words = screened ? words + 2 * (size_t)R * T + 2 * (size_t)R * kScreenParts : 0;
+    const size_t range_words = screened ? 2 * (size_t)R : 0;
+    // the dense lists: a count and every tile of the set
+    const size_t next_words = 1 + k3x::PER_BLOCK * 2 * (size_t)R, rest_words = 1 + k3x::PER_BLOCK * (size_t)R * R;
+    const size_t list_words = screened ? next_words + rest_words : 0;
+    if (scratch_alloc((void **)&scratch, (8 * words + diag + 2 * scr_words + range_words + list_words) * 4, s) != cudaSuccess) {
       cudaGetLastError();
       return APSP_ENOMEM;
     }
@@ -1086,7 +1474,35 @@ static int run_fw_f32(float *D, int64_t n64, int64_t ld, int32_t *P, void *strea
     }
     ops.A = reinterpret_cast<unsigned long long *>(scratch + 8 * words * 4);
     ops.B = ops.A + T * T / 2;
+    if (screened) {
+      uint32_t *base = reinterpret_cast<uint32_t *>(scratch + (8 * words + diag) * 4);
+      for (int q = 0; q < 2; ++q, base += scr_words) {
+        scr[q].EA = base;
+        scr[q].EB = base + words / 2;
+        scr[q].base_a = reinterpret_cast<float *>(base + words);
+        scr[q].base_b = scr[q].base_a + (size_t)R * T;
+        scr[q].whole_a = reinterpret_cast<int *>(scr[q].base_b + (size_t)R * T);
+        scr[q].whole_b = scr[q].whole_a + (size_t)R * kScreenParts;
+      }
+      ranges = base;
+      dense_next = reinterpret_cast<int *>(base + range_words);
+      dense_rest = dense_next + next_words;
+      if (cudaMemsetAsync(ranges, 0, range_words * 4, s) != cudaSuccess) {
+        cudaFreeAsync(scratch, s);
+        cudaGetLastError();
+        return APSP_ECUDA;
+      }
+    }
   }
+  // The round's screening data, or none where the round is not screened.
+  auto screen_of = [&](int r) {
+    if (!screened || r < kScreenFrom) return Screen{};
+    Screen sc = scr[r & 1];
+    sc.range = ranges + 2 * r;
+    sc.dense_next = dense_next;
+    sc.dense_rest = dense_rest;
+    return sc;
+  };
   const bool aligned = ld % 4 == 0;
   const int vec = (aligned && (reinterpret_cast<uintptr_t>(D) & 15) == 0 ? kVecD : 0) |
                   (aligned && (reinterpret_cast<uintptr_t>(P) & 15) == 0 ? kVecP : 0);
@@ -1105,17 +1521,24 @@ static int run_fw_f32(float *D, int64_t n64, int64_t ld, int32_t *P, void *strea
   auto diag = [&](int r, cudaStream_t st) {
     PhaseScope ps(1, st);
     launch_after(P ? fw_phase1_diag_f32<true> : fw_phase1_diag_f32<false>, k1::CTAS, 32 * k1::WARPS, sizeof(k1::Smem),
-                 st, overlap, D, ld, P, n, r, vec, (int)(P && r == 0), ops);
+                 st, overlap, D, ld, P, n, r, vec, (int)(P && r == 0), ops, screen_of(r).range);
   };
   auto panels = [&](int r, cudaStream_t st) {
     PhaseScope ps(2, st);
     launch_after(lines_kernel, 2 * (R - 1) * k2s::parts(lines), k2s::THREADS, lines_smem, st, overlap, D, ld, P, n, r, R,
-                 vec, ops, pan[r & 1]);
+                 vec, ops, pan[r & 1], screen_of(r));
   };
   auto phase4 = [&](int r, int set, int blocks, cudaStream_t st) {
     if (blocks <= 0) return;
     PhaseScope ps(3, st);
-    if (R <= kR32 || (set == kSetNext && R <= kRNext32))
+    if (screened && r >= kScreenFrom) {
+      const Screen sc = screen_of(r);
+      cudaMemsetAsync(set == kSetNext ? sc.dense_next : sc.dense_rest, 0, sizeof(int), st);
+      launch_after(P ? fw_phase3_screen_f32<true> : fw_phase3_screen_f32<false>, k3x::PER_BLOCK * blocks, k3x::THREADS,
+                   sizeof(k3x::Smem), st, overlap, D, ld, P, n, r, R, vec_ok, pan[r & 1], sc, set);
+      launch_after(P ? fw_phase3_listed_f32<true> : fw_phase3_listed_f32<false>, std::min(4 * blocks, 3 * kSms),
+                   k3s::THREADS, sizeof(k3s::Smem<64>), st, overlap, D, ld, P, n, r, R, vec_ok, pan[r & 1], sc, set);
+    } else if (R <= kR32 || (set == kSetNext && R <= kRNext32))
       launch_after(kernel32, k3s::per_block(32) * blocks, k3s::THREADS, sizeof(k3s::Smem<32>), st, overlap, D, ld, P, n,
                    r, R, vec_ok, pan[r & 1], set);
     else if (P ? r < kDenseRounds : R <= kR64)

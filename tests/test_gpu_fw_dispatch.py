@@ -102,3 +102,46 @@ def test_batched_blocks_at_quad_and_tile_edges(d_off, with_path):
         np.testing.assert_array_equal(D, oracle.fw(m)[0])
         if with_path:
             assert oracle.check_paths(m, D, P[int(o):int(o) + n * n].view(n, n).cpu().numpy()) == 0
+
+
+def _screened_graph(kind, n):
+    """Weights for the screened rounds (more than 21 blocks a side, from round 8 on)."""
+    rng = np.random.default_rng(3)
+    if kind == "integers":
+        return graphgen.dense_graph(n, 0.1, 21)
+    if kind == "halves":
+        return graphgen.dense_graph(n, 0.1, 22) * np.float32(0.5)
+    if kind == "beyond 2^22":  # integers, but not all of them below 2^22
+        return graphgen.dense_graph(n, 0.02, 23, lo=1, hi=9_000_000)
+    if kind == "sparse":  # most pairs far apart, some unreachable; diagonal blocks nearly empty
+        return graphgen.dense_graph(n, 0.001, 24, weights="real", lo=0.5, hi=2.0)
+    if kind == "no edges":
+        return graphgen.dense_graph(n, 0.0, 25)
+    W = graphgen.dense_graph(n, 0.05, 26, weights="real", lo=0.5, hi=2.0)
+    if kind == "negative":  # shifted by potentials: negative edges, no negative cycle but by rounding
+        h = rng.integers(-64, 65, n).astype(np.float32)
+        W = graphgen.dense_graph(n, 0.05, 26, lo=1, hi=100) + h[:, None] - h[None, :]
+    if kind == "clusters":  # distances within a cluster near 1e-3, between clusters near 1e6
+        c = np.arange(n) % 3
+        W = np.where(c[:, None] == c[None, :], W * np.float32(1e-3), W + np.float32(1e6)).astype(np.float32)
+    np.fill_diagonal(W, 0)
+    return W
+
+
+@pytest.mark.parametrize("kind", ["integers", "halves", "beyond 2^22", "sparse", "no edges", "real", "negative",
+                                  "clusters"])
+def test_screened_rounds_bitwise(kind):
+    n = 2900
+    W = _screened_graph(kind, n)
+    Db, Pb = oracle.bfw(W, 128)
+    ld = n + 1 if kind in ("real", "integers") else n  # rows off 16-byte boundaries too
+    D = torch.empty((n, ld), device=DEV)[:, :n]
+    P = torch.empty((n, ld), dtype=torch.int32, device=DEV)[:, :n]
+    D.copy_(torch.from_numpy(W))
+    apsp.apsp_fw(D, P)
+    np.testing.assert_array_equal(D.cpu().numpy(), Db)
+    np.testing.assert_array_equal(P.cpu().numpy(), Pb)
+    D.copy_(torch.from_numpy(W))
+    apsp.apsp_fw(D)
+    np.testing.assert_array_equal(D.cpu().numpy(), Db)
+    assert apsp.device_status() == apsp.APSP_OK
