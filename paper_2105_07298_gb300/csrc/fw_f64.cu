@@ -299,33 +299,37 @@ __device__ __forceinline__ void relax_lines(WarpLines &L, int kq, bool own, int 
   __syncwarp();
 }
 
-// K1: phase 1 on block (r,r) by one cluster of eight CTAs of four warps, as
+// K1: phase 1 on block (r,r) by one cluster of eight CTAs of four row warps, as
 // the FP32 path's: a warp owns four adjacent rows, lane l their columns
 // 4l..4l+3, and takes the four steps of a quad together.  The quad's own rows
-// are brought to their steps by all four warps of the owning CTA (a column a
-// lane) and passed around the ring of CTAs by st.async.  The buffers hold
-// eight quads (so that the kernel leaves room beside phase-4 CTAs): a CTA's
-// four quads reuse the space of the quads eight before, which every CTA has
-// left behind by then (a split cluster barrier per four quads).
+// are brought to their steps by four helper warps of the owning CTA (a column a
+// lane) while the others bring their pivots up; the helpers also pass the quads
+// around the ring of CTAs by st.async.  The buffers hold eight quads (so that
+// the kernel leaves room beside phase-4 CTAs): a CTA's four quads reuse the
+// space of the quads eight before, which every CTA has left behind by then (a
+// split cluster barrier per four quads).
 // Bound: the chain of 32 quads (up to six dependent FP64 adds each), and while
 // many elements still improve the FP64 adds of their candidates.  Measured per
-// launch at n = 1000, real weights: 65-105 us, of which 1.9 us a quad (one CTA
-// that took each flagged element in a serial loop per step: 245-600 us);
-// taking a lane's own flagged elements in place instead of listing them for
-// the warp 125-218 us.
+// launch at n = 1000, real weights: 61-95 us, 1.9 us a quad (one CTA that took
+// each flagged element in a serial loop per step: 245-600 us; this split with
+// the row warps doing the helpers' work: 65-105 us, the whole solve 1.14 ms
+// against 1.08); taking a lane's own flagged elements in place instead of
+// listing them for the warp 125-218 us.
 namespace k1 {
-constexpr int CTAS = 8, WARPS = 4, RING = 2 * WARPS;
+constexpr int CTAS = 8, WARPS = 4, RING = 2 * WARPS;  // WARPS: that own rows; as many help
+constexpr int THREADS = 64 * WARPS;
 struct Smem {
   double r64[RING][4][T];              // row s of the quad at its step
   unsigned long long rlo[RING][2][T];  // their lower bounds, rows (0, 1) and (2, 3)
   WarpLines wl[WARPS];
   double es[3][4];                     // the own quad's rows at its columns, at their steps
+  float eslo[3][4];                    // their lower bounds
   uint64_t bar[QUADS];
 };
 constexpr uint32_t QUAD_BYTES = 4 * T * 8 + 2 * T * 8;
 }  // namespace k1
 
-__global__ void __cluster_dims__(k1::CTAS, 1, 1) __launch_bounds__(32 * k1::WARPS, 1)
+__global__ void __cluster_dims__(k1::CTAS, 1, 1) __launch_bounds__(k1::THREADS, 2)
     fw64_diag(double *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r, int vec, int first,
               DiagOps64 ops) {
   using namespace k1;
@@ -333,17 +337,18 @@ __global__ void __cluster_dims__(k1::CTAS, 1, 1) __launch_bounds__(32 * k1::WARP
   Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
   const int base = r * T, m = min(T, n - base), nquad = (m + 3) / 4;
   const int cta = (int)cluster_cta_rank(), tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const int own = cta * WARPS + w;  // this warp's row quad
-  const int i0 = 4 * own, j0 = 4 * lane;
+  const bool helper = w >= WARPS;
+  const int own = helper ? -1 : cta * WARPS + w;  // this warp's row quad
+  const int i0 = 4 * own, j0 = 4 * lane, ht = tid - 32 * WARPS;  // ht: a helper's column
   if (tid < QUADS) {
     mbar_init(&sm.bar[tid], 1);
     fence_mbar_init();
     if (tid / WARPS != cta) mbar_expect_tx(&sm.bar[tid], QUAD_BYTES);
   }
   grid_dep_wait();
-  WarpLines &L = sm.wl[w];
+  WarpLines &L = sm.wl[w % WARPS];
 #pragma unroll
-  for (int rr = 0; rr < 4; ++rr) {
+  for (int rr = 0; rr < 4 && !helper; ++rr) {
     const double *row = D + (int64_t)(base + i0 + rr) * ld + base;
     *reinterpret_cast<unsigned *>(&L.pk[rr][j0]) = 0xFFFFFFFFu;
 #pragma unroll
@@ -370,33 +375,40 @@ __global__ void __cluster_dims__(k1::CTAS, 1, 1) __launch_bounds__(32 * k1::WARP
   for (int kq = 0; kq < nquad; ++kq) {
     const int g = kq / WARPS, ow = kq % WARPS, slot = kq % RING;
     const bool mine = kq == own;
-    double v = L.d[(lane >> 2) & 3][4 * kq + (lane & 3)];
+    double v = 0.0;
     float vlo;
+    auto keep_pivots = [&]() {
+      if (lane < 16) {
+        (&L.ps[0][0])[lane] = v;
+        (&L.plo[0][0])[lane] = vlo;
+      }
+    };
+    if (!helper) v = L.d[(lane >> 2) & 3][4 * kq + (lane & 3)];
     if (cta == g) {
       if (mine) {
         double e[3];
         quad_pivots_own(v, vlo, e, lane);
         if (lane < 4) {
 #pragma unroll
-          for (int u = 0; u < 3; ++u) sm.es[u][lane] = e[u];
+          for (int u = 0; u < 3; ++u) {
+            sm.es[u][lane] = e[u];
+            sm.eslo[u][lane] = f64_down(e[u]);
+          }
         }
-        if (lane < 16) {
-          (&L.ps[0][0])[lane] = v;
-          (&L.plo[0][0])[lane] = vlo;
-        }
+        keep_pivots();
       }
       __syncthreads();
-      {  // column tid: the quad's rows at their steps
+      if (helper) {  // column ht: the quad's rows at their steps
         double q[4];
         float qlo[4];
         bool may = false;
 #pragma unroll
         for (int s = 0; s < 4; ++s) {
-          q[s] = sm.wl[ow].d[s][tid];
+          q[s] = sm.wl[ow].d[s][ht];
           qlo[s] = f64_down(q[s]);
 #pragma unroll
           for (int u = 0; u < 3; ++u)
-            if (u < s) may |= __fadd_rd(sm.wl[ow].plo[s][u], qlo[u]) < sm.wl[ow].hi[s][tid];
+            if (u < s) may |= __fadd_rd(sm.wl[ow].plo[s][u], qlo[u]) < sm.wl[ow].hi[s][ht];
         }
         if (may) {  // (a column whose rows cannot improve keeps its values)
 #pragma unroll
@@ -411,47 +423,44 @@ __global__ void __cluster_dims__(k1::CTAS, 1, 1) __launch_bounds__(32 * k1::WARP
           }
         }
 #pragma unroll
-        for (int s = 0; s < 4; ++s) sm.r64[slot][s][tid] = q[s];
-        sm.rlo[slot][0][tid] = packf2(qlo[0], qlo[1]);
-        sm.rlo[slot][1][tid] = packf2(qlo[2], qlo[3]);
-      }
-      if (!mine) {
-        float elo[3];
-#pragma unroll
-        for (int s = 0; s < 3; ++s) elo[s] = f64_down(sm.es[s][lane & 3]);
+        for (int s = 0; s < 4; ++s) sm.r64[slot][s][ht] = q[s];
+        sm.rlo[slot][0][ht] = packf2(qlo[0], qlo[1]);
+        sm.rlo[slot][1][ht] = packf2(qlo[2], qlo[3]);
+      } else if (!mine) {
+        const float elo[3] = {sm.eslo[0][lane & 3], sm.eslo[1][lane & 3], sm.eslo[2][lane & 3]};
         quad_pivots(v, vlo, elo, lane, [&](int s) { return sm.es[s][lane & 3]; });
+        keep_pivots();
       }
       __syncthreads();
     } else {
       if (ok) ok = mbar_spin(&sm.bar[kq], 0);
     }
-    if (next != (unsigned)g) {  // pass the quad on to the next CTA of the ring
-      const uint32_t bar = next_base + smem_addr(&sm.bar[kq]);
-      const ulonglong2 *src = reinterpret_cast<const ulonglong2 *>(&sm.r64[slot][0][0]);
-      const ulonglong2 *srl = reinterpret_cast<const ulonglong2 *>(&sm.rlo[slot][0][0]);
+    if (helper) {
+      if (next != (unsigned)g) {  // pass the quad on to the next CTA of the ring
+        const uint32_t bar = next_base + smem_addr(&sm.bar[kq]);
+        const ulonglong2 *src = reinterpret_cast<const ulonglong2 *>(&sm.r64[slot][0][0]);
+        const ulonglong2 *srl = reinterpret_cast<const ulonglong2 *>(&sm.rlo[slot][0][0]);
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const ulonglong2 t = src[tid + 128 * u];
-        st_async16(next_base + smem_addr(src + tid + 128 * u), t.x, t.y, bar);
+        for (int u = 0; u < 2; ++u) {
+          const ulonglong2 t = src[ht + 128 * u];
+          st_async16(next_base + smem_addr(src + ht + 128 * u), t.x, t.y, bar);
+        }
+        const ulonglong2 t = srl[ht];
+        st_async16(next_base + smem_addr(srl + ht), t.x, t.y, bar);
       }
-      const ulonglong2 t = srl[tid];
-      st_async16(next_base + smem_addr(srl + tid), t.x, t.y, bar);
-    }
-    if (!mine) {
+    } else {
       if (cta != g) {
         const int t = 4 * kq + (lane & 3);
         const unsigned long long e01 = sm.rlo[slot][0][t], e23 = sm.rlo[slot][1][t];
         const float elo[3] = {__uint_as_float((unsigned)e01), __uint_as_float((unsigned)(e01 >> 32)),
                               __uint_as_float((unsigned)e23)};
         quad_pivots(v, vlo, elo, lane, [&](int s) { return sm.r64[slot][s][t]; });
+        keep_pivots();
       }
-      if (lane < 16) {
-        (&L.ps[0][0])[lane] = v;
-        (&L.plo[0][0])[lane] = vlo;
-      }
+      __syncwarp();
+      relax_lines(L, kq, mine, lane, sm.rlo[slot][0], sm.rlo[slot][1],
+                  [&](int s, int pos) { return sm.r64[slot][s][pos]; });
     }
-    __syncwarp();
-    relax_lines(L, kq, mine, lane, sm.rlo[slot][0], sm.rlo[slot][1], [&](int s, int pos) { return sm.r64[slot][s][pos]; });
     if (ow == WARPS - 1 || kq + 1 == nquad) {  // done with CTA g's quads
       if (g > 0) cluster_wait();               // and so is everyone with CTA g-1's, whose space comes next
       cluster_arrive();
@@ -463,6 +472,7 @@ __global__ void __cluster_dims__(k1::CTAS, 1, 1) __launch_bounds__(32 * k1::WARP
     report_wait_timeout();
     return;
   }
+  if (helper) return;
   double d[4][4];
 #pragma unroll
   for (int rr = 0; rr < 4; ++rr)
@@ -886,7 +896,7 @@ int run_fw_f64_interval(double *D, int n, int64_t ld, int32_t *P, cudaStream_t s
   };
   auto diag = [&](int r, cudaStream_t stm) {
     PhaseScope sc(1, stm);
-    launch_after(fw64_diag, k1::CTAS, 32 * k1::WARPS, sizeof(k1::Smem), stm, overlap, D, ld, P, n, r, vec,
+    launch_after(fw64_diag, k1::CTAS, k1::THREADS, sizeof(k1::Smem), stm, overlap, D, ld, P, n, r, vec,
                  (int)(P && r == 0), ops);
   };
   auto panels = [&](int r, cudaStream_t stm) {
