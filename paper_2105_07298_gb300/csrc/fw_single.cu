@@ -1206,7 +1206,8 @@ __global__ void __launch_bounds__(k3x::THREADS, 4)
   const float inv = screen_scale(scr.range);
   if (tid < 2 * H) {  // the bases in units of s, less their share of the argument's error
     const float v = tid < H ? scr.base_a[I * T + hI * H + tid] : scr.base_b[J * T + hJ * H + tid - H];
-    (&sm.base_a[0])[tid] = fmaf(v, inv, -fabsf(v) * (4.76837158203125e-7f * inv) - 0.03f);
+    const float b = fmaf(v, inv, -fabsf(v) * (4.76837158203125e-7f * inv) - 0.03f);
+    (&sm.base_a[0])[tid] = fabsf(b) < 1e38f ? b : -INF;  // beyond the floats: the line's outputs are all flagged
   }
   bool whole = true;
 #pragma unroll
@@ -1259,7 +1260,8 @@ __global__ void __launch_bounds__(k3x::THREADS, 4)
           for (int q = 0; q < 2; ++q) {
             const float t = limit(q ? o[a][h][b].y : o[a][h][b].x);
             const float arg = fmaf(-fabsf(t), kErr * inv, fmaf(-t, inv, ai + (q ? bj.y : bj.x)));
-            if (x[a][b][2 * h + q] > ex2(arg)) mine[a][h] |= 1u << (2 * b + q);
+            // (NaN, where t / s and the bases overflow, is flagged; nothing is below -inf)
+            if (!(x[a][b][2 * h + q] <= ex2(arg)) && t > -INF) mine[a][h] |= 1u << (2 * b + q);
           }
         }
         found += __popc(mine[a][h]);

@@ -124,12 +124,17 @@ def _screened_graph(kind, n):
     if kind == "clusters":  # distances within a cluster near 1e-3, between clusters near 1e6
         c = np.arange(n) % 3
         W = np.where(c[:, None] == c[None, :], W * np.float32(1e-3), W + np.float32(1e6)).astype(np.float32)
+    if kind == "huge":  # far above the diagonal blocks' spread: in its units the weights overflow
+        c = np.arange(n) // 128
+        near = rng.uniform(0.005, 0.02, (n, n)).astype(np.float32)
+        far = graphgen.dense_graph(n, 1e-4, 27, weights="real", lo=0.5, hi=2.0) * np.float32(5e37)
+        W = np.where(c[:, None] == c[None, :], near, far)
     np.fill_diagonal(W, 0)
     return W
 
 
 @pytest.mark.parametrize("kind", ["integers", "halves", "beyond 2^22", "sparse", "no edges", "real", "negative",
-                                  "clusters"])
+                                  "clusters", "huge"])
 def test_screened_rounds_bitwise(kind):
     n = 2900
     W = _screened_graph(kind, n)
