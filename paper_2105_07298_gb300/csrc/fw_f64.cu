@@ -21,7 +21,9 @@
 //  K1  fw64_diag     phase 1: Algorithm 1 on block (r,r), k sequential.
 //  K2  fw64_lines    phases 2 and 3: the row blocks (r,J) and column blocks
 //                    (I,r), k sequential per line; writes the phase-4 operands.
-//  K3  fw64_pieces   phase 4: (I,J) <- min(C, D(I,r) (x) D(r,J)).
+//  K3  fw64_pieces   phase 4: (I,J) <- min(C, D(I,r) (x) D(r,J)); in the later
+//      fw64_screen   rounds of large matrices only where a screen on the
+//      fw64_listed   tensor cores finds that outputs may improve.
 // Rounds overlap as in the FP32 path (rounds.cuh).
 // Every candidate sum is one IEEE FP64 addition rounded to nearest, taken in
 // the order of the sequential blocked FW, so D and P are bit-exact with it on
@@ -29,11 +31,14 @@
 #include <float.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "bulk.cuh"
 #include "common.cuh"
 #include "scratch.h"
 #include "profile.h"
 #include "rounds.cuh"
+#include "screen.cuh"
 
 namespace apsp {
 namespace f64 {
@@ -46,9 +51,12 @@ constexpr int T = 128, PAIRS = T / 2, QUADS = T / 4;
 //                       A64[I][i][k] = D[i][k]
 //   row block (r,J):    B[J][j/64][kp][j%64] = (rd D[2kp][j], rd D[2kp+1][j]),
 //                       B64[J][j][k] = D[k][j]
+// and in a screened round the lower bounds as rows too: Alo[I][i][k] = rd
+// A64[I][i][k], Blo[J][j][k] = rd B64[J][j][k].
 struct Panels64 {
   unsigned long long *A, *B;
   double *A64, *B64;
+  float *Alo, *Blo;
 };
 // The closed diagonal block in K2's layouts, written by K1: lower bounds
 // k-paired, Alo[kp][i] = (rd D[i][2kp], rd D[i][2kp+1]), Blo[kp][j] =
@@ -331,7 +339,7 @@ constexpr uint32_t QUAD_BYTES = 4 * T * 8 + 2 * T * 8;
 
 __global__ void __cluster_dims__(k1::CTAS, 1, 1) __launch_bounds__(k1::THREADS, 2)
     fw64_diag(double *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r, int vec, int first,
-              DiagOps64 ops) {
+              DiagOps64 ops, unsigned *__restrict__ range) {
   using namespace k1;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
@@ -478,6 +486,20 @@ __global__ void __cluster_dims__(k1::CTAS, 1, 1) __launch_bounds__(k1::THREADS, 
   for (int rr = 0; rr < 4; ++rr)
 #pragma unroll
     for (int c = 0; c < 4; ++c) d[rr][c] = L.d[rr][j0 + c];
+  if (range) {  // of the lower bounds
+    unsigned hi = 0u, lo = 0u;
+#pragma unroll
+    for (int rr = 0; rr < 4; ++rr)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const float x = f64_down(d[rr][c]);
+        if (x < inf<float>()) {
+          hi = max(hi, fkey(x));
+          lo = max(lo, fkey(-x));
+        }
+      }
+    screen_range(range, hi, lo);
+  }
   if (ops.Alo) {
 #pragma unroll
     for (int h = 0; h < 2; ++h)
@@ -533,7 +555,7 @@ struct Smem {
 
 __global__ void __launch_bounds__(32 * k2::WARPS, 2)
     fw64_lines(double *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r, int R, int vec,
-               DiagOps64 ops, Panels64 pan) {
+               DiagOps64 ops, Panels64 pan, Screen scr) {
   using namespace k2;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
@@ -640,6 +662,32 @@ __global__ void __launch_bounds__(32 * k2::WARPS, 2)
 #pragma unroll
     for (int q = 0; q < 4; q += 2)
       *reinterpret_cast<double2 *>(&rows[(blk * T + line0 + c) * T + p0 + q]) = make_double2(v[c][q], v[c][q + 1]);
+  if (scr.EA) {
+    const float inv = screen_scale(scr.range);
+    uint32_t *E = (is_row ? scr.EB : scr.EA) + blk * (T * T / 2);
+    float *rlo = is_row ? pan.Blo : pan.Alo;
+    bool whole = true;
+#pragma unroll
+    for (int c = 0; c < LINES; ++c) {
+      const int line = line0 + c;
+      float lo[4], e[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) lo[q] = f64_down(v[c][q]);
+      *reinterpret_cast<float4 *>(&rlo[(blk * T + line) * T + p0]) = make_float4(lo[0], lo[1], lo[2], lo[3]);
+      const float least = screen_least(lo[0], lo[1], lo[2], lo[3]);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        e[q] = screen_weight(lo[q], least, inv);
+        whole = whole && screen_whole(lo[q]) && lo[q] == f64_up(v[c][q]);
+      }
+      // k = 4 lane .. 4 lane + 3: half of chunk lane / 2
+      *reinterpret_cast<uint2 *>(&E[line * (T / 2) + ((lane >> 1) ^ (line & 7)) * 4 + 2 * (lane & 1)]) =
+          make_uint2(bf16x2(e[0], e[1]), bf16x2(e[2], e[3]));
+      if (lane == 0) (is_row ? scr.base_b : scr.base_a)[blk * T + line] = least;
+    }
+    whole = __syncthreads_and(whole);
+    if (tid == 0) (is_row ? scr.whole_b : scr.whole_a)[blk * PARTS + part] = whole;
+  }
 #pragma unroll
   for (int c = 0; c < LINES; ++c)
 #pragma unroll
@@ -679,17 +727,12 @@ struct Smem {
 };
 }  // namespace k3
 
-template <int CTAS_PER_SM>
-__global__ void __launch_bounds__(k3::THREADS, CTAS_PER_SM)
-    fw64_pieces(double *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r, int R, Panels64 pan,
-                int set) {
+__device__ __forceinline__ void piece64(double *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r,
+                                        int I, int J, int sub, const Panels64 &pan) {
   using namespace k3;
   constexpr int CW = 2;  // columns per thread
   extern __shared__ __align__(128) unsigned char smem_raw[];
   Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
-  const int tile = blockIdx.x / PER_BLOCK, sub = blockIdx.x % PER_BLOCK;
-  int I, J;
-  block_of(set, tile, r, R, I, J);
   const int si = sub >> 1, hJ = sub & 1;
   const int baseI = I * T + si * TR, baseJ = J * T + hJ * TC, baseK = r * T;
   const int mI = min(TR, n - baseI), mJ = min(TC, n - baseJ), mK = min(T, n - baseK);
@@ -840,13 +883,144 @@ __global__ void __launch_bounds__(k3::THREADS, CTAS_PER_SM)
   }
 }
 
-static int g_smem_k1[64], g_smem_k2[64], g_smem_k3[2][64];
+template <int CTAS_PER_SM>
+__global__ void __launch_bounds__(k3::THREADS, CTAS_PER_SM)
+    fw64_pieces(double *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r, int R, Panels64 pan,
+                int set) {
+  int I, J;
+  block_of(set, blockIdx.x / k3::PER_BLOCK, r, R, I, J);
+  piece64(D, ld, P, n, r, I, J, blockIdx.x % k3::PER_BLOCK, pan);
+}
+
+// K3 screened (screen.cuh), on the lower bounds of the panels and the upper
+// bounds of the old values: a candidate below the old value has a lower-bound
+// sum below its upper bound.  Eight lanes settle a flagged output, four outputs
+// a warp: lane s takes entries 4 (s + 8 u) + q (u, q < 4) of the row of Alo and
+// the row of Blo; the candidate of the least sum is added in FP64 first, then
+// those whose lower-bound sum its value does not exclude.
+// Bound: as the FP32 screen, the latency of the loads; at n = 4096 the next
+// round's chain (K1 90, K2 60, row and column r+1 50 us) sets the pace.  n =
+// 4096 / 6000 with P, integers: 9.8 / 27.2 -> 8.7 / 21.1 ms.
+__global__ void __launch_bounds__(k3x::THREADS, 4)
+    fw64_screen(double *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r, int R, int vec, Panels64 pan,
+                Screen scr, int set) {
+  using namespace k3x;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
+  const float FINF = inf<float>();
+  Tile tile;
+  const int count = screen_tile<k2::PARTS>(sm, tile, n, r, R, scr, set, [&](int i, int j, int left) {
+    const double *p = D + (int64_t)i * ld + j;
+    if (vec && left > 1) {
+      const double2 t = *reinterpret_cast<const double2 *>(p);
+      return make_float2(f64_up(t.x), f64_up(t.y));
+    }
+    return make_float2(left > 0 ? f64_up(p[0]) : -FINF, left > 1 ? f64_up(p[1]) : -FINF);
+  });
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, s8 = lane & 7;
+  const float4 *alo = reinterpret_cast<const float4 *>(pan.Alo + (int64_t)tile.baseI * T);
+  const float4 *blo = reinterpret_cast<const float4 *>(pan.Blo + (int64_t)tile.baseJ * T);
+#pragma unroll 1
+  for (int g = 4 * w; g < count; g += THREADS / 32 * 4) {
+    const int it = g + (lane >> 3), e = sm.list[min(it, count - 1)], i = e / H, j = e % H;
+    double *out = D + (int64_t)(tile.baseI + i) * ld + tile.baseJ + j;
+    float4 av[4], bv[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      av[u] = alo[i * (T / 4) + s8 + 8 * u];
+      bv[u] = blo[j * (T / 4) + s8 + 8 * u];
+    }
+    const double was = *out;
+    float c[16], m = FINF;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      c[4 * u] = __fadd_rd(av[u].x, bv[u].x);
+      c[4 * u + 1] = __fadd_rd(av[u].y, bv[u].y);
+      c[4 * u + 2] = __fadd_rd(av[u].z, bv[u].z);
+      c[4 * u + 3] = __fadd_rd(av[u].w, bv[u].w);
+      m = min3f(min3f(m, c[4 * u], c[4 * u + 1]), c[4 * u + 2], c[4 * u + 3]);
+    }
+    float least = m;
+#pragma unroll
+    for (int d = 1; d < 8; d <<= 1) least = fminf(least, __shfl_xor_sync(kFullMask, least, d));
+    const bool may = it < count && least < f64_up(was);
+    if (!__any_sync(kFullMask, may)) continue;
+    const double *ra = pan.A64 + (int64_t)(tile.baseI + i) * T, *rb = pan.B64 + (int64_t)(tile.baseJ + j) * T;
+    // k of this lane's entry t: 4 (s8 + 8 (t / 4)) + t % 4, ascending with t
+    auto k_of = [&](int t) { return 4 * (s8 + 8 * (t >> 2)) + (t & 3); };
+    double best = inf<double>();
+    int k = T;
+    if (may && m == least) {
+      int t = 0;
+#pragma unroll
+      for (int u = 15; u >= 0; --u) t = c[u] == m ? u : t;
+      k = k_of(t);
+      best = __dadd_rn(ra[k], rb[k]);
+    }
+    __syncwarp();
+    auto reduce = [&]() {  // the least value of the output's lanes, the first k that has it
+#pragma unroll
+      for (int d = 1; d < 8; d <<= 1) {
+        const double v = __shfl_xor_sync(kFullMask, best, d);
+        const int kv = __shfl_xor_sync(kFullMask, k, d);
+        if (dless(v, best) || (!dless(best, v) && kv < k)) best = v, k = kv;
+      }
+    };
+    const int first = k;
+    reduce();
+    const float up = f64_up(best);
+    unsigned bits = 0u;
+#pragma unroll
+    for (int u = 0; u < 16; ++u) bits |= (c[u] <= up && k_of(u) != first ? 1u : 0u) << u;
+    if (!may) bits = 0u;
+    if (__any_sync(kFullMask, bits != 0u)) {
+#pragma unroll 1
+      for (; bits; bits &= bits - 1) {
+        const int kk = k_of(__ffs(bits) - 1);
+        const double v = __dadd_rn(ra[kk], rb[kk]);
+        if (dless(v, best) || (!dless(best, v) && kk < k)) best = v, k = kk;
+      }
+      __syncwarp();
+      reduce();
+    }
+    if (may && s8 == 0 && dless(best, was)) {
+      *out = best;
+      if (P) P[out - D] = r * T + k;
+    }
+  }
+}
+
+// The tiles the screen listed, relaxed densely: CTAs take pieces in turn.
+__global__ void __launch_bounds__(k3::THREADS, 4)
+    fw64_listed(double *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r, int R, Panels64 pan,
+                Screen scr, int set) {
+  constexpr int PER = k3x::H / k3::TR;  // pieces a tile, one above the other
+  grid_dep_wait();
+  const k3x::Listed listed(scr, set, R);
+  const int pieces = PER * listed.count;
+#pragma unroll 1
+  for (int t = blockIdx.x; t < pieces; t += gridDim.x) {
+    const int tile = listed.tile(t / PER), q = tile % k3x::PER_BLOCK;
+    int I, J;
+    block_of(set, tile / k3x::PER_BLOCK, r, R, I, J);
+    fence_proxy_async_smem();
+    __syncthreads();  // everyone is done with the previous piece's shared memory
+    piece64(D, ld, P, n, r, I, J, 2 * ((q >> 1) * PER + t % PER) + (q & 1), pan);
+  }
+}
+
+static int g_smem_k1[64], g_smem_k2[64], g_smem_k3[2][64], g_smem_k3x[64], g_smem_k3l[64];
 
 // Four CTAs of 64 registers per SM where phase 4 has many waves (n = 4096 /
 // 8192: 10.6 / 68.9 ms against 11.1 / 72.2 with three, before the outputs were
 // settled a lane at a time), three of 80 up to 24 blocks a side, where K1 must
 // find room beside them (int32 n = 2048: 2.96 against 3.09 ms).
 constexpr int kFewBlocks = 24;
+// Phase 4 is screened from round 16 on from 32 blocks a side (n = 3328: 6.0 against
+// 5.8 ms unscreened, 3584: 6.9 / 7.0, 3840: 7.9 / 8.3, integers; where most
+// outputs improve, U(0, 1), screening costs 2-3 % at every size).  From round 8
+// on: 9.0 ms at n = 4096 against 8.7, since settling an output costs more here.
+constexpr int kScreenMinR = 32, kScreenFrom = 16;
 
 }  // namespace f64
 
@@ -861,14 +1035,21 @@ int run_fw_f64_interval(double *D, int n, int64_t ld, int32_t *P, cudaStream_t s
   if ((st = ensure_smem(fw64_lines, (int)sizeof(k2::Smem), g_smem_k2))) return st;
   const auto pieces = R <= kFewBlocks ? fw64_pieces<3> : fw64_pieces<4>;
   if ((st = ensure_smem(pieces, (int)sizeof(k3::Smem), g_smem_k3[R <= kFewBlocks]))) return st;
+  if ((st = ensure_smem(fw64_screen, (int)sizeof(k3x::Smem), g_smem_k3x))) return st;
+  if ((st = ensure_smem(fw64_listed, (int)sizeof(k3::Smem), g_smem_k3l))) return st;
   // Phase-4 operands: two sets by round parity, each R blocks of A and of B;
-  // then K1's copies of the closed diagonal block.
+  // then K1's copies of the closed diagonal block.  With screened rounds the
+  // sets also hold the rows of lower bounds and the screen's share.
   Panels64 pan[2]{};
   DiagOps64 ops{};
   char *scratch = nullptr;
+  const bool screened = R >= kScreenMinR;
+  ScreenSets scr(R, k2::PARTS);
   if (R > 1) {
-    const size_t elems = (size_t)R * T * T, set = elems * (4 + 4 + 8 + 8);
-    if (scratch_alloc((void **)&scratch, 2 * set + (size_t)T * T * 24, s) != cudaSuccess) {
+    const size_t elems = (size_t)R * T * T, plain = elems * (4 + 4 + 8 + 8);
+    const size_t set = plain + (screened ? elems * (4 + 4) + scr.set_bytes() : 0);
+    if (scratch_alloc((void **)&scratch, 2 * set + (size_t)T * T * 24 + (screened ? scr.list_bytes() : 0), s) !=
+        cudaSuccess) {
       cudaGetLastError();
       return APSP_ENOMEM;
     }
@@ -878,12 +1059,22 @@ int run_fw_f64_interval(double *D, int n, int64_t ld, int32_t *P, cudaStream_t s
       pan[q].B64 = pan[q].A64 + elems;
       pan[q].A = reinterpret_cast<unsigned long long *>(pan[q].B64 + elems);
       pan[q].B = pan[q].A + elems / 2;
+      if (!screened) continue;
+      pan[q].Alo = reinterpret_cast<float *>(base + plain);
+      pan[q].Blo = pan[q].Alo + elems;
+      scr.place_set(q, pan[q].Blo + elems);
     }
     ops.A64 = reinterpret_cast<double *>(scratch + 2 * set);
     ops.B64 = ops.A64 + T * T;
     ops.Alo = reinterpret_cast<unsigned long long *>(ops.B64 + T * T);
     ops.Blo = ops.Alo + T * T / 2;
+    if (screened && scr.place_lists(ops.Blo + T * T / 2, s) != cudaSuccess) {
+      cudaFreeAsync(scratch, s);
+      cudaGetLastError();
+      return APSP_ECUDA;
+    }
   }
+  auto screen_of = [&](int r) { return screened && r >= kScreenFrom ? scr.round(r, 2) : Screen{}; };
   bool capturing = false;
   if ((st = stream_capturing(s, &capturing))) {
     if (scratch) cudaFreeAsync(scratch, s);
@@ -897,16 +1088,24 @@ int run_fw_f64_interval(double *D, int n, int64_t ld, int32_t *P, cudaStream_t s
   auto diag = [&](int r, cudaStream_t stm) {
     PhaseScope sc(1, stm);
     launch_after(fw64_diag, k1::CTAS, k1::THREADS, sizeof(k1::Smem), stm, overlap, D, ld, P, n, r, vec,
-                 (int)(P && r == 0), ops);
+                 (int)(P && r == 0), ops, screen_of(r).range);
   };
   auto panels = [&](int r, cudaStream_t stm) {
     PhaseScope sc(2, stm);
     launch_after(fw64_lines, 2 * (R - 1) * k2::PARTS, 32 * k2::WARPS, sizeof(k2::Smem), stm, overlap, D, ld, P, n, r, R,
-                 vec, ops, pan[r & 1]);
+                 vec, ops, pan[r & 1], screen_of(r));
   };
   auto phase4 = [&](int r, int set, int blocks, cudaStream_t stm) {
     if (blocks <= 0) return;
     PhaseScope sc(3, stm);
+    if (screened && r >= kScreenFrom) {
+      const Screen sr = screen_of(r);
+      launch_after(fw64_screen, k3x::PER_BLOCK * blocks, k3x::THREADS, sizeof(k3x::Smem), stm, overlap, D, ld, P, n, r,
+                   R, vec, pan[r & 1], sr, set);
+      launch_after(fw64_listed, std::min(k3::PER_BLOCK * blocks, kListedCtas * kSms), k3::THREADS, sizeof(k3::Smem), stm, overlap,
+                   D, ld, P, n, r, R, pan[r & 1], sr, set);
+      return;
+    }
     launch_after(pieces, k3::PER_BLOCK * blocks, k3::THREADS, sizeof(k3::Smem), stm, overlap, D, ld, P, n, r, R,
                  pan[r & 1], set);
   };

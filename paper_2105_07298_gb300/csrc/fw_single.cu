@@ -45,6 +45,7 @@
 #include "phases_f32.cuh"
 #include "profile.h"
 #include "rounds.cuh"
+#include "screen.cuh"
 
 namespace apsp {
 
@@ -65,48 +66,12 @@ __global__ void fw_path_init(int32_t *__restrict__ P, int64_t n, int64_t ld, int
 // 16-byte boundary.
 constexpr int kVecD = 1, kVecP = 2;
 
+constexpr int kScreenParts = 4;  // parts of a block K2 reports on in a screened round
+
 // The closed diagonal block of a round in K2's operand layouts (K1 writes them).
 struct DiagOps {
   unsigned long long *A, *B;
 };
-
-// What the screened phase 4 needs of a round besides the panels (all NULL in a
-// round that is not screened), see fw_phase3_screen_f32.
-//   EA[I][i][k], EB[J][j][k]: bf16 weights of the column and the row panel, 8-k
-//     chunks of a line moved to chunk (k / 8) ^ (line % 8);
-//   base_a[I][i], base_b[J][j]: the least entry of the line (0 if none is finite);
-//   whole_a[I][p], whole_b[J][p]: part p of the block holds only integers below
-//     2^22 in magnitude (and +inf);
-//   range: of the closed diagonal block, ordered keys of its largest finite
-//     entry and of minus its smallest;
-//   dense_next, dense_rest: lists the screen makes for the dense kernel.
-struct Screen {
-  uint32_t *EA, *EB;
-  float *base_a, *base_b;
-  int *whole_a, *whole_b;
-  unsigned *range;
-  int *dense_next, *dense_rest;  // [0]: tiles listed, [1..]: the tiles to relax densely, by block set
-};
-constexpr int kScreenParts = 4;  // parts of a block K2 reports on
-
-// Unsigned keys with the order of the floats (no NaN), and back.
-__device__ __forceinline__ unsigned fkey(float x) {
-  const unsigned u = __float_as_uint(x);
-  return (u >> 31) ? ~u : u | 0x80000000u;
-}
-__device__ __forceinline__ float fkey_value(unsigned k) { return __uint_as_float((k >> 31) ? k & 0x7fffffffu : ~k); }
-
-// 1 / s of a round, s = (largest - smallest finite entry of the diagonal block) / 48.
-__device__ __forceinline__ float screen_scale(const unsigned *range) {
-  const unsigned hi = range[0], lo = range[1];
-  const float span = hi && lo ? fkey_value(hi) + fkey_value(lo) : 0.0f;
-  return span > 0.0f ? fminf(fmaxf(48.0f / span, 1e-30f), 1e30f) : 1e-30f;
-}
-__device__ __forceinline__ float ex2(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
 
 // __byte_perm selector that replaces byte c of its first operand with byte 0 of its second.
 __device__ __forceinline__ constexpr unsigned byte_sel(int c) {
@@ -308,12 +273,7 @@ __global__ void __cluster_dims__(k1::CTAS, 1, 1) __launch_bounds__(32 * k1::WARP
             hi = max(hi, fkey(d[rr][c]));
             lo = max(lo, fkey(-d[rr][c]));
           }
-      hi = __reduce_max_sync(kFullMask, hi);
-      lo = __reduce_max_sync(kFullMask, lo);
-      if (lane == 0) {
-        atomicMax(&range[0], hi);
-        atomicMax(&range[1], lo);
-      }
+      screen_range(range, hi, lo);
     }
     if (ops.A) {
 #pragma unroll
@@ -545,23 +505,16 @@ __global__ void __launch_bounds__(k2s::THREADS, 2)
 #pragma unroll
     for (int c = 0; c < LINES; ++c) {
       const int line = line0 + c;
-      float least = fminf(mp32::min3f(v[c][0], v[c][1], v[c][2]), v[c][3]);
-      least = fkey_value(__reduce_min_sync(kFullMask, fkey(least)));
-      least = least < INF ? least : 0.0f;
+      const float least = screen_least(v[c][0], v[c][1], v[c][2], v[c][3]);
       float e[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        const float x = v[c][q];
-        // at least 2^-(x - least) / s: 1/128 above what covers ex2's error and the rounding to bf16
-        e[q] = x < INF ? ex2(-fminf(__fmul_rn(__fsub_rn(x, least), inv), 60.0f)) * 1.0078125f : 0.0f;
-        whole = whole && (!(x < INF) || (x == rintf(x) && fabsf(x) < 4194304.0f));
+        e[q] = screen_weight(v[c][q], least, inv);
+        whole = whole && screen_whole(v[c][q]);
       }
 #pragma unroll
-      for (int hq = 0; hq < 2; ++hq) {  // k = 2 lane + 64 hq, + 1: chunk lane / 4 + 8 hq
-        uint32_t two;
-        asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(two) : "f"(e[2 * hq + 1]), "f"(e[2 * hq]));
-        E[line * (T / 2) + (((lane >> 2) + 8 * hq) ^ (line & 7)) * 4 + (lane & 3)] = two;
-      }
+      for (int hq = 0; hq < 2; ++hq)  // k = 2 lane + 64 hq, + 1: chunk lane / 4 + 8 hq
+        E[line * (T / 2) + (((lane >> 2) + 8 * hq) ^ (line & 7)) * 4 + (lane & 3)] = bf16x2(e[2 * hq], e[2 * hq + 1]);
       if (lane == 0) (is_row ? scr.base_b : scr.base_a)[blk * T + line] = least;
     }
     whole = __syncthreads_and(whole);
@@ -1090,67 +1043,10 @@ __global__ void __launch_bounds__(k3s::THREADS, TR == 32 ? 4 : 3)
   piece_f32<PATH, TR>(D, ld, P, n, r, I, J, blockIdx.x % PER, vec_ok, pan);
 }
 
-// --------------------------------------------------------------------------
-// K3 screened: phase 4 in rounds where few outputs improve.  A bf16 product on
-// the tensor cores finds the outputs that may improve, and only those are
-// relaxed in FP32.
-//
-// With s > 0 and any bases a_i, b_j, a candidate below the old value, D[i][k] +
-// D[k][j] < old, gives 2^-(D[i][k] - a_i)/s * 2^-(D[k][j] - b_j)/s >
-// 2^-(old - a_i - b_j)/s =: T.  K2 writes weights at least as large as the two
-// factors (the bases are the lines' least entries, so weights are at most about
-// 1; entries further than 60 s above get the weight of 60 s, +inf gets 0), so
-// the sum X of a row's products over the round's k exceeds T whenever any
-// candidate improves.  Outputs with X <= 0.96 T', T' lowered by what rounding
-// in its argument can amount to, are left as they are; the FP32 accumulation of
-// at most 128 non-negative normal products loses less than the factor covers.
-// The other outputs may or may not improve: the test sees a candidate within
-// about s log2(how many) of the old value.  Where both blocks hold only
-// integers, a candidate below the old value is at most ceil(old) - 1, and with
-// s <= 1/8 (128 ties at the old value weigh half of one a step below) the test
-// is exact.
-//
-// Flagged outputs are listed and settled four to a warp, eight lanes each: the
-// lanes add the row of A and the row of B^T, and the minimum and its first k are
-// taken over them - the values and the tie rule of the sequential loop.
-// A tile with more than kScreenDense flagged outputs is listed for
-// fw_phase3_listed_f32, which relaxes it densely.
-//
-// Bound: the latency of a tile's loads (weights, old values, then the flagged
-// outputs' rows), overlapped over four CTAs per SM; a tile of 128 x 64 with two
-// CTAs measured 8 % slower, settling one output a warp 25 %.  Measured per round
-// at n = 16384 (U[1, 100], p = 0.5): 0.64 ms from round 60 on, of which the
-// screen 0.58 (the dense kernel 2.0 ms); the product itself 0.22 ms on mma.sync
-// with 128 x 128 tiles, so its rate is not what counts.  Solves with P: n = 4096
-// 6.2 -> 4.4 ms, 8192 40.9 -> 24.3, 16384 289 -> 120; real weights and sparse
-// graphs gain likewise (n = 8192: U[0.5, 2) 22.2 ms, 16 edges a vertex 52.9
-// against 81).
-// --------------------------------------------------------------------------
-namespace k3x {
-constexpr int T = mp32::T, THREADS = 256;
-constexpr int H = T / 2, PER_BLOCK = 4;  // a CTA's tile: H x H, a quarter of a block
-constexpr int kScreenDense = 800;  // of H H outputs (625, 800, 1000: within 1 %)
-struct Smem {
-  uint32_t EA[H][T / 2], EB[H][T / 2];
-  float base_a[H], base_b[H];  // adjacent; base_b is read in pairs
-  uint64_t bar;
-  int count, next;
-  unsigned short list[kScreenDense];  // flagged outputs, i H + j
-};
-static_assert(offsetof(Smem, base_b) % 8 == 0 && offsetof(Smem, EB) % 128 == 0, "pairs and bulk copies");
-__device__ __forceinline__ void ldmatrix4(uint32_t (&f)[4], uint32_t addr) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
-               : "=r"(f[0]), "=r"(f[1]), "=r"(f[2]), "=r"(f[3])
-               : "r"(addr));
-}
-__device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
-               "{%0, %1, %2, %3};"
-               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-               : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-}  // namespace k3x
-
+// The FP32 screen.  Eight lanes settle an output, a warp four: lane s of an
+// output adds entries 4 (s + 8 u) + c (u, c < 4) of the row of A and the row of
+// B^T, and the minimum and its first k are taken over the lanes - the values and
+// the tie rule of the sequential loop.
 template <bool PATH>
 __global__ void __launch_bounds__(k3x::THREADS, 4)
     fw_phase3_screen_f32(float *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r, int R, int vec_ok,
@@ -1158,149 +1054,16 @@ __global__ void __launch_bounds__(k3x::THREADS, 4)
   using namespace k3x;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
-  int I, J;
-  block_of(set, blockIdx.x / PER_BLOCK, r, R, I, J);
-  const int hI = (blockIdx.x >> 1) & 1, hJ = blockIdx.x & 1;
-  const int baseI = I * T + hI * H, baseJ = J * T + hJ * H, baseK = r * T;
-  const int mI = min(H, n - baseI), mJ = min(H, n - baseJ);
-  if (mI <= 0 || mJ <= 0) return;  // past the matrix (uniform exit)
-  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const float INF = inf<float>();
-  if (tid == 0) {
-    mbar_init(&sm.bar, 1);
-    fence_mbar_init();
-    mbar_expect_tx(&sm.bar, 2 * H * T * 2);
-    sm.count = sm.next = 0;
-  }
-  grid_dep_wait();
-  if (tid == 0) {
-    fence_proxy_async_global();
-    bulk_g2s(&sm.EA[0][0], scr.EA + (int64_t)I * (T * T / 2) + hI * (H * T / 2), H * T * 2, &sm.bar);
-    bulk_g2s(&sm.EB[0][0], scr.EB + (int64_t)J * (T * T / 2) + hJ * (H * T / 2), H * T * 2, &sm.bar);
-  }
-  // Warp (w / 4, w % 4): rows wi .. wi + 31, columns wj .. wj + 15.  Output (a, h,
-  // b, q) of lane l: row wi + 16 a + 8 h + l / 4, column wj + 8 b + 2 (l % 4) + q.
-  // The old values are under way while the weights arrive and are multiplied.
-  const int wi = 32 * (w >> 2), wj = 16 * (w & 3);
-  float2 o[2][2][2];
-#pragma unroll
-  for (int a = 0; a < 2; ++a)
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int i = wi + 16 * a + 8 * h + (lane >> 2);
-      const float *row = D + (int64_t)(baseI + i) * ld + baseJ;
-#pragma unroll
-      for (int b = 0; b < 2; ++b) {
-        const int j = wj + 8 * b + 2 * (lane & 3);
-        o[a][h][b] = make_float2(-INF, -INF);  // outside the matrix: never flagged
-        if (i < mI) {
-          if (vec_ok && j + 1 < mJ) {
-            o[a][h][b] = *reinterpret_cast<const float2 *>(row + j);
-          } else {
-            if (j < mJ) o[a][h][b].x = row[j];
-            if (j + 1 < mJ) o[a][h][b].y = row[j + 1];
-          }
-        }
-      }
-    }
-  const float inv = screen_scale(scr.range);
-  if (tid < 2 * H) {  // the bases in units of s, less their share of the argument's error
-    const float v = tid < H ? scr.base_a[I * T + hI * H + tid] : scr.base_b[J * T + hJ * H + tid - H];
-    const float b = fmaf(v, inv, -fabsf(v) * (4.76837158203125e-7f * inv) - 0.03f);
-    (&sm.base_a[0])[tid] = fabsf(b) < 1e38f ? b : -INF;  // beyond the floats: the line's outputs are all flagged
-  }
-  bool whole = true;
-#pragma unroll
-  for (int p = 0; p < kScreenParts; ++p)
-    whole = whole && scr.whole_a[I * kScreenParts + p] && scr.whole_b[J * kScreenParts + p];
-  __syncthreads();
-  const bool ok = mbar_wait(&sm.bar, 0);
-  if (__syncthreads_or(!ok)) {  // the weights never arrived: the block stays as it is
-    if (tid == 0) report_wait_timeout();
-    return;
-  }
-  float x[2][2][4];
-#pragma unroll
-  for (int a = 0; a < 2; ++a)
-#pragma unroll
-    for (int b = 0; b < 2; ++b)
-#pragma unroll
-      for (int c = 0; c < 4; ++c) x[a][b][c] = 0.0f;
-  const uint32_t sa = smem_addr(&sm.EA[0][0]), sb = smem_addr(&sm.EB[0][0]);
-  const int ar = wi + (lane & 15), ac = lane >> 4;                       // A: row, chunk
-  const int br = wj + (lane & 7) + 8 * (lane >> 4), bc = (lane >> 3) & 1;  // B: line, chunk
-#pragma unroll
-  for (int ks = 0; ks < T / 16; ++ks) {
-    uint32_t fb[4];
-    ldmatrix4(fb, sb + (uint32_t)(br * (T * 2) + (((2 * ks + bc) ^ (br & 7)) << 4)));
-#pragma unroll
-    for (int a = 0; a < 2; ++a) {
-      uint32_t fa[4];
-      ldmatrix4(fa, sa + (uint32_t)((ar + 16 * a) * (T * 2) + (((2 * ks + ac) ^ (ar & 7)) << 4)));
-      mma_bf16(x[a][0], fa, fb[0], fb[1]);
-      mma_bf16(x[a][1], fa, fb[2], fb[3]);
-    }
-  }
-  // log2(0.96 T') = (a_i + b_j - t) / s, less what its roundings and ex2's can
-  // amount to: kErr of each of its three terms, and 0.06.
-  constexpr float kErr = 4.76837158203125e-7f;  // 2^-21
-  unsigned mine[2][2];  // [a][h]: bit 2 b + q
-  int found = 0;
-  auto test = [&](auto limit) {  // limit(old): the largest value a candidate below old can have
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        mine[a][h] = 0u;
-        const float ai = sm.base_a[wi + 16 * a + 8 * h + (lane >> 2)];
-#pragma unroll
-        for (int b = 0; b < 2; ++b) {
-          const float2 bj = *reinterpret_cast<const float2 *>(&sm.base_b[wj + 8 * b + 2 * (lane & 3)]);
-#pragma unroll
-          for (int q = 0; q < 2; ++q) {
-            const float t = limit(q ? o[a][h][b].y : o[a][h][b].x);
-            const float arg = fmaf(-fabsf(t), kErr * inv, fmaf(-t, inv, ai + (q ? bj.y : bj.x)));
-            // (NaN, where t / s and the bases overflow, is flagged; nothing is below -inf)
-            if (!(x[a][b][2 * h + q] <= ex2(arg)) && t > -INF) mine[a][h] |= 1u << (2 * b + q);
-          }
-        }
-        found += __popc(mine[a][h]);
-      }
-  };
-  if (whole)
-    test([](float old) {  // the largest integer below old, by rounding to nearest (old itself beyond 2^22)
-      const float near = __fadd_rn(__fadd_rn(old, 12582912.0f), -12582912.0f);
-      return fabsf(old) < 4194304.0f ? (near < old ? near : near - 1.0f) : old;
-    });
-  else test([](float old) { return old; });
-  found = __reduce_add_sync(kFullMask, found);
-  if (lane == 0 && found) atomicAdd(&sm.count, found);
-  __syncthreads();
-  const int count = sm.count;
-  if (count == 0) return;
-  if (count > kScreenDense) {  // left to the dense kernel
-    if (tid == 0) {
-      int *list = set == kSetNext ? scr.dense_next : scr.dense_rest;
-      list[1 + atomicAdd(&list[0], 1)] = blockIdx.x;
-    }
-    return;
-  }
-  // The flagged outputs as a list, in any order.
-  int at = __popc(mine[0][0]) + __popc(mine[0][1]) + __popc(mine[1][0]) + __popc(mine[1][1]);
-  if (at) at = atomicAdd(&sm.next, at);
-#pragma unroll
-  for (int a = 0; a < 2; ++a)
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-      for (unsigned bits = mine[a][h]; bits; bits &= bits - 1) {
-        const int t = __ffs(bits) - 1;
-        sm.list[at++] = (unsigned short)((wi + 16 * a + 8 * h + (lane >> 2)) * H + wj + 8 * (t >> 1) + 2 * (lane & 3) + (t & 1));
-      }
-  __syncthreads();
-  // Eight lanes an output, four outputs a warp: lane s of an output adds
-  // entries 4 (s + 8 u) + c (u, c < 4) of the row of A and the row of B^T.
-  const float4 *acp = reinterpret_cast<const float4 *>(pan.Acp + ((int64_t)I * T + hI * H) * T);
-  const float4 *bt = reinterpret_cast<const float4 *>(pan.Bt + ((int64_t)J * T + hJ * H) * T);
+  Tile tile;
+  const int count = screen_tile<kScreenParts>(sm, tile, n, r, R, scr, set, [&](int i, int j, int left) {
+    const float *p = D + (int64_t)i * ld + j;
+    if (vec_ok && left > 1) return *reinterpret_cast<const float2 *>(p);
+    return make_float2(left > 0 ? p[0] : -INF, left > 1 ? p[1] : -INF);
+  });
+  const int baseI = tile.baseI, baseJ = tile.baseJ, baseK = r * T, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const float4 *acp = reinterpret_cast<const float4 *>(pan.Acp + (int64_t)baseI * T);
+  const float4 *bt = reinterpret_cast<const float4 *>(pan.Bt + (int64_t)baseJ * T);
   const int s8 = lane & 7;
 #pragma unroll 1
   for (int g = 4 * w; g < count; g += THREADS / 32 * 4) {
@@ -1348,11 +1111,10 @@ __global__ void __launch_bounds__(k3s::THREADS, 3)
     fw_phase3_listed_f32(float *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r, int R, int vec_ok,
                          Panels pan, Screen scr, int set) {
   grid_dep_wait();
-  const int *list = set == kSetNext ? scr.dense_next : scr.dense_rest;
-  const int tiles = list[0];
+  const k3x::Listed listed(scr, set, R);
 #pragma unroll 1
-  for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
-    const int tile = list[1 + t];
+  for (int t = blockIdx.x; t < listed.count; t += gridDim.x) {
+    const int tile = listed.tile(t);
     int I, J;
     block_of(set, tile / k3x::PER_BLOCK, r, R, I, J);
     fence_proxy_async_smem();
@@ -1376,7 +1138,6 @@ std::vector<cudaEvent_t> g_prof_pool;
 constexpr int kMaxN = 1 << 18;
 
 constexpr int kT32 = mp32::T, kT64 = 128;
-constexpr int kSms = 152;
 // Phase-4 kernels by blocks per side R (measured, whole solves, ms):
 //  * 32-row pieces for every launch while the whole of phase 4 is about a wave
 //    of CTAs or less (n = 2049: 0.93 against 0.97 with 64 rows, 1.12 with the
@@ -1451,19 +1212,12 @@ static int run_fw_f32(float *D, int64_t n64, int64_t ld, int32_t *P, void *strea
   Panels pan[2]{};
   DiagOps ops{};
   char *scratch = nullptr;
-  Screen scr[2]{};
-  unsigned *ranges = nullptr;
-  int *dense_next = nullptr, *dense_rest = nullptr;
   const bool screened = R >= kScreenMinR;
+  ScreenSets scr(R, kScreenParts);
   if (R > 1) {
     const size_t words = (size_t)R * T * T, diag = 2 * (size_t)T * T;
-    // per set: EA, EB (half a word per entry), bases, whole flags; per round: the range
-    const size_t scr_words = screened ? words + 2 * (size_t)R * T + 2 * (size_t)R * kScreenParts : 0;
-    const size_t range_words = screened ? 2 * (size_t)R : 0;
-    // the dense lists: a count and every tile of the set
-    const size_t next_words = 1 + k3x::PER_BLOCK * 2 * (size_t)R, rest_words = 1 + k3x::PER_BLOCK * (size_t)R * R;
-    const size_t list_words = screened ? next_words + rest_words : 0;
-    if (scratch_alloc((void **)&scratch, (8 * words + diag + 2 * scr_words + range_words + list_words) * 4, s) != cudaSuccess) {
+    const size_t screen_bytes = screened ? 2 * scr.set_bytes() + scr.list_bytes() : 0;
+    if (scratch_alloc((void **)&scratch, (8 * words + diag) * 4 + screen_bytes, s) != cudaSuccess) {
       cudaGetLastError();
       return APSP_ENOMEM;
     }
@@ -1477,19 +1231,9 @@ static int run_fw_f32(float *D, int64_t n64, int64_t ld, int32_t *P, void *strea
     ops.A = reinterpret_cast<unsigned long long *>(scratch + 8 * words * 4);
     ops.B = ops.A + T * T / 2;
     if (screened) {
-      uint32_t *base = reinterpret_cast<uint32_t *>(scratch + (8 * words + diag) * 4);
-      for (int q = 0; q < 2; ++q, base += scr_words) {
-        scr[q].EA = base;
-        scr[q].EB = base + words / 2;
-        scr[q].base_a = reinterpret_cast<float *>(base + words);
-        scr[q].base_b = scr[q].base_a + (size_t)R * T;
-        scr[q].whole_a = reinterpret_cast<int *>(scr[q].base_b + (size_t)R * T);
-        scr[q].whole_b = scr[q].whole_a + (size_t)R * kScreenParts;
-      }
-      ranges = base;
-      dense_next = reinterpret_cast<int *>(base + range_words);
-      dense_rest = dense_next + next_words;
-      if (cudaMemsetAsync(ranges, 0, range_words * 4, s) != cudaSuccess) {
+      char *base = scratch + (8 * words + diag) * 4;
+      for (int q = 0; q < 2; ++q, base += scr.set_bytes()) scr.place_set(q, base);
+      if (scr.place_lists(base, s) != cudaSuccess) {
         cudaFreeAsync(scratch, s);
         cudaGetLastError();
         return APSP_ECUDA;
@@ -1497,14 +1241,9 @@ static int run_fw_f32(float *D, int64_t n64, int64_t ld, int32_t *P, void *strea
     }
   }
   // The round's screening data, or none where the round is not screened.
-  auto screen_of = [&](int r) {
-    if (!screened || r < kScreenFrom) return Screen{};
-    Screen sc = scr[r & 1];
-    sc.range = ranges + 2 * r;
-    sc.dense_next = dense_next;
-    sc.dense_rest = dense_rest;
-    return sc;
-  };
+  // It is left out where the last probe listed half of the tiles, without a path
+  // matrix a quarter (the dense kernel then costs less).
+  auto screen_of = [&](int r) { return screened && r >= kScreenFrom ? scr.round(r, P ? 2 : 4) : Screen{}; };
   const bool aligned = ld % 4 == 0;
   const int vec = (aligned && (reinterpret_cast<uintptr_t>(D) & 15) == 0 ? kVecD : 0) |
                   (aligned && (reinterpret_cast<uintptr_t>(P) & 15) == 0 ? kVecP : 0);
@@ -1535,10 +1274,9 @@ static int run_fw_f32(float *D, int64_t n64, int64_t ld, int32_t *P, void *strea
     PhaseScope ps(3, st);
     if (screened && r >= kScreenFrom) {
       const Screen sc = screen_of(r);
-      cudaMemsetAsync(set == kSetNext ? sc.dense_next : sc.dense_rest, 0, sizeof(int), st);
       launch_after(P ? fw_phase3_screen_f32<true> : fw_phase3_screen_f32<false>, k3x::PER_BLOCK * blocks, k3x::THREADS,
                    sizeof(k3x::Smem), st, overlap, D, ld, P, n, r, R, vec_ok, pan[r & 1], sc, set);
-      launch_after(P ? fw_phase3_listed_f32<true> : fw_phase3_listed_f32<false>, std::min(4 * blocks, 3 * kSms),
+      launch_after(P ? fw_phase3_listed_f32<true> : fw_phase3_listed_f32<false>, std::min(4 * blocks, kListedCtas * kSms),
                    k3s::THREADS, sizeof(k3s::Smem<64>), st, overlap, D, ld, P, n, r, R, vec_ok, pan[r & 1], sc, set);
     } else if (R <= kR32 || (set == kSetNext && R <= kRNext32))
       launch_after(kernel32, k3s::per_block(32) * blocks, k3s::THREADS, sizeof(k3s::Smem<32>), st, overlap, D, ld, P, n,

@@ -14,10 +14,16 @@
 
 namespace apsp {
 
+constexpr int kSms = 152;
+
 // Block sets of one phase-4 launch.
 constexpr int kSetAll = 0;   // all (R-1)^2 blocks off row/column r
 constexpr int kSetNext = 1;  // the 2R-3 blocks in row r+1 or column r+1
 constexpr int kSetRest = 2;  // the (R-2)^2 blocks off rows/columns r and r+1
+
+__host__ __device__ constexpr int set_blocks(int set, int R) {
+  return set == kSetNext ? 2 * R - 3 : set == kSetRest ? (R - 2) * (R - 2) : (R - 1) * (R - 1);
+}
 
 // The output block (I, J) of a launch's tile-th block in round r (R blocks a side).
 __device__ __forceinline__ void block_of(int set, int tile, int r, int R, int &I, int &J) {

@@ -105,7 +105,7 @@ def test_batched_blocks_at_quad_and_tile_edges(d_off, with_path):
 
 
 def _screened_graph(kind, n):
-    """Weights for the screened rounds (more than 21 blocks a side, from round 8 on)."""
+    """Weights for the screened rounds (FP32: from 22 blocks a side and round 8 on; FP64: 32, 16)."""
     rng = np.random.default_rng(3)
     if kind == "integers":
         return graphgen.dense_graph(n, 0.1, 21)
@@ -117,6 +117,8 @@ def _screened_graph(kind, n):
         return graphgen.dense_graph(n, 0.001, 24, weights="real", lo=0.5, hi=2.0)
     if kind == "no edges":
         return graphgen.dense_graph(n, 0.0, 25)
+    if kind == "most improve":  # rounds between two probes go without the screen
+        return graphgen.dense_graph(n, 0.4, 28, weights="real", lo=0.0, hi=1.0)
     W = graphgen.dense_graph(n, 0.05, 26, weights="real", lo=0.5, hi=2.0)
     if kind == "negative":  # shifted by potentials: negative edges, no negative cycle but by rounding
         h = rng.integers(-64, 65, n).astype(np.float32)
@@ -134,13 +136,48 @@ def _screened_graph(kind, n):
 
 
 @pytest.mark.parametrize("kind", ["integers", "halves", "beyond 2^22", "sparse", "no edges", "real", "negative",
-                                  "clusters", "huge"])
+                                  "clusters", "huge", "most improve"])
 def test_screened_rounds_bitwise(kind):
     n = 2900
     W = _screened_graph(kind, n)
     Db, Pb = oracle.bfw(W, 128)
     ld = n + 1 if kind in ("real", "integers") else n  # rows off 16-byte boundaries too
     D = torch.empty((n, ld), device=DEV)[:, :n]
+    P = torch.empty((n, ld), dtype=torch.int32, device=DEV)[:, :n]
+    D.copy_(torch.from_numpy(W))
+    apsp.apsp_fw(D, P)
+    np.testing.assert_array_equal(D.cpu().numpy(), Db)
+    np.testing.assert_array_equal(P.cpu().numpy(), Pb)
+    D.copy_(torch.from_numpy(W))
+    apsp.apsp_fw(D)
+    np.testing.assert_array_equal(D.cpu().numpy(), Db)
+    assert apsp.device_status() == apsp.APSP_OK
+
+
+def _screened_graph_f64(kind, n):
+    rng = np.random.default_rng(5)
+    if kind == "real":
+        return graphgen.dense_graph(n, 0.05, 31, weights="real", lo=0.5, hi=2.0, dtype=np.float64)
+    if kind == "one float":  # all sums within a float step of each other
+        W = 1.0 + rng.integers(0, 3, (n, n)) * 2.0 ** -40 + rng.integers(0, 3, (n, n)) * 2.0 ** -52
+        W[rng.random((n, n)) >= 0.05] = np.inf
+    elif kind == "beyond the floats":  # edges of either sign, exact sums
+        h = rng.integers(-64, 65, n) * 2.0 ** 1000
+        W = graphgen.dense_graph(n, 0.02, 32, lo=1, hi=100).astype(np.float64) * 2.0 ** 1000 + h[:, None] - h[None, :]
+    else:
+        return _screened_graph(kind, n).astype(np.float64)
+    np.fill_diagonal(W, 0)
+    return W
+
+
+@pytest.mark.parametrize("kind", ["real", "one float", "beyond the floats", "integers", "beyond 2^22", "sparse",
+                                  "negative", "clusters", "huge", "most improve"])
+def test_screened_rounds_f64_bitwise(kind):
+    n = 4000
+    W = _screened_graph_f64(kind, n)
+    Db, Pb = oracle.bfw(W, 128)
+    ld = n + 1 if kind in ("real", "integers") else n  # rows off 16-byte boundaries too
+    D = torch.empty((n, ld), device=DEV, dtype=torch.float64)[:, :n]
     P = torch.empty((n, ld), dtype=torch.int32, device=DEV)[:, :n]
     D.copy_(torch.from_numpy(W))
     apsp.apsp_fw(D, P)
