@@ -84,12 +84,15 @@ int apsp_fw_block_size(int elem_bytes);
  *            it is fully written (P as described above).  May be NULL.
  *   stream : cudaStream_t as void*.  All work is ordered after earlier work
  *            on `stream`, and later work on `stream` sees the results.  With
- *            more than two blocks per side the next round's phases 1-3 run
- *            on an internal second stream (created and destroyed by the call,
- *            joined to `stream` by events), except while `stream` is being
- *            captured into a CUDA graph: then every phase runs on `stream`.
- *            Scratch (operand panels: about 32 n TB bytes for FP32, 48 n TB
- *            bytes for FP64; 128 MiB / 192 MiB at n = 32768) is stream-ordered
+ *            more than two blocks per side what the next round waits for
+ *            (phase 4 on its row and column, then its phases 1-3) runs on an
+ *            internal second stream of higher priority (created and destroyed
+ *            by the call, joined to `stream` by events), except while `stream`
+ *            is being captured into a CUDA graph: then every phase runs on
+ *            `stream`.
+ *            Scratch (operand panels: about 16 n TB bytes for FP32 up to
+ *            n = 2688 and 40 n TB above, 48 n TB for FP64 up to n = 3968 and
+ *            72 n TB above; 160 MiB / 288 MiB at n = 32768) is stream-ordered
  *            (allocated on `stream` from a memory pool of the library's own,
  *            which keeps at most 256 MiB per device between calls, and freed
  *            with cudaFreeAsync; cudaMallocAsync while `stream` is captured).

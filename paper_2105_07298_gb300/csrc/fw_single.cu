@@ -490,6 +490,7 @@ __global__ void __launch_bounds__(k2s::THREADS, 2)
     for (int c = 0; c < LINES; c += 2)
       *reinterpret_cast<ulonglong2 *>(dst + c) = make_ulonglong2(mp32::pack2(v[c][2 * hq], v[c][2 * hq + 1]),
                                                                  mp32::pack2(v[c + 1][2 * hq], v[c + 1][2 * hq + 1]));
+    if (!scr.EA) continue;  // the rows are the screen's
 #pragma unroll
     for (int c = 0; c < LINES; ++c)
       *reinterpret_cast<float2 *>(&rows[(blk * T + line0 + c) * T + 2 * kp]) = make_float2(v[c][2 * hq], v[c][2 * hq + 1]);
@@ -903,33 +904,34 @@ static int run_fw_f32(float *D, int64_t n64, int64_t ld, int32_t *P, void *strea
     return st;
   cudaGetLastError();  // clear any stale error so the checks below are ours
   // Phase-4 operand panels, written by K2 each round: two sets (round parity)
-  // of 4 arrays of R*T*T 4-byte words, so that K2 of round r+1 can run while
-  // phase 4 of round r still reads round r's panels; then K1's two copies of
-  // the closed diagonal block.  Stream-ordered scratch, freed after the last
-  // round.
+  // of R*T*T 4-byte words each for Apan and Bpan, and with screened rounds for
+  // the rows Acp and Bt, so that K2 of round r+1 can run while phase 4 of round
+  // r still reads round r's panels; then K1's two copies of the closed diagonal
+  // block.  Stream-ordered scratch, freed after the last round.
   Panels pan[2]{};
   DiagOps ops{};
   char *scratch = nullptr;
   const bool screened = R >= kScreenMinR;
   ScreenSets scr(R, kScreenParts);
   if (R > 1) {
-    const size_t words = (size_t)R * T * T, diag = 2 * (size_t)T * T;
+    const size_t words = (size_t)R * T * T, diag = 2 * (size_t)T * T, set = (screened ? 4 : 2) * words;
     const size_t screen_bytes = screened ? 2 * scr.set_bytes() + scr.list_bytes() : 0;
-    if (scratch_alloc((void **)&scratch, (8 * words + diag) * 4 + screen_bytes, s) != cudaSuccess) {
+    if (scratch_alloc((void **)&scratch, (2 * set + diag) * 4 + screen_bytes, s) != cudaSuccess) {
       cudaGetLastError();
       return APSP_ENOMEM;
     }
     for (int q = 0; q < 2; ++q) {
-      char *base = scratch + (size_t)q * 4 * words * 4;
+      char *base = scratch + (size_t)q * set * 4;
       pan[q].Apan = reinterpret_cast<unsigned long long *>(base);
       pan[q].Bpan = reinterpret_cast<unsigned long long *>(base + words * 4);
+      if (!screened) continue;
       pan[q].Acp = reinterpret_cast<float *>(base + 2 * words * 4);
       pan[q].Bt = reinterpret_cast<float *>(base + 3 * words * 4);
     }
-    ops.A = reinterpret_cast<unsigned long long *>(scratch + 8 * words * 4);
+    ops.A = reinterpret_cast<unsigned long long *>(scratch + 2 * set * 4);
     ops.B = ops.A + T * T / 2;
     if (screened) {
-      char *base = scratch + (8 * words + diag) * 4;
+      char *base = scratch + (2 * set + diag) * 4;
       for (int q = 0; q < 2; ++q, base += scr.set_bytes()) scr.place_set(q, base);
       if (scr.place_lists(base, s) != cudaSuccess) {
         cudaFreeAsync(scratch, s);
