@@ -909,13 +909,14 @@ __global__ void __launch_bounds__(k3x::THREADS, 4)
   Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
   const float FINF = inf<float>();
   Tile tile;
-  const int count = screen_tile<k2::PARTS>(sm, tile, n, r, R, scr, set, [&](int i, int j, int left) {
+  const int count = screen_tile<k2::PARTS>(sm, tile, n, r, R, scr, set, vec != 0,
+                                            [&](int i, int j, int left, auto whole_tile) {
     const double *p = D + (int64_t)i * ld + j;
-    if (vec && left > 1) {
+    if constexpr (decltype(whole_tile)::value) {
       const double2 t = *reinterpret_cast<const double2 *>(p);
       return make_float2(f64_up(t.x), f64_up(t.y));
     }
-    return make_float2(left > 0 ? f64_up(p[0]) : -FINF, left > 1 ? f64_up(p[1]) : -FINF);
+    return make_float2(left > 0 ? f64_up(p[0]) : 0.0f, left > 1 ? f64_up(p[1]) : 0.0f);
   });
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, s8 = lane & 7;
   const float4 *alo = reinterpret_cast<const float4 *>(pan.Alo + (int64_t)tile.baseI * T);

@@ -761,10 +761,11 @@ __global__ void __launch_bounds__(k3x::THREADS, 4)
   Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
   const float INF = inf<float>();
   Tile tile;
-  const int count = screen_tile<kScreenParts>(sm, tile, n, r, R, scr, set, [&](int i, int j, int left) {
+  const int count = screen_tile<kScreenParts>(sm, tile, n, r, R, scr, set, vec_ok != 0,
+                                              [&](int i, int j, int left, auto whole_tile) {
     const float *p = D + (int64_t)i * ld + j;
-    if (vec_ok && left > 1) return *reinterpret_cast<const float2 *>(p);
-    return make_float2(left > 0 ? p[0] : -INF, left > 1 ? p[1] : -INF);
+    if constexpr (decltype(whole_tile)::value) return *reinterpret_cast<const float2 *>(p);
+    return make_float2(left > 0 ? p[0] : 0.0f, left > 1 ? p[1] : 0.0f);
   });
   const int baseI = tile.baseI, baseJ = tile.baseJ, baseK = r * T, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const float4 *acp = reinterpret_cast<const float4 *>(pan.Acp + (int64_t)baseI * T);

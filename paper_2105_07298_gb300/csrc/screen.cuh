@@ -4,6 +4,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "bulk.cuh"
 #include "common.cuh"
 #include "minplus_f32.cuh"
@@ -17,7 +19,7 @@ namespace apsp {
 //     chunks of a line moved to chunk (k / 8) ^ (line % 8);
 //   base_a[I][i], base_b[J][j]: the least entry of the line (0 if none is finite);
 //   whole_a[I][p], whole_b[J][p]: part p of the block (K2 divides it into PARTS
-//     parts, lines in order) holds only integers below 2^22 in magnitude (and +inf);
+//     parts, lines in order) holds only integers below 2^21 in magnitude (and +inf);
 //   range: of the closed diagonal block, ordered keys of its largest finite
 //     entry and of minus its smallest;
 //   next, rest: the tiles the screen lists for the dense kernel, by block set, and
@@ -116,7 +118,7 @@ __device__ __forceinline__ float screen_least(float a, float b, float c, float d
   return least < inf<float>() ? least : 0.0f;
 }
 __device__ __forceinline__ bool screen_whole(float x) {
-  return !(x < inf<float>()) || (x == rintf(x) && fabsf(x) < 4194304.0f);
+  return !(x < inf<float>()) || (x == rintf(x) && fabsf(x) < 2097152.0f);
 }
 __device__ __forceinline__ uint32_t bf16x2(float lo, float hi) {
   uint32_t two;
@@ -161,7 +163,8 @@ __device__ __forceinline__ void screen_range(unsigned *range, unsigned hi, unsig
 //
 // Bound: the latency of a tile's loads (weights, old values, then the flagged
 // outputs' rows), overlapped over four CTAs per SM; a tile of 128 x 64 with two
-// CTAs measured 8 % slower, settling one output a warp 25 %.  Measured per round
+// CTAs measured 8 % slower, settling one output a warp 25 %, a test with twice the
+// instructions per output 1.7 % (n = 16384: 120.9 against 118.9 ms).  Measured per round
 // in FP32 at n = 16384 (U[1, 100], p = 0.5): 0.64 ms from round 60 on, of which
 // the screen 0.58 (the dense kernel 2.0 ms); the product itself 0.22 ms on
 // mma.sync with 128 x 128 tiles, so its rate is not what counts.  FP32 solves
@@ -200,10 +203,12 @@ struct Tile {
 
 // One CTA screens its tile: returns how many of its outputs are in sm.list, for
 // the caller to settle; 0 if there are none or the tile was listed for the dense
-// kernel.  old(i, j, left): the values (FP64: upper bounds) of outputs (i, j) and
-// (i, j + 1), -inf where `left` columns of the matrix end before them.
+// kernel.  old(i, j, left, whole_tile): the values (FP64: upper bounds) of outputs
+// (i, j) and (i, j + 1), anything where `left` columns of the matrix end before
+// them; whole_tile: a std::true_type says that they lie inside it, aligned (pairs).
 template <int PARTS, typename Old>
-__device__ __forceinline__ int screen_tile(Smem &sm, Tile &t, int n, int r, int R, const Screen &scr, int set, Old old) {
+__device__ __forceinline__ int screen_tile(Smem &sm, Tile &t, int n, int r, int R, const Screen &scr, int set, bool pairs,
+                                           Old old) {
   block_of(set, blockIdx.x / PER_BLOCK, r, R, t.I, t.J);
   const int I = t.I, J = t.J;
   const int hI = (blockIdx.x >> 1) & 1, hJ = blockIdx.x & 1;
@@ -229,18 +234,23 @@ __device__ __forceinline__ int screen_tile(Smem &sm, Tile &t, int n, int r, int 
   // b, q) of lane l: row wi + 16 a + 8 h + l / 4, column wj + 8 b + 2 (l % 4) + q.
   // The old values are under way while the weights arrive and are multiplied.
   const int wi = 32 * (w >> 2), wj = 16 * (w & 3);
+  const bool full = mI == H && mJ == H;
   float2 o[2][2][2];
+  auto load = [&](auto whole_tile) {
 #pragma unroll
-  for (int a = 0; a < 2; ++a)
+    for (int a = 0; a < 2; ++a)
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int i = wi + 16 * a + 8 * h + (lane >> 2);
+      for (int h = 0; h < 2; ++h) {
+        const int i = wi + 16 * a + 8 * h + (lane >> 2);
 #pragma unroll
-      for (int b = 0; b < 2; ++b) {
-        const int j = wj + 8 * b + 2 * (lane & 3);
-        o[a][h][b] = i < mI ? old(baseI + i, baseJ + j, mJ - j) : make_float2(-INF, -INF);
+        for (int b = 0; b < 2; ++b) {
+          const int j = wj + 8 * b + 2 * (lane & 3);
+          o[a][h][b] = decltype(whole_tile)::value || i < mI ? old(baseI + i, baseJ + j, mJ - j, whole_tile) : make_float2(0.0f, 0.0f);
+        }
       }
-    }
+  };
+  if (full && pairs) load(std::true_type{});
+  else load(std::false_type{});
   const float inv = screen_scale(scr.range);
   if (tid < 2 * H) {  // the bases in units of s, less their share of the argument's error
     const float v = tid < H ? scr.base_a[I * T + hI * H + tid] : scr.base_b[J * T + hJ * H + tid - H];
@@ -280,8 +290,9 @@ __device__ __forceinline__ int screen_tile(Smem &sm, Tile &t, int n, int r, int 
     }
   }
   // log2(0.96 T') = (a_i + b_j - t) / s, less what its roundings and ex2's can
-  // amount to: kErr of each of its three terms, and 0.06.
-  constexpr float kErr = 4.76837158203125e-7f;  // 2^-21
+  // amount to: the bases have 2^-21 of a_i / s and b_j / s taken off, and 0.06,
+  // and t / s only enters a fused multiply-add, whose own rounding is within
+  // 2^-24 of the result: nothing below 2^-200, where T' is 0, needs more.
   unsigned mine[2][2];  // [a][h]: bit 2 b + q
   int found = 0;
   auto test = [&](auto limit) {  // limit(old): the largest value a candidate below old can have
@@ -296,20 +307,26 @@ __device__ __forceinline__ int screen_tile(Smem &sm, Tile &t, int n, int r, int 
           const float2 bj = *reinterpret_cast<const float2 *>(&sm.base_b[wj + 8 * b + 2 * (lane & 3)]);
 #pragma unroll
           for (int q = 0; q < 2; ++q) {
-            const float lim = limit(q ? o[a][h][b].y : o[a][h][b].x);
-            const float arg = fmaf(-fabsf(lim), kErr * inv, fmaf(-lim, inv, ai + (q ? bj.y : bj.x)));
-            // (NaN, where t / s and the bases overflow, is flagged; nothing is below -inf)
-            if (!(x[a][b][2 * h + q] <= ex2(arg)) && lim > -INF) mine[a][h] |= 1u << (2 * b + q);
+            const float arg = fmaf(-limit(q ? o[a][h][b].y : o[a][h][b].x), inv, ai + (q ? bj.y : bj.x));
+            // (NaN, where t / s and the bases overflow, is flagged)
+            if (!(x[a][b][2 * h + q] <= ex2(arg))) mine[a][h] |= 1u << (2 * b + q);
           }
+        }
+        if (!full) {
+          const int i = wi + 16 * a + 8 * h + (lane >> 2), j = wj + 2 * (lane & 3);
+          if (i >= mI) mine[a][h] = 0u;
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (j + 8 * (q >> 1) + (q & 1) >= mJ) mine[a][h] &= ~(1u << q);
         }
         found += __popc(mine[a][h]);
       }
   };
   if (whole)
-    test([](float old) {  // the largest integer below old, by rounding to nearest (old itself beyond 2^22)
-      const float near = __fadd_rn(__fadd_rn(old, 12582912.0f), -12582912.0f);
-      return fabsf(old) < 4194304.0f ? (near < old ? near : near - 1.0f) : old;
-    });
+    // ceil(old) - 1, by rounding up at 1.5 2^23.  From 2^22 on the result is at least
+    // min(ceil(old) - 1, 2^23), which no sum of these blocks passes; below -2^22, where
+    // the rounding may be finer, no sum of theirs lies.
+    test([](float old) { return __fadd_rn(__fadd_ru(old, 12582912.0f), -12582913.0f); });
   else test([](float old) { return old; });
   found = __reduce_add_sync(kFullMask, found);
   if (lane == 0 && found) atomicAdd(&sm.count, found);
