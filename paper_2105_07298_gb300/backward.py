@@ -80,18 +80,22 @@ def _solve_stack(D, P):
     persistent launch: directly when every graph starts 16-byte aligned (n^2 a
     multiple of 4), otherwise through a copy in the aligned packed layout.
     Larger graphs are solved one by one by the single-graph path."""
-    from . import apsp_fw_f32
+    import torch
+    from . import ApspError, APSP_ECUDA, apsp_fw_f32
     from .batched import apsp_fw_batched_f32, packed_offsets, packed_numel, MAX_N
     B, n, _ = D.shape
     if n > MAX_N:
         for b in range(B):
             apsp_fw_f32(D[b], P[b])
         return
+    # The batch's work list is host memory of this call: a graph that replays its
+    # upload would read what is no longer there.
+    if torch.cuda.is_current_stream_capturing():
+        raise ApspError(APSP_ECUDA, "batched solve during graph capture")
     sizes = [n] * B
     if (n * n) % 4 == 0:
         apsp_fw_batched_f32(D.view(-1), sizes, [b * n * n for b in range(B)], P.view(-1))
         return
-    import torch
     off = packed_offsets(sizes)
     total = packed_numel(sizes)
     idx = (torch.from_numpy(off).to(D.device)[:, None] + torch.arange(n * n, device=D.device)[None, :])
