@@ -153,7 +153,7 @@ int apsp_fw_i32(int32_t *d_dist, int64_t n, int64_t ld, int32_t *d_path, void *s
  * blocks with 8 x 4 tiles (2), the single-graph phases run by one CTA, which
  * gives apsp_fw_f32's results bit for bit on any weights.  Variant 2 needs
  * per-CTA operand panels: (graph-dependent) scratch of up to
- * 2 MiB per resident CTA, held by the plan.
+ * 1 MiB per resident CTA, held by the plan.
  *
  * Planning splits the graphs into size classes, orders them largest first
  * (longest-processing-time order) and uploads the work list.  A plan holds

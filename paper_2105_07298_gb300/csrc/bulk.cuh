@@ -78,10 +78,6 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t by
       : "memory");
 }
 
-__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
-}
-
 // Thread-block clusters: this CTA's rank, the address of a peer's shared
 // memory, the cluster-wide barrier, and a 16-byte asynchronous store to a
 // peer that completes on that peer's mbarrier as 16 transaction bytes.

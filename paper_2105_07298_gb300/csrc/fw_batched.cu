@@ -71,10 +71,10 @@ static const int kVariantTileRows[kNumVariants] = {4, 4, 8};
 static const int kVariantTileCols[kNumVariants] = {4, 4, 4};
 static const int kVariantEager[kNumVariants] = {0, 1, 1};
 constexpr int kT128 = mp32::T;
-// Per-CTA operand panels of the 128-block variants: Apan, Bpan, Acp and Bt of
-// every block of one round (R <= 8 blocks for n <= 1024), 4-byte words.
+// Per-CTA operand panels of the 128-block variants: Apan and Bpan of every
+// block of one round (R <= 8 blocks for n <= 1024), 4-byte words.
 __host__ __device__ constexpr size_t panel_words_per_array(int rmax) { return (size_t)rmax * kT128 * kT128; }
-__host__ __device__ constexpr size_t panel_bytes_per_cta(int rmax) { return 4 * panel_words_per_array(rmax) * 4; }
+__host__ __device__ constexpr size_t panel_bytes_per_cta(int rmax) { return 2 * panel_words_per_array(rmax) * 4; }
 
 static int class_of(int32_t n) { return class_of_n(n); }
 
@@ -618,9 +618,8 @@ __device__ __forceinline__ void solve_graph_pipe_f32(float *__restrict__ D, int3
 }
 
 // The 128-block variant: the single-graph phases run by this CTA alone.
-// The panels (this CTA's scratch) are rewritten every round, so the product's
-// path recovery reads them through the coherent path (NC = false), and every
-// thread fences its generic writes before the bulk copies read them.
+// The panels (this CTA's scratch) are rewritten every round: every thread fences
+// its generic writes before the bulk copies read them.
 // Returns false if a bounded copy wait ran out (error word set).
 __device__ __forceinline__ bool solve_graph128_f32(float *__restrict__ D, int32_t *__restrict__ P, int n,
                                                    const Panels &pan, bool aligned, unsigned char *smem_raw) {
@@ -653,7 +652,7 @@ __device__ __forceinline__ bool solve_graph128_f32(float *__restrict__ D, int32_
         if (J == r) continue;
         for (int hJ = 0; hJ < 2; ++hJ) {
           __syncthreads();  // the previous product's epilogue is done with the shared memory
-          if (!minplus_half_f32<true, false>(D, ld, P, n, I, J, hJ, r, vec_ok, pan)) return false;
+          if (!minplus_half_f32(D, ld, P, n, I, J, hJ, r, vec_ok, pan)) return false;
         }
       }
     }
@@ -681,8 +680,6 @@ __device__ __forceinline__ void persistent_body(float *__restrict__ Dp, int32_t 
     const size_t words = panel_words_per_array(rmax);
     pan.Apan = reinterpret_cast<unsigned long long *>(base);
     pan.Bpan = reinterpret_cast<unsigned long long *>(base + words * 4);
-    pan.Acp = reinterpret_cast<float *>(base + 2 * words * 4);
-    pan.Bt = reinterpret_cast<float *>(base + 3 * words * 4);
   }
   for (;;) {
     if (threadIdx.x == 0) s_next = atomicAdd(counter, 1);
