@@ -775,6 +775,7 @@ __device__ __forceinline__ void piece64(double *__restrict__ D, int64_t ld, int3
     if (tid == 0) report_wait_timeout();
     return;
   }
+  if (tid == 0) mbar_inval(&sm.bar);  // its one phase is over: the next piece may set it up again
 #pragma unroll 1
   for (int g = 0; g < ng; ++g) {
     float m[4][CW];
