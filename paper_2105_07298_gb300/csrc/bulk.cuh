@@ -145,4 +145,22 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, uint32
   return false;
 }
 
+// What one thread of a CTA does whose wait ran out, before the CTA leaves:
+// records it, and waits once more (bounded) for the copies still on their way, so
+// that none lands in shared memory that has passed to another CTA.
+__device__ __forceinline__ void give_up(uint64_t *bar, uint32_t parity) {
+  report_wait_timeout();
+  mbar_wait(bar, parity);
+}
+
+// The same for a CTA of a cluster to which others send (call it after the cluster's
+// last barrier, when all is sent): bar[q], q < count, is completed by CTA q / own,
+// phase 0 alone.  Out of line, since it is not expected to run: inside phase 1 of
+// FP64 it cost 2 % of an n = 1000 solve.
+static __device__ __noinline__ void drain_ring(uint64_t *bar, int count, int own, int cta) {
+#pragma unroll 1
+  for (int q = 0; q < count; ++q)
+    if (q / own != cta) mbar_spin(&bar[q], 0, kWaitLimit / 32);
+}
+
 }  // namespace apsp

@@ -478,6 +478,7 @@ __global__ void __cluster_dims__(k1::CTAS, 1, 1) __launch_bounds__(k1::THREADS, 
   cluster_wait();  // no CTA leaves while another may still write its buffers
   if (!ok) {       // D and P stay as they are
     report_wait_timeout();
+    drain_ring(sm.bar, nquad, WARPS, cta);
     return;
   }
   if (helper) return;
@@ -617,7 +618,7 @@ __global__ void __launch_bounds__(32 * k2::WARPS, 2)
   __syncthreads();
   const bool ok = mbar_wait(&sm.bar, 0);
   if (__syncthreads_or(!ok)) {  // the diagonal block never arrived: leave D, P and the operands as they are
-    if (tid == 0) report_wait_timeout();
+    if (tid == 0) give_up(&sm.bar, 0);
     return;
   }
 #pragma unroll 1
@@ -727,7 +728,9 @@ struct Smem {
 };
 }  // namespace k3
 
-__device__ __forceinline__ void piece64(double *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r,
+// False if the wait for the operands ran out: the CTA must then not set the
+// barrier up again.
+__device__ __forceinline__ bool piece64(double *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r,
                                         int I, int J, int sub, const Panels64 &pan) {
   using namespace k3;
   constexpr int CW = 2;  // columns per thread
@@ -736,7 +739,7 @@ __device__ __forceinline__ void piece64(double *__restrict__ D, int64_t ld, int3
   const int si = sub >> 1, hJ = sub & 1;
   const int baseI = I * T + si * TR, baseJ = J * T + hJ * TC, baseK = r * T;
   const int mI = min(TR, n - baseI), mJ = min(TC, n - baseJ), mK = min(T, n - baseK);
-  if (mI <= 0 || mJ <= 0) return;  // past the matrix (uniform exit)
+  if (mI <= 0 || mJ <= 0) return true;  // past the matrix (uniform exit)
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   // Whole groups: the operands are +inf past the matrix.
   const int ng = (mK + 2 * GP - 1) / (2 * GP);
@@ -772,8 +775,8 @@ __device__ __forceinline__ void piece64(double *__restrict__ D, int64_t ld, int3
   __syncwarp();
   const bool ok = mbar_wait(&sm.bar, 0);
   if (__syncthreads_or(!ok)) {  // the operands never arrived: the block stays as it is
-    if (tid == 0) report_wait_timeout();
-    return;
+    if (tid == 0) give_up(&sm.bar, 0);
+    return false;
   }
   if (tid == 0) mbar_inval(&sm.bar);  // its one phase is over: the next piece may set it up again
 #pragma unroll 1
@@ -882,6 +885,7 @@ __device__ __forceinline__ void piece64(double *__restrict__ D, int64_t ld, int3
       if (P) P[e] = baseK + k;
     }
   }
+  return true;
 }
 
 template <int CTAS_PER_SM>
@@ -1007,7 +1011,7 @@ __global__ void __launch_bounds__(k3::THREADS, 4)
     block_of(set, tile / k3x::PER_BLOCK, r, R, I, J);
     fence_proxy_async_smem();
     __syncthreads();  // everyone is done with the previous piece's shared memory
-    piece64(D, ld, P, n, r, I, J, 2 * ((q >> 1) * PER + t % PER) + (q & 1), pan);
+    if (!piece64(D, ld, P, n, r, I, J, 2 * ((q >> 1) * PER + t % PER) + (q & 1), pan)) return;
   }
 }
 

@@ -310,7 +310,8 @@ __global__ void __cluster_dims__(k1::CTAS, 1, 1) __launch_bounds__(32 * k1::WARP
       }
     }
   }
-  cluster_sync();  // no CTA leaves while another may still write its history
+  cluster_sync();  // no CTA leaves while another may still send to its history
+  if (!ok) drain_ring(sm.bar, nquad, WARPS, cta);  // nor while one may still arrive
 }
 
 // --------------------------------------------------------------------------
@@ -427,7 +428,7 @@ __global__ void __launch_bounds__(k2s::THREADS, 2)
   __syncthreads();
   const bool ok = mbar_wait(&sm.bar, 0);
   if (__syncthreads_or(!ok)) {  // the diagonal block never arrived: leave D, P and the panels as they are
-    if (tid == 0) report_wait_timeout();
+    if (tid == 0) give_up(&sm.bar, 0);
     return;
   }
   // Positions 2 kp, 2 kp + 1: slots 2 h, 2 h + 1 of lane kp mod 32, h = kp / 32.
@@ -591,9 +592,10 @@ struct Smem {
 }  // namespace k3s
 
 // Piece `sub` of output block (I, J): all 256 threads, the launch's dynamic
-// shared memory from offset 0, its barrier in phase 0.
+// shared memory from offset 0, its barrier in phase 0.  False if the wait for the
+// operands ran out: the CTA must then not set the barrier up again.
 template <bool PATH, int TR>
-__device__ __forceinline__ void piece_f32(float *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r,
+__device__ __forceinline__ bool piece_f32(float *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r,
                                           int I, int J, int sub, int vec_ok, const Panels &pan) {
   using namespace k3s;
   static_assert(TR == 32 || TR == 64, "eight warps of 16 x 16 or 16 x 32 outputs");
@@ -603,7 +605,7 @@ __device__ __forceinline__ void piece_f32(float *__restrict__ D, int64_t ld, int
   const int si = sub >> 1, hJ = sub & 1;
   const int baseI = I * T + si * TR, baseJ = J * T + hJ * TC, baseK = r * T;
   const int mI = min(TR, n - baseI), mJ = min(TC, n - baseJ), mK = min(T, n - baseK);
-  if (mI <= 0 || mJ <= 0) return;  // past the matrix (uniform exit)
+  if (mI <= 0 || mJ <= 0) return true;  // past the matrix (uniform exit)
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int nkp = (mK + 1) / 2;
   if (tid == 0) {
@@ -653,8 +655,8 @@ __device__ __forceinline__ void piece_f32(float *__restrict__ D, int64_t ld, int
   __syncwarp();
   const bool ok = mbar_wait(&sm.bar, 0);
   if (__syncthreads_or(!ok)) {  // the operands never arrived: the block stays as it is
-    if (tid == 0) report_wait_timeout();
-    return;
+    if (tid == 0) give_up(&sm.bar, 0);
+    return false;
   }
   if (tid == 0) mbar_inval(&sm.bar);  // its one phase is over: the next piece may set it up again
   auto step = [&](int kp) {
@@ -704,7 +706,7 @@ __device__ __forceinline__ void piece_f32(float *__restrict__ D, int64_t ld, int
         // (improved outputs lie inside the matrix)
         if (acc[a][c] < prev[a][c]) D[(int64_t)(baseI + i) * ld + baseJ + j] = acc[a][c];
       }
-    return;
+    return true;
   }
   // Each lane takes its own next improved output, so that the warp runs the
   // rest as often as its fullest lane needs and not once per output.
@@ -736,6 +738,7 @@ __device__ __forceinline__ void piece_f32(float *__restrict__ D, int64_t ld, int
     D[e] = x;
     P[e] = baseK + k;
   }
+  return true;
 }
 
 template <bool PATH, int TR>
@@ -825,7 +828,7 @@ __global__ void __launch_bounds__(k3s::THREADS, 3)
     block_of(set, tile / k3x::PER_BLOCK, r, R, I, J);
     fence_proxy_async_smem();
     __syncthreads();  // everyone is done with the previous piece's shared memory
-    piece_f32<PATH, 64>(D, ld, P, n, r, I, J, tile % k3x::PER_BLOCK, vec_ok, pan);
+    if (!piece_f32<PATH, 64>(D, ld, P, n, r, I, J, tile % k3x::PER_BLOCK, vec_ok, pan)) return;
   }
 }
 

@@ -200,10 +200,10 @@ __device__ __forceinline__ bool minplus_half_f32(float *__restrict__ D, int64_t 
     const int st = s % STAGES;
     const bool ok = mbar_wait(&sm.bar[st], (s / STAGES) & 1);
     if (__syncthreads_or(!ok)) {
-      // A copy never completed: record it, wait (bounded) for the other
-      // copies this CTA issued, and leave without touching D or P.
+      // A copy never completed: record it, wait (bounded) for every copy of
+      // this CTA still on its way, and leave without touching D or P.
       if (tid == 0) {
-        report_wait_timeout();
+        give_up(&sm.bar[st], (s / STAGES) & 1);
         for (int s2 = s + 1; s2 < nslab && s2 < s + STAGES; ++s2)
           mbar_wait(&sm.bar[s2 % STAGES], (s2 / STAGES) & 1);
       }

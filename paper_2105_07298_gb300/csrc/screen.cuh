@@ -264,7 +264,7 @@ __device__ __forceinline__ int screen_tile(Smem &sm, Tile &t, int n, int r, int 
   __syncthreads();
   const bool ok = mbar_wait(&sm.bar, 0);
   if (__syncthreads_or(!ok)) {  // the weights never arrived: the block stays as it is
-    if (tid == 0) report_wait_timeout();
+    if (tid == 0) give_up(&sm.bar, 0);
     return 0;
   }
   float x[2][2][4];
