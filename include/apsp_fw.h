@@ -167,7 +167,10 @@ int apsp_fw_i32(int32_t *d_dist, int64_t n, int64_t ld, int32_t *d_path, void *s
  *   d_dist     : packed FP32 distances, overwritten in place.
  *   d_path     : packed int32 path matrices (same offsets), or NULL.
  * apsp_fw_batched_f32 = plan + run + destroy (allocates and frees its work
- * list and panels with stream-ordered allocation on `stream`).
+ * list and panels with stream-ordered allocation on `stream`).  It returns
+ * APSP_ECUDA, with nothing enqueued, while `stream` is being captured into a
+ * CUDA graph, whose replays would read its work list from host memory of the
+ * call: capture the run of a plan instead.
  * ---------------------------------------------------------------------- */
 typedef struct apsp_batched_plan apsp_batched_plan;
 

@@ -91,7 +91,8 @@ class BatchedPlan:
 
 
 def apsp_fw_batched_f32(dist, sizes, offsets=None, path=None, stream=None):
-    """One-shot batched solve (plan, run and free in one call)."""
+    """One-shot batched solve (plan, run and free in one call).  Refused while the
+    stream is being captured into a CUDA graph: capture a BatchedPlan's run."""
     from . import load, _check, _stream_ptr
     n, off = _host_arrays(sizes, offsets)
     _check_buffers(dist, path, _layout_numel(n, off))

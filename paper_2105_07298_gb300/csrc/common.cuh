@@ -23,6 +23,17 @@ __device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(
 
 inline int status_from(cudaError_t e) { return e == cudaSuccess ? APSP_OK : APSP_ECUDA; }
 
+// Whether `s` is being captured into a CUDA graph.
+inline int stream_capturing(cudaStream_t s, bool *capturing) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
+    cudaGetLastError();
+    return APSP_ECUDA;
+  }
+  *capturing = cap != cudaStreamCaptureStatusNone;
+  return APSP_OK;
+}
+
 // Sets the dynamic shared-memory limit of a kernel once per (kernel, device).
 template <typename K>
 inline int ensure_smem(K kernel, int bytes, int *done_flags /*[64]*/) {

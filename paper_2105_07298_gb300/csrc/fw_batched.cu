@@ -867,6 +867,11 @@ APSP_EXPORT int apsp_fw_batched_f32(float *d_dist, int32_t *d_path, const int32_
   if (num == 0) return APSP_OK;
   if (!d_dist) return APSP_EINVAL;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+  // A graph would replay the upload of the work list from host memory of this
+  // call, which is gone by then.
+  bool capturing = false;
+  if ((st = apsp::stream_capturing(s, &capturing))) return st;
+  if (capturing) return APSP_ECUDA;
   int rmax = 0;
   std::vector<int32_t> order = lpt_order(h_n, num, &rmax);
   int grid = grid_for(num, rmax > 0);

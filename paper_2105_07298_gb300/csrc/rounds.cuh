@@ -65,17 +65,6 @@ inline void launch_after(void (*kernel)(A...), int grid, int threads, size_t sme
   cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-// Whether `s` is being captured into a CUDA graph.
-inline int stream_capturing(cudaStream_t s, bool *capturing) {
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
-    cudaGetLastError();
-    return APSP_ECUDA;
-  }
-  *capturing = cap != cudaStreamCaptureStatusNone;
-  return APSP_OK;
-}
-
 // All rounds of an R-block solve.  diag(r, stream) and panels(r, stream)
 // enqueue phases 1 and 2+3, phase4(r, set, blocks, stream) phase 4 on a block
 // set, init(stream) what must precede every panel but not the first diagonal

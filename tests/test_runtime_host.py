@@ -1,0 +1,29 @@
+"""Host code of the library on a CUDA runtime that only keeps count (fake_cudart)."""
+import ctypes
+
+import pytest
+
+import paper_2105_07298_gb300 as apsp
+from fake_cudart import load, word
+
+DEV = ctypes.c_void_p(256)  # stands for any device buffer: nothing reads it
+
+
+@pytest.fixture()
+def lib(tmp_path):
+    return load(tmp_path)
+
+
+def _one_shot(lib):
+    n, off = (ctypes.c_int32 * 2)(8, 16), (ctypes.c_int64 * 2)(0, 64)
+    return lib.apsp_fw_batched_f32(DEV, DEV, n, off, 2, None)
+
+
+def test_one_shot_batch_refuses_graph_capture(lib):
+    """Its work list is uploaded from memory of the call, which a replay would not find."""
+    word(lib, "capturing").value = 1
+    assert _one_shot(lib) == apsp.APSP_ECUDA
+    assert not any(word(lib, w).value for w in ("launches", "copies", "allocs", "pool_allocs", "live"))
+    word(lib, "capturing").value = 0
+    assert _one_shot(lib) == apsp.APSP_OK
+    assert word(lib, "launches").value == word(lib, "copies").value == 1 and word(lib, "live").value == 0
