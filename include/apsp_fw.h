@@ -300,9 +300,10 @@ int apsp_profile_records(int32_t *phase, float *ms, int64_t cap, int64_t *count)
 int apsp_measure_peak(int dtype_bytes, double *relax_per_clk_per_sm, void *stream);
 
 /* Synchronizes `stream`, then returns and clears the error words that the
- * single-graph kernels set on the device when one of their bounded waits for
- * an asynchronous copy runs out (the kernel then leaves its block unchanged,
- * so the result of that solve is incomplete): APSP_OK if no wait ran out
+ * single-graph and the batched kernels set on the device when one of their
+ * bounded waits for an asynchronous copy runs out (the kernel then leaves its
+ * block, a batched one its graph, unfinished, so the result of that solve is
+ * incomplete): APSP_OK if no wait ran out
  * since the last call, APSP_ETIMEOUT if one did, APSP_EUNSUPPORTED if
  * apsp_fw_i32 saturated a distance, APSP_ECUDA if the stream or the
  * read-back failed. */

@@ -730,6 +730,8 @@ __global__ void __launch_bounds__(mp32::THREADS, 2)
   persistent_body<true>(Dp, Pp, order, ns, offs, num, counter, scratch, rmax);
 }
 
+int take_device_error_batched() { return take_tu_device_error(); }
+
 }  // namespace apsp
 
 struct apsp_batched_plan {

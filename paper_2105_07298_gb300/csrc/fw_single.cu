@@ -866,6 +866,7 @@ int run_fw_f64_interval(double *D, int n, int64_t ld, int32_t *P, cudaStream_t s
 int take_device_error_f64();
 int take_device_error_checks();
 int take_device_error_int32();
+int take_device_error_batched();
 
 static void path_init(int32_t *P, int64_t n, int64_t ld, int64_t skip, cudaStream_t s) {
   const int64_t total = n * n;
@@ -1090,5 +1091,6 @@ APSP_EXPORT int apsp_device_status(void *stream) {
   const int v64 = apsp::take_device_error_f64();
   const int vc = apsp::take_device_error_checks();
   const int vi = apsp::take_device_error_int32();
-  return v != 0 ? v : v64 != 0 ? v64 : vc != 0 ? vc : vi;
+  const int vb = apsp::take_device_error_batched();
+  return v != 0 ? v : v64 != 0 ? v64 : vc != 0 ? vc : vi != 0 ? vi : vb;
 }

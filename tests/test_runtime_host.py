@@ -27,3 +27,13 @@ def test_one_shot_batch_refuses_graph_capture(lib):
     word(lib, "capturing").value = 0
     assert _one_shot(lib) == apsp.APSP_OK
     assert word(lib, "launches").value == word(lib, "copies").value == 1 and word(lib, "live").value == 0
+
+
+def test_device_status_reads_and_clears_every_error_word(lib):
+    """Each source file's kernels have a word of their own."""
+    words = [lib.var_at(i) for i in range(word(lib, "num_vars").value) if b"g_device_error" in lib.var_name(i)]
+    assert len(words) >= 5 and lib.apsp_device_status(None) == apsp.APSP_OK
+    for w in words:
+        ctypes.c_int.from_address(w).value = apsp.APSP_ETIMEOUT
+        assert lib.apsp_device_status(None) == apsp.APSP_ETIMEOUT
+        assert lib.apsp_device_status(None) == apsp.APSP_OK
