@@ -6,17 +6,19 @@
 namespace apsp {
 
 static std::mutex g_mu;
-static cudaMemPool_t g_pool[64];  // per device, created on first use
+static cudaMemPool_t g_pool[64];  // per device, created on first use, kept to the end of the process
 
-static cudaError_t create_pool(int dev, cudaMemPool_t *pool) {
+static cudaMemPool_t create_pool(int dev) {
   cudaMemPoolProps props{};
   props.allocType = cudaMemAllocationTypePinned;
   props.location.type = cudaMemLocationTypeDevice;
   props.location.id = dev;
-  cudaError_t e = cudaMemPoolCreate(pool, &props);
-  if (e != cudaSuccess) return e;
+  cudaMemPool_t pool = nullptr;
+  if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) return nullptr;
   unsigned long long keep = kKeepBytes;
-  return cudaMemPoolSetAttribute(*pool, cudaMemPoolAttrReleaseThreshold, &keep);
+  if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess) return pool;
+  cudaMemPoolDestroy(pool);
+  return nullptr;
 }
 
 cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t s) {
@@ -26,16 +28,12 @@ cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t s) {
       cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64)
     return cudaMallocAsync(p, bytes, s);
   std::lock_guard<std::mutex> lock(g_mu);
-  // A second attempt with a new pool: a device reset has taken the old one.
-  for (int attempt = 0; attempt < 2; ++attempt) {
-    if (!g_pool[dev] && create_pool(dev, &g_pool[dev]) != cudaSuccess) break;
-    const cudaError_t e = cudaMallocFromPoolAsync(p, bytes, g_pool[dev], s);
-    if (e == cudaSuccess || e == cudaErrorMemoryAllocation) return e;
-    cudaGetLastError();
-    g_pool[dev] = nullptr;
+  if (!g_pool[dev]) g_pool[dev] = create_pool(dev);
+  if (g_pool[dev]) {
+    if (cudaMallocFromPoolAsync(p, bytes, g_pool[dev], s) == cudaSuccess) return cudaSuccess;
+    cudaMemPoolTrimTo(g_pool[dev], 0);
   }
   cudaGetLastError();
-  g_pool[dev] = nullptr;
   return cudaMallocAsync(p, bytes, s);
 }
 

@@ -14,7 +14,9 @@ namespace apsp {
 constexpr size_t kKeepBytes = size_t(256) << 20;
 
 // cudaMallocAsync while `s` is being captured (the allocation then belongs to
-// the graph).
+// the graph), and where the pool cannot be had or cannot hold the block: what it
+// keeps is then given back first, and the default pool may have room that other
+// code of the process keeps there.
 cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t s);
 
 }  // namespace apsp

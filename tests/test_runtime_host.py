@@ -37,3 +37,28 @@ def test_device_status_reads_and_clears_every_error_word(lib):
         ctypes.c_int.from_address(w).value = apsp.APSP_ETIMEOUT
         assert lib.apsp_device_status(None) == apsp.APSP_ETIMEOUT
         assert lib.apsp_device_status(None) == apsp.APSP_OK
+
+
+def _counts(lib, *names):
+    return tuple(word(lib, w).value for w in names)
+
+
+@pytest.mark.parametrize("error", [2, 1])  # out of memory, and any other
+def test_scratch_falls_back_to_the_default_pool(lib, error):
+    word(lib, "pool_error").value = error
+    for call in (1, 2):
+        assert _one_shot(lib) == apsp.APSP_OK
+        assert _counts(lib, "pools_created", "pools_destroyed", "pool_allocs", "pools_trimmed", "allocs",
+                       "live") == (1, 0, call, call, call, 0)
+    word(lib, "alloc_error").value = 2
+    assert _one_shot(lib) == apsp.APSP_ENOMEM
+    word(lib, "pool_error").value = word(lib, "alloc_error").value = 0
+    assert _one_shot(lib) == apsp.APSP_OK
+    assert _counts(lib, "pools_created", "allocs", "live") == (1, 3, 0)
+
+
+def test_scratch_pool_without_its_bound_is_not_kept(lib):
+    """The bound on what it keeps could not be set: the default pool serves."""
+    word(lib, "pool_attr_error").value = 1
+    assert _one_shot(lib) == apsp.APSP_OK
+    assert _counts(lib, "pools_created", "pools_destroyed", "pool_allocs", "allocs") == (1, 1, 0, 1)
