@@ -279,10 +279,12 @@ int apsp_fw_backward_packed_f32(const float *d_grad_dist, const int32_t *d_path,
 int apsp_profile_enable(int on);
 int apsp_profile_collect(double *ms, int64_t *launches);
 
-/* The same records one by one, in launch order (per-round timing: the r-th
- * phase-4 record is round r of the last solve when one solve was recorded).
+/* The same records one by one, in the order they were enqueued (per-round
+ * timing: phase 4 of a round is one record, or two where the next round
+ * overlaps it: its row and column, then the rest).  A record is one launch, or
+ * in a screened round of phase 4 the two of a screen and its dense kernel.
  * Waits for the recorded events; writes min(cap, records) entries to
- * phase[] (index as above) and ms[] (device time of that launch), and the
+ * phase[] (index as above) and ms[] (device time of that record), and the
  * number of records to *count.  phase and ms may be NULL when cap is 0.
  * Returns APSP_EINVAL for a NULL count, a negative cap, or NULL arrays with
  * cap > 0. */

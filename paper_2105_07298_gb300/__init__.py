@@ -255,7 +255,7 @@ def profile_collect() -> dict:
 
 
 def profile_records() -> list:
-    """[(phase, ms)] of every recorded launch, in launch order."""
+    """[(phase, ms)] of every record, in launch order (a screened part of phase 4 is one, of two launches)."""
     lib = load()
     count = _i64(0)
     _check(lib.apsp_profile_records(None, None, 0, ctypes.byref(count)), "apsp_profile_records")

@@ -1103,8 +1103,9 @@ int run_fw_f64_interval(double *D, int n, int64_t ld, int32_t *P, cudaStream_t s
   };
   auto phase4 = [&](int r, int set, int blocks, cudaStream_t stm) {
     if (blocks <= 0) return;
-    PhaseScope sc(3, stm);
-    if (screened && r >= kScreenFrom) {
+    const bool screen = screened && r >= kScreenFrom;
+    PhaseScope sc(3, stm, screen ? 2 : 1);
+    if (screen) {
       const Screen sr = screen_of(r);
       launch_after(fw64_screen, k3x::PER_BLOCK * blocks, k3x::THREADS, sizeof(k3x::Smem), stm, overlap, D, ld, P, n, r,
                    R, vec, pan[r & 1], sr, set);

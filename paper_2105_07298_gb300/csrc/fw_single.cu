@@ -976,8 +976,9 @@ static int run_fw_f32(float *D, int64_t n64, int64_t ld, int32_t *P, void *strea
   };
   auto phase4 = [&](int r, int set, int blocks, cudaStream_t st) {
     if (blocks <= 0) return;
-    PhaseScope ps(3, st);
-    if (screened && r >= kScreenFrom) {
+    const bool screen = screened && r >= kScreenFrom;
+    PhaseScope ps(3, st, screen ? 2 : 1);
+    if (screen) {
       const Screen sc = screen_of(r);
       launch_after(P ? fw_phase3_screen_f32<true> : fw_phase3_screen_f32<false>, k3x::PER_BLOCK * blocks, k3x::THREADS,
                    sizeof(k3x::Smem), st, overlap, D, ld, P, n, r, R, vec_ok, pan[r & 1], sc, set);
@@ -1062,7 +1063,7 @@ APSP_EXPORT int apsp_profile_collect(double *ms, int64_t *launches) {
     float t = 0.f;
     if (cudaEventElapsedTime(&t, r.a, r.b) != cudaSuccess) return APSP_ECUDA;
     ms[r.phase] += t;
-    launches[r.phase] += 1;
+    launches[r.phase] += r.launches;
   }
   return APSP_OK;
 }

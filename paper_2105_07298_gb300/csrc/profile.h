@@ -1,6 +1,7 @@
 // Host-side phase timing shared by the translation units (internal).  When
-// enabled through apsp_profile_enable, each bracketed launch gets two CUDA
-// events on its stream; apsp_profile_collect sums them per phase.
+// enabled through apsp_profile_enable, each bracketed launch (or pair: a screened
+// part of phase 4 is two launches, one behind the other) gets two CUDA events on
+// its stream; apsp_profile_collect sums them per phase.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -10,7 +11,7 @@
 namespace apsp {
 
 struct PhaseRec {
-  int phase;
+  int phase, launches;
   cudaEvent_t a, b;
 };
 
@@ -31,16 +32,17 @@ inline cudaEvent_t prof_event() {
   return e;
 }
 
-// RAII bracket around the launches of one phase (no-op when profiling is off).
+// RAII bracket around a launch, or several, of one phase (no-op when profiling is off).
 struct PhaseScope {
   bool on;
   PhaseRec rec;
   cudaStream_t s;
-  PhaseScope(int phase, cudaStream_t st) : on(false), s(st) {
+  PhaseScope(int phase, cudaStream_t st, int launches = 1) : on(false), s(st) {
     std::lock_guard<std::mutex> g(g_prof_mu);
     if (!g_prof_on) return;
     on = true;
     rec.phase = phase;
+    rec.launches = launches;
     rec.a = prof_event();
     rec.b = prof_event();
     cudaEventRecord(rec.a, s);

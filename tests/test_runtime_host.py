@@ -62,3 +62,16 @@ def test_scratch_pool_without_its_bound_is_not_kept(lib):
     word(lib, "pool_attr_error").value = 1
     assert _one_shot(lib) == apsp.APSP_OK
     assert _counts(lib, "pools_created", "pools_destroyed", "pool_allocs", "allocs") == (1, 1, 0, 1)
+
+
+@pytest.mark.parametrize("fn,n", [("apsp_fw_f32", 2900), ("apsp_fw_f64", 4000), ("apsp_fw_f32", 1000)])
+def test_phase_timing_counts_every_launch(lib, fn, n):
+    """Also the dense kernel behind each screen."""
+    lib.apsp_profile_enable(1)
+    assert getattr(lib, fn)(DEV, ctypes.c_int64(n), ctypes.c_int64(n), DEV, None) == apsp.APSP_OK
+    ms, launches = (ctypes.c_double * 4)(), (ctypes.c_int64 * 4)()
+    assert lib.apsp_profile_collect(ms, launches) == apsp.APSP_OK
+    assert sum(launches) == word(lib, "launches").value
+    R = (n + 127) // 128
+    assert launches[:3] == [1, R, R] and (launches[3] == 2 * R - 1) == (n == 1000)
+    lib.apsp_profile_enable(0)
