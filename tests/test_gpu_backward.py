@@ -162,3 +162,83 @@ def test_autograd_stack_odd_and_large_n(Bn, n):
         ref = oracle.fw_backward(gD[b], Ph[b], Dh[b])
         bound = _grad_tol(gD[b], Ph[b], Dh[b])
         assert (np.abs(gW[b] - ref) <= 1e-5 * np.maximum(bound, 1e-30) + 1e-30).all()
+
+
+def _oracle_grad(W, gD):
+    """(P, D, gradient, bound of its rounding) of one graph, by the oracle alone."""
+    D, P = oracle.bfw(W, 64)
+    return P, D, oracle.fw_backward(gD, P, D), 1e-5 * np.maximum(_grad_tol(gD, P, D), 1e-30) + 1e-30
+
+
+# A thread per pair up to 128 vertices, a warp per row above.
+@pytest.mark.parametrize("Bn,n", [(5, 1), (700, 2), (300, 5), (9, 31), (3, 33), (2, 128), (2, 129)])
+def test_backward_small_graphs_strided(Bn, n):
+    """Rows and graphs apart (ld > n, stride > n ld); nothing between them is written."""
+    import ctypes
+    ld, stride = n + 3, n * (n + 3) + 5
+    Ws = [graphgen.dense_graph(n, 0.6, 1300 + b, weights="real", lo=0.5, hi=2.0) for b in range(Bn)]
+    gD = graphgen.normal((Bn, n, n), 17)
+    host = {k: np.full(Bn * stride, 7, np.int32 if k == "P" else np.float32) for k in ("g", "P", "D", "w")}
+    at = [np.arange(n)[:, None] * ld + np.arange(n) + b * stride for b in range(Bn)]
+    refs = []
+    for b in range(Bn):
+        P, D, ref, bound = _oracle_grad(Ws[b], gD[b])
+        host["g"][at[b]], host["P"][at[b]], host["D"][at[b]] = gD[b], P, D
+        refs.append((ref, bound))
+    dev = {k: torch.from_numpy(v).to(DEV) for k, v in host.items()}
+    status = torch.full((1,), 9, dtype=torch.int32, device=DEV)
+    p = [ctypes.c_void_p(dev[k].data_ptr()) for k in ("g", "P", "D", "w")]
+    assert apsp.load().apsp_fw_backward_f32(*p, n, ld, Bn, stride, ctypes.c_void_p(status.data_ptr()), None) == apsp.APSP_OK
+    torch.cuda.synchronize()
+    got = dev["w"].cpu().numpy()
+    for b in range(Bn):
+        ref, bound = refs[b]
+        assert (np.abs(got[at[b]] - ref) <= bound).all(), b
+        got[at[b]] = 7
+    assert (got == 7).all() and int(status.item()) == apsp.APSP_OK
+
+
+# Fewer graphs than warps' slices, enough for eight zeroing warps each, and many.
+@pytest.mark.parametrize("count", [3, 1300, 5000])
+def test_backward_packed_small_graphs(count):
+    """Sizes around the limit of a thread per pair, and graphs with no vertex between them."""
+    from paper_2105_07298_gb300 import batched as B
+    rng = np.random.default_rng(count)
+    sizes = rng.integers(1, 9, count)
+    sizes[[0, count // 2, count - 1]] = 128, 129, 40
+    off, total = B.packed_offsets(sizes), B.packed_numel(sizes)
+    host = {k: np.full(total, 7, np.int32 if k == "P" else np.float32) for k in ("g", "P", "D", "w")}
+    ref, bound = np.full(total, 7.0), np.zeros(total)
+    seen = {}  # (n, variant): graphs repeat
+    for g, (n, o) in enumerate(zip(sizes, off)):
+        key = (int(n), g % 7)
+        if key not in seen:
+            W = graphgen.dense_graph(int(n), 0.6, 2100 + 7 * int(n) + g % 7, weights="real", lo=0.5, hi=2.0)
+            gD = graphgen.normal((int(n), int(n)), 5 + g % 7)
+            seen[key] = (gD, *_oracle_grad(W, gD))
+        s = slice(o, o + n * n)
+        for dst, src in zip((host["g"], host["P"], host["D"], ref, bound), seen[key], strict=True):
+            dst[s] = src.reshape(-1)
+    skipped = np.array([1, count - 2])  # no vertices: left alone
+    ns = sizes.astype(np.int32)
+    ns[skipped] = 0
+    for g in skipped:
+        s = slice(off[g], off[g] + sizes[g] ** 2)
+        ref[s], bound[s] = 7, 0
+    dev = {k: torch.from_numpy(v).to(DEV) for k, v in host.items()}
+    nd, od = torch.from_numpy(ns).to(DEV), torch.from_numpy(off).to(DEV)
+    apsp.apsp_fw_backward_packed_f32(dev["g"], dev["P"], dev["D"], nd, od, dev["w"])
+    assert (np.abs(dev["w"].cpu().numpy() - ref) <= bound).all()
+    nd[1] = -1
+    with pytest.raises(apsp.ApspError):
+        apsp.apsp_fw_backward_packed_f32(dev["g"], dev["P"], dev["D"], nd, od, dev["w"])
+
+
+def test_backward_more_pairs_than_32_bits_index():
+    """2^31 pairs and a few: graphs in which every pair is its own edge."""
+    Bn, n = (1 << 17) + 1, 128
+    gD = torch.randn((Bn, n, n), device=DEV)
+    P = torch.full((Bn, n, n), -1, dtype=torch.int32, device=DEV)
+    gW = apsp.apsp_fw_backward_f32(gD, P, torch.ones_like(gD))
+    gD.diagonal(dim1=1, dim2=2).zero_()
+    assert torch.equal(gW, gD)
