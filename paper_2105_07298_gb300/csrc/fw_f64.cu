@@ -906,6 +906,7 @@ __global__ void __launch_bounds__(k3::THREADS, CTAS_PER_SM)
 // Bound: as the FP32 screen, the latency of the loads; at n = 4096 the next
 // round's chain (K1 90, K2 60, row and column r+1 50 us) sets the pace.  n =
 // 4096 / 6000 with P, integers: 9.8 / 27.2 -> 8.7 / 21.1 ms.
+template <bool PROBE>
 __global__ void __launch_bounds__(k3x::THREADS, 4)
     fw64_screen(double *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r, int R, int vec, Panels64 pan,
                 Screen scr, int set) {
@@ -914,8 +915,8 @@ __global__ void __launch_bounds__(k3x::THREADS, 4)
   Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
   const float FINF = inf<float>();
   Tile tile;
-  const int count = screen_tile<k2::PARTS>(sm, tile, n, r, R, scr, set, vec != 0,
-                                            [&](int i, int j, int left, auto whole_tile) {
+  const int count = screen_tile<k2::PARTS, PROBE>(sm, tile, n, r, R, scr, set, vec != 0,
+                                                  [&](int i, int j, int left, auto whole_tile) {
     const double *p = D + (int64_t)i * ld + j;
     if constexpr (decltype(whole_tile)::value) {
       const double2 t = *reinterpret_cast<const double2 *>(p);
@@ -1015,7 +1016,7 @@ __global__ void __launch_bounds__(k3::THREADS, 4)
   }
 }
 
-static int g_smem_k1[64], g_smem_k2[64], g_smem_k3[2][64], g_smem_k3x[64], g_smem_k3l[64];
+static int g_smem_k1[64], g_smem_k2[64], g_smem_k3[2][64], g_smem_k3x[2][64], g_smem_k3l[64];
 
 // Four CTAs of 64 registers per SM where phase 4 has many waves (n = 4096 /
 // 8192: 10.6 / 68.9 ms against 11.1 / 72.2 with three, before the outputs were
@@ -1027,6 +1028,8 @@ constexpr int kFewBlocks = 24;
 // outputs improve, U(0, 1), screening costs 2-3 % at every size).  From round 8
 // on: 9.0 ms at n = 4096 against 8.7, since settling an output costs more here.
 constexpr int kScreenMinR = 32, kScreenFrom = 16;
+// (As FP32 with P; limits of 12 to 14 within 1 % at n = 4096 and 6000.)
+constexpr ScreenCost kCost{18, 15};
 
 }  // namespace f64
 
@@ -1041,7 +1044,8 @@ int run_fw_f64_interval(double *D, int n, int64_t ld, int32_t *P, cudaStream_t s
   if ((st = ensure_smem(fw64_lines, (int)sizeof(k2::Smem), g_smem_k2))) return st;
   const auto pieces = R <= kFewBlocks ? fw64_pieces<3> : fw64_pieces<4>;
   if ((st = ensure_smem(pieces, (int)sizeof(k3::Smem), g_smem_k3[R <= kFewBlocks]))) return st;
-  if ((st = ensure_smem(fw64_screen, (int)sizeof(k3x::Smem), g_smem_k3x))) return st;
+  if ((st = ensure_smem(fw64_screen<false>, (int)sizeof(k3x::Smem), g_smem_k3x[0]))) return st;
+  if ((st = ensure_smem(fw64_screen<true>, (int)sizeof(k3x::Smem), g_smem_k3x[1]))) return st;
   if ((st = ensure_smem(fw64_listed, (int)sizeof(k3::Smem), g_smem_k3l))) return st;
   // Phase-4 operands: two sets by round parity, each R blocks of A and of B;
   // then K1's copies of the closed diagonal block.  With screened rounds the
@@ -1080,13 +1084,14 @@ int run_fw_f64_interval(double *D, int n, int64_t ld, int32_t *P, cudaStream_t s
       return APSP_ECUDA;
     }
   }
-  auto screen_of = [&](int r) { return screened && r >= kScreenFrom ? scr.round(r, 2) : Screen{}; };
   bool capturing = false;
   if ((st = stream_capturing(s, &capturing))) {
     if (scratch) cudaFreeAsync(scratch, s);
     return st;
   }
   const bool overlap = !capturing;
+  const int probed = set_blocks(capturing ? kSetAll : kSetRest, R);
+  auto screen_of = [&](int r) { return screened && r >= kScreenFrom ? scr.round(r, kScreenFrom, probed, kCost) : Screen{}; };
   const int vec = ld % 2 == 0 && (reinterpret_cast<uintptr_t>(D) & 15) == 0;
   auto init = [&](cudaStream_t stm) {
     if (P) path_init(P, n, ld, T, stm);
@@ -1107,8 +1112,8 @@ int run_fw_f64_interval(double *D, int n, int64_t ld, int32_t *P, cudaStream_t s
     PhaseScope sc(3, stm, screen ? 2 : 1);
     if (screen) {
       const Screen sr = screen_of(r);
-      launch_after(fw64_screen, k3x::PER_BLOCK * blocks, k3x::THREADS, sizeof(k3x::Smem), stm, overlap, D, ld, P, n, r,
-                   R, vec, pan[r & 1], sr, set);
+      launch_after(sr.cost ? fw64_screen<true> : fw64_screen<false>, k3x::PER_BLOCK * blocks, k3x::THREADS,
+                   sizeof(k3x::Smem), stm, overlap, D, ld, P, n, r, R, vec, pan[r & 1], sr, set);
       launch_after(fw64_listed, std::min(k3::PER_BLOCK * blocks, kListedCtas * kSms), k3::THREADS, sizeof(k3::Smem), stm, overlap,
                    D, ld, P, n, r, R, pan[r & 1], sr, set);
       return;

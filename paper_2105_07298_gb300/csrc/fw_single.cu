@@ -755,7 +755,7 @@ __global__ void __launch_bounds__(k3s::THREADS, TR == 32 ? 4 : 3)
 // output adds entries 4 (s + 8 u) + c (u, c < 4) of the row of A and the row of
 // B^T, and the minimum and its first k are taken over the lanes - the values and
 // the tie rule of the sequential loop.
-template <bool PATH>
+template <bool PATH, bool PROBE>
 __global__ void __launch_bounds__(k3x::THREADS, 4)
     fw_phase3_screen_f32(float *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r, int R, int vec_ok,
                          Panels pan, Screen scr, int set) {
@@ -764,7 +764,7 @@ __global__ void __launch_bounds__(k3x::THREADS, 4)
   Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
   const float INF = inf<float>();
   Tile tile;
-  const int count = screen_tile<kScreenParts>(sm, tile, n, r, R, scr, set, vec_ok != 0,
+  const int count = screen_tile<kScreenParts, PROBE>(sm, tile, n, r, R, scr, set, vec_ok != 0,
                                               [&](int i, int j, int left, auto whole_tile) {
     const float *p = D + (int64_t)i * ld + j;
     if constexpr (decltype(whole_tile)::value) return *reinterpret_cast<const float2 *>(p);
@@ -858,8 +858,13 @@ constexpr int kR32 = 21, kRNext32 = 40;
 // above 21 blocks a side, where the chain of the next round no longer sets the
 // pace.
 constexpr int kScreenMinR = 22, kScreenFrom = 8;
+// From a round at n = 8192: a tile takes the dense kernel 34 ns (with P 52) and the
+// screen 9, 64 settled outputs 2.4 (2.9).  Limits of 9 and 11 without P: 36.6 and 36.3
+// ms against 36.3 (n = 8192, U(0, 1)); of 14 and 16 with P 51.9 and 51.4 against 51.4.
+constexpr ScreenCost kCost{14, 10}, kCostP{18, 15};
+static_assert(kScreenFrom % kProbeRounds == 0, "the first screened round probes");
 static_assert(2 * (kScreenMinR - 1) * k2s::parts(4) >= kSms, "a screened round's K2 runs kScreenParts parts");
-static int g_smem_k1[2][64], g_smem_k2[2][2][64], g_smem_k3s[2][2][64], g_smem_k3x[2][64], g_smem_k3l[2][64];
+static int g_smem_k1[2][64], g_smem_k2[2][2][64], g_smem_k3s[2][2][64], g_smem_k3x[2][2][64], g_smem_k3l[2][64];
 
 int run_fw_f64_interval(double *D, int n, int64_t ld, int32_t *P, cudaStream_t s,
                         void (*path_init)(int32_t *, int64_t, int64_t, int64_t, cudaStream_t));
@@ -902,8 +907,10 @@ static int run_fw_f32(float *D, int64_t n64, int64_t ld, int32_t *P, void *strea
   const auto kernel64 = P ? fw_phase3_small_f32<true, 64> : fw_phase3_small_f32<false, 64>;
   if ((st = ensure_smem(kernel32, (int)sizeof(k3s::Smem<32>), g_smem_k3s[0][P != nullptr]))) return st;
   if ((st = ensure_smem(kernel64, (int)sizeof(k3s::Smem<64>), g_smem_k3s[1][P != nullptr]))) return st;
-  if ((st = ensure_smem(P ? fw_phase3_screen_f32<true> : fw_phase3_screen_f32<false>, (int)sizeof(k3x::Smem),
-                        g_smem_k3x[P != nullptr])) ||
+  const auto screen_kernel = P ? fw_phase3_screen_f32<true, false> : fw_phase3_screen_f32<false, false>;
+  const auto probe_kernel = P ? fw_phase3_screen_f32<true, true> : fw_phase3_screen_f32<false, true>;
+  if ((st = ensure_smem(screen_kernel, (int)sizeof(k3x::Smem), g_smem_k3x[0][P != nullptr])) ||
+      (st = ensure_smem(probe_kernel, (int)sizeof(k3x::Smem), g_smem_k3x[1][P != nullptr])) ||
       (st = ensure_smem(P ? fw_phase3_listed_f32<true> : fw_phase3_listed_f32<false>, (int)sizeof(k3s::Smem<64>),
                         g_smem_k3l[P != nullptr])))
     return st;
@@ -945,10 +952,6 @@ static int run_fw_f32(float *D, int64_t n64, int64_t ld, int32_t *P, void *strea
       }
     }
   }
-  // The round's screening data, or none where the round is not screened.
-  // It is left out where the last probe listed half of the tiles, without a path
-  // matrix a quarter (the dense kernel then costs less).
-  auto screen_of = [&](int r) { return screened && r >= kScreenFrom ? scr.round(r, P ? 2 : 4) : Screen{}; };
   const bool aligned = ld % 4 == 0;
   const int vec = (aligned && (reinterpret_cast<uintptr_t>(D) & 15) == 0 ? kVecD : 0) |
                   (aligned && (reinterpret_cast<uintptr_t>(P) & 15) == 0 ? kVecP : 0);
@@ -959,6 +962,11 @@ static int run_fw_f32(float *D, int64_t n64, int64_t ld, int32_t *P, void *strea
     return st;
   }
   const bool overlap = !capturing;
+  // The round's screening data, or none where the round is not screened.
+  const int probed = set_blocks(capturing ? kSetAll : kSetRest, R);
+  auto screen_of = [&](int r) {
+    return screened && r >= kScreenFrom ? scr.round(r, kScreenFrom, probed, P ? kCostP : kCost) : Screen{};
+  };
   // K1 of round 0 writes all of P's first block; the rest of P is set to -1
   // beside it.
   auto init = [&](cudaStream_t st) {
@@ -980,8 +988,8 @@ static int run_fw_f32(float *D, int64_t n64, int64_t ld, int32_t *P, void *strea
     PhaseScope ps(3, st, screen ? 2 : 1);
     if (screen) {
       const Screen sc = screen_of(r);
-      launch_after(P ? fw_phase3_screen_f32<true> : fw_phase3_screen_f32<false>, k3x::PER_BLOCK * blocks, k3x::THREADS,
-                   sizeof(k3x::Smem), st, overlap, D, ld, P, n, r, R, vec_ok, pan[r & 1], sc, set);
+      launch_after(sc.cost ? probe_kernel : screen_kernel, k3x::PER_BLOCK * blocks, k3x::THREADS, sizeof(k3x::Smem), st,
+                   overlap, D, ld, P, n, r, R, vec_ok, pan[r & 1], sc, set);
       launch_after(P ? fw_phase3_listed_f32<true> : fw_phase3_listed_f32<false>, std::min(4 * blocks, kListedCtas * kSms),
                    k3s::THREADS, sizeof(k3s::Smem<64>), st, overlap, D, ld, P, n, r, R, vec_ok, pan[r & 1], sc, set);
     } else if (R <= kR32 || (set == kSetNext && R <= kRNext32))

@@ -24,29 +24,49 @@ namespace apsp {
 //     entry and of minus its smallest;
 //   next, rest: the tiles the screen lists for the dense kernel, by block set, and
 //     listed_next, listed_rest: how many;
-//   probe: how many the last probing round listed of its rest (NULL in a probing
-//     round): if more than half, this round is relaxed densely without a screen.
+//   cost: in a probing round, what every kSample-th tile of its rest (or of all, where
+//     that is one launch) costs beside the screen itself, in units of 64 settled
+//     outputs, `dense` for a listed tile; NULL otherwise;
+//   probe: the last probing round's cost (in a probing round that of the one before,
+//     NULL in the first): above `enough` this round is relaxed densely without a
+//     screen, but for those tiles of a probing round.
 struct Screen {
   uint32_t *EA, *EB;
   float *base_a, *base_b;
   int *whole_a, *whole_b;
   unsigned *range;
   int *next, *rest, *listed_next, *listed_rest;
+  int *cost;
   const int *probe;
-  int enough;  // of the tiles, where to leave the screen out
-  // Whether the screen is left out (read after grid_dep_wait).
-  __device__ __forceinline__ bool skip() const { return probe && *probe > enough; }
+  int dense, enough;
+  // (Read after grid_dep_wait.)  Whether the last probe did not pay, and whether
+  // the screen is left out.
+  __device__ __forceinline__ bool failed() const { return probe && *probe > enough; }
+  __device__ __forceinline__ bool skip() const { return !cost && failed(); }
 };
 // Every eighth round probes.  Where many outputs improve in every round (weights
 // down to 0), screening them all costs more than it saves: n = 8192, U(0, 1),
-// without P 33 ms unscreened, 41.6 with every round screened, 36.9 with these
-// probes; with P 51.4 against 53.7 (every 4 / 16 rounds: 51.5 / 51.8).
-constexpr int kProbeRounds = 8;
+// without P 33.4 ms unscreened, 41.6 with every round screened, 36.3 with these
+// probes (37.3 with the number of listed tiles as their measure and no samples; every
+// 16 / 32 rounds 38.3 / 39.6 then).  Of what is left over 33.4, 0.9 ms are the screens
+// of rounds that go without (their CTAs start, read the probe's cost and end) and
+// the dense kernel's CTAs beside them; the chain's kernels find SMs later, too.  A
+// probe that follows one that failed takes every eighth tile alone (all of them: 0.15
+// ms a probe there, and 36.7); the cost is always added up over these (0.013 ms a
+// probe at n = 16384).
+constexpr int kProbeRounds = 8, kSample = 8;
 // CTAs of the dense kernel per SM of the chip: each takes its pieces in turn, and
 // ends early enough that the next round's chain finds room (three per SM, n =
 // 4096, U(0, 1): 9.2 ms, twelve 7.8, thirty-two 7.8; n = 16384: 124.3 / 124.5 /
 // 124.8).
 constexpr int kListedCtas = 12;
+
+// What a tile costs the solve's kernels, in units of 64 settled outputs: relaxed by
+// the dense kernel, and the same less the screen itself (a probing round must cost
+// less than that beside its screens).
+struct ScreenCost {
+  int dense, enough;
+};
 
 // The scratch of a solve with screened rounds: two sets by round parity (as the
 // panels), then the ranges and counts of all rounds and the two lists.
@@ -54,11 +74,11 @@ struct ScreenSets {
   size_t R, parts;
   Screen set[2]{};
   unsigned *ranges = nullptr;
-  int *listed = nullptr, *next = nullptr, *rest = nullptr;
+  int *listed = nullptr, *costs = nullptr, *next = nullptr, *rest = nullptr;
   ScreenSets(int R, int parts) : R((size_t)R), parts((size_t)parts) {}
   static constexpr size_t kT = mp32::T, kTiles = 4;  // tiles of a block
   size_t set_bytes() const { return (R * kT * kT + 2 * R * kT + 2 * R * parts) * 4; }  // EA, EB: half a word an entry
-  size_t list_bytes() const { return (4 * R + kTiles * 2 * R + kTiles * R * R) * 4; }
+  size_t list_bytes() const { return (5 * R + kTiles * 2 * R + kTiles * R * R) * 4; }
   void place_set(int q, void *at) {
     Screen &sc = set[q];
     sc.EA = static_cast<uint32_t *>(at);
@@ -71,19 +91,25 @@ struct ScreenSets {
   cudaError_t place_lists(void *at, cudaStream_t s) {
     ranges = static_cast<unsigned *>(at);
     listed = reinterpret_cast<int *>(ranges + 2 * R);
-    next = listed + 2 * R;
+    costs = listed + 2 * R;
+    next = costs + R;
     rest = next + kTiles * 2 * R;
-    return cudaMemsetAsync(ranges, 0, 4 * R * 4, s);
+    return cudaMemsetAsync(ranges, 0, 5 * R * 4, s);
   }
-  Screen round(int r, int part) const {
+  // `blocks`: of the set whose cost a probing round adds up.
+  // `first`: the first screened round (a probing one).
+  Screen round(int r, int first, int blocks, ScreenCost c) const {
     Screen sc = set[r & 1];
-    sc.enough = (int)(kTiles * (R - 2) * (R - 2)) / part;
+    const int at = r - r % kProbeRounds;
+    sc.dense = c.dense;
+    sc.enough = c.enough * ((int)kTiles * blocks / kSample);
     sc.range = ranges + 2 * r;
     sc.next = next;
     sc.rest = rest;
     sc.listed_next = listed + 2 * r;
     sc.listed_rest = sc.listed_next + 1;
-    sc.probe = r % kProbeRounds ? listed + 2 * (r - r % kProbeRounds) + 1 : nullptr;
+    sc.cost = r == at ? costs + at : nullptr;
+    sc.probe = r != at ? costs + at : at > first ? costs + at - kProbeRounds : nullptr;
     return sc;
   }
 };
@@ -201,12 +227,20 @@ struct Tile {
   int I, J, baseI, baseJ;  // block, first row and column of the H x H outputs
 };
 
+// Leaves this CTA's tile to the dense kernel.
+__device__ __forceinline__ void list_tile(const Screen &scr, int set) {
+  const bool nx = set == kSetNext;
+  (nx ? scr.next : scr.rest)[atomicAdd(nx ? scr.listed_next : scr.listed_rest, 1)] = blockIdx.x;
+}
+
 // One CTA screens its tile: returns how many of its outputs are in sm.list, for
 // the caller to settle; 0 if there are none or the tile was listed for the dense
 // kernel.  old(i, j, left, whole_tile): the values (FP64: upper bounds) of outputs
 // (i, j) and (i, j + 1), anything where `left` columns of the matrix end before
 // them; whole_tile: a std::true_type says that they lie inside it, aligned (pairs).
-template <int PARTS, typename Old>
+// PROBE: of a probing round (an instance of its own: with its tests in the one
+// kernel n = 16384 with P, integers, took 119.6 ms against 118.9).
+template <int PARTS, bool PROBE, typename Old>
 __device__ __forceinline__ int screen_tile(Smem &sm, Tile &t, int n, int r, int R, const Screen &scr, int set, bool pairs,
                                            Old old) {
   block_of(set, blockIdx.x / PER_BLOCK, r, R, t.I, t.J);
@@ -224,7 +258,10 @@ __device__ __forceinline__ int screen_tile(Smem &sm, Tile &t, int n, int r, int 
     sm.count = sm.next = 0;
   }
   grid_dep_wait();
-  if (scr.skip()) return 0;  // (uniform)
+  if (scr.failed() && (!PROBE || blockIdx.x % kSample)) {  // (uniform)
+    if (PROBE && tid == 0) list_tile(scr, set);
+    return 0;
+  }
   if (tid == 0) {
     fence_proxy_async_global();
     bulk_g2s(&sm.EA[0][0], scr.EA + (int64_t)I * (T * T / 2) + hI * (H * T / 2), H * T * 2, &sm.bar);
@@ -333,11 +370,10 @@ __device__ __forceinline__ int screen_tile(Smem &sm, Tile &t, int n, int r, int 
   __syncthreads();
   const int count = sm.count;
   if (count == 0) return 0;
-  if (count > kScreenDense) {  // left to the dense kernel
-    if (tid == 0) {
-      const bool nx = set == kSetNext;
-      (nx ? scr.next : scr.rest)[atomicAdd(nx ? scr.listed_next : scr.listed_rest, 1)] = blockIdx.x;
-    }
+  if (PROBE && tid == 0 && set != kSetNext && blockIdx.x % kSample == 0)
+    atomicAdd(scr.cost, count > kScreenDense ? scr.dense : (count + 63) / 64);
+  if (count > kScreenDense) {
+    if (tid == 0) list_tile(scr, set);
     return 0;
   }
   // The flagged outputs as a list, in any order.
