@@ -103,12 +103,6 @@ __device__ __forceinline__ void st_async16(uint32_t addr, unsigned long long a, 
                : "memory");
 }
 
-// Programmatic dependent launch: wait until the kernel this one was launched
-// behind has ended and its writes are visible (returns at once after an
-// ordinary launch); let the next such kernel start once every CTA has got here.
-__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(

@@ -353,7 +353,6 @@ __global__ void __cluster_dims__(k1::CTAS, 1, 1) __launch_bounds__(k1::THREADS, 
     fence_mbar_init();
     if (tid / WARPS != cta) mbar_expect_tx(&sm.bar[tid], QUAD_BYTES);
   }
-  grid_dep_wait();
   WarpLines &L = sm.wl[w % WARPS];
 #pragma unroll
   for (int rr = 0; rr < 4 && !helper; ++rr) {
@@ -474,7 +473,6 @@ __global__ void __cluster_dims__(k1::CTAS, 1, 1) __launch_bounds__(k1::THREADS, 
       cluster_arrive();
     }
   }
-  grid_dep_launch();
   cluster_wait();  // no CTA leaves while another may still write its buffers
   if (!ok) {       // D and P stay as they are
     report_wait_timeout();
@@ -571,9 +569,6 @@ __global__ void __launch_bounds__(32 * k2::WARPS, 2)
     mbar_init(&sm.bar, 1);
     fence_mbar_init();
     mbar_expect_tx(&sm.bar, sizeof(sm.M));
-  }
-  grid_dep_wait();
-  if (tid == 0) {
     fence_proxy_async_global();
     bulk_g2s(&sm.M[0][0], is_row ? ops.Alo : ops.Blo, sizeof(sm.M), &sm.bar);
   }
@@ -643,7 +638,6 @@ __global__ void __launch_bounds__(32 * k2::WARPS, 2)
   for (int c = 0; c < LINES; ++c)
 #pragma unroll
     for (int q = 0; q < 4; ++q) v[c][q] = L.d[c][p0 + q];
-  grid_dep_launch();
   // The phase-4 operands everywhere (padded), D and P where the line improved.
   const int64_t blk = other;
 #pragma unroll
@@ -747,9 +741,6 @@ __device__ __forceinline__ bool piece64(double *__restrict__ D, int64_t ld, int3
     mbar_init(&sm.bar, 1);
     fence_mbar_init();
     mbar_expect_tx(&sm.bar, (uint32_t)(GP * ng * (TR + TC) * 8));
-  }
-  grid_dep_wait();
-  if (tid == 0) {
     fence_proxy_async_global();
     bulk_g2s(&sm.B[0][0], pan.B + ((int64_t)J * 2 + hJ) * PAIRS * TC, (uint32_t)(GP * ng * TC * 8), &sm.bar);
   }
@@ -813,7 +804,6 @@ __device__ __forceinline__ bool piece64(double *__restrict__ D, int64_t ld, int3
         X[a][c] = fminf(X[a][c], m[a][c]);
       }
   }
-  grid_dep_launch();
   double old[4][CW];
   unsigned left = 0u;  // bit 4 c + a: output (a, c) may improve
 #pragma unroll
@@ -1002,7 +992,6 @@ __global__ void __launch_bounds__(k3::THREADS, 4)
     fw64_listed(double *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r, int R, Panels64 pan,
                 Screen scr, int set) {
   constexpr int PER = k3x::H / k3::TR;  // pieces a tile, one above the other
-  grid_dep_wait();
   const k3x::Listed listed(scr, set, R);
   const int pieces = PER * listed.count;
 #pragma unroll 1
@@ -1089,7 +1078,6 @@ int run_fw_f64_interval(double *D, int n, int64_t ld, int32_t *P, cudaStream_t s
     if (scratch) cudaFreeAsync(scratch, s);
     return st;
   }
-  const bool overlap = !capturing;
   const int probed = set_blocks(capturing ? kSetAll : kSetRest, R);
   auto screen_of = [&](int r) { return screened && r >= kScreenFrom ? scr.round(r, kScreenFrom, probed, kCost) : Screen{}; };
   const int vec = ld % 2 == 0 && (reinterpret_cast<uintptr_t>(D) & 15) == 0;
@@ -1098,13 +1086,13 @@ int run_fw_f64_interval(double *D, int n, int64_t ld, int32_t *P, cudaStream_t s
   };
   auto diag = [&](int r, cudaStream_t stm) {
     PhaseScope sc(1, stm);
-    launch_after(fw64_diag, k1::CTAS, k1::THREADS, sizeof(k1::Smem), stm, overlap, D, ld, P, n, r, vec,
-                 (int)(P && r == 0), ops, screen_of(r).range);
+    fw64_diag<<<k1::CTAS, k1::THREADS, sizeof(k1::Smem), stm>>>(D, ld, P, n, r, vec, (int)(P && r == 0), ops,
+                                                                screen_of(r).range);
   };
   auto panels = [&](int r, cudaStream_t stm) {
     PhaseScope sc(2, stm);
-    launch_after(fw64_lines, 2 * (R - 1) * k2::PARTS, 32 * k2::WARPS, sizeof(k2::Smem), stm, overlap, D, ld, P, n, r, R,
-                 vec, ops, pan[r & 1], screen_of(r));
+    fw64_lines<<<2 * (R - 1) * k2::PARTS, 32 * k2::WARPS, sizeof(k2::Smem), stm>>>(D, ld, P, n, r, R, vec, ops,
+                                                                                   pan[r & 1], screen_of(r));
   };
   auto phase4 = [&](int r, int set, int blocks, cudaStream_t stm) {
     if (blocks <= 0) return;
@@ -1112,14 +1100,13 @@ int run_fw_f64_interval(double *D, int n, int64_t ld, int32_t *P, cudaStream_t s
     PhaseScope sc(3, stm, screen ? 2 : 1);
     if (screen) {
       const Screen sr = screen_of(r);
-      launch_after(sr.cost ? fw64_screen<true> : fw64_screen<false>, k3x::PER_BLOCK * blocks, k3x::THREADS,
-                   sizeof(k3x::Smem), stm, overlap, D, ld, P, n, r, R, vec, pan[r & 1], sr, set);
-      launch_after(fw64_listed, std::min(k3::PER_BLOCK * blocks, kListedCtas * kSms), k3::THREADS, sizeof(k3::Smem), stm, overlap,
-                   D, ld, P, n, r, R, pan[r & 1], sr, set);
+      (sr.cost ? fw64_screen<true> : fw64_screen<false>)<<<k3x::PER_BLOCK * blocks, k3x::THREADS, sizeof(k3x::Smem), stm>>>(
+          D, ld, P, n, r, R, vec, pan[r & 1], sr, set);
+      fw64_listed<<<std::min(k3::PER_BLOCK * blocks, kListedCtas * kSms), k3::THREADS, sizeof(k3::Smem), stm>>>(
+          D, ld, P, n, r, R, pan[r & 1], sr, set);
       return;
     }
-    launch_after(pieces, k3::PER_BLOCK * blocks, k3::THREADS, sizeof(k3::Smem), stm, overlap, D, ld, P, n, r, R,
-                 pan[r & 1], set);
+    pieces<<<k3::PER_BLOCK * blocks, k3::THREADS, sizeof(k3::Smem), stm>>>(D, ld, P, n, r, R, pan[r & 1], set);
   };
   st = run_rounds(R, s, capturing, init, diag, panels, phase4);
   cudaError_t e = cudaGetLastError();

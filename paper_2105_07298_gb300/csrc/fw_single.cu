@@ -136,7 +136,6 @@ __global__ void __cluster_dims__(k1::CTAS, 1, 1) __launch_bounds__(32 * k1::WARP
     fence_mbar_init();
     if (tid / WARPS != cta) mbar_expect_tx(&sm.bar[tid], 4 * T * 4);
   }
-  grid_dep_wait();
   float d[4][4];
 #pragma unroll
   for (int rr = 0; rr < 4; ++rr) {
@@ -255,7 +254,6 @@ __global__ void __cluster_dims__(k1::CTAS, 1, 1) __launch_bounds__(32 * k1::WARP
         }
     }
   }
-  grid_dep_launch();
   __syncwarp();
   if (!ok) report_wait_timeout();  // D and P stay as they are
   if (ok) {
@@ -374,9 +372,6 @@ __global__ void __launch_bounds__(k2s::THREADS, 2)
     mbar_init(&sm.bar, 1);
     fence_mbar_init();
     mbar_expect_tx(&sm.bar, sizeof(sm.M));
-  }
-  grid_dep_wait();
-  if (tid == 0) {
     fence_proxy_async_global();
     bulk_g2s(&sm.M[0][0], is_row ? ops.A : ops.B, sizeof(sm.M), &sm.bar);
   }
@@ -470,7 +465,6 @@ __global__ void __launch_bounds__(k2s::THREADS, 2)
           }
     }
   }
-  grid_dep_launch();
   __syncwarp();  // lane 0's history writes
   if (!PATH) {  // which positions improved (prev still holds the input)
 #pragma unroll
@@ -612,9 +606,6 @@ __device__ __forceinline__ bool piece_f32(float *__restrict__ D, int64_t ld, int
     mbar_init(&sm.bar, 1);
     fence_mbar_init();
     mbar_expect_tx(&sm.bar, (uint32_t)(nkp * (TR + TC) * 8));
-  }
-  grid_dep_wait();
-  if (tid == 0) {
     fence_proxy_async_global();
     bulk_g2s(&sm.B[0][0], pan.Bpan + ((int64_t)J * 2 + hJ) * PAIRS * TC, (uint32_t)(nkp * TC * 8), &sm.bar);
   }
@@ -696,7 +687,6 @@ __device__ __forceinline__ bool piece_f32(float *__restrict__ D, int64_t ld, int
     for (int kp = 8 * g; kp < nkp; ++kp) step(kp);
     if (PATH) note(g);
   }
-  grid_dep_launch();
   if (!PATH) {
 #pragma unroll
     for (int a = 0; a < 4; ++a)
@@ -819,7 +809,6 @@ template <bool PATH>
 __global__ void __launch_bounds__(k3s::THREADS, 3)
     fw_phase3_listed_f32(float *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r, int R, int vec_ok,
                          Panels pan, Screen scr, int set) {
-  grid_dep_wait();
   const k3x::Listed listed(scr, set, R);
 #pragma unroll 1
   for (int t = blockIdx.x; t < listed.count; t += gridDim.x) {
@@ -961,7 +950,6 @@ static int run_fw_f32(float *D, int64_t n64, int64_t ld, int32_t *P, void *strea
     if (scratch) cudaFreeAsync(scratch, s);
     return st;
   }
-  const bool overlap = !capturing;
   // The round's screening data, or none where the round is not screened.
   const int probed = set_blocks(capturing ? kSetAll : kSetRest, R);
   auto screen_of = [&](int r) {
@@ -974,13 +962,13 @@ static int run_fw_f32(float *D, int64_t n64, int64_t ld, int32_t *P, void *strea
   };
   auto diag = [&](int r, cudaStream_t st) {
     PhaseScope ps(1, st);
-    launch_after(P ? fw_phase1_diag_f32<true> : fw_phase1_diag_f32<false>, k1::CTAS, 32 * k1::WARPS, sizeof(k1::Smem),
-                 st, overlap, D, ld, P, n, r, vec, (int)(P && r == 0), ops, screen_of(r).range);
+    (P ? fw_phase1_diag_f32<true> : fw_phase1_diag_f32<false>)<<<k1::CTAS, 32 * k1::WARPS, sizeof(k1::Smem), st>>>(
+        D, ld, P, n, r, vec, (int)(P && r == 0), ops, screen_of(r).range);
   };
   auto panels = [&](int r, cudaStream_t st) {
     PhaseScope ps(2, st);
-    launch_after(lines_kernel, 2 * (R - 1) * k2s::parts(lines), k2s::THREADS, lines_smem, st, overlap, D, ld, P, n, r, R,
-                 vec, ops, pan[r & 1], screen_of(r));
+    lines_kernel<<<2 * (R - 1) * k2s::parts(lines), k2s::THREADS, lines_smem, st>>>(D, ld, P, n, r, R, vec, ops,
+                                                                                    pan[r & 1], screen_of(r));
   };
   auto phase4 = [&](int r, int set, int blocks, cudaStream_t st) {
     if (blocks <= 0) return;
@@ -988,16 +976,17 @@ static int run_fw_f32(float *D, int64_t n64, int64_t ld, int32_t *P, void *strea
     PhaseScope ps(3, st, screen ? 2 : 1);
     if (screen) {
       const Screen sc = screen_of(r);
-      launch_after(sc.cost ? probe_kernel : screen_kernel, k3x::PER_BLOCK * blocks, k3x::THREADS, sizeof(k3x::Smem), st,
-                   overlap, D, ld, P, n, r, R, vec_ok, pan[r & 1], sc, set);
-      launch_after(P ? fw_phase3_listed_f32<true> : fw_phase3_listed_f32<false>, std::min(4 * blocks, kListedCtas * kSms),
-                   k3s::THREADS, sizeof(k3s::Smem<64>), st, overlap, D, ld, P, n, r, R, vec_ok, pan[r & 1], sc, set);
+      (sc.cost ? probe_kernel : screen_kernel)<<<k3x::PER_BLOCK * blocks, k3x::THREADS, sizeof(k3x::Smem), st>>>(
+          D, ld, P, n, r, R, vec_ok, pan[r & 1], sc, set);
+      (P ? fw_phase3_listed_f32<true> : fw_phase3_listed_f32<false>)<<<std::min(4 * blocks, kListedCtas * kSms),
+                                                                       k3s::THREADS, sizeof(k3s::Smem<64>), st>>>(
+          D, ld, P, n, r, R, vec_ok, pan[r & 1], sc, set);
     } else if (R <= kR32 || (set == kSetNext && R <= kRNext32))
-      launch_after(kernel32, k3s::per_block(32) * blocks, k3s::THREADS, sizeof(k3s::Smem<32>), st, overlap, D, ld, P, n,
-                   r, R, vec_ok, pan[r & 1], set);
+      kernel32<<<k3s::per_block(32) * blocks, k3s::THREADS, sizeof(k3s::Smem<32>), st>>>(D, ld, P, n, r, R, vec_ok,
+                                                                                        pan[r & 1], set);
     else
-      launch_after(kernel64, k3s::per_block(64) * blocks, k3s::THREADS, sizeof(k3s::Smem<64>), st, overlap, D, ld, P, n,
-                   r, R, vec_ok, pan[r & 1], set);
+      kernel64<<<k3s::per_block(64) * blocks, k3s::THREADS, sizeof(k3s::Smem<64>), st>>>(D, ld, P, n, r, R, vec_ok,
+                                                                                        pan[r & 1], set);
   };
   st = run_rounds(R, s, capturing, init, diag, panels, phase4);
   cudaError_t e = cudaGetLastError();

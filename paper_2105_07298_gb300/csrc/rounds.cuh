@@ -6,6 +6,11 @@
 // round r+1.  The rest of round r's phase 4 runs on the caller's stream beside
 // it, filling the SMs the chain leaves free; the two touch disjoint blocks and
 // write/read different operand sets (round parity).
+//
+// No launch is programmatic (griddepcontrol), although that hides about 2.5 us a
+// kernel of the chain: a dependent waits on the SMs for everything before it in its
+// hardware queue, other streams' kernels among it where they share the queue, and
+// these may find no SM with room beside the waiting CTAs.  Two solves at once hung so.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -44,25 +49,6 @@ __device__ __forceinline__ void block_of(int set, int tile, int r, int R, int &I
     I += (I >= r + 1);
     J += (J >= r + 1);
   }
-}
-
-// Launches `kernel` so that it may start before the previous kernel of the
-// stream has ended (it waits for it with grid_dep_wait before it reads or
-// writes anything that kernel does): the launch latency, about 3 us, is hidden.
-template <typename... A>
-inline void launch_after(void (*kernel)(A...), int grid, int threads, size_t smem, cudaStream_t s, bool overlap,
-                         A... args) {
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3((unsigned)threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr{};
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = overlap ? 1 : 0;
-  cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
 // All rounds of an R-block solve.  diag(r, stream) and panels(r, stream)

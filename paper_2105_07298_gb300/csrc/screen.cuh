@@ -39,8 +39,7 @@ struct Screen {
   int *cost;
   const int *probe;
   int dense, enough;
-  // (Read after grid_dep_wait.)  Whether the last probe did not pay, and whether
-  // the screen is left out.
+  // Whether the last probe did not pay, and whether the screen is left out.
   __device__ __forceinline__ bool failed() const { return probe && *probe > enough; }
   __device__ __forceinline__ bool skip() const { return !cost && failed(); }
 };
@@ -257,7 +256,6 @@ __device__ __forceinline__ int screen_tile(Smem &sm, Tile &t, int n, int r, int 
     mbar_expect_tx(&sm.bar, 2 * H * T * 2);
     sm.count = sm.next = 0;
   }
-  grid_dep_wait();
   if (scr.failed() && (!PROBE || blockIdx.x % kSample)) {  // (uniform)
     if (PROBE && tid == 0) list_tile(scr, set);
     return 0;

@@ -13,7 +13,7 @@ _SRC = r"""
 #include <stdlib.h>
 #include <string.h>
 int capturing, pool_error, pool_attr_error, alloc_error;
-int launches, copies, memsets, pools_created, pools_destroyed, pools_trimmed, pool_allocs, allocs, frees, live;
+int programmatic, launches, copies, memsets, pools_created, pools_destroyed, pools_trimmed, pool_allocs, allocs, frees, live;
 static void *vars[256]; static const char *names[256]; int num_vars;
 void *var_at(int i) { return vars[i]; }
 const char *var_name(int i) { return names[i]; }
@@ -44,7 +44,12 @@ int cudaEventCreateWithFlags(void **e) { *e = (void *)1; return 0; }
 int cudaEventCreate(void **e) { *e = (void *)1; return 0; }
 int cudaEventElapsedTime(float *ms) { *ms = 1.0f; return 0; }
 int __cudaLaunchKernel(void) { ++launches; return 0; }
-int cudaLaunchKernelExC(void) { ++launches; return 0; }
+struct config { unsigned grid[3], block[3]; size_t smem; void *stream; int *attrs; unsigned num; };
+int cudaLaunchKernelExC(const struct config *c) { /* attribute 6: may start before its predecessor ends */
+  for (unsigned i = 0; i < c->num; ++i) programmatic += c->attrs[18 * i] == 6;
+  ++launches;
+  return 0;
+}
 static int fatbin;
 void **__cudaRegisterFatBinary(void *f) { return (void **)&fatbin; }
 void __cudaRegisterVar(void **f, void *host, char *dev, const char *name) {

@@ -1,4 +1,6 @@
-"""Calls while a stream is being captured into a CUDA graph."""
+"""Calls while a stream is being captured into a CUDA graph, and from several streams at once."""
+from concurrent.futures import ThreadPoolExecutor
+
 import pytest
 import torch
 
@@ -57,4 +59,30 @@ def test_screened_solve_captured_in_cuda_graph(n, dtype, lo):
         g.replay()
         torch.cuda.synchronize()
         assert torch.equal(D, Dd) and torch.equal(P, Pd)
+    assert apsp.device_status() == apsp.APSP_OK
+
+
+@pytest.mark.parametrize("n,dtype", SCREENED)
+def test_solves_on_two_streams_at_once(n, dtype):
+    """Each with its own scratch from the one pool, again and again, from two host threads."""
+    cases = []
+    for lo in (1, 0):
+        W = _weights(n, lo, dtype)
+        Dd, Pd = W.clone(), torch.empty((n, n), dtype=torch.int32, device=DEV)
+        apsp.apsp_fw(Dd, Pd)
+        cases.append((W, Dd, Pd, torch.cuda.Stream()))
+    torch.cuda.synchronize()
+
+    def solve(case):
+        W, Dd, Pd, s = case
+        same = True
+        with torch.cuda.stream(s):
+            for _ in range(3):
+                D, P = W.clone(), torch.full_like(Pd, 77)
+                apsp.apsp_fw(D, P)
+                same = same and torch.equal(D, Dd) and torch.equal(P, Pd)
+        return same
+
+    with ThreadPoolExecutor(2) as pool:
+        assert list(pool.map(solve, cases)) == [True, True]
     assert apsp.device_status() == apsp.APSP_OK

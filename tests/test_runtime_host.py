@@ -75,3 +75,11 @@ def test_phase_timing_counts_every_launch(lib, fn, n):
     R = (n + 127) // 128
     assert launches[:3] == [1, R, R] and (launches[3] == 2 * R - 1) == (n == 1000)
     lib.apsp_profile_enable(0)
+
+
+@pytest.mark.parametrize("fn,n", [("apsp_fw_f32", 1000), ("apsp_fw_f32", 2900), ("apsp_fw_f64", 4000)])
+def test_no_launch_starts_before_its_predecessor_ends(lib, fn, n):
+    """Its waiting CTAs could hold the SMs that another stream's kernel, which they come to wait
+    for in a shared hardware queue, needs."""
+    assert getattr(lib, fn)(DEV, ctypes.c_int64(n), ctypes.c_int64(n), DEV, None) == apsp.APSP_OK
+    assert word(lib, "launches").value > 0 and word(lib, "programmatic").value == 0
