@@ -894,8 +894,8 @@ __global__ void __launch_bounds__(k3::THREADS, CTAS_PER_SM)
 // the row of Blo; the candidate of the least sum is added in FP64 first, then
 // those whose lower-bound sum its value does not exclude.
 // Bound: as the FP32 screen, the latency of the loads; at n = 4096 the next
-// round's chain (K1 90, K2 60, row and column r+1 50 us) sets the pace.  n =
-// 4096 / 6000 with P, integers: 9.8 / 27.2 -> 8.7 / 21.1 ms.
+// round's chain (K1 90, K2 75, row and column r+1 50 us) sets the pace.  n =
+// 4096 / 6000 with P, integers: 9.8 / 27.3 -> 8.6 / 20.2 ms.
 template <bool PROBE>
 __global__ void __launch_bounds__(k3x::THREADS, 4)
     fw64_screen(double *__restrict__ D, int64_t ld, int32_t *__restrict__ P, int n, int r, int R, int vec, Panels64 pan,
@@ -1008,14 +1008,14 @@ __global__ void __launch_bounds__(k3::THREADS, 4)
 static int g_smem_k1[64], g_smem_k2[64], g_smem_k3[2][64], g_smem_k3x[2][64], g_smem_k3l[64];
 
 // Four CTAs of 64 registers per SM where phase 4 has many waves (n = 4096 /
-// 8192: 10.6 / 68.9 ms against 11.1 / 72.2 with three, before the outputs were
-// settled a lane at a time), three of 80 up to 24 blocks a side, where K1 must
-// find room beside them (int32 n = 2048: 2.96 against 3.09 ms).
+// 8192: 8.56 / 41.0 ms against 8.63 / 41.2 with three), three of 80 up to 24 blocks
+// a side, where K1 must find room beside them (int32 n = 2048: 2.88 against 2.99 ms).
 constexpr int kFewBlocks = 24;
-// Phase 4 is screened from round 16 on from 32 blocks a side (n = 3328: 6.0 against
-// 5.8 ms unscreened, 3584: 6.9 / 7.0, 3840: 7.9 / 8.3, integers; where most
-// outputs improve, U(0, 1), screening costs 2-3 % at every size).  From round 8
-// on: 9.0 ms at n = 4096 against 8.7, since settling an output costs more here.
+// Phase 4 is screened from round 16 on from 32 blocks a side (n = 4096: 8.56 against
+// 9.83 ms unscreened, 6000: 20.2 / 27.3; n = 3328: 5.66 / 5.83, 3840: 7.65 / 8.31,
+// integers, but where most outputs improve screening costs up to 3 % at every
+// size).  From round 8 on 3 % more at n = 4096, since settling an output costs more
+// here.
 constexpr int kScreenMinR = 32, kScreenFrom = 16;
 // (As FP32 with P; limits of 12 to 14 within 1 % at n = 4096 and 6000.)
 constexpr ScreenCost kCost{18, 15};

@@ -4,8 +4,8 @@
 // weights the relaxation is carried out exactly by the FP64 path: every int32
 // value and every sum of fewer than 2^22 of them is an integer below 2^53, so
 // each FP64 addition is exact and the distances equal the integer ones.  The
-// FP64 path runs its main loop on FP32 lower bounds (about 1.2e13
-// relaxations/s on GB300).  A native integer main loop was measured instead
+// FP64 path works on FP32 lower bounds (2.7e13 relaxations/s at n = 32768,
+// integers up to 100).  A native integer main loop was measured instead
 // (apsp_measure_peak with dtype_bytes = -4): the DPX fused add-then-min
 // sustains fewer relaxations per clock than the FP32 instruction pair, so it
 // would not be faster.

@@ -836,12 +836,12 @@ std::vector<cudaEvent_t> g_prof_pool;
 constexpr int kMaxN = 1 << 18;
 
 constexpr int kT32 = mp32::T, kT64 = 128;
-// Phase 4 by blocks per side R (measured, whole solves, ms): 32-row pieces for
-// every launch while the whole of phase 4 is about a wave of CTAs or less (n =
-// 2049: 0.93 against 0.97 with 64 rows; with P 1.29 / 1.38), and for row and
-// column r+1 alone, which the next round waits for, a little longer; 64-row pieces
-// otherwise, until the rounds are screened.
-constexpr int kR32 = 21, kRNext32 = 40;
+// Phase 4 by blocks per side R (measured, whole solves, ms): 32-row pieces while
+// the whole of phase 4 is about a wave of CTAs or less (n = 2049: 0.96 against 1.02
+// with 64 rows, with P 1.35 / 1.41; n = 1024 with P 0.45 / 0.50); 64-row pieces
+// otherwise, until the rounds are screened (n = 4096: 32 rows for row and column
+// r+1 within 0.3 %).
+constexpr int kR32 = 21;
 // Phase 4 is screened from round 8 on (5 and 12 rounds: within 2 % at n = 4096
 // and 16384; about one output in r + 1 improves in round r of a random graph)
 // above 21 blocks a side, where the chain of the next round no longer sets the
@@ -981,7 +981,7 @@ static int run_fw_f32(float *D, int64_t n64, int64_t ld, int32_t *P, void *strea
       (P ? fw_phase3_listed_f32<true> : fw_phase3_listed_f32<false>)<<<std::min(4 * blocks, kListedCtas * kSms),
                                                                        k3s::THREADS, sizeof(k3s::Smem<64>), st>>>(
           D, ld, P, n, r, R, vec_ok, pan[r & 1], sc, set);
-    } else if (R <= kR32 || (set == kSetNext && R <= kRNext32))
+    } else if (R <= kR32)
       kernel32<<<k3s::per_block(32) * blocks, k3s::THREADS, sizeof(k3s::Smem<32>), st>>>(D, ld, P, n, r, R, vec_ok,
                                                                                         pan[r & 1], set);
     else

@@ -193,9 +193,9 @@ __device__ __forceinline__ void screen_range(unsigned *range, unsigned hi, unsig
 // in FP32 at n = 16384 (U[1, 100], p = 0.5): 0.64 ms from round 60 on, of which
 // the screen 0.58 (the dense kernel 2.0 ms); the product itself 0.22 ms on
 // mma.sync with 128 x 128 tiles, so its rate is not what counts.  FP32 solves
-// with P: n = 4096 6.2 -> 4.5 ms, 8192 40.9 -> 22.8, 16384 289 -> 120; real
-// weights and sparse graphs gain likewise (n = 8192: U[0.5, 2) 22.2 ms, 16 edges
-// a vertex 38.5 against 71).  FP64: n = 4096 9.8 -> 8.7 ms, 6000 27.2 -> 21.1.
+// with P: n = 4096 6.2 -> 4.6 ms, 8192 42.3 -> 22.5, 16384 289 -> 119; real
+// weights and sparse graphs gain likewise (n = 8192: U[0.5, 2) 41.8 -> 22.3 ms, 16
+// edges a vertex 46.5 -> 38.9).  FP64: n = 4096 9.8 -> 8.6 ms, 6000 27.3 -> 20.2.
 // --------------------------------------------------------------------------
 namespace k3x {
 constexpr int T = mp32::T, THREADS = 256;

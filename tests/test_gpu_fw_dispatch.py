@@ -21,8 +21,7 @@ def _expect(n, p, seed, dtype=np.float32):
 
 # One quad of the diagonal block; a block less one; two blocks, the last one
 # vertex wide; the last size with two lines a warp in the panels and the first
-# with four; the first past the 32-row pieces; the first that leaves them for row
-# and column r+1 too.
+# with four; the first past the 32-row pieces; one well past it.
 @pytest.mark.parametrize("n", [1, 3, 5, 127, 129, 258, 2305, 2433, 2689, 5121])
 def test_real_weights_bitwise_at_dispatch_limits(n):
     W, Db, Pb = _expect(n, 0.3 if n < 300 else 0.05, 900 + n)
