@@ -3,7 +3,8 @@
 //
 // A copy of `bytes` (multiple of 16, both addresses 16-byte aligned) from
 // global to shared memory completes on an mbarrier as transaction bytes.
-// Every wait is bounded: after kWaitLimit polls it reports failure, and the
+// Every wait is bounded: after kWaitLimit polls (kPollLimit of the kind that
+// suspends the thread, about 3 us each) it reports failure, and the
 // caller records APSP_ETIMEOUT in the translation unit's error word
 // (report_wait_timeout) and leaves instead of spinning forever.
 #pragma once
@@ -14,7 +15,7 @@
 
 namespace apsp {
 
-constexpr uint32_t kWaitLimit = 1u << 22;
+constexpr uint32_t kWaitLimit = 1u << 22, kPollLimit = 1u << 18;  // both under a second
 
 // Error word the kernels of a translation unit set when a bounded wait runs
 // out (read back by apsp_device_status).
@@ -133,7 +134,7 @@ __device__ __forceinline__ bool mbar_spin(uint64_t *bar, uint32_t parity, uint32
 }
 
 // Waits for phase `parity` of `bar` to complete; false if `limit` polls ran out.
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, uint32_t limit = kWaitLimit) {
+__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, uint32_t limit = kPollLimit) {
   for (uint32_t it = 0; it < limit; ++it)
     if (mbar_try_wait(bar, parity)) return true;
   return false;

@@ -41,3 +41,10 @@ def test_ctas_whose_wait_ran_out_wait_for_their_copies():
             end = src[m.end():src.index("\n}", m.end())]
             assert "drain_ring(sm.bar, nquad, WARPS, cta)" in end, file
         assert "give_up(&sm.bar" in src, file
+
+
+def test_default_wait_is_the_short_one():
+    """A poll that suspends the thread takes about 3 us: 2^18 of them, not 2^22 (13 s)."""
+    src = open(os.path.join(CSRC, "bulk.cuh")).read()
+    assert re.search(r"kPollLimit = 1u << 18;", src)
+    assert re.search(r"bool mbar_wait\(uint64_t \*bar, uint32_t parity, uint32_t limit = kPollLimit\)", src)

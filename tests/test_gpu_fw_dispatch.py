@@ -187,3 +187,16 @@ def test_screened_rounds_f64_bitwise(kind):
     apsp.apsp_fw(D)
     np.testing.assert_array_equal(D.cpu().numpy(), Db)
     assert apsp.device_status() == apsp.APSP_OK
+
+
+def test_bounded_wait_ends_within_seconds():
+    """As many polls as the kernels' waits for their copies make (csrc/bulk.cuh): a wait that runs
+    out must not hold the GPU for long."""
+    apsp.wait_timeout_selftest(1 << 10)
+    assert apsp.device_status() == apsp.APSP_ETIMEOUT
+    t0, t1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+    t0.record()
+    apsp.wait_timeout_selftest(1 << 18)
+    t1.record()
+    assert apsp.device_status() == apsp.APSP_ETIMEOUT
+    assert t0.elapsed_time(t1) < 3000.0
